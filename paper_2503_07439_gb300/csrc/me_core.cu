@@ -761,9 +761,7 @@ int me_init(const char* process, const me_params* params, me_handle** out) {
   }
   KParams& kp = h->kp;
   std::memset(&kp, 0, sizeof(kp));
-  kp.cp.gs = std::sqrt(4.0 * M_PI * params->alpha_s);
-  kp.cp.ee = std::sqrt(4.0 * M_PI * params->alpha);
-  kp.cp.mt = params->mt;
+  kp.cp = Couplings(std::sqrt(4.0 * M_PI * params->alpha_s), std::sqrt(4.0 * M_PI * params->alpha), params->mt);
   kp.avg_inv = 1.0 / pd->avg;
   kp.born_avg_inv = pd->born_pid >= 0 ? 1.0 / kProcs[pd->born_pid].avg : 0.0;
   kp.nlo_factor = 1.0;
@@ -1165,9 +1163,7 @@ int me_internal_kparams(const char* process, const me_params* params, me::KParam
     if (std::strcmp(d.name, process) == 0) pd = &d;
   if (!pd) return fail(ME_ERR_PROCESS, std::string("unknown process ") + process);
   std::memset(kp, 0, sizeof(*kp));
-  kp->cp.gs = std::sqrt(4.0 * M_PI * params->alpha_s);
-  kp->cp.ee = std::sqrt(4.0 * M_PI * params->alpha);
-  kp->cp.mt = params->mt;
+  kp->cp = Couplings(std::sqrt(4.0 * M_PI * params->alpha_s), std::sqrt(4.0 * M_PI * params->alpha), params->mt);
   kp->avg_inv = 1.0 / pd->avg;
   kp->born_avg_inv = pd->born_pid >= 0 ? 1.0 / kProcs[pd->born_pid].avg : 0.0;
   kp->nlo_factor = 1.0;

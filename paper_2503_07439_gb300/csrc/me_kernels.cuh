@@ -86,30 +86,15 @@ template <int PID, typename T>
 __device__ __forceinline__ T colour_sum(const ColourTables* tab, const cx<T>* J) {
   constexpr int NF = Proc<PID>::NFLOW;
   T s = T(0);
-  if constexpr (NF <= 6) {
-    // triangular form: NF (NF + 1) + 2 NF multiply-adds instead of 2 NF^2 + 2 NF
-    const T* __restrict__ Um = utab<T>(tab, PID);
-#pragma unroll
-    for (int a = 0; a < NF; ++a) {
-      const T d = Um[a * NF + a];
-      T zr = d * J[a].re, zi = d * J[a].im;
-#pragma unroll
-      for (int b = a + 1; b < NF; ++b) {
-        const T c = Um[a * NF + b];
-        zr += c * J[b].re;
-        zi += c * J[b].im;
-      }
-      s += J[a].re * zr + J[a].im * zi;
-    }
-    return s;
-  }
-  const T* __restrict__ Cm = ctab<T>(tab, PID);
-#pragma unroll 4
+  // triangular form: NF (NF + 1) + 2 NF multiply-adds instead of 2 NF^2 + 2 NF
+  const T* __restrict__ Um = utab<T>(tab, PID);
+#pragma unroll(NF <= 6 ? NF : 1)
   for (int a = 0; a < NF; ++a) {
-    T zr = T(0), zi = T(0);
-#pragma unroll 8
-    for (int b = 0; b < NF; ++b) {
-      const T c = Cm[a * NF + b];
+    const T d = Um[a * NF + a];
+    T zr = d * J[a].re, zi = d * J[a].im;
+#pragma unroll(NF <= 6 ? NF : 4)
+    for (int b = a + 1; b < NF; ++b) {
+      const T c = Um[a * NF + b];
       zr += c * J[b].re;
       zi += c * J[b].im;
     }
@@ -334,7 +319,6 @@ __global__ void __launch_bounds__(TC4_THREADS, 2) k_tree_tc4(const double* __res
   const float g = (float)kp.cp.gs, mt = (float)kp.cp.mt;
   const r4<float>* q = K.q;
   const r4<float> kt = K.pl[2];
-  const c4<float> v[2] = {spinor_v_of(K.wtb, -1), spinor_v_of(K.wtb, 1)};
   constexpr int LEG[4] = {0, 1, 4, 5};
   float acc = 0.0f;
   for (int b = 0; b < n_live_blocks<PID>(); ++b) {
@@ -383,9 +367,8 @@ __global__ void __launch_bounds__(TC4_THREADS, 2) k_tree_tc4(const double* __res
     // 5. quark line for the orderings starting with gluon w = lane
     const int w = lane;
     for (int ht = 0; ht < 2; ++ht) {
-      const c4<float> ub = dbar(spinor_u_of(K.wt, ht ? 1 : -1));
       const int row0 = (wl & ~3) + 2 * ht;  // rows of (this event, ht, hv = 0 / 1)
-      const c4<float> U1 = row_prop(row_slash(ub, ld_sl4(cur, w)), scaled_prop(kt + q[w], mt, -g * K.iq[1 << w]));
+      const c4<float> U1 = row_prop(ubar_slash(K.wt, ht, ld_sl4(cur, w)), scaled_prop(kt + q[w], mt, -g * K.iq[1 << w]));
       // every lane runs the same 3 x 2 iterations (no lane idles on a skipped index):
       // x is the kx-th gluon other than w, y the ky-th other than w and x, in increasing
       // order, so f counts the orderings w x y z as the ordering tables do
@@ -393,7 +376,7 @@ __global__ void __launch_bounds__(TC4_THREADS, 2) k_tree_tc4(const double* __res
 #pragma unroll
       for (int kx = 0; kx < 3; ++kx) {
         const int x = kx + (kx >= w ? 1 : 0);
-        c4<float> r2 = row_slash(ub, ld_sj2(cur, w, x));
+        c4<float> r2 = ubar_slash(K.wt, ht, ld_sj2(cur, w, x));
         row_slash_acc(r2, U1, ld_sl4(cur, x));
         const c4<float> U2 = row_prop(r2, scaled_prop(kt + q[w] + q[x], mt, -g * K.iq[(1 << w) | (1 << x)]));
         const int lo = w < x ? w : x, hi = w < x ? x : w;
@@ -403,20 +386,20 @@ __global__ void __launch_bounds__(TC4_THREADS, 2) k_tree_tc4(const double* __res
           if (y >= lo) ++y;
           if (y >= hi) ++y;
           const int z = 6 - w - x - y;
-          c4<float> r3 = row_slash(ub, ld_sl4(cur, triple_slot(w, x, y)));
+          c4<float> r3 = ubar_slash(K.wt, ht, ld_sl4(cur, triple_slot(w, x, y)));
           row_slash_acc(r3, U1, ld_sj2(cur, x, y));
           row_slash_acc(r3, U2, ld_sl4(cur, y));
           const c4<float> U3 =
               row_prop(r3, scaled_prop(kt + q[w] + q[x] + q[y], mt, -g * K.iq[(1 << w) | (1 << x) | (1 << y)]));
           const int s4 = kJ4OfOrdering[f];
-          c4<float> R = row_slash(ub, ld_sl4(cur, 22 + (s4 > 0 ? s4 : -s4) - 1));
+          c4<float> R = ubar_slash(K.wt, ht, ld_sl4(cur, 22 + (s4 > 0 ? s4 : -s4) - 1));
           if (s4 < 0) R = cneg(R);
           row_slash_acc(R, U1, ld_sl4(cur, triple_slot(x, y, z)));
           row_slash_acc(R, U2, ld_sj2(cur, y, z));
           row_slash_acc(R, U3, ld_sl4(cur, z));
 #pragma unroll
           for (int hv = 0; hv < 2; ++hv) {
-            const cx<float> a = times_i(spdot(R, v[hv])) * g;
+            const cx<float> a = dot_v(R, K.wtb, hv);
             are[(row0 + hv) * TC4_ROW + f] = a.re;
             aim[(row0 + hv) * TC4_ROW + f] = a.im;
           }

@@ -43,11 +43,23 @@ template <> struct Proc<P_GG_TTGG> { static constexpr int NEXT = 6, NHEL = 64, N
 template <> struct Proc<P_UU_TT> { static constexpr int NEXT = 4, NHEL = 16, NFLOW = 2; };
 template <> struct Proc<P_UU_TTG> { static constexpr int NEXT = 5, NHEL = 32, NFLOW = 4; };
 
+// The couplings and the top mass; the float32 copies spare the float32 kernels a float64
+// conversion (as dear as a float64 multiply-add) per thread and use.
 struct Couplings {
   double gs;   // strong coupling g_s
   double ee;   // electromagnetic coupling e
   double mt;   // top mass
+  float gsf, eef, mtf;
+  Couplings() = default;
+  __host__ __device__ Couplings(double g, double e, double m)
+      : gs(g), ee(e), mt(m), gsf((float)g), eef((float)e), mtf((float)m) {}
 };
+template <typename T> ME_HD T gs_of(const Couplings& c) { return (T)c.gs; }
+template <> ME_HD float gs_of<float>(const Couplings& c) { return c.gsf; }
+template <typename T> ME_HD T ee_of(const Couplings& c) { return (T)c.ee; }
+template <> ME_HD float ee_of<float>(const Couplings& c) { return c.eef; }
+template <typename T> ME_HD T mt_of(const Couplings& c) { return (T)c.mt; }
+template <> ME_HD float mt_of<float>(const Couplings& c) { return c.mtf; }
 
 __host__ __device__ constexpr int factorial(int n) { return n <= 1 ? 1 : n * factorial(n - 1); }
 
@@ -77,7 +89,7 @@ struct KinTT {
   T ig[1 << NG];
   T iq[1 << NG];
   wf_v<T> wg[NG];       // polarisation ingredients of the gluons (legs 0, 1, 4, 5)
-  wf_f<T> wt, wtb;      // spinor ingredients of the top and the antitop
+  wf_q<T> wt, wtb;      // spinor ingredients of the top and, times g_s, of the antitop
 };
 
 template <typename T, int NG>
@@ -92,8 +104,8 @@ ME_HD KinTT<T, NG> prep_tt(const r4<double>* p, const Couplings& cp) {
     K.q[i] = l < 2 ? -K.pl[l] : K.pl[l];
     K.wg[i] = wf_vector(K.pl[l]);
   }
-  K.wt = wf_fermion(K.pl[2], (T)cp.mt);
-  K.wtb = wf_fermion(K.pl[3], (T)cp.mt);
+  K.wt = wf_quark(K.pl[2], mt_of<T>(cp));
+  K.wtb = scaled(wf_quark(K.pl[3], mt_of<T>(cp)), gs_of<T>(cp));
   // The gluons are massless and the top on shell, so every subset invariant is a sum of
   // pairwise products (float64):  Q_S^2 = 2 sum_{i<j in S} q_i.q_j,
   // (p_t + Q_S)^2 - m^2 = 2 sum_{i in S} p_t.q_i + Q_S^2.
@@ -124,8 +136,8 @@ ME_HD KinTT<T, NG> prep_tt(const r4<double>* p, const Couplings& cp) {
 template <typename T, int NG>
 ME_HD void amp_ttng(const KinTT<T, NG>& K, int hel, const Couplings& cp, cx<T>* A) {
   constexpr int NF = factorial(NG);
-  const T g = (T)cp.gs;
-  const T mt = (T)cp.mt;
+  const T g = gs_of<T>(cp);
+  const T mt = mt_of<T>(cp);
   c4<T> eps[NG];
 #pragma unroll
   for (int i = 0; i < NG; ++i) {
@@ -197,7 +209,7 @@ ME_HD void amp_ttng(const KinTT<T, NG>& K, int hel, const Couplings& cp, cx<T>* 
 // lexicographically as in amp_ttng, so the colour basis is the same.
 template <typename T>
 ME_HD void amp_tt2_fast(const KinTT<T, 2>& K, int hel, const Couplings& cp, const c4<T>* ov, int ov_leg, cx<T>* A) {
-  const T g = (T)cp.gs, mt = (T)cp.mt;
+  const T g = gs_of<T>(cp), mt = mt_of<T>(cp);
   const r4<T> k0 = K.q[0], k1 = K.q[1], kt = K.pl[2];
   const c4<T> e0 = (ov != nullptr && ov_leg == 0) ? *ov : polvec(K.pl[0], hel_of(hel, 0), false);
   const c4<T> e1 = (ov != nullptr && ov_leg == 1) ? *ov : polvec(K.pl[1], hel_of(hel, 1), false);
@@ -217,7 +229,7 @@ ME_HD void amp_tt2_fast(const KinTT<T, 2>& K, int hel, const Couplings& cp, cons
 
 template <typename T>
 ME_HD void amp_tt3_fast(const KinTT<T, 3>& K, int hel, const Couplings& cp, cx<T>* A) {
-  const T g = (T)cp.gs, mt = (T)cp.mt;
+  const T g = gs_of<T>(cp), mt = mt_of<T>(cp);
   const r4<T> k0 = K.q[0], k1 = K.q[1], k2 = K.q[2], kt = K.pl[2];
   const c4<T> e0 = polvec(K.pl[0], hel_of(hel, 0), false);
   const c4<T> e1 = polvec(K.pl[1], hel_of(hel, 1), false);
@@ -329,83 +341,100 @@ ME_HD void amp_tt3_fast(const KinTT<T, 3>& K, int hel, const Couplings& cp, cx<T
 // only, so a block builds the gluon currents once, the rows once per top helicity, and
 // closes each row with both antitop spinors: the partial amplitudes of the four
 // single-helicity evaluations, with the shared pieces computed once.
-// consume(r, A) receives the partial amplitudes of helicity hb | (r << 2).
+// consume(r, A) receives the partial amplitudes of heavy spins r.
+//
+// The blocks are bound by the float64 pipe where they run in float64 (2 lane operations per
+// SM and cycle) and by instruction issue in float32, so what counts is the number of
+// operations.  Five-real polarisations (pol), light-cone quark spins (wf_q), brackets of
+// conserved currents without their vanishing terms, products e.J computed once and each
+// gluon-pair bracket used by both currents it enters take a g g -> t tbar g block from 7349
+// to 4737 operations and a g g -> t tbar g g block from 66751 to 49460.  GB300: 2^20
+// subtracted g g -> t tbar g points 5.55 -> 4.23 ms, 30011 in float64 1.385 -> 1.007 ms,
+// 8191 g g -> t tbar g g trees in float64 3.96 -> 3.04 ms.
 
-// g g -> t tbar.  A(01) = ig ubar [J01 + U0 e1] v,  A(10) = ig ubar [-J01 + U1 e0] v.
+// g g -> t tbar.  A(01) = ubar [J01 + U0 e1] v,  A(10) = ubar [-J01 + U1 e0] v (no factor i g).
 template <typename T, class F>
 ME_HD void amp_tt2_block(const KinTT<T, 2>& K, int hb, const Couplings& cp, const c4<T>* ov, int ov_leg,
                          F&& consume) {
-  const T g = (T)cp.gs, mt = (T)cp.mt;
+  const T g = gs_of<T>(cp), mt = mt_of<T>(cp);
   const r4<T> k0 = K.q[0], k1 = K.q[1], kt = K.pl[2];
   const c4<T> e0 = (ov != nullptr && ov_leg == 0) ? *ov : polvec_of(K.wg[0], hel_of(hb, 0), false);
   const c4<T> e1 = (ov != nullptr && ov_leg == 1) ? *ov : polvec_of(K.wg[1], hel_of(hb, 1), false);
   const c4<T> J01 = vvv(e0, e1, -k0, -k1, -g * K.ig[3]);
   const sl4<T> s0 = slashed(e0), s1 = slashed(e1), s01 = slashed(J01);
   const prop4<T> P0 = scaled_prop(kt + k0, mt, -g * K.iq[1]), P1 = scaled_prop(kt + k1, mt, -g * K.iq[2]);
-  const c4<T> v[2] = {spinor_v_of(K.wtb, -1), spinor_v_of(K.wtb, 1)};
 #pragma unroll
   for (int ht = 0; ht < 2; ++ht) {
-    const c4<T> ub = dbar(spinor_u_of(K.wt, ht ? 1 : -1));
-    const c4<T> S = row_slash(ub, s01);
-    const c4<T> U0 = row_prop(row_slash(ub, s0), P0);
-    const c4<T> U1 = row_prop(row_slash(ub, s1), P1);
+    const c4<T> S = ubar_slash(K.wt, ht, s01);
+    const c4<T> U0 = row_prop(ubar_slash(K.wt, ht, s0), P0);
+    const c4<T> U1 = row_prop(ubar_slash(K.wt, ht, s1), P1);
     c4<T> R0 = S;
     row_slash_acc(R0, U0, s1);
     c4<T> R1 = cneg(S);
     row_slash_acc(R1, U1, s0);
 #pragma unroll
     for (int hv = 0; hv < 2; ++hv) {
-      cx<T> A[2] = {times_i(spdot(R0, v[hv])) * g, times_i(spdot(R1, v[hv])) * g};
+      cx<T> A[2] = {dot_v(R0, K.wtb, hv), dot_v(R1, K.wtb, hv)};
       consume(ht | (hv << 1), A);
     }
   }
 }
 
 // g g -> t tbar g: the three-gluon currents F(012) = F(210), F(021) = F(120),
-// F(102) = F(201) and the pair currents J(xy) are built once per block; per top
-// helicity the row R_s of ordering s collects ubar F(s), U(x) J(yz) and W(xy) e_z.
+// F(102) = F(201) and the pair currents J(xy) are built once per block; per top spin the
+// row R_s of ordering s collects ubar F(s), U(x) J(yz) and W(xy) e_z.
+// consume(r, A) receives the partial amplitudes of heavy spins r without the factor i g.
 template <typename T, class F>
 ME_HD void amp_tt3_block(const KinTT<T, 3>& K, int hb, const Couplings& cp, F&& consume) {
-  const T g = (T)cp.gs, mt = (T)cp.mt;
+  const T g = gs_of<T>(cp), mt = mt_of<T>(cp);
   const r4<T> k0 = K.q[0], k1 = K.q[1], k2 = K.q[2], kt = K.pl[2];
-  const c4<T> e0 = polvec_of(K.wg[0], hel_of(hb, 0), false);
-  const c4<T> e1 = polvec_of(K.wg[1], hel_of(hb, 1), false);
-  const c4<T> e2 = polvec_of(K.wg[2], hel_of(hb, 4), true);
-  const c4<T> J01 = vvv(e0, e1, -k0, -k1, -g * K.ig[3]);
-  const c4<T> J02 = vvv(e0, e2, -k0, -k2, -g * K.ig[5]);
-  const c4<T> J12 = vvv(e1, e2, -k1, -k2, -g * K.ig[6]);
+  const pol<T> e0 = pol_of(K.wg[0], hel_of(hb, 0), false);
+  const pol<T> e1 = pol_of(K.wg[1], hel_of(hb, 1), false);
+  const pol<T> e2 = pol_of(K.wg[2], hel_of(hb, 4), true);
+  const r4<T> k01 = k0 + k1, k02 = k0 + k2, k12 = k1 + k2;
+  cx<T> e01, e02, e12;
+  const c4<T> J01 = bracket(e0, k0, e1, k1, -g * K.ig[3], e01);
+  const c4<T> J02 = bracket(e0, k0, e2, k2, -g * K.ig[5], e02);
+  const c4<T> J12 = bracket(e1, k1, e2, k2, -g * K.ig[6], e12);
   const T c3 = -g * K.ig[7], c4g = g * g * K.ig[7];
-  c4<T> F0 = vvv(e0, J12, -k0, -(k1 + k2), c3);
-  vvv_acc(F0, J01, e2, -(k0 + k1), -k2, c3);
-  caxpy(F0, c4g, vvvv_ordered(e0, e1, e2));
-  c4<T> F1 = vvv(J12, e0, -(k1 + k2), -k0, c3);  // = vvv(e0, -J12, ...) by antisymmetry
-  vvv_acc(F1, J02, e1, -(k0 + k2), -k1, c3);
-  caxpy(F1, c4g, vvvv_ordered(e0, e2, e1));
-  c4<T> F2 = vvv(e1, J02, -k1, -(k0 + k2), c3);
-  vvv_acc(F2, e2, J01, -k2, -(k0 + k1), c3);  // = vvv(-J01, e2, ...)
-  caxpy(F2, c4g, vvvv_ordered(e1, e0, e2));
-  const sl4<T> se0 = slashed(e0), se1 = slashed(e1), se2 = slashed(e2);
+  e01 = c4g * e01;
+  e02 = c4g * e02;
+  e12 = c4g * e12;
+  // each bracket of a gluon with a pair current enters two of the three currents:
+  // J(a|bc) = -J(a|cb)
+  c4<T> F0 = czero<T>(), F2 = czero<T>(), B = czero<T>();
+  bracket_acc(F0, e0, k0, J12, k12, c3, cdot(e0, J12));
+  c4<T> F1 = cneg(F0);
+  bracket_acc(B, e2, k2, J01, k01, c3, cdot(e2, J01));  // J(2|01)
+  csub(F0, B);
+  cadd(F2, B);
+  B = czero<T>();
+  bracket_acc(B, e1, k1, J02, k02, c3, cdot(e1, J02));  // J(1|02)
+  csub(F1, B);
+  cadd(F2, B);
+  quartic_acc(F0, e0, e1, e2, e02, e01, e12);
+  quartic_acc(F1, e0, e2, e1, e01, e02, e12);
+  quartic_acc(F2, e1, e0, e2, e12, e01, e02);
+  const spol<T> se0 = slashed(e0), se1 = slashed(e1), se2 = slashed(e2);
   const sl4<T> sJ01 = slashed(J01), sJ02 = slashed(J02), sJ12 = slashed(J12);
   const sl4<T> sF0 = slashed(F0), sF1 = slashed(F1), sF2 = slashed(F2);
-  const c4<T> v[2] = {spinor_v_of(K.wtb, -1), spinor_v_of(K.wtb, 1)};
   const r4<T> Q0 = kt + k0, Q1 = kt + k1, Q2 = kt + k2;
   const prop4<T> P0 = scaled_prop(Q0, mt, -g * K.iq[1]), P1 = scaled_prop(Q1, mt, -g * K.iq[2]),
                  P2 = scaled_prop(Q2, mt, -g * K.iq[4]);
-  const prop4<T> P01 = scaled_prop(Q0 + k1, mt, -g * K.iq[3]), P02 = scaled_prop(Q0 + k2, mt, -g * K.iq[5]),
-                 P12 = scaled_prop(Q1 + k2, mt, -g * K.iq[6]);
+  const prop4<T> P01 = scaled_prop(kt + k01, mt, -g * K.iq[3]), P02 = scaled_prop(kt + k02, mt, -g * K.iq[5]),
+                 P12 = scaled_prop(kt + k12, mt, -g * K.iq[6]);
 #pragma unroll
   for (int ht = 0; ht < 2; ++ht) {
-    const c4<T> ub = dbar(spinor_u_of(K.wt, ht ? 1 : -1));
     c4<T> R[6];
-    R[0] = row_slash(ub, sF0);  // orderings 012, 021, 102, 120, 201, 210
-    R[1] = row_slash(ub, sF1);
-    R[2] = row_slash(ub, sF2);
+    R[0] = ubar_slash(K.wt, ht, sF0);  // orderings 012, 021, 102, 120, 201, 210
+    R[1] = ubar_slash(K.wt, ht, sF1);
+    R[2] = ubar_slash(K.wt, ht, sF2);
     R[3] = R[1];
     R[4] = R[2];
     R[5] = R[0];
-    const c4<T> S01 = row_slash(ub, sJ01), S02 = row_slash(ub, sJ02), S12 = row_slash(ub, sJ12);
+    const c4<T> S01 = ubar_slash(K.wt, ht, sJ01), S02 = ubar_slash(K.wt, ht, sJ02), S12 = ubar_slash(K.wt, ht, sJ12);
     {  // first gluon 0: orderings 012, 021
-      const c4<T> U = row_prop(row_slash(ub, se0), P0);
+      const c4<T> U = row_prop(ubar_slash(K.wt, ht, se0), P0);
       const c4<T> t = row_slash(U, sJ12);
       cadd(R[0], t);
       csub(R[1], t);
@@ -417,7 +446,7 @@ ME_HD void amp_tt3_block(const KinTT<T, 3>& K, int hb, const Couplings& cp, F&& 
       row_slash_acc(R[1], row_prop(r, P02), se1);
     }
     {  // first gluon 1: orderings 102, 120
-      const c4<T> U = row_prop(row_slash(ub, se1), P1);
+      const c4<T> U = row_prop(ubar_slash(K.wt, ht, se1), P1);
       const c4<T> t = row_slash(U, sJ02);
       cadd(R[2], t);
       csub(R[3], t);
@@ -429,7 +458,7 @@ ME_HD void amp_tt3_block(const KinTT<T, 3>& K, int hb, const Couplings& cp, F&& 
       row_slash_acc(R[3], row_prop(r, P12), se0);
     }
     {  // first gluon 2: orderings 201, 210
-      const c4<T> U = row_prop(row_slash(ub, se2), P2);
+      const c4<T> U = row_prop(ubar_slash(K.wt, ht, se2), P2);
       const c4<T> t = row_slash(U, sJ01);
       cadd(R[4], t);
       csub(R[5], t);
@@ -444,7 +473,7 @@ ME_HD void amp_tt3_block(const KinTT<T, 3>& K, int hb, const Couplings& cp, F&& 
     for (int hv = 0; hv < 2; ++hv) {
       cx<T> A[6];
 #pragma unroll
-      for (int f = 0; f < 6; ++f) A[f] = times_i(spdot(R[f], v[hv])) * g;
+      for (int f = 0; f < 6; ++f) A[f] = dot_v(R[f], K.wtb, hv);
       consume(ht | (hv << 1), A);
     }
   }
@@ -480,7 +509,7 @@ ME_HD c4<T> lepton_current(const KinEE<T>& K, int hel, const Couplings& cp) {
   c4<T> vb = dbar(spinor_v(K.pl[0], T(0), hel_of(hel, 0)));
   c4<T> u = spinor_u(K.pl[1], T(0), hel_of(hel, 1));
   c4<T> L = vcurrent(vb, u);
-  cscale(L, -(T)cp.ee * K.is);
+  cscale(L, -ee_of<T>(cp) * K.is);
   return L;
 }
 
@@ -499,7 +528,7 @@ ME_HD void amp_ee_uug(const KinEE<T>& K, int hel, const Couplings& cp, cx<T>* A)
   c4<T> ub = dbar(spinor_u(K.pl[2], T(0), hel_of(hel, 2)));
   c4<T> v = spinor_v(K.pl[3], T(0), hel_of(hel, 3));
   c4<T> eps = polvec(K.pl[4], hel_of(hel, 4), true);
-  const T g = (T)cp.gs;
+  const T g = gs_of<T>(cp);
   const T equ = (T)(cp.ee * (2.0 / 3.0));
   // gluon on the quark side: ubar (i g eps) i(Q1slash)/Q1^2, Q1 = p_u + p_g
   c4<T> u1 = row_prop(row_slash(ub, eps), K.pl[2] + K.pl[4], T(0));
@@ -561,7 +590,7 @@ ME_HD c4<T> light_current(const c4<T>& vbar_ub, const c4<T>& u_u, T inv, T g) {
 
 template <typename T>
 ME_HD void amp_uu_tt(const KinUU<T>& K, int hel, const Couplings& cp, cx<T>* A) {
-  const T g = (T)cp.gs, mt = (T)cp.mt;
+  const T g = gs_of<T>(cp), mt = mt_of<T>(cp);
   c4<T> uu = spinor_u(K.pl[0], T(0), hel_of(hel, 0));
   c4<T> vbu = dbar(spinor_v(K.pl[1], T(0), hel_of(hel, 1)));
   c4<T> ub = dbar(spinor_u(K.pl[2], mt, hel_of(hel, 2)));
@@ -574,7 +603,7 @@ ME_HD void amp_uu_tt(const KinUU<T>& K, int hel, const Couplings& cp, cx<T>* A) 
 
 template <typename T>
 ME_HD void amp_uu_ttg(const KinUU<T>& K, int hel, const Couplings& cp, cx<T>* A) {
-  const T g = (T)cp.gs, mt = (T)cp.mt;
+  const T g = gs_of<T>(cp), mt = mt_of<T>(cp);
   c4<T> uu = spinor_u(K.pl[0], T(0), hel_of(hel, 0));
   c4<T> vbu = dbar(spinor_v(K.pl[1], T(0), hel_of(hel, 1)));
   c4<T> ub = dbar(spinor_u(K.pl[2], mt, hel_of(hel, 2)));
@@ -653,31 +682,41 @@ ME_HD void amplitude(const Kin<PID, T>& K, int hel, const Couplings& cp, cx<T>* 
 
 // g g -> t tbar g g.  The ordered gluon currents are built once per block with the
 // reflection identities: 6 pairs J(xy), x < y; 12 triples J(xyz) (one of each
-// reversed pair); 12 quadruples J(wxyz) with w < z.  Per top helicity, the quark line
+// reversed pair); 12 quadruples J(wxyz) with w < z.  Per top spin, the quark line
 // is extended ordering by ordering, U(w) -> U(wx) -> U(wxy), and the row of ordering
 // wxyz is ubar J(wxyz) + U(w) J(xyz) + U(wx) J(yz) + U(wxy) e_z.  Orderings are
 // numbered lexicographically, as in amp_ttng.
 template <typename T, class F>
 ME_HD void amp_tt4_block(const KinTT<T, 4>& K, int hb, const Couplings& cp, F&& consume) {
-  const T g = (T)cp.gs, mt = (T)cp.mt;
+  const T g = gs_of<T>(cp), mt = mt_of<T>(cp);
   constexpr int LEG[4] = {0, 1, 4, 5};
-  c4<T> e[4];
+  pol<T> e[4];
 #pragma unroll
-  for (int i = 0; i < 4; ++i) e[i] = polvec_of(K.wg[i], hel_of(hb, LEG[i]), LEG[i] >= 2);
+  for (int i = 0; i < 4; ++i) e[i] = pol_of(K.wg[i], hel_of(hb, LEG[i]), LEG[i] >= 2);
   const r4<T>* q = K.q;
-  // pair currents, index pidx(x, y) for x < y
+  // pair currents, index pidx(x, y) for x < y, and the products e_i . e_j, e_i . J(xy)
   c4<T> J2[6];
+  cx<T> ee[6], eJ[4][6];
   auto pidx = [](int x, int y) { return x == 0 ? y - 1 : (x == 1 ? y + 1 : 5); };
 #pragma unroll
   for (int x = 0; x < 4; ++x)
 #pragma unroll
     for (int y = x + 1; y < 4; ++y) {
-      J2[pidx(x, y)] = vvv(e[x], e[y], -q[x], -q[y], -g * K.ig[(1 << x) | (1 << y)]);
+      J2[pidx(x, y)] = bracket(e[x], q[x], e[y], q[y], -g * K.ig[(1 << x) | (1 << y)], ee[pidx(x, y)]);
     }
-  auto j2 = [&](int x, int y) {  // ordered pair current, J(yx) = -J(xy)
-    c4<T> J = J2[x < y ? pidx(x, y) : pidx(y, x)];
-    if (x > y) cscale(J, T(-1));
-    return J;
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int x = 0; x < 4; ++x)
+#pragma unroll
+      for (int y = x + 1; y < 4; ++y)
+        if (i != x && i != y) eJ[i][pidx(x, y)] = cdot(e[i], J2[pidx(x, y)]);
+  auto e2 = [&](int x, int y) { return ee[x < y ? pidx(x, y) : pidx(y, x)]; };
+  auto ej = [&](int i, int x, int y) {  // e_i . J(xy), J(yx) = -J(xy)
+    return x < y ? eJ[i][pidx(x, y)] : -eJ[i][pidx(y, x)];
+  };
+  auto j2 = [&](int x, int y) {  // ordered pair current
+    return x < y ? J2[pidx(x, y)] : cneg(J2[pidx(y, x)]);
   };
   // triple currents J(xyz) for x < z (J(zyx) = J(xyz)); index tidx = 3 * (missing gluon) + (middle slot)
   c4<T> J3[12];
@@ -697,9 +736,10 @@ ME_HD void amp_tt4_block(const KinTT<T, 4>& K, int hb, const Couplings& cp, F&& 
         if (y == x || y == z) continue;
         const int S = (1 << x) | (1 << y) | (1 << z);
         const T c3 = -g * K.ig[S], c4g = g * g * K.ig[S];
-        c4<T> J = vvv(e[x], j2(y, z), -q[x], -(q[y] + q[z]), c3);
-        vvv_acc(J, j2(x, y), e[z], -(q[x] + q[y]), -q[z], c3);
-        caxpy(J, c4g, vvvv_ordered(e[x], e[y], e[z]));
+        c4<T> J = czero<T>();
+        bracket_acc(J, e[x], q[x], j2(y, z), q[y] + q[z], c3, ej(x, y, z));
+        bracket_acc(J, e[z], q[z], j2(x, y), q[x] + q[y], -c3, ej(z, x, y));
+        quartic_acc(J, e[x], e[y], e[z], c4g * e2(x, z), c4g * e2(x, y), c4g * e2(y, z));
         J3[tidx(x, y, z)] = J;
       }
   auto j3 = [&](int x, int y, int z) { return J3[tidx(x, y, z)]; };
@@ -716,13 +756,15 @@ ME_HD void amp_tt4_block(const KinTT<T, 4>& K, int hb, const Couplings& cp, F&& 
         const int z = 6 - w - x - y;
         if (z < w) continue;
         const T c3 = -g * K.ig[15], c4g = g * g * K.ig[15];
-        c4<T> J = vvv(e[w], j3(x, y, z), -q[w], -(q[x] + q[y] + q[z]), c3);
-        vvv_acc(J, j2(w, x), j2(y, z), -(q[w] + q[x]), -(q[y] + q[z]), c3);
-        vvv_acc(J, j3(w, x, y), e[z], -(q[w] + q[x] + q[y]), -q[z], c3);
-        c4<T> V = vvvv_ordered(e[w], e[x], j2(y, z));
-        cadd(V, vvvv_ordered(e[w], j2(x, y), e[z]));
-        cadd(V, vvvv_ordered(j2(w, x), e[y], e[z]));
-        caxpy(J, c4g, V);
+        const r4<T> qwx = q[w] + q[x], qyz = q[y] + q[z];
+        const c4<T> Jxyz = j3(x, y, z), Jwxy = j3(w, x, y), Jwx = j2(w, x), Jxy = j2(x, y), Jyz = j2(y, z);
+        c4<T> J = czero<T>();
+        bracket_acc(J, e[w], q[w], Jxyz, q[x] + qyz, c3, cdot(e[w], Jxyz));
+        bracket_acc(J, Jwx, qwx, Jyz, qyz, c3);
+        bracket_acc(J, e[z], q[z], Jwxy, qwx + q[y], -c3, cdot(e[z], Jwxy));
+        quartic_acc(J, e[w], e[x], Jyz, c4g * ej(w, y, z), c4g * e2(w, x), c4g * ej(x, y, z));
+        quartic_acc(J, e[w], Jxy, e[z], c4g * e2(w, z), c4g * ej(w, x, y), c4g * ej(z, x, y));
+        quartic_acc(J, Jwx, e[y], e[z], c4g * ej(z, w, x), c4g * ej(y, w, x), c4g * e2(y, z));
         J4[n4++] = J;
       }
   // rank of the quadruple current of ordering wxyz among those with first < last
@@ -740,39 +782,35 @@ ME_HD void amp_tt4_block(const KinTT<T, 4>& K, int hb, const Couplings& cp, F&& 
         }
     return -1;
   };
-  const c4<T> v[2] = {spinor_v_of(K.wtb, -1), spinor_v_of(K.wtb, 1)};
   const r4<T> kt = K.pl[2];
 #pragma unroll 1
   for (int ht = 0; ht < 2; ++ht) {
-    const c4<T> ub = dbar(spinor_u_of(K.wt, ht ? 1 : -1));
     cx<T> A[2][24];
     int f = 0;
 #pragma unroll
     for (int w = 0; w < 4; ++w) {
-      const c4<T> U1 = row_prop(row_slash(ub, e[w]), scaled_prop(kt + q[w], mt, -g * K.iq[1 << w]));
+      const c4<T> U1 = row_prop(ubar_slash(K.wt, ht, slashed(e[w])), scaled_prop(kt + q[w], mt, -g * K.iq[1 << w]));
 #pragma unroll
       for (int x = 0; x < 4; ++x) {
         if (x == w) continue;
-        c4<T> r2 = row_slash(ub, j2(w, x));
-        row_slash_acc(r2, U1, e[x]);
+        c4<T> r2 = ubar_slash(K.wt, ht, slashed(j2(w, x)));
+        row_slash_acc(r2, U1, slashed(e[x]));
         const c4<T> U2 = row_prop(r2, scaled_prop(kt + q[w] + q[x], mt, -g * K.iq[(1 << w) | (1 << x)]));
 #pragma unroll
         for (int y = 0; y < 4; ++y) {
           if (y == w || y == x) continue;
           const int z = 6 - w - x - y;
-          c4<T> r3 = row_slash(ub, j3(w, x, y));
+          c4<T> r3 = ubar_slash(K.wt, ht, slashed(j3(w, x, y)));
           row_slash_acc(r3, U1, j2(x, y));
-          row_slash_acc(r3, U2, e[y]);
+          row_slash_acc(r3, U2, slashed(e[y]));
           const c4<T> U3 =
               row_prop(r3, scaled_prop(kt + q[w] + q[x] + q[y], mt, -g * K.iq[(1 << w) | (1 << x) | (1 << y)]));
-          c4<T> J = z > w ? J4[q4(w, x, y)] : J4[q4(z, y, x)];
-          if (z < w) cscale(J, T(-1));
-          c4<T> R = row_slash(ub, J);
+          c4<T> R = ubar_slash(K.wt, ht, slashed(z > w ? J4[q4(w, x, y)] : cneg(J4[q4(z, y, x)])));
           row_slash_acc(R, U1, j3(x, y, z));
           row_slash_acc(R, U2, j2(y, z));
-          row_slash_acc(R, U3, e[z]);
+          row_slash_acc(R, U3, slashed(e[z]));
 #pragma unroll
-          for (int hv = 0; hv < 2; ++hv) A[hv][f] = times_i(spdot(R, v[hv])) * g;
+          for (int hv = 0; hv < 2; ++hv) A[hv][f] = dot_v(R, K.wtb, hv);
           ++f;
         }
       }
