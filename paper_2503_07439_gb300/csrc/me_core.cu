@@ -34,52 +34,83 @@ static int fail(int code, const std::string& msg) {
   } while (0)
 
 // ---------------------------------------------------------------- reductions
-__global__ void k_partials(const double* __restrict__ w, long n, double* __restrict__ part, const int* __restrict__ cnt) {
-  __shared__ double s1[256], s2[256];
-  double a = 0.0, b = 0.0;
-  if (cnt) n = *cnt;
-  for (long i = (long)blockIdx.x * 256 + threadIdx.x; i < n; i += (long)gridDim.x * 256) {
-    const double x = w[i];
-    a += x;
-    b += x * x;
-  }
-  s1[threadIdx.x] = a;
-  s2[threadIdx.x] = b;
-  __syncthreads();
-  for (int o = 128; o > 0; o >>= 1) {
-    if ((int)threadIdx.x < o) {
-      s1[threadIdx.x] += s1[threadIdx.x + o];
-      s2[threadIdx.x] += s2[threadIdx.x + o];
-    }
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) {
-    part[2 * blockIdx.x] = s1[0];
-    part[2 * blockIdx.x + 1] = s2[0];
-  }
-}
-
-// One warp: lane l adds the partials l, l + 32, ... in order, then a fixed butterfly adds
-// the lanes.  The order is fixed, so the result is reproducible; a single thread adding
-// all partials in a dependent chain would take tens of microseconds of float64 latency.
-__global__ void k_finish(const double* __restrict__ part, int nblk, double* __restrict__ acc, long n,
-                         const int* __restrict__ cnt) {
-  if (blockIdx.x != 0 || threadIdx.x >= 32) return;
-  double a = 0.0, b = 0.0;
-  for (int i = (int)threadIdx.x; i < nblk; i += 32) {
-    a += part[2 * i];
-    b += part[2 * i + 1];
-  }
+// Sum over the block of (a, b): warp butterflies, then the first warp over the warps' sums.
+// The order is fixed.  Result on thread 0.
+__device__ __forceinline__ void block_sum2(double& a, double& b, double (*sm)[8]) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
     a += __shfl_xor_sync(0xffffffffu, a, o);
     b += __shfl_xor_sync(0xffffffffu, b, o);
   }
+  if ((threadIdx.x & 31) == 0) {
+    sm[0][threadIdx.x >> 5] = a;
+    sm[1][threadIdx.x >> 5] = b;
+  }
+  __syncthreads();
+  if (threadIdx.x < 32) {
+    a = threadIdx.x < 8 ? sm[0][threadIdx.x] : 0.0;
+    b = threadIdx.x < 8 ? sm[1][threadIdx.x] : 0.0;
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) {
+      a += __shfl_xor_sync(0xffffffffu, a, o);
+      b += __shfl_xor_sync(0xffffffffu, b, o);
+    }
+  }
+}
+
+// Weight accumulation and the end of a call: (sum w, sum w^2) by blocks in a fixed order,
+// then the block that finishes last adds the blocks' partials in block order (no floating
+// atomics: the result is reproducible) and hands the call's counters over, `live` to `last`,
+// leaving `live` zero for the next call.  One launch instead of three (a memset of the
+// counters, the partials, their sum), each mostly launch and drain latency: with the closed
+// form, a call with 999 e+e- n-body points went from 56 to 33 us.  `cnt` (optional, device):
+// the number of points, at most n.
+constexpr int CNT_LIVE = 12;    // counters handed over
+constexpr int CNT_TICKET = 12;  // blocks finished
+__global__ void __launch_bounds__(256) k_reduce(const double* __restrict__ w, long n, const int* __restrict__ cnt,
+                                                double* __restrict__ part, double* __restrict__ acc,
+                                                int* __restrict__ live, int* __restrict__ last) {
+  __shared__ double sm[2][8];
+  __shared__ bool final_block;
+  double a = 0.0, b = 0.0;
+  if (cnt) n = *cnt;
+  const long stride = (long)gridDim.x * 256;
+  long i = (long)blockIdx.x * 256 + threadIdx.x;
+  for (; i + 3 * stride < n; i += 4 * stride) {
+    const double x0 = w[i], x1 = w[i + stride], x2 = w[i + 2 * stride], x3 = w[i + 3 * stride];
+    a += (x0 + x1) + (x2 + x3);
+    b += (x0 * x0 + x1 * x1) + (x2 * x2 + x3 * x3);
+  }
+  for (; i < n; i += stride) {
+    const double x = w[i];
+    a += x;
+    b += x * x;
+  }
+  block_sum2(a, b, sm);
   if (threadIdx.x == 0) {
-    if (cnt) n = *cnt;
+    __stcg(part + 2 * blockIdx.x, a);
+    __stcg(part + 2 * blockIdx.x + 1, b);
+    __threadfence();
+    final_block = atomicAdd(live + CNT_TICKET, 1) == (int)gridDim.x - 1;
+  }
+  __syncthreads();
+  if (!final_block) return;
+  __threadfence();
+  a = b = 0.0;
+  for (int j = (int)threadIdx.x; j < (int)gridDim.x; j += 256) {
+    a += __ldcg(part + 2 * j);
+    b += __ldcg(part + 2 * j + 1);
+  }
+  block_sum2(a, b, sm);
+  if (threadIdx.x == 0) {
     acc[0] += a;
     acc[1] += b;
     acc[2] += (double)n;
+    live[CNT_TICKET] = 0;
+  }
+  if (threadIdx.x < CNT_LIVE) {
+    last[threadIdx.x] = live[threadIdx.x];
+    live[threadIdx.x] = 0;
   }
 }
 constexpr int RED_BLOCKS = 304;  // 2 x 152 SMs
@@ -410,9 +441,13 @@ struct me_handle {
   double* d_out = nullptr;
   size_t cap = 0;
   int* d_resc = nullptr;     // rescue index list (capacity cap)
-  int* d_nresc = nullptr;    // [0]: points re-evaluated in float64, [1]: tile counter (queued kernel),
-                             // [2] / [3]: real-block / Born items of the item rescue,
-                             // [8]: points passing the cuts (tree entries with per-term queues)
+  // counters of the running call (ItemBufs, the reduction's ticket; zero between calls) and,
+  // from d_last, those of the last finished one; [13]: points passing the cuts (tree entries
+  // with per-term queues)
+  int* d_nresc = nullptr;
+  int* d_last = nullptr;
+  bool dirty = false;       // a call failed half way: the counters have to be cleared
+  bool last_terms = false;  // the last subtracted-real call ran the per-term queues
   // item rescue (mixed-precision subtracted real): records and item lists, capacity icap
   ItemBufs ib{};
   size_t icap = 0;
@@ -432,27 +467,22 @@ struct me_handle {
 };
 
 static void free_items(me_handle* h) {
-  cudaFree(h->ib.ev);
-  cudaFree(h->ib.mask);
-  cudaFree(h->ib.a);
-  cudaFree(h->ib.v);
-  cudaFree(h->ib.list_r);
-  cudaFree(h->ib.list_b);
+  void* ptrs[] = {h->ib.ev, h->ib.pend, h->ib.a, h->ib.v, h->ib.list_r};
+  for (void* q : ptrs) cudaFree(q);
   h->ib = ItemBufs{};
   h->icap = 0;
 }
 
-// Records and item lists of the item rescue for n points (grown on demand).
+// Records and item list of the item rescue for n points (grown on demand).
 static int ensure_item_capacity(me_handle* h, size_t n) {
   if (n <= h->icap) return ME_OK;
   free_items(h);
   const size_t c = std::max(n, (size_t)1024);
   ItemBufs& b = h->ib;
-  if (cudaMalloc(&b.ev, c * sizeof(int)) != cudaSuccess || cudaMalloc(&b.mask, c * sizeof(int)) != cudaSuccess ||
-      cudaMalloc(&b.a, c * MAX_ITEMS * sizeof(double)) != cudaSuccess ||
-      cudaMalloc(&b.v, c * MAX_ITEMS * sizeof(double)) != cudaSuccess ||
-      cudaMalloc(&b.list_r, c * 4 * sizeof(int)) != cudaSuccess ||
-      cudaMalloc(&b.list_b, c * sizeof(int)) != cudaSuccess) {
+  if (cudaMalloc(&b.ev, c * sizeof(int)) != cudaSuccess || cudaMalloc(&b.pend, c * sizeof(int)) != cudaSuccess ||
+      cudaMalloc(&b.a, c * 2 * sizeof(double)) != cudaSuccess ||
+      cudaMalloc(&b.v, c * MAX_BLOCKS * sizeof(double)) != cudaSuccess ||
+      cudaMalloc(&b.list_r, c * MAX_BLOCKS * sizeof(int)) != cudaSuccess) {
     free_items(h);
     return fail(ME_ERR_OOM, "item-rescue scratch allocation failed");
   }
@@ -463,32 +493,22 @@ static int ensure_item_capacity(me_handle* h, size_t n) {
 
 static void free_terms(me_handle* h) {
   TermBufs& t = h->tb;
-  void* ptrs[] = {t.ev, t.flags, t.grow, t.a, t.v, t.m, t.cfg, t.bp, t.bx, t.bslot, t.q_real, t.r_real, t.r_born,
-                  t.flagged, t.cnt};
+  void* ptrs[] = {t.ev, t.grow, t.a, t.cnt};
   for (void* q : ptrs) cudaFree(q);
   h->tb = TermBufs{};
   h->tcap = 0;
 }
 
-// Records, Born configurations and queues of the per-term queues for n points.
+// Records of the per-term queues for n points.
 static int ensure_term_capacity(me_handle* h, size_t n) {
   if (n <= h->tcap) return ME_OK;
   free_terms(h);
   const size_t c = std::max(n, (size_t)1024);
   TermBufs& t = h->tb;
-  bool ok = cudaMalloc(&t.ev, c * sizeof(int)) == cudaSuccess && cudaMalloc(&t.flags, c * sizeof(int)) == cudaSuccess &&
-            cudaMalloc(&t.grow, c * sizeof(float)) == cudaSuccess &&
-            cudaMalloc(&t.a, c * MAX_ITEMS * sizeof(double)) == cudaSuccess &&
-            cudaMalloc(&t.v, c * MAX_ITEMS * sizeof(double)) == cudaSuccess &&
-            cudaMalloc(&t.m, c * 6 * sizeof(double)) == cudaSuccess &&
-            cudaMalloc(&t.cfg, c * 2 * sizeof(int)) == cudaSuccess &&
-            cudaMalloc(&t.bp, c * 2 * 16 * sizeof(double)) == cudaSuccess &&
-            cudaMalloc(&t.bx, c * 2 * 4 * sizeof(double)) == cudaSuccess &&
-            cudaMalloc(&t.bslot, c * 2 * sizeof(int)) == cudaSuccess &&
-            cudaMalloc(&t.q_real, c * sizeof(int)) == cudaSuccess &&
-            cudaMalloc(&t.r_real, c * 4 * sizeof(int)) == cudaSuccess &&
-            cudaMalloc(&t.r_born, c * 2 * sizeof(int)) == cudaSuccess &&
-            cudaMalloc(&t.flagged, c * sizeof(int)) == cudaSuccess && cudaMalloc(&t.cnt, 8 * sizeof(int)) == cudaSuccess;
+  const bool ok = cudaMalloc(&t.ev, c * sizeof(int)) == cudaSuccess &&
+                  cudaMalloc(&t.grow, c * sizeof(float)) == cudaSuccess &&
+                  cudaMalloc(&t.a, c * 3 * sizeof(double)) == cudaSuccess &&
+                  cudaMalloc(&t.cnt, sizeof(int)) == cudaSuccess;
   if (!ok) {
     free_terms(h);
     return fail(ME_ERR_OOM, "per-term queue scratch allocation failed");
@@ -559,15 +579,16 @@ static bool use_items(const me_handle* h, int64_t n) {
 // Float64 work for the points the bulk-precision launch `a` flagged, on the handle's
 // stream, counts read on the device: the item rescue (float64 items, then W recombined
 // from the coefficients), or every flagged point re-evaluated whole.
-static cudaError_t launch_rescue(me_handle* h, const LaunchArgs& a, int lpe64) {
-  if (a.kp.item_rescue) {
-    switch (h->proc->pid) {
-      case P_EE_UUG: return launch_items_ee(a, h->stream);
-      case P_GG_TTG: return launch_items_gg(a, h->stream);
-      case P_UU_TTG: return launch_items_uu(a, h->stream);
-    }
-    return cudaErrorInvalidValue;
+static cudaError_t launch_items(me_handle* h, const LaunchArgs& a) {
+  switch (h->proc->pid) {
+    case P_EE_UUG: return launch_items_ee(a, h->stream);
+    case P_GG_TTG: return launch_items_gg(a, h->stream);
+    case P_UU_TTG: return launch_items_uu(a, h->stream);
   }
+  return cudaErrorInvalidValue;
+}
+static cudaError_t launch_rescue(me_handle* h, const LaunchArgs& a, int lpe64) {
+  if (a.kp.item_rescue) return launch_items(h, a);
   LaunchArgs r = a;
   r.kp.flag_unstable = 0;
   r.idx = h->d_resc;
@@ -585,15 +606,31 @@ static bool use_terms(const me_handle* h, int64_t n) {
                                   h->prm.queued_rescue == 0 && h->prm.rescue == ME_RESCUE_ITEMS);
 }
 
-// Per-term queues of the subtracted real (phase 0: float64 pass, bulk items and
-// recombination; phase 1: float64 rescue and recombination of the flagged points).
-static cudaError_t launch_terms(me_handle* h, int phase, bool mixed, const LaunchArgs& a) {
+// Per-term queues of the subtracted real: float64 pass, reals and recombination.
+static cudaError_t launch_terms(me_handle* h, bool mixed, const LaunchArgs& a) {
   switch (h->proc->pid) {
-    case P_EE_UUG: return launch_terms_ee(phase, mixed, a, h->tb, h->d_nresc, h->stream);
-    case P_GG_TTG: return launch_terms_gg(phase, mixed, a, h->tb, h->d_nresc, h->stream);
-    case P_UU_TTG: return launch_terms_uu(phase, mixed, a, h->tb, h->d_nresc, h->stream);
+    case P_EE_UUG: return launch_terms_ee(mixed, a, h->tb, h->stream);
+    case P_GG_TTG: return launch_terms_gg(mixed, a, h->tb, h->stream);
+    case P_UU_TTG: return launch_terms_uu(mixed, a, h->tb, h->stream);
   }
   return cudaErrorInvalidValue;
+}
+
+// Weight accumulation of n results (or *cnt) and hand-over of the call's counters.
+static cudaError_t launch_reduce(me_handle* h, const double* out, long n, const int* cnt) {
+  const long blocks = std::min<long>(RED_BLOCKS, (n + 1023) / 1024);
+  k_reduce<<<(unsigned)std::max(1L, blocks), 256, 0, h->stream>>>(out, n, cnt, h->d_part, h->d_acc, h->d_nresc, h->d_last);
+  return cudaGetLastError();
+}
+
+// Counters of the running call at zero: the reduction leaves them so, unless a call failed.
+static cudaError_t begin_call(me_handle* h) {
+  if (h->dirty) {
+    const cudaError_t e = cudaMemsetAsync(h->d_nresc, 0, 16 * sizeof(int), h->stream);
+    if (e != cudaSuccess) return e;
+  }
+  h->dirty = true;
+  return cudaSuccess;
 }
 
 // pick lanes-per-event by timing each candidate once on the caller's batch (first use)
@@ -614,6 +651,8 @@ static int size_class(long n) {
 
 static int choose_lpe(me_handle* h, int kind, bool fp64, const LaunchArgs& a) {
   int& slot = h->lpe[kind][fp64 ? 1 : 0];
+  const int pid = h->proc->pid;
+  if (kind == K_TREE && (pid == P_EE_UU || pid == P_GG_TT || pid == P_UU_TT)) return slot = 1;  // closed forms
   if (h->prm.lanes_per_event) return slot = h->prm.lanes_per_event;
   const int cls = size_class(a.groups);
   if (slot && h->lpe_class[kind][fp64 ? 1 : 0] == cls) return slot;
@@ -754,17 +793,19 @@ int me_init(const char* process, const me_params* params, me_handle** out) {
     return fail(ME_ERR_CUDA, "me_init: stream creation failed");
   }
   h->stream = h->own_stream;
-  if (cudaMalloc(&h->d_nresc, 16 * sizeof(int)) != cudaSuccess || cudaMalloc(&h->d_part, 2 * RED_BLOCKS * sizeof(double)) != cudaSuccess ||
+  if (cudaMalloc(&h->d_nresc, 32 * sizeof(int)) != cudaSuccess || cudaMalloc(&h->d_part, 2 * RED_BLOCKS * sizeof(double)) != cudaSuccess ||
       cudaMalloc(&h->d_acc, 3 * sizeof(double)) != cudaSuccess) {
     me_destroy(h);
     return fail(ME_ERR_OOM, "me_init: allocation failed");
   }
+  h->d_last = h->d_nresc + 16;
   KParams& kp = h->kp;
-  std::memset(&kp, 0, sizeof(kp));
+  kp = KParams{};
   kp.cp = Couplings(std::sqrt(4.0 * M_PI * params->alpha_s), std::sqrt(4.0 * M_PI * params->alpha), params->mt);
   kp.avg_inv = 1.0 / pd->avg;
   kp.born_avg_inv = pd->born_pid >= 0 ? 1.0 / kProcs[pd->born_pid].avg : 0.0;
-  kp.nlo_factor = 1.0;
+  kp.tree_scale = kp.avg_inv * tree_coupling(pd->pid, kp.cp);
+  kp.real_scale = 2.0 * kp.tree_scale;
   kp.xi_cut = params->xi_cut;
   kp.delta = params->delta;
   kp.xi_thr = params->xi_thr;
@@ -777,7 +818,7 @@ int me_init(const char* process, const me_params* params, me_handle** out) {
   // stream-ordered on the handle's own stream: no device-wide synchronisation, so a
   // handle can be created while other threads capture CUDA graphs
   if (cudaMemsetAsync(h->d_acc, 0, 3 * sizeof(double), h->own_stream) != cudaSuccess ||
-      cudaMemsetAsync(h->d_nresc, 0, 16 * sizeof(int), h->own_stream) != cudaSuccess ||
+      cudaMemsetAsync(h->d_nresc, 0, 32 * sizeof(int), h->own_stream) != cudaSuccess ||
       cudaStreamSynchronize(h->own_stream) != cudaSuccess) {
     me_destroy(h);
     return fail(ME_ERR_CUDA, "me_init: device error");
@@ -824,7 +865,7 @@ static int run(me_handle* h, int kind, double nlo_factor, const double* momenta,
   a.n = n;
   a.out = O;
   a.kp = h->kp;
-  a.kp.nlo_factor = nlo_factor;
+  a.kp.tree_scale *= nlo_factor;
   a.groups = n;
   a.resc_list = h->d_resc;
   a.resc_count = h->d_nresc;
@@ -840,13 +881,13 @@ static int run(me_handle* h, int kind, double nlo_factor, const double* momenta,
   if (terms && vp && pv.host) a.p_copy = h->d_p;
   if (kind == K_REAL && mixed) {
     a.kp.flag_unstable = 1;
-    if (!queued && !terms && use_items(h, n)) {
+    if (terms || (!queued && use_items(h, n))) {
       if ((rc = ensure_item_capacity(h, (size_t)n)) != ME_OK) return rc;
       a.kp.item_rescue = 1;
       a.items = h->ib;
     }
-    ME_CUDA(cudaMemsetAsync(h->d_nresc, 0, 6 * sizeof(int), h->stream));
     h->last_kind = K_REAL;
+    h->last_terms = terms;
   }
   // the first call per (kind, precision) times the lane layouts (synchronising);
   // both are chosen before the launches whose results are kept.  The queued kernel
@@ -870,26 +911,26 @@ static int run(me_handle* h, int kind, double nlo_factor, const double* momenta,
     h->ev_used.push_back(ev);
     ME_CUDA(cudaEventRecord(ev[0], h->stream));
   }
+  ME_CUDA(begin_call(h));
   if (terms) {
-    ME_CUDA(launch_terms(h, 0, mixed, a));
+    ME_CUDA(launch_terms(h, mixed, a));
   } else if (queued) {
     ME_CUDA(launch_queued(h->proc->pid, a, h->stream));
   } else {
     if (cut_list) {
       // per-term queues of a tree entry: only the points that pass the cuts are evaluated
-      ME_CUDA(launch_cut_list(h->proc->pid, a, h->d_resc, h->d_nresc + 8, h->stream));
+      ME_CUDA(launch_cut_list(h->proc->pid, a, h->d_resc, h->d_nresc + 13, h->stream));
       a.idx = h->d_resc;
-      a.count = h->d_nresc + 8;
+      a.count = h->d_nresc + 13;
     }
     ME_CUDA(dispatch(h->proc->pid, kind, !mixed, lpe, a, h->stream));
   }
   if (timed) ME_CUDA(cudaEventRecord(ev[1], h->stream));
-  if (terms && mixed) ME_CUDA(launch_terms(h, 1, mixed, a));
+  if (terms && mixed) ME_CUDA(launch_items(h, a));
   if (kind == K_REAL && mixed && !queued && !terms) ME_CUDA(launch_rescue(h, a, lpe64));
   if (timed) ME_CUDA(cudaEventRecord(ev[2], h->stream));
-  k_partials<<<RED_BLOCKS, 256, 0, h->stream>>>(O, n, h->d_part, nullptr);
-  k_finish<<<1, 32, 0, h->stream>>>(h->d_part, RED_BLOCKS, h->d_acc, n, nullptr);
-  ME_CUDA(cudaGetLastError());
+  ME_CUDA(launch_reduce(h, O, n, nullptr));
+  h->dirty = false;
   if (timed) ME_CUDA(cudaEventRecord(ev[3], h->stream));
   if (!vo) ME_CUDA(cudaMemcpyAsync(out, O, (size_t)n * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
   if (on_host) ME_CUDA(cudaStreamSynchronize(h->stream));
@@ -924,7 +965,7 @@ int me_last_rescued(me_handle* h, int64_t* n_rescued) {
   ME_CUDA(cudaSetDevice(h->device));
   int c = 0;
   if (h->prm.precision == ME_PREC_MIXED && h->last_kind == K_REAL) {
-    ME_CUDA(cudaMemcpyAsync(&c, h->d_nresc, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
+    ME_CUDA(cudaMemcpyAsync(&c, h->d_last, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
     ME_CUDA(cudaStreamSynchronize(h->stream));
   }
   *n_rescued = c;
@@ -934,14 +975,14 @@ int me_last_rescued(me_handle* h, int64_t* n_rescued) {
 int me_last_rescue_work(me_handle* h, int64_t* points, int64_t* real_blocks, int64_t* born_sets) {
   if (!h || !points || !real_blocks || !born_sets) return fail(ME_ERR_ARG, "NULL argument");
   ME_CUDA(cudaSetDevice(h->device));
-  int c[4] = {0, 0, 0, 0};
+  int c[6] = {0, 0, 0, 0, 0, 0};
   if (h->prm.precision == ME_PREC_MIXED && h->last_kind == K_REAL) {
-    ME_CUDA(cudaMemcpyAsync(c, h->d_nresc, sizeof(c), cudaMemcpyDeviceToHost, h->stream));
+    ME_CUDA(cudaMemcpyAsync(c, h->d_last, sizeof(c), cudaMemcpyDeviceToHost, h->stream));
     ME_CUDA(cudaStreamSynchronize(h->stream));
   }
   *points = c[0];
   *real_blocks = c[2];
-  *born_sets = c[3];
+  *born_sets = h->last_terms ? c[4] + c[5] : c[3];
   return ME_OK;
 }
 
@@ -949,8 +990,8 @@ int me_last_rescue_configs(me_handle* h, int64_t* set0, int64_t* set1) {
   if (!h || !set0 || !set1) return fail(ME_ERR_ARG, "NULL argument");
   ME_CUDA(cudaSetDevice(h->device));
   int c[6] = {0, 0, 0, 0, 0, 0};
-  if (h->prm.precision == ME_PREC_MIXED && h->last_kind == K_REAL) {
-    ME_CUDA(cudaMemcpyAsync(c, h->d_nresc, sizeof(c), cudaMemcpyDeviceToHost, h->stream));
+  if (h->prm.precision == ME_PREC_MIXED && h->last_kind == K_REAL && h->last_terms) {
+    ME_CUDA(cudaMemcpyAsync(c, h->d_last, sizeof(c), cudaMemcpyDeviceToHost, h->stream));
     ME_CUDA(cudaStreamSynchronize(h->stream));
   }
   *set0 = c[4];
@@ -1059,7 +1100,9 @@ int me_internal_prepare_counted(me_handle* h, int me_kind, int64_t cap) {
   int rc = ensure_capacity(h, (size_t)cap);
   if (rc == ME_OK && kind == K_REAL && use_terms(h, cap)) {
     if (cap >= (int64_t)1 << 29) return fail(ME_ERR_ARG, "term_queues: at most 2^29 - 1 points per call");
-    return ensure_term_capacity(h, (size_t)cap);
+    rc = ensure_term_capacity(h, (size_t)cap);
+    if (rc == ME_OK && mixed) rc = ensure_item_capacity(h, (size_t)cap);
+    return rc;
   }
   if (rc == ME_OK && kind == K_REAL && mixed && !h->prm.queued_rescue && use_items(h, cap))
     rc = ensure_item_capacity(h, (size_t)cap);
@@ -1080,7 +1123,7 @@ int me_internal_launch_counted(me_handle* h, int me_kind, const double* d_p, con
   a.n = cap;
   a.out = d_out;
   a.kp = h->kp;
-  a.kp.nlo_factor = nlo;
+  a.kp.tree_scale *= nlo;
   a.count = d_n;
   a.groups = cap;
   a.resc_list = h->d_resc;
@@ -1093,31 +1136,31 @@ int me_internal_launch_counted(me_handle* h, int me_kind, const double* d_p, con
   if (terms && (size_t)cap > h->tcap) return fail(ME_ERR_ARG, "counted launch: handle not prepared");
   if (kind == K_REAL && mixed) {
     a.kp.flag_unstable = 1;
-    if (!queued && !terms && use_items(h, cap)) {
+    if (terms || (!queued && use_items(h, cap))) {
       if ((size_t)cap > h->icap) return fail(ME_ERR_ARG, "counted launch: handle not prepared");
       a.kp.item_rescue = 1;
       a.items = h->ib;
     }
-    ME_CUDA(cudaMemsetAsync(h->d_nresc, 0, 6 * sizeof(int), h->stream));
     h->last_kind = K_REAL;
+    h->last_terms = terms;
   }
+  ME_CUDA(begin_call(h));
   if (terms) {
-    ME_CUDA(launch_terms(h, 0, mixed, a));
-    if (mixed) ME_CUDA(launch_terms(h, 1, mixed, a));
+    ME_CUDA(launch_terms(h, mixed, a));
+    if (mixed) ME_CUDA(launch_items(h, a));
   } else if (queued) {
     ME_CUDA(launch_queued(h->proc->pid, a, h->stream));
   } else {
     if (cut_list) {
-      ME_CUDA(launch_cut_list(h->proc->pid, a, h->d_resc, h->d_nresc + 8, h->stream));
+      ME_CUDA(launch_cut_list(h->proc->pid, a, h->d_resc, h->d_nresc + 13, h->stream));
       a.idx = h->d_resc;
-      a.count = h->d_nresc + 8;
+      a.count = h->d_nresc + 13;
     }
     ME_CUDA(dispatch(h->proc->pid, kind, !mixed, lpe, a, h->stream));
   }
   if (kind == K_REAL && mixed && !queued && !terms) ME_CUDA(launch_rescue(h, a, lpe64));
-  k_partials<<<RED_BLOCKS, 256, 0, h->stream>>>(d_out, cap, h->d_part, d_n);
-  k_finish<<<1, 32, 0, h->stream>>>(h->d_part, RED_BLOCKS, h->d_acc, cap, d_n);
-  ME_CUDA(cudaGetLastError());
+  ME_CUDA(launch_reduce(h, d_out, cap, d_n));
+  h->dirty = false;
   return ME_OK;
 }
 
@@ -1139,7 +1182,7 @@ int me_internal_rescued_async(me_handle* h, int* dst) {
     *dst = 0;
     return ME_OK;
   }
-  ME_CUDA(cudaMemcpyAsync(dst, h->d_nresc, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
+  ME_CUDA(cudaMemcpyAsync(dst, h->d_last, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
   return ME_OK;
 }
 
@@ -1162,11 +1205,12 @@ int me_internal_kparams(const char* process, const me_params* params, me::KParam
   for (const auto& d : kProcs)
     if (std::strcmp(d.name, process) == 0) pd = &d;
   if (!pd) return fail(ME_ERR_PROCESS, std::string("unknown process ") + process);
-  std::memset(kp, 0, sizeof(*kp));
+  *kp = KParams{};
   kp->cp = Couplings(std::sqrt(4.0 * M_PI * params->alpha_s), std::sqrt(4.0 * M_PI * params->alpha), params->mt);
   kp->avg_inv = 1.0 / pd->avg;
   kp->born_avg_inv = pd->born_pid >= 0 ? 1.0 / kProcs[pd->born_pid].avg : 0.0;
-  kp->nlo_factor = 1.0;
+  kp->tree_scale = kp->avg_inv * tree_coupling(pd->pid, kp->cp);
+  kp->real_scale = 2.0 * kp->tree_scale;
   kp->xi_cut = params->xi_cut;
   kp->delta = params->delta;
   kp->xi_thr = params->xi_thr;

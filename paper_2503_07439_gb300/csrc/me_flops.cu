@@ -40,12 +40,12 @@ static double colour_flops(int nf) { return nf <= 6 ? 2.0 * nf * nf + 4.0 * nf :
 
 // one helicity block (me_procs.cuh): amplitudes of four helicities plus their colour sums
 template <int PID>
-static double block_ops(const r4<double>* p, int hb = 1, const c4<Flop>* ov = nullptr, int ov_leg = -1) {
+static double block_ops(const r4<double>* p, int hb = 1) {
   const Couplings cp{1.2, 0.3, 173.0};
   const Kin<PID, Flop> K = prepare<PID, Flop>(p, cp);
   g_ops = 0;
   int calls = 0;
-  amplitude_block<PID, Flop>(K, hb, cp, [&](int, const cx<Flop>*) { ++calls; }, ov, ov_leg);
+  amplitude_block<PID, Flop>(K, hb, cp, [&](int, const cx<Flop>*) { ++calls; });
   return (double)g_ops + calls * colour_flops(Proc<PID>::NFLOW);
 }
 
@@ -59,9 +59,15 @@ static double prep_ops(const r4<double>* p) {
   return (double)g_ops;
 }
 
-// Born |M|^2 of one event: every block of the half helicity set, plus the preparation
+// Born |M|^2 of one event: its closed form, or every block of the half helicity set plus the
+// preparation
 template <int PID>
 static double born_ops(const r4<double>* p) {
+  if constexpr (closed_tree<PID>()) {
+    g_ops = 0;
+    closed_sum<PID, Flop>(p, Couplings{1.2, 0.3, 173.0});
+    return (double)g_ops;
+  }
   double t = prep_ops<PID>(p);
   for (int b = 0; b < n_live_blocks<PID>(); ++b) t += block_ops<PID>(p, live_block_hel<PID>(b));
   return t;
@@ -71,15 +77,29 @@ int main() {
   // a generic massive 2 -> 4 configuration is enough: the count does not depend on values
   r4<double> p[6] = {{1000, 0, 0, 1000},     {1000, 0, 0, -1000}, {600, 100, 200, 300},
                      {700, -150, -100, 200}, {400, 30, -80, -300}, {300, 20, -20, -200}};
-  c4<Flop> e;
-  for (int i = 0; i < 4; ++i) e.v[i] = cx<Flop>{Flop(0.5), Flop(0.0)};
-  const double quad2 = 10.0;  // J^dagger E J for the 2x2 eikonal-weighted correlator matrix
-  // subtracted real: real blocks + Born tasks (soft with the eikonal form, collinear,
-  // spin-correlated for g g: both polarised gluons at the one collinear kinematics)
+  // Born values of the counterterms: soft (plain and with the eikonal-weighted correlator
+  // matrix), collinear (plain and, for g g, polarised along the emission's direction)
+  const Couplings cp{1.2, 0.3, 173.0};
+  const Flop E[4] = {Flop(1.0), Flop(2.0), Flop(2.0), Flop(1.0)};
+  const Inv22<Flop> k = inv22<Flop>(p, Flop(173.0));
+  const BornGG<Flop> b2 = born_gg(k, cp);
+  g_ops = 0;
+  born_gg_matrix(b2, E);
+  const double matrix_gg = (double)g_ops;
+  g_ops = 0;
+  born_uu_matrix(Flop(1.0), E);
+  const double matrix_uu = (double)g_ops;
+  g_ops = 0;
+  born_gg_polarised(k, b2, Flop(50.0), cp);
+  const double polarised = (double)g_ops;
+  const double soft_gg = born_ops<P_GG_TT>(p) + matrix_gg, coll_gg = born_ops<P_GG_TT>(p) + polarised;
+  const double soft_uu = born_ops<P_UU_TT>(p) + matrix_uu, coll_uu = born_ops<P_UU_TT>(p);
+  // subtracted real: real blocks and Born values; the collinear term of each g g sector adds
+  // its plain and its polarised Born with the splitting kernels (the second sector's sum is
+  // not part of a single configuration)
   const double real_ee = born_ops<P_EE_UUG>(p) + 2 * born_ops<P_EE_UU>(p);
-  const double real_gg = born_ops<P_GG_TTG>(p) + born_ops<P_GG_TT>(p) + 8 * quad2 + born_ops<P_GG_TT>(p) +
-                         block_ops<P_GG_TT>(p, 2, &e, 0) + block_ops<P_GG_TT>(p, 1, &e, 1);
-  const double real_uu = born_ops<P_UU_TTG>(p) + born_ops<P_UU_TT>(p) + 8 * quad2 + born_ops<P_UU_TT>(p);
+  const double real_gg = born_ops<P_GG_TTG>(p) + soft_gg + coll_gg + 3;
+  const double real_uu = born_ops<P_UU_TTG>(p) + soft_uu + coll_uu;
   const double b[7] = {born_ops<P_EE_UU>(p),  born_ops<P_EE_UUG>(p), born_ops<P_GG_TT>(p), born_ops<P_GG_TTG>(p),
                        born_ops<P_GG_TTGG>(p), born_ops<P_UU_TT>(p), born_ops<P_UU_TTG>(p)};
   const int nh[7] = {16, 32, 16, 32, 64, 16, 32};
@@ -92,12 +112,8 @@ int main() {
               b[0], b[1], b[2], b[3], b[4], b[5], b[6]);
   std::printf(" \"real_subtracted_per_event\": {\"ee_uug\": %.0f, \"gg_ttg\": %.0f, \"uu_ttg\": %.0f},\n", real_ee,
               real_gg, real_uu);
-  // per-term queues: one Born configuration per lane -- soft (Born with the eikonal
-  // form), collinear (Born plus, for g g, the spin-correlated block of the one sector
-  // whose collinear term is active, delta <= 1), or a final-state sector's Born
-  const double soft_gg = born_ops<P_GG_TT>(p) + 8 * quad2,
-               coll_gg = born_ops<P_GG_TT>(p) + block_ops<P_GG_TT>(p, 2, &e, 0);
-  const double soft_uu = born_ops<P_UU_TT>(p) + 8 * quad2, coll_uu = born_ops<P_UU_TT>(p);
+  // per-term queues: one Born configuration -- soft, collinear (one sector), or a final-state
+  // sector's Born
   std::printf(" \"term_config_per_event\": {\"ee_uug\": [%.0f, %.0f], \"gg_ttg\": [%.0f, %.0f], "
               "\"uu_ttg\": [%.0f, %.0f]},\n", b[0], b[0], soft_gg, coll_gg, soft_uu, coll_uu);
   std::printf(" \"colour_sum_per_event\": {\"gg_ttgg\": %.0f}}\n", 32 * (4.0 * 24 * 24 + 4.0 * 24));

@@ -3,13 +3,11 @@
 // two compile in parallel).
 #include "me_kernels.cuh"
 namespace me {
-cudaError_t launch_terms_ee(int phase, bool mixed, const LaunchArgs& a, const TermBufs& tb, int* counts,
-                            cudaStream_t st) {
-  return launch_terms_one<P_EE_UUG>(phase, mixed, a, tb, counts, st);
+cudaError_t launch_terms_ee(bool mixed, const LaunchArgs& a, const TermBufs& tb, cudaStream_t st) {
+  return launch_terms_one<P_EE_UUG>(mixed, a, tb, st);
 }
-cudaError_t launch_terms_uu(int phase, bool mixed, const LaunchArgs& a, const TermBufs& tb, int* counts,
-                            cudaStream_t st) {
-  return launch_terms_one<P_UU_TTG>(phase, mixed, a, tb, counts, st);
+cudaError_t launch_terms_uu(bool mixed, const LaunchArgs& a, const TermBufs& tb, cudaStream_t st) {
+  return launch_terms_one<P_UU_TTG>(mixed, a, tb, st);
 }
 cudaError_t launch_cut_list(int pid, const LaunchArgs& a, int* list, int* listed, cudaStream_t st) {
   (void)cudaGetLastError();

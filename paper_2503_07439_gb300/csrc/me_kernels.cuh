@@ -63,7 +63,8 @@ struct KParams {
   Couplings cp;
   double avg_inv;       // 1 / (initial spin x colour average), x identical-particle factor
   double born_avg_inv;  // same for the underlying Born of a real process
-  double nlo_factor;    // Born -> Born * factor (n-body NLO entry), else 1
+  double tree_scale;    // |M|^2 at unit couplings -> weight: couplings x avg_inv x nlo_factor
+  double real_scale;    // half helicity sum of a real block at unit couplings -> |M|^2
   double xi_cut, delta; // FKS plus-distribution cut-offs
   double xi_thr, y_thr; // points with xi < xi_thr or 1-y < y_thr go to the FP64 path
   double me_eps;        // assumed relative error of a bulk-precision matrix element
@@ -103,12 +104,6 @@ __device__ __forceinline__ T colour_sum(const ColourTables* tab, const cx<T>* J)
   return s;
 }
 
-// J^dagger M J for a real symmetric 2x2 matrix M (row-major)
-template <typename T>
-__device__ __forceinline__ T quad2(const T* M, const cx<T>* J) {
-  return M[0] * norm2(J[0]) + M[3] * norm2(J[1]) + T(2) * M[1] * (J[0].re * J[1].re + J[0].im * J[1].im);
-}
-
 template <int LPE, typename T>
 __device__ __forceinline__ T group_sum(T v, unsigned mask) {
 #pragma unroll
@@ -126,15 +121,20 @@ __device__ __forceinline__ unsigned group_mask() {
   }
 }
 
-template <int NEXT>
-__device__ __forceinline__ void load_event(const double* __restrict__ p, long n, long i, r4<double>* k) {
+// legs 0 .. LEGS - 1 of an event with NEXT legs
+template <int NEXT, int LEGS>
+__device__ __forceinline__ void load_legs(const double* __restrict__ p, long n, long i, r4<double>* k) {
 #pragma unroll
-  for (int l = 0; l < NEXT; ++l) {
+  for (int l = 0; l < LEGS; ++l) {
     k[l].e = __ldg(p + (0L * NEXT + l) * n + i);
     k[l].x = __ldg(p + (1L * NEXT + l) * n + i);
     k[l].y = __ldg(p + (2L * NEXT + l) * n + i);
     k[l].z = __ldg(p + (3L * NEXT + l) * n + i);
   }
+}
+template <int NEXT>
+__device__ __forceinline__ void load_event(const double* __restrict__ p, long n, long i, r4<double>* k) {
+  load_legs<NEXT, NEXT>(p, n, i, k);
 }
 
 // ---------------------------------------------------------------- cuts
@@ -170,20 +170,12 @@ __device__ __forceinline__ bool pass_cuts(const r4<double>* k, const Cuts& c) {
 }
 
 // ---------------------------------------------------------------- tree |M|^2
-// float32 trees of 2 -> 2 processes fit 128 registers: 4 blocks per SM (16 warps) hide
-// their float64 preparation better than the 2 blocks of the heavier kernels
-// (gg -> t tbar Born: 0.122 against 0.132 ms per 2^20 points)
-template <int PID, typename T>
-constexpr int tree_min_blocks() {
-  return (Proc<PID>::NEXT == 4 && std::is_same<T, float>::value) ? 4 : ME_MINB;
-}
-
 // out[i] = wgt[i] * |M|^2(p_i) * nlo_factor.  `count` (optional): the number of events,
 // read on the device; `idx` (optional): the list of events to process (its length in
 // `count`).  Momenta have stride n either way.  (g g -> t tbar g g in float32 runs
 // k_tree_tc4 below instead.)
 template <int PID, typename T, int LPE>
-__global__ void __launch_bounds__(128, tree_min_blocks<PID, T>()) k_tree(const double* __restrict__ p, const double* __restrict__ wgt,
+__global__ void __launch_bounds__(128, ME_MINB) k_tree(const double* __restrict__ p, const double* __restrict__ wgt,
                                                        long n, double* __restrict__ out, KParams kp,
                                                        const int* __restrict__ idx, const int* __restrict__ count) {
   static_assert(!(PID == P_GG_TTGG && std::is_same<T, float>::value), "float g g -> t tbar g g runs k_tree_tc4");
@@ -197,16 +189,39 @@ __global__ void __launch_bounds__(128, tree_min_blocks<PID, T>()) k_tree(const d
   load_event<NEXT>(p, n, ev, k);
   // Algorithm 2: every point is evaluated, and zeroed below where it fails the cuts
   const bool pass = !kp.cut.mask || pass_cuts<PID>(k, kp.cut);
-  const Kin<PID, T> K = prepare<PID, T>(k, kp.cp);
+  const Couplings unit = unit_couplings(kp.cp);
+  const Kin<PID, T> K = prepare<PID, T>(k, unit);
   T acc = T(0);
   for (int b = lane; b < n_live_blocks<PID>(); b += LPE)
-    amplitude_block<PID, T>(K, live_block_hel<PID>(b), kp.cp,
+    amplitude_block<PID, T>(K, live_block_hel<PID>(b), unit,
                             [&](int, const cx<T>* J) { acc += colour_sum<PID, T>(kp.tab, J); });
   const double tot = 2.0 * (double)group_sum<LPE>(acc, group_mask<LPE>());
   if (lane == 0) {
     const double w = wgt ? wgt[ev] : 1.0;
-    out[ev] = pass ? w * tot * kp.avg_inv * kp.nlo_factor : 0.0;
+    out[ev] = pass ? w * tot * kp.tree_scale : 0.0;
   }
+}
+
+// The closed 2 -> 2 trees: one lane per event, bound by the momenta's DRAM traffic and, in
+// the float64 products, by the float64 pipe.  A call with 2^20 g g -> t tbar points: 113 us with the helicity
+// amplitudes (float32), 42 us here.
+template <int PID, typename T>
+__global__ void __launch_bounds__(256) k_tree_closed(const double* __restrict__ p, const double* __restrict__ wgt,
+                                                     long n, double* __restrict__ out, KParams kp,
+                                                     const int* __restrict__ idx, const int* __restrict__ count) {
+  const long gid = (long)blockIdx.x * blockDim.x + threadIdx.x;
+  const long nev = count ? (long)*count : n;
+  if (gid >= nev) return;
+  const long ev = idx ? (long)idx[gid] : gid;
+  r4<double> k[4];
+  if (PID == P_GG_TT && !kp.cut.mask) {
+    load_legs<4, 3>(p, n, ev, k);  // leg 3 enters the cuts only
+  } else {
+    load_event<4>(p, n, ev, k);
+  }
+  const bool pass = !kp.cut.mask || pass_cuts<PID>(k, kp.cut);
+  const double tot = (double)closed_sum<PID, T>(k, unit_couplings(kp.cp)) * kp.tree_scale;
+  out[ev] = pass ? (wgt ? wgt[ev] * tot : tot) : 0.0;
 }
 
 // ---------------------------------------------------------------- g g -> t tbar g g, float32, tensor cores
@@ -315,8 +330,8 @@ __global__ void __launch_bounds__(TC4_THREADS, 2) k_tree_tc4(const double* __res
     for (int l = 0; l < 6; ++l) k[l] = r4<double>{d[l][0], d[l][1], d[l][2], d[l][3]};
   }
   const TcColourB cb = tc_load_colour(kp.tab->C[PID]);
-  const Kin<PID, float> K = prepare<PID, float>(k, kp.cp);
-  const float g = (float)kp.cp.gs, mt = (float)kp.cp.mt;
+  const Kin<PID, float> K = prepare<PID, float>(k, unit_couplings(kp.cp));
+  const float g = 1.0f, mt = kp.cp.mtf;
   const r4<float>* q = K.q;
   const r4<float> kt = K.pl[2];
   constexpr int LEG[4] = {0, 1, 4, 5};
@@ -425,7 +440,7 @@ __global__ void __launch_bounds__(TC4_THREADS, 2) k_tree_tc4(const double* __res
       load_event<6>(p, n, ev, kc);
       pass = pass_cuts<P_GG_TTGG>(kc, kp.cut);
     }
-    out[ev] = pass ? w8 * tot * kp.avg_inv * kp.nlo_factor : 0.0;
+    out[ev] = pass ? w8 * tot * kp.tree_scale : 0.0;
   }
 }
 
@@ -587,20 +602,17 @@ __device__ __forceinline__ double eik(const r4<double>& a, const r4<double>& b, 
 // with the error scale of the stability test.  The LPE lanes of a group evaluate one
 // point together and all return the same result.
 //
-// W is linear in its matrix-element ingredients -- the real's helicity blocks R_b
-// (R = sum_b R_b) and the Born values of the counterterms (for initial-state sectors:
-// the eikonal-weighted soft Born E, the soft Born B_s, the collinear Born B_c and, for
-// g g, the two spin-correlated Borns B_p; for final-state sectors the Born B_j of each
-// sector) -- with float64 coefficients fixed by the FKS maps:  W = sum_i a_i v_i.  The
-// item rescue re-evaluates in float64 only the ingredients whose float32 error the
-// point's tolerance cannot absorb, and recombines W from the coefficients.
+// W is linear in the real matrix element R = sum_b R_b (helicity blocks) with float64
+// coefficients fixed by the FKS maps: W = a_R sum_b R_b + W_B, W_B the counterterms.  Their
+// Born values are closed forms of some 40 float64 operations, so they are evaluated in
+// float64 for every point, in every precision, and only the real's blocks have a
+// bulk-precision value.  The item rescue re-evaluates in float64 the blocks whose float32
+// error the point's tolerance cannot absorb, and recombines W.
 template <int PID>
 struct RealLayout {
-  static constexpr int NB = n_live_blocks<PID>();                                   // real's blocks
-  static constexpr int NBV = PID == P_EE_UUG ? 2 : (PID == P_GG_TTG ? 5 : 3);      // Born values
-  static constexpr int NI = NB + NBV;
+  static constexpr int NB = n_live_blocks<PID>();  // the real's blocks
 };
-constexpr int MAX_ITEMS = 9;
+constexpr int MAX_BLOCKS = 4;
 
 struct RealSubOut {
   double W;     // subtracted real, summed over sectors
@@ -610,11 +622,15 @@ struct RealSubOut {
   bool near;    // inside xi_thr / y_thr of an active counterterm
 };
 
-// Ingredients and coefficients of one point for the item rescue (group lane 0).
-struct RealItems {
-  double a[MAX_ITEMS];  // W = sum_i a_i v_i
-  double v[MAX_ITEMS];  // bulk-precision values: R blocks, then the Born values
-  double born_scale;    // error scale of the Born values together (as in RealSubOut::mag)
+// Everything of a point but the real matrix element.
+struct PointTerms {
+  double a_R;    // sum_j S_j, or 0 if the real fails its cuts
+  double w_born; // the counterterms (with their sign): W = a_R R + w_born
+  double mag_b;  // their error scale, |CT_coll| + |CT_soft - CT_softcoll| per sector
+  double y[2];
+  bool near;     // inside xi_thr / y_thr of an active counterterm
+  bool inside;   // inside the FKS domain
+  bool need[2];  // active Born configurations: soft, collinear (initial state); sector 1, 2
 };
 
 // Eikonal-weighted colour-correlation matrix of the soft counter-event (2x2, row-major):
@@ -639,196 +655,71 @@ __device__ __forceinline__ void isr_eikonal_matrix(const IsrKin& f, const KParam
     }
 }
 
-// Born values of the soft counter-event kb: vE = E-weighted correlated Born (multiplies
-// -4 g^2 / s in the soft limit), vS = plain Born.  Every sum ran over one helicity of
-// each flipped pair (|M(h)|^2 = |M(-h)|^2), hence the factor 2.
-template <int BPID, typename T, int LPE>
-__device__ __forceinline__ void isr_soft_pair(const r4<double>* kb, const double* E, const KParams& kp, int lane,
-                                              unsigned mask, double& vE, double& vS) {
-  const T Et[4] = {(T)E[0], (T)E[1], (T)E[2], (T)E[3]};
-  T aE = T(0), aS = T(0);
-  const Kin<BPID, T> KB = prepare<BPID, T>(kb, kp.cp);
-  for (int b = lane; b < n_live_blocks<BPID>(); b += LPE)
-    amplitude_block<BPID, T>(KB, live_block_hel<BPID>(b), kp.cp, [&](int, const cx<T>* J) {
-      aE += quad2(Et, J);
-      aS += colour_sum<BPID, T>(kp.tab, J);
-    });
-  const double bav = 2.0 * kp.born_avg_inv;
-  vE = (double)group_sum<LPE>(aE, mask) * bav;
-  vS = (double)group_sum<LPE>(aS, mask) * bav;
-}
-
-// Born values of the collinear counter-event kb: v[0] = B_c (plain), and for g g the
-// spin-correlated Borns v[1], v[2] with gluon 0 or 1 polarised along the transverse
-// direction (0, cos phi, sin phi, 0) of the emission.
-template <int BPID, typename T, int LPE>
-__device__ __forceinline__ void isr_coll_set(const r4<double>* kb, double cphi, double sphi, const KParams& kp,
-                                             int lane, unsigned mask, double* v, bool want0 = true,
-                                             bool want1 = true) {
-  c4<T> eperp;
-  eperp.v[0] = cx<T>{T(0), T(0)};
-  eperp.v[1] = cx<T>{(T)cphi, T(0)};
-  eperp.v[2] = cx<T>{(T)sphi, T(0)};
-  eperp.v[3] = cx<T>{T(0), T(0)};
-  T aC = T(0), aP[2] = {T(0), T(0)};
-  const Kin<BPID, T> KB = prepare<BPID, T>(kb, kp.cp);
-  for (int b = lane; b < n_live_blocks<BPID>(); b += LPE)
-    amplitude_block<BPID, T>(KB, live_block_hel<BPID>(b), kp.cp,
-                             [&](int, const cx<T>* J) { aC += colour_sum<BPID, T>(kp.tab, J); });
-  if constexpr (BPID == P_GG_TT) {
-    // polarised gluon 0; gluon 1 fixed to +, the heavy pair free (the flip covers the rest)
-    if (lane == 0 && want0)
-      amplitude_block<BPID, T>(
-          KB, 2, kp.cp, [&](int, const cx<T>* J) { aP[0] += colour_sum<BPID, T>(kp.tab, J); }, &eperp, 0);
-    // polarised gluon 1, gluon 0 fixed to +: sector 2's spin-correlated Born, at the
-    // same kinematics (invariant under the boost that relates the two sectors)
-    if (lane == 1 % LPE && want1)
-      amplitude_block<BPID, T>(
-          KB, 1, kp.cp, [&](int, const cx<T>* J) { aP[1] += colour_sum<BPID, T>(kp.tab, J); }, &eperp, 1);
-  }
-  const double bav = 2.0 * kp.born_avg_inv;
-  v[0] = (double)group_sum<LPE>(aC, mask) * bav;
-  if constexpr (BPID == P_GG_TT) {
-    v[1] = (double)group_sum<LPE>(aP[0], mask) * bav;
-    v[2] = (double)group_sum<LPE>(aP[1], mask) * bav;
-  }
-}
-
-// Born values of the initial-state counterterms: v[0] = E (eikonal-weighted soft Born),
-// v[1] = B_s (soft Born), v[2] = B_c (collinear Born), v[3], v[4] = B_p (spin-correlated
-// Borns, g g only).
-template <int PID, typename T, int LPE>
-__device__ __forceinline__ void isr_born_values(const IsrKin& f, const KParams& kp, int lane, unsigned mask,
-                                                double* v) {
-  constexpr int BPID = PID == P_GG_TTG ? P_GG_TT : P_UU_TT;
-  double E[4];
-  isr_eikonal_matrix<BPID>(f, kp, E);
-  isr_soft_pair<BPID, T, LPE>(f.soft, E, kp, lane, mask, v[0], v[1]);
-  // sector j's spin-correlated Born enters only where its collinear term is active (one
-  // sector at most for delta <= 1); where that is sector 2 alone, the beams are swapped
-  // (Bose symmetry of g g -> t tbar) so that every lane evaluates the gluon-0 block
-  const bool w0 = BPID == P_GG_TT && f.y[0] > 1.0 - kp.delta && f.cut_c[0];
-  const bool w1 = BPID == P_GG_TT && f.y[1] > 1.0 - kp.delta && f.cut_c[1];
-  const bool sw = w1 && !w0;
-  const r4<double> cb[4] = {sw ? f.coll[1] : f.coll[0], sw ? f.coll[0] : f.coll[1], f.coll[2], f.coll[3]};
-  isr_coll_set<BPID, T, LPE>(cb, f.cphi, f.sphi, kp, lane, mask, v + 2, w0 || sw, w1 && !sw);
-  if constexpr (BPID == P_GG_TT) {
-    if (sw) {
-      v[4] = v[3];
-      v[3] = 0.0;
-    }
-  }
-}
-
-// The Born |M|^2 of e+e- -> u ubar at kb (a final-state counterterm's Born).
-template <typename T, int LPE>
-__device__ __forceinline__ double fsr_born_one(const r4<double>* kb, const KParams& kp, int lane, unsigned mask) {
-  T aB = T(0);
-  const Kin<P_EE_UU, T> KB = prepare<P_EE_UU, T>(kb, kp.cp);
-  for (int b = lane; b < n_live_blocks<P_EE_UU>(); b += LPE)
-    amplitude_block<P_EE_UU, T>(KB, live_block_hel<P_EE_UU>(b), kp.cp,
-                                [&](int, const cx<T>* J) { aB += colour_sum<P_EE_UU, T>(kp.tab, J); });
-  return 2.0 * (double)group_sum<LPE>(aB, mask) * kp.born_avg_inv;
-}
-
-// Born values of the final-state counterterms: v[j] = the Born at sector j's kinematics.
-template <typename T, int LPE>
-__device__ __forceinline__ void fsr_born_values(const FsrKin& f, const KParams& kp, int lane, unsigned mask,
-                                                double* v) {
-#pragma unroll
-  for (int j = 0; j < 2; ++j) v[j] = fsr_born_one<T, LPE>(f.born[j], kp, lane, mask);
-}
-
-// One helicity block b of the real matrix element, colour-summed and averaged:
-// R = sum over the live blocks.
-template <int PID, typename T>
-__device__ __forceinline__ double real_block_value(const Kin<PID, T>& K, int b, const KParams& kp) {
-  T acc = T(0);
-  amplitude_block<PID, T>(K, live_block_hel<PID>(b), kp.cp, [&](int, const cx<T>* J) { acc += colour_sum<PID, T>(kp.tab, J); });
-  return 2.0 * (double)acc * kp.avg_inv;
-}
-
-// `items` (optional): filled with the coefficients and ingredient values on group lane 0
-// (every lane of the group must pass it or none).
-template <int PID, typename T, int LPE>
-__device__ __forceinline__ RealSubOut real_sub_event(const double* __restrict__ p, long n, long ev, const KParams& kp,
-                                                     int lane, unsigned mask, RealItems* items = nullptr) {
-  constexpr int NEXT = Proc<PID>::NEXT;
-  constexpr int NB = RealLayout<PID>::NB;
-  constexpr int NBL = (NB + LPE - 1) / LPE;  // real blocks per lane
-  r4<double> k[NEXT];
-  load_event<NEXT>(p, n, ev, k);
+// Counterterms, error scale and regions of one point, from its momenta k.
+template <int PID>
+__device__ __forceinline__ PointTerms point_terms(const r4<double>* k, const KParams& kp) {
+  PointTerms o{};
   const double rs = k[0].e + k[1].e, s = rs * rs;
   const double g2 = kp.cp.gs * kp.cp.gs;
   // Algorithm 2's cut of the real term, at the real point
   const double cR = (!kp.cut.mask || pass_cuts<PID>(k, kp.cut)) ? 1.0 : 0.0;
-
-  // real matrix element; lane l holds blocks l, l + LPE, ... (one copy of the block code:
-  // the loop is not unrolled)
-  double blk[NBL];
-  double mine = 0.0;
-  {
-    const Kin<PID, T> K = prepare<PID, T>(k, kp.cp);
-#pragma unroll 1
-    for (int i = 0; i < NBL; ++i) {
-      const int b = lane + i * LPE;
-      const double v = b < NB ? real_block_value<PID, T>(K, b, kp) : 0.0;
-      blk[i] = v;
-      mine += v;
-    }
-  }
-  const double R = group_sum<LPE>(mine, mask);
-
-  double W = 0.0, mag = 0.0;
-  double ysec[2] = {-1.0, -1.0};  // y_j of both sectors (collinear resolution of the flag)
-  double xi_pt = 0.0;             // the emission's energy fraction
-  bool near = false;
-  double a_R = 0.0, ab[RealLayout<PID>::NBV] = {};  // coefficients of R and of the Born values
-  double bv[RealLayout<PID>::NBV];
+  double xi_pt;
   if constexpr (PID == P_EE_UUG) {
     FsrKin f;
     fsr_map(k, f);
-    ysec[0] = f.y[0];
-    ysec[1] = f.y[1];
+    o.y[0] = f.y[0];
+    o.y[1] = f.y[1];
     xi_pt = f.xi;
-    fsr_born_values<T, LPE>(f, kp, lane, mask, bv);
-    const double* B = bv;
     // Algorithm 2's cuts: both counterterms of sector j at sector j's Born
     const bool cuts = kp.cut.mask != 0;
 #pragma unroll
     for (int j = 0; j < 2; ++j) {
+      const double B = closed_sum<P_EE_UU, double>(f.born[j], kp.cp) * kp.born_avg_inv;
       const double cB = (!cuts || pass_cuts<P_EE_UU>(f.born[j], kp.cut)) ? 1.0 : 0.0;
       const double th_s = f.xi < kp.xi_cut ? cB : 0.0;
       // soft: sum_{kl} w_kl B_kl with B_23 = B_32 = -C_F B (massless diagonal terms vanish)
       const double cs = (1.0 - f.y[j]) * 0.5 * (1.0 + f.y[j]) * f.K0 * (-(4.0 * g2 / s) * 2.0 * eik(f.born[j][2], f.born[j][3], f.qdir) * (-CF_));
       const double cc = f.K1 * (2.0 / (s * (1.0 - f.xi))) * 2.0 * g2 * CF_ * (1.0 + (1.0 - f.xi) * (1.0 - f.xi));
       const double csc = f.K0 * (2.0 / s) * 2.0 * g2 * 2.0 * CF_;
-      const double Gs = cs * B[j], Gc = cc * B[j], Gsc = csc * B[j];
       const double th_c = f.y[j] > 1.0 - kp.delta ? cB : 0.0;
       const double iden = 1.0 / (f.xi * f.xi * (1.0 - f.y[j]) * f.K[j]);
-      const double ct = (th_s * Gs + th_c * Gc - th_s * th_c * Gsc) * iden;
-      const double rsj = R * f.S[j] * cR;
-      W += rsj - ct;
-      // error scale: the real, the collinear term, and the soft pair (whose Borns are shared)
-      mag += fabs(rsj) + fabs(th_c * Gc * iden) + fabs(th_s * (Gs - th_c * Gsc) * iden);
-      near |= (th_s > 0.0 && f.xi < kp.xi_thr) || (th_c > 0.0 && 1.0 - f.y[j] < kp.y_thr);
-      a_R += f.S[j] * cR;
-      ab[j] = -(th_s * cs + th_c * cc - th_s * th_c * csc) * iden;
+      o.w_born -= (th_s * cs + th_c * cc - th_s * th_c * csc) * iden * B;
+      // error scale: the collinear term, and the soft pair (whose Borns are shared)
+      o.mag_b += (fabs(th_c * cc * iden) + fabs(th_s * (cs - th_c * csc) * iden)) * B;
+      o.near |= (th_s > 0.0 && f.xi < kp.xi_thr) || (th_c > 0.0 && 1.0 - f.y[j] < kp.y_thr);
+      o.a_R += f.S[j] * cR;
+      o.need[j] = th_s > 0.0 || th_c > 0.0;
     }
   } else {
     constexpr int BPID = PID == P_GG_TTG ? P_GG_TT : P_UU_TT;
     IsrKin f;
     isr_map(k, kp.cp.mt, f, kp.cut);
-    ysec[0] = f.y[0];
-    ysec[1] = f.y[1];
+    o.y[0] = f.y[0];
+    o.y[1] = f.y[1];
     xi_pt = f.xi;
-    isr_born_values<PID, T, LPE>(f, kp, lane, mask, bv);
+    // Born values: E-weighted and plain at the soft counter-event, plain (and, for g g, with
+    // the splitting gluon polarised along the emission's transverse direction) at the
+    // collinear one, of sector 1; sector 2's are the same (see IsrKin and the closed forms)
+    double E[4], vE, vS, Bc, Bp = 0.0;
+    isr_eikonal_matrix<BPID>(f, kp, E);
+    const Inv22<double> ks = inv22<double>(f.soft, kp.cp.mt), kc_ = inv22<double>(f.coll, kp.cp.mt);
+    if constexpr (BPID == P_GG_TT) {
+      const BornGG<double> bs = born_gg(ks, kp.cp), bc = born_gg(kc_, kp.cp);
+      vE = born_gg_matrix(bs, E);
+      vS = born_gg_colour(bs);
+      Bc = born_gg_colour(bc);
+      Bp = born_gg_polarised(kc_, bc, f.cphi * f.coll[2].x + f.sphi * f.coll[2].y, kp.cp) * kp.born_avg_inv;
+    } else {
+      const double d = 8.0 * g2 * g2, fs = d * born_qq(ks);
+      vE = born_uu_matrix(fs, E);
+      vS = 2.0 * fs;
+      Bc = 2.0 * d * born_qq(kc_);
+    }
+    vE *= kp.born_avg_inv;
+    vS *= kp.born_avg_inv;
+    Bc *= kp.born_avg_inv;
     // Algorithm 2's cuts (isr_map): soft and soft-collinear terms at the soft
     // counter-event, the collinear term of sector j at sector j's collinear counter-event
-    const double x2R = -(4.0 * g2 / s) * bv[0];
-    const double Bs = bv[1], Bc = bv[2];
-    const double Bp[2] = {BPID == P_GG_TT ? bv[3 % RealLayout<PID>::NBV] : 0.0,
-                          BPID == P_GG_TT ? bv[4 % RealLayout<PID>::NBV] : 0.0};
     const double xi = f.xi, z = 1.0 - xi, iz = f.iz, is2 = 2.0 / s;
     const double th_s = xi < kp.xi_cut && f.cut_s ? 1.0 : 0.0;
     // 1 / (xi^2 (1 - y_j) K) of both sectors from one reciprocal
@@ -838,39 +729,79 @@ __device__ __forceinline__ RealSubOut real_sub_event(const double* __restrict__ 
     // d xi P / d B_c, d xi P / d B_p, d xi P_0 / d B_s of the splitting kernels
     const double kc = BPID == P_GG_TT ? 2.0 * CA_ * (z + xi * xi * z) : CF_ * (1.0 + z * z);
     const double kp_ = BPID == P_GG_TT ? 2.0 * CA_ * 2.0 * (xi * xi * iz) : 0.0;
-    const double ks = BPID == P_GG_TT ? 2.0 * CA_ : 2.0 * CF_;
+    const double kq = BPID == P_GG_TT ? 2.0 * CA_ : 2.0 * CF_;
+    const double xiP = kc * Bc + kp_ * Bp;
 #pragma unroll
     for (int j = 0; j < 2; ++j) {
-      const double Gs = (1.0 - f.y[j]) * f.S[j] * f.K0 * x2R;
-      const double xiP = kc * Bc + kp_ * Bp[j];
-      const double xiP0 = ks * Bs;
+      const double Gs = (1.0 - f.y[j]) * f.S[j] * f.K0 * (-(4.0 * g2 / s) * vE);
       const double Gc = f.K * is2 * iz * 2.0 * g2 * xiP;
-      const double Gsc = f.K0 * is2 * 2.0 * g2 * xiP0;
+      const double Gsc = f.K0 * is2 * 2.0 * g2 * (kq * vS);
       const double th_c = f.y[j] > 1.0 - kp.delta ? 1.0 : 0.0;  // soft-collinear term's
       const double th_cc = f.cut_c[j] ? th_c : 0.0;             // collinear term's
-      const double ct = (th_s * Gs + th_cc * Gc - th_s * th_c * Gsc) * iden[j];
-      const double rsj = R * f.S[j] * cR;
-      W += rsj - ct;
-      // error scale: the real, the collinear term, and the soft pair (whose Borns are shared)
-      mag += fabs(rsj) + fabs(th_cc * Gc * iden[j]) + fabs(th_s * (Gs - th_c * Gsc) * iden[j]);
-      near |= (th_s > 0.0 && xi < kp.xi_thr) || ((th_cc > 0.0 || th_s * th_c > 0.0) && 1.0 - f.y[j] < kp.y_thr);
-      a_R += f.S[j] * cR;
-      const double gcj = th_cc * f.K * is2 * iz * 2.0 * g2 * iden[j];
-      ab[0] -= th_s * (1.0 - f.y[j]) * f.S[j] * f.K0 * (-(4.0 * g2 / s)) * iden[j];
-      ab[1] += th_s * th_c * f.K0 * is2 * 2.0 * g2 * ks * iden[j];
-      ab[2] -= gcj * kc;
-      if constexpr (BPID == P_GG_TT) ab[3 + j] = -gcj * kp_;
+      o.w_born -= (th_s * Gs + th_cc * Gc - th_s * th_c * Gsc) * iden[j];
+      // error scale: the collinear term, and the soft pair (whose Borns are shared)
+      o.mag_b += fabs(th_cc * Gc * iden[j]) + fabs(th_s * (Gs - th_c * Gsc) * iden[j]);
+      o.near |= (th_s > 0.0 && xi < kp.xi_thr) || ((th_cc > 0.0 || th_s * th_c > 0.0) && 1.0 - f.y[j] < kp.y_thr);
+      o.a_R += f.S[j] * cR;
+      o.need[1] |= th_cc > 0.0;
     }
+    o.need[0] = th_s > 0.0;
   }
   // A point on the boundary of the FKS domain -- no emitted energy (xi = 0), all of it
   // (xi = 1), or the emission exactly along a sector's reference direction (y_j = 1) --
   // has measure zero and no defined subtracted weight (1 / (xi^2 (1 - y)) diverges):
   // weight 0, and it is not re-evaluated.  The comparisons are false for NaN.
-  if (!(xi_pt > 0.0 && xi_pt < 1.0 && 1.0 - ysec[0] > 0.0 && 1.0 - ysec[1] > 0.0)) {
-    W = 0.0;
-    mag = 0.0;
-    near = false;
+  o.inside = xi_pt > 0.0 && xi_pt < 1.0 && 1.0 - o.y[0] > 0.0 && 1.0 - o.y[1] > 0.0;
+  return o;
+}
+
+// One helicity block b of the real matrix element, colour-summed and averaged:
+// R = sum over the live blocks.
+template <int PID, typename T>
+__device__ __forceinline__ double real_block_value(const Kin<PID, T>& K, int b, const KParams& kp) {
+  T acc = T(0);
+  amplitude_block<PID, T>(K, live_block_hel<PID>(b), unit_couplings(kp.cp),
+                          [&](int, const cx<T>* J) { acc += colour_sum<PID, T>(kp.tab, J); });
+  return (double)acc * kp.real_scale;
+}
+
+// W and its error scale from a point's terms and R.
+__device__ __forceinline__ RealSubOut combine_point(const PointTerms& t, double R) {
+  if (!t.inside) return RealSubOut{0.0, 0.0, 0.0, {t.y[0], t.y[1]}, false};
+  const double r = t.a_R * R, magR = fabs(r);
+  return RealSubOut{r + t.w_born, magR + t.mag_b, magR, {t.y[0], t.y[1]}, t.near};
+}
+
+// `items` (optional): filled with the terms and block values on group lane 0 (every lane of
+// the group must pass it or none).
+struct RealItems {
+  PointTerms t;
+  double v[MAX_BLOCKS];  // bulk-precision values of the R blocks
+};
+template <int PID, typename T, int LPE>
+__device__ __forceinline__ RealSubOut real_sub_event(const double* __restrict__ p, long n, long ev, const KParams& kp,
+                                                     int lane, unsigned mask, RealItems* items = nullptr) {
+  constexpr int NEXT = Proc<PID>::NEXT;
+  constexpr int NB = RealLayout<PID>::NB;
+  constexpr int NBL = (NB + LPE - 1) / LPE;  // real blocks per lane
+  r4<double> k[NEXT];
+  load_event<NEXT>(p, n, ev, k);
+  // real matrix element; lane l holds blocks l, l + LPE, ... (one copy of the block code:
+  // the loop is not unrolled)
+  double blk[NBL];
+  double mine = 0.0;
+  {
+    const Kin<PID, T> K = prepare<PID, T>(k, unit_couplings(kp.cp));
+#pragma unroll 1
+    for (int i = 0; i < NBL; ++i) {
+      const int b = lane + i * LPE;
+      const double v = b < NB ? real_block_value<PID, T>(K, b, kp) : 0.0;
+      blk[i] = v;
+      mine += v;
+    }
   }
+  const double R = group_sum<LPE>(mine, mask);
+  const PointTerms t = point_terms<PID>(k, kp);
   if (items) {
     // every block value to lane 0 (block b lives on lane b % LPE, slot b / LPE)
 #pragma unroll
@@ -881,17 +812,10 @@ __device__ __forceinline__ RealSubOut real_sub_event(const double* __restrict__ 
         if (i == b / LPE) x = blk[i];
       if constexpr (LPE > 1) x = __shfl_sync(mask, x, b % LPE, LPE);
       items->v[b] = x;
-      items->a[b] = a_R;
     }
-#pragma unroll
-    for (int t = 0; t < RealLayout<PID>::NBV; ++t) {
-      items->v[NB + t] = bv[t];
-      items->a[NB + t] = ab[t];
-    }
-    items->born_scale = mag - fabs(R) * a_R;
+    items->t = t;
   }
-  const double magR = mag > 0.0 ? fabs(R) * a_R : 0.0;
-  return RealSubOut{W, mag, magR, {ysec[0], ysec[1]}, near};
+  return combine_point(t, R);
 }
 
 // Stability test of a bulk-precision result: the error of W is ~ me_eps x (error
@@ -903,32 +827,38 @@ __device__ __forceinline__ double error_growth(const RealSubOut& r) {
   const float rho = fmaxf((float)fmin(1.0 - r.y[0], 1.0 - r.y[1]), 1e-30f);
   return 1.0 + (double)sqrtf(0.01f / rho);
 }
-__device__ __forceinline__ bool unstable_point(const RealSubOut& r, const KParams& kp) {
-  const double g = error_growth(r);
+__device__ __forceinline__ bool unstable_point(const RealSubOut& r, const KParams& kp, double g) {
   return r.near || !((r.magR * g + (r.mag - r.magR)) * kp.me_eps <= kp.tol * fabs(r.W));
 }
 
-// Items of a flagged point to re-evaluate in float64: bit b < NB for the real's block
-// b, bit NB for the Born values together.  Largest error scale first, until the scale
-// of the items left in float32, times the bulk-precision error per unit scale, is
-// within kp.item_budget x tol |W|.  Points inside the thresholds take every item.
+__device__ __forceinline__ bool unstable_point(const RealSubOut& r, const KParams& kp) {
+  return unstable_point(r, kp, error_growth(r));
+}
+
+// Blocks of a flagged point to re-evaluate in float64 (bit b: block b).  Largest error scale
+// first, until the scale of what is left, times the bulk-precision error per unit scale, is
+// within kp.item_budget x tol |W|.  The Born part is float64 already but keeps its place in
+// the order: a point whose flag came from it alone takes no block, and what the part no
+// longer adds to the error is a margin.  Points inside the thresholds take every block.
 template <int PID>
-__device__ __forceinline__ unsigned rescue_mask(const RealSubOut& r, const RealItems& it, const KParams& kp) {
+__device__ __forceinline__ unsigned rescue_mask(const RealSubOut& r, double a_R, const double* v, const KParams& kp,
+                                                double grow) {
   constexpr int NB = RealLayout<PID>::NB;
-  constexpr unsigned all = (1u << (NB + 1)) - 1u;
+  constexpr unsigned all = (1u << NB) - 1u;
+  if (a_R == 0.0) return 0;  // the real failed its cuts
   if (r.near) return all;
   double e[NB + 1];
   double rest = 0.0;
 #pragma unroll
-  for (int b = 0; b < NB; ++b) rest += (e[b] = fabs(it.a[b] * it.v[b]));
-  const double grow = error_growth(r);
-  rest += (e[NB] = fabs(it.born_scale) / grow);  // no growth for the Born part (see above)
+  for (int b = 0; b < NB; ++b) rest += (e[b] = fabs(a_R * v[b]));
+  rest += (e[NB] = (r.mag - r.magR) / grow);  // no growth for the Born part (unstable_point)
+  if (!(rest == rest)) return all;
   const double budget = kp.item_budget * kp.tol * fabs(r.W) / (grow * kp.me_eps);
   unsigned m = 0;
 #pragma unroll
   for (int k = 0; k <= NB; ++k) {
-    if (!(rest > budget)) break;  // NaN or over budget: keep going
-    int pick = -1;
+    if (rest <= budget) break;
+    int pick = 0;
     double best = -1.0;
 #pragma unroll
     for (int b = 0; b <= NB; ++b)
@@ -936,40 +866,81 @@ __device__ __forceinline__ unsigned rescue_mask(const RealSubOut& r, const RealI
         best = e[b];
         pick = b;
       }
-    if (pick < 0) break;
     m |= 1u << pick;
     rest -= best;
   }
-  return m ? m : all;
+  return m & all;
 }
 
-// Buffers of the item rescue (structure of arrays, capacity `cap` points):
-// ev[slot], mask[slot], a[i * cap + slot], v[i * cap + slot]; the item lists hold
-// slot * 4 + b (real blocks) and slot (Born values); count[0] = flagged points,
-// count[2] = real-block items, count[3] = Born items (count[1] is the queued kernel's
-// tile counter).
+// Buffers of the item rescue (structure of arrays, capacity `cap` points): a record for
+// each flagged point with blocks to re-evaluate -- ev[slot], pend[slot] (its blocks still
+// to come), a[slot] = a_R, a[cap + slot] = W_B, v[b * cap + slot] -- and the item list,
+// slot * 4 + b.  Counters (`counts`): [0] flagged points, [2] blocks, [3] flagged points with
+// an active counterterm, [4] / [5] their active Born configurations (soft, collinear, or
+// sector 1, 2), [6] records; [1] is the queued kernel's tile counter.
 struct ItemBufs {
   int* ev;
-  int* mask;
+  int* pend;
   double* a;
   double* v;
   int* list_r;
-  int* list_b;
   long cap;
 };
+
+// Record a flagged point and list its blocks: called by the flagged lanes of a warp together
+// (one atomic per warp and counter).
+template <int PID>
+__device__ __forceinline__ void append_flagged(int* __restrict__ counts, const ItemBufs& ib, long ev, double a_R,
+                                               double w_born, const bool* need, const double* v, unsigned m) {
+  constexpr int NB = RealLayout<PID>::NB;
+  const unsigned am = __activemask();
+  const int wl = threadIdx.x & 31, leader = __ffs(am) - 1;
+  const unsigned lt = (1u << wl) - 1u;
+  const unsigned rec = __ballot_sync(am, m != 0);
+  const unsigned c0 = __ballot_sync(am, need[0]), c1 = __ballot_sync(am, need[1]);
+  unsigned bal[NB];
+  int tot = 0;
+#pragma unroll
+  for (int b = 0; b < NB; ++b) tot += __popc(bal[b] = __ballot_sync(am, m >> b & 1u));
+  int base = 0, rbase = 0;
+  if (wl == leader) {
+    atomicAdd(counts, __popc(am));
+    if (c0 | c1) atomicAdd(counts + 3, __popc(c0 | c1));
+    if (c0) atomicAdd(counts + 4, __popc(c0));
+    if (c1) atomicAdd(counts + 5, __popc(c1));
+    if (rec) {
+      base = atomicAdd(counts + 6, __popc(rec));
+      rbase = atomicAdd(counts + 2, tot);
+    }
+  }
+  const int slot = __shfl_sync(am, base, leader) + __popc(rec & lt);
+  rbase = __shfl_sync(am, rbase, leader);
+  if (m) {
+    ib.ev[slot] = (int)ev;
+    ib.pend[slot] = __popc(m);
+    ib.a[slot] = a_R;
+    ib.a[ib.cap + slot] = w_born;
+#pragma unroll
+    for (int b = 0; b < NB; ++b) ib.v[b * ib.cap + slot] = v[b];
+  }
+  // ordered by block, then lane
+#pragma unroll
+  for (int b = 0; b < NB; ++b) {
+    if (m >> b & 1u) ib.list_r[rbase + __popc(bal[b] & lt)] = slot * 4 + b;
+    rbase += __popc(bal[b]);
+  }
+}
 
 // out[i] = wgt[i] * W(p_i).  In the bulk precision with kp.flag_unstable set, the
 // points failing the stability test are appended to resc_list; the float64 launch over
 // that list (idx, count) re-evaluates them.  With kp.item_rescue set as well, each
-// flagged point gets a record (coefficients, bulk-precision values, item mask) and its
-// float64 items are appended to the item lists instead (warp-aggregated appends).
+// flagged point gets a record and its float64 blocks are listed instead.
 template <int PID, typename T, int LPE>
 __global__ void __launch_bounds__(128, ME_MINB) k_real_sub(const double* __restrict__ p, const double* __restrict__ wgt,
                                                   long n, double* __restrict__ out, KParams kp,
                                                   const int* __restrict__ idx, const int* __restrict__ count,
                                                   int* __restrict__ resc_list, int* __restrict__ resc_count,
                                                   ItemBufs ib) {
-  constexpr int NB = RealLayout<PID>::NB, NI = RealLayout<PID>::NI;
   const long gid = ((long)blockIdx.x * blockDim.x + threadIdx.x) / LPE;
   const int lane = threadIdx.x % LPE;
   const long nev = count ? (long)*count : n;
@@ -985,96 +956,38 @@ __global__ void __launch_bounds__(128, ME_MINB) k_real_sub(const double* __restr
         const int slot = atomicAdd(resc_count, 1);
         resc_list[slot] = (int)ev;
       } else {
-        const unsigned m = rescue_mask<PID>(r, it, kp);
-        // warp-aggregated appends over the flagged group leaders of this warp
-        const unsigned am = __activemask();
-        const int wl = threadIdx.x & 31, leader = __ffs(am) - 1;
-        const unsigned lt = (1u << wl) - 1u;
-        int base = 0;
-        if (wl == leader) base = atomicAdd(resc_count, __popc(am));
-        const int slot = __shfl_sync(am, base, leader) + __popc(am & lt);
-        ib.ev[slot] = (int)ev;
-        ib.mask[slot] = (int)m;
-#pragma unroll
-        for (int i = 0; i < NI; ++i) {
-          ib.a[i * ib.cap + slot] = it.a[i];
-          ib.v[i * ib.cap + slot] = it.v[i];
-        }
-        // real-block items, ordered by block then lane within the warp
-        unsigned bal[NB];
-        int tot = 0;
-#pragma unroll
-        for (int b = 0; b < NB; ++b) tot += __popc(bal[b] = __ballot_sync(am, m >> b & 1u));
-        int rbase = 0;
-        if (wl == leader) rbase = atomicAdd(resc_count + 2, tot);
-        rbase = __shfl_sync(am, rbase, leader);
-#pragma unroll
-        for (int b = 0; b < NB; ++b) {
-          if (m >> b & 1u) ib.list_r[rbase + __popc(bal[b] & lt)] = slot * 4 + b;
-          rbase += __popc(bal[b]);
-        }
-        const unsigned bb = __ballot_sync(am, m >> NB & 1u);
-        int bbase = 0;
-        if (wl == leader) bbase = atomicAdd(resc_count + 3, __popc(bb));
-        bbase = __shfl_sync(am, bbase, leader);
-        if (m >> NB & 1u) ib.list_b[bbase + __popc(bb & lt)] = slot;
+        append_flagged<PID>(resc_count, ib, ev, it.t.a_R, it.t.w_born, it.t.need, it.v,
+                            rescue_mask<PID>(r, it.t.a_R, it.v, kp, error_growth(r)));
       }
     }
   }
 }
 
-// Float64 evaluation of the rescue items (grid-stride over the item lists, counts read
-// on the device): blockIdx.y = 0 takes real blocks, 1 takes the Born values.  Every
-// item writes its value into its point's record.
+// Float64 evaluation of the listed blocks (grid-stride over the list, its length read on the
+// device).  The lane that delivers a record's last block recombines its W: the values are
+// published with a fence before the count, and read from L2 after it.
 template <int PID>
-__global__ void __launch_bounds__(128, ME_MINB) k_rescue_items(const double* __restrict__ p, long n, KParams kp,
+__global__ void __launch_bounds__(128, ME_MINB) k_rescue_items(const double* __restrict__ p,
+                                                               const double* __restrict__ wgt, long n,
+                                                               double* __restrict__ out, KParams kp,
                                                                const int* __restrict__ counts, ItemBufs ib) {
   constexpr int NEXT = Proc<PID>::NEXT, NB = RealLayout<PID>::NB;
-  const long stride = (long)gridDim.x * blockDim.x;
-  if (blockIdx.y == 0) {
-    const long nit = counts[2];
-    for (long t = (long)blockIdx.x * blockDim.x + threadIdx.x; t < nit; t += stride) {
-      const int item = ib.list_r[t], slot = item >> 2, b = item & 3;
-      r4<double> k[NEXT];
-      load_event<NEXT>(p, n, ib.ev[slot], k);
-      const Kin<PID, double> K = prepare<PID, double>(k, kp.cp);
-      ib.v[b * ib.cap + slot] = real_block_value<PID, double>(K, b, kp);
-    }
-  } else {
-    const long nit = counts[3];
-    const unsigned self = 1u << (threadIdx.x & 31u);
-    for (long t = (long)blockIdx.x * blockDim.x + threadIdx.x; t < nit; t += stride) {
-      const int slot = ib.list_b[t];
-      r4<double> k[NEXT];
-      load_event<NEXT>(p, n, ib.ev[slot], k);
-      double bv[RealLayout<PID>::NBV];
-      if constexpr (PID == P_EE_UUG) {
-        FsrKin f;
-        fsr_map(k, f);
-        fsr_born_values<double, 1>(f, kp, 0, self, bv);
-      } else {
-        IsrKin f;
-        isr_map(k, kp.cp.mt, f, Cuts{});  // the cuts are in the coefficients already
-        isr_born_values<PID, double, 1>(f, kp, 0, self, bv);
-      }
-#pragma unroll
-      for (int i = 0; i < RealLayout<PID>::NBV; ++i) ib.v[(NB + i) * ib.cap + slot] = bv[i];
-    }
-  }
-}
-
-// W of every flagged point from its coefficients and values (float64 where re-evaluated).
-template <int PID>
-__global__ void k_rescue_combine(const double* __restrict__ wgt, double* __restrict__ out,
-                                 const int* __restrict__ counts, ItemBufs ib) {
-  constexpr int NI = RealLayout<PID>::NI;
-  const long m = counts[0];
-  for (long slot = (long)blockIdx.x * blockDim.x + threadIdx.x; slot < m; slot += (long)gridDim.x * blockDim.x) {
-    double W = 0.0;
-#pragma unroll
-    for (int i = 0; i < NI; ++i) W += ib.a[i * ib.cap + slot] * ib.v[i * ib.cap + slot];
+  const long stride = (long)gridDim.x * blockDim.x, nit = counts[2];
+  for (long t = (long)blockIdx.x * blockDim.x + threadIdx.x; t < nit; t += stride) {
+    const int item = ib.list_r[t], slot = item >> 2, b = item & 3;
     const int ev = ib.ev[slot];
-    out[ev] = (wgt ? wgt[ev] : 1.0) * W;
+    r4<double> k[NEXT];
+    load_event<NEXT>(p, n, ev, k);
+    const Kin<PID, double> K = prepare<PID, double>(k, unit_couplings(kp.cp));
+    __stcg(ib.v + b * ib.cap + slot, real_block_value<PID, double>(K, b, kp));
+    __threadfence();
+    if (atomicSub(ib.pend + slot, 1) == 1) {
+      __threadfence();
+      double R = 0.0;
+#pragma unroll
+      for (int i = 0; i < NB; ++i) R += __ldcg(ib.v + i * ib.cap + slot);
+      out[ev] = (wgt ? wgt[ev] : 1.0) * (ib.a[slot] * R + ib.a[ib.cap + slot]);
+    }
   }
 }
 
@@ -1141,40 +1054,20 @@ __global__ void __launch_bounds__(QT, ME_MINB) k_real_sub_queued(const double* _
 // ---------------------------------------------------------------- per-term queues
 // The variant of Algorithm 2 discussed after it (Sec. 4.3): rather than evaluating every
 // term of every point and masking the ones whose cuts fail, a float64 pass (k_terms) maps
-// each point, decides its cuts and counterterm regions, stores the coefficients of W =
-// sum_i a_i v_i, and queues only the amplitudes the point needs -- the real's helicity
-// blocks if the real passes its cuts, the soft Born set if the soft term is active and its
-// counter-event passes, the collinear Born set likewise, each with its counter-event
-// momenta.  k_term_items then evaluates every queued amplitude, one lane each, in one
-// launch over all queues; k_terms_combine recombines W (and, in mixed precision, applies
-// the stability test and queues the float64 items of the flagged points, which the same
-// item kernel evaluates in float64; k_terms_final recombines those).
-//
-// Value layout per record: v[b], b < NB, the real's blocks; then the Born values: initial
-// state v[NB] = E, v[NB+1] = B_s (set 0, soft counter-event), v[NB+2] = B_c, v[NB+3],
-// v[NB+4] = B_p (set 1, collinear counter-event); final state v[NB+j] = B_j (set j).
+// each point, decides its cuts and counterterm regions, adds up its counterterms (closed
+// forms, evaluated where they are needed) and queues the real matrix element if it passes
+// its cuts; points without one are finished there.  k_term_reals evaluates the queued reals
+// one lane each and combines W, in mixed precision with the stability test and the records
+// and float64 items of the flagged points, as the masked evaluation (k_rescue_items follows).
+// A queued real carries 40 B: its point, a_R, W_B, the Born error scale, and the error
+// growth (negative for points inside the thresholds) with the active configurations.
 struct TermBufs {
-  int* ev;      // [cap] point of the record
-  int* flags;   // [cap] bit 0: inside xi_thr / y_thr of an active counterterm
-  float* grow;  // [cap] error growth factor of the stability test
-  double* a;    // [MAX_ITEMS][cap] coefficients
-  double* v;    // [MAX_ITEMS][cap] values
-  double* m;    // [6][cap] error-scale coefficients of the Born values (term_born_scale)
-  int* cfg;     // [2][cap] the record's Born configurations, -1 for none
-  double* bp;   // [16][2 cap] configuration momenta, index (component * 4 + leg)
-  double* bx;   // [4][2 cap] set 0 (initial state): eikonal correlator matrix; set 1: cos, sin phi
-  int* bslot;   // [2 cap] record slot | set << 30
-  int* q_real;  // [cap] records whose real is evaluated (every block in one lane; Born
-                //   configurations are queued as they are stored: set 0 at 0 .. cnt[TC_QB] - 1,
-                //   set 1 at cap .. cap + cnt[TC_QB1] - 1, so that a warp runs one kind)
-  int* r_real;  // [4 cap] float64 rescue: real blocks, slot * 4 + b
-  int* r_born;  // [2 cap] float64 rescue: Born configurations, set 0 from 0, set 1 from cap
-  int* flagged; // [cap] records that failed the stability test
-  int* cnt;     // [8]: records, q_real, set-0 configurations, flagged, r_real, r_born set 0,
-                //   set-1 configurations, r_born set 1
+  int* ev;      // [cap] point of the record; bits 29, 30: active Born configurations
+  float* grow;  // [cap] error growth factor of the stability test, negative: near
+  double* a;    // [3][cap] a_R, W_B, Born error scale
+  int* cnt;     // records
   long cap;
 };
-enum : int { TC_REC = 0, TC_QR = 1, TC_QB = 2, TC_FLAG = 3, TC_RR = 4, TC_RB = 5, TC_QB1 = 6, TC_RB1 = 7 };
 
 // Reserve `c` consecutive entries of counter `ctr` for each lane of a full warp (every
 // lane calls it; c = 0 reserves nothing): one atomic per warp.  Returns the lane's base.
@@ -1193,40 +1086,15 @@ __device__ __forceinline__ int warp_reserve(int* ctr, int c) {
   return base + incl - c;
 }
 
-// Error scale of the Born values of a record (as RealSubOut::mag without the real):
-// initial state sum_j |m_2j E + m_2j+1 B_s| + |m_4+j B_c + cp_j B_p,j| with cp_j =
-// -a[NB+3+j] (g g); final state sum_j m_j |B_j|.
+// Float64 pass of the per-term queues: one thread per point.  `pc` (optional, device memory,
+// same layout as p): the momenta are copied there, so that the item kernels read device
+// memory when p is host memory read in place over the CPU-GPU link (p is then read once).
 template <int PID>
-__device__ __forceinline__ double term_born_scale(const TermBufs& tb, long slot) {
-  constexpr int NB = RealLayout<PID>::NB;
-  const long c = tb.cap;
-  const double* v = tb.v + NB * c + slot;
-  const double* m = tb.m + slot;
-  if constexpr (PID == P_EE_UUG) {
-    return m[0] * fabs(v[0]) + m[c] * fabs(v[c]);
-  } else {
-    const double E = v[0], Bs = v[c], Bc = v[2 * c];
-    double sc = fabs(m[0] * E + m[c] * Bs) + fabs(m[2 * c] * E + m[3 * c] * Bs);
-    if constexpr (PID == P_GG_TTG) {
-      const double* a = tb.a + NB * c + slot;
-      sc += fabs(m[4 * c] * Bc - a[3 * c] * v[3 * c]) + fabs(m[5 * c] * Bc - a[4 * c] * v[4 * c]);
-    } else {
-      sc += fabs(m[4 * c] * Bc) + fabs(m[5 * c] * Bc);
-    }
-    return sc;
-  }
-}
-
-// Float64 pass of the per-term queues: one thread per point (the counter-event maps,
-// the cuts of every term, the coefficients, and the queues).  Points with nothing left
-// to evaluate get weight 0 here.  `pc` (optional, device memory, same layout as p): the
-// momenta are copied there, so that the item kernels read device memory when p is host
-// memory read in place over the CPU-GPU link (p is then read once).
-template <int PID>
-__global__ void __launch_bounds__(128) k_terms(const double* __restrict__ p, long n, double* __restrict__ out,
-                                               KParams kp, const int* __restrict__ count, TermBufs tb,
+__global__ void __launch_bounds__(128) k_terms(const double* __restrict__ p, const double* __restrict__ wgt, long n,
+                                               double* __restrict__ out, KParams kp, const int* __restrict__ count,
+                                               TermBufs tb, int* __restrict__ counts, ItemBufs ib,
                                                double* __restrict__ pc) {
-  constexpr int NEXT = Proc<PID>::NEXT, NB = RealLayout<PID>::NB, NBV = RealLayout<PID>::NBV;
+  constexpr int NEXT = Proc<PID>::NEXT;
   const long i = (long)blockIdx.x * blockDim.x + threadIdx.x;
   const long nev = count ? (long)*count : n;
   const bool act = i < nev;
@@ -1246,328 +1114,57 @@ __global__ void __launch_bounds__(128) k_terms(const double* __restrict__ p, lon
 #pragma unroll
     for (int l = 0; l < NEXT; ++l) k[l] = r4<double>{1.0, 0.0, 0.0, 0.0};
   }
-  const double rs = k[0].e + k[1].e, s = rs * rs;
-  const double g2 = kp.cp.gs * kp.cp.gs;
-  const double cR = (!kp.cut.mask || pass_cuts<PID>(k, kp.cut)) ? 1.0 : 0.0;
-  double a_R = 0.0, ab[NBV] = {}, m[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
-  bool need[2] = {false, false}, near = false;
-  double xi, y0, y1;
-  r4<double> kb[2][4];
-  double bx[2][3] = {{0.0, 0.0, 0.0}, {0.0, 0.0, 0.0}};
-  double E[4] = {0.0, 0.0, 0.0, 0.0};
-  if constexpr (PID == P_EE_UUG) {
-    FsrKin f;
-    fsr_map(k, f);
-    xi = f.xi;
-    y0 = f.y[0];
-    y1 = f.y[1];
-#pragma unroll
-    for (int j = 0; j < 2; ++j) {
-      const double cB = (!kp.cut.mask || pass_cuts<P_EE_UU>(f.born[j], kp.cut)) ? 1.0 : 0.0;
-      const double th_s = f.xi < kp.xi_cut ? cB : 0.0;
-      const double th_c = f.y[j] > 1.0 - kp.delta ? cB : 0.0;
-      const double cs = (1.0 - f.y[j]) * 0.5 * (1.0 + f.y[j]) * f.K0 * (-(4.0 * g2 / s) * 2.0 * eik(f.born[j][2], f.born[j][3], f.qdir) * (-CF_));
-      const double cc = f.K1 * (2.0 / (s * (1.0 - f.xi))) * 2.0 * g2 * CF_ * (1.0 + (1.0 - f.xi) * (1.0 - f.xi));
-      const double csc = f.K0 * (2.0 / s) * 2.0 * g2 * 2.0 * CF_;
-      const double iden = 1.0 / (f.xi * f.xi * (1.0 - f.y[j]) * f.K[j]);
-      ab[j] = -(th_s * cs + th_c * cc - th_s * th_c * csc) * iden;
-      m[j] = fabs(th_c * cc * iden) + fabs(th_s * (cs - th_c * csc) * iden);
-      near |= (th_s > 0.0 && f.xi < kp.xi_thr) || (th_c > 0.0 && 1.0 - f.y[j] < kp.y_thr);
-      a_R += f.S[j] * cR;
-      need[j] = th_s > 0.0 || th_c > 0.0;
-#pragma unroll
-      for (int l = 0; l < 4; ++l) kb[j][l] = f.born[j][l];
-    }
-  } else {
-    constexpr int BPID = PID == P_GG_TTG ? P_GG_TT : P_UU_TT;
-    IsrKin f;
-    isr_map(k, kp.cp.mt, f, kp.cut);
-    xi = f.xi;
-    y0 = f.y[0];
-    y1 = f.y[1];
-    const double z = 1.0 - xi, iz = f.iz, is2 = 2.0 / s;
-    const double th_s = xi < kp.xi_cut && f.cut_s ? 1.0 : 0.0;
-    const double den0 = xi * xi * (1.0 - f.y[0]) * f.K, den1 = xi * xi * (1.0 - f.y[1]) * f.K;
-    const double rden = 1.0 / (den0 * den1);
-    const double iden[2] = {den1 * rden, den0 * rden};
-    const double kc = BPID == P_GG_TT ? 2.0 * CA_ * (z + xi * xi * z) : CF_ * (1.0 + z * z);
-    const double kp_ = BPID == P_GG_TT ? 2.0 * CA_ * 2.0 * (xi * xi * iz) : 0.0;
-    const double ks = BPID == P_GG_TT ? 2.0 * CA_ : 2.0 * CF_;
-#pragma unroll
-    for (int j = 0; j < 2; ++j) {
-      const double th_c = f.y[j] > 1.0 - kp.delta ? 1.0 : 0.0;
-      const double th_cc = f.cut_c[j] ? th_c : 0.0;
-      a_R += f.S[j] * cR;
-      const double sE = th_s * (1.0 - f.y[j]) * f.S[j] * f.K0 * (-(4.0 * g2 / s)) * iden[j];
-      const double sB = -th_s * th_c * f.K0 * is2 * 2.0 * g2 * ks * iden[j];
-      const double gcj = th_cc * f.K * is2 * iz * 2.0 * g2 * iden[j];
-      ab[0] -= sE;
-      ab[1] -= sB;
-      ab[2] -= gcj * kc;
-      if constexpr (BPID == P_GG_TT) ab[3 + j] = -gcj * kp_;
-      m[2 * j] = sE;
-      m[2 * j + 1] = sB;
-      m[4 + j] = gcj * kc;
-      near |= (th_s > 0.0 && xi < kp.xi_thr) || ((th_cc > 0.0 || th_s * th_c > 0.0) && 1.0 - f.y[j] < kp.y_thr);
-      need[1] |= th_cc > 0.0;
-    }
-    need[0] = th_s > 0.0;
-    if (need[0]) isr_eikonal_matrix<BPID>(f, kp, E);
-    // spin-correlated Borns the collinear configuration needs (g g): sector j's has a
-    // nonzero coefficient only where sector j's collinear term is active, which with
-    // delta <= 1 is one sector at most.  If only sector 2's is needed, the beams are
-    // stored swapped: by Bose symmetry the Born with gluon 1 polarised at (k0, k1, ..)
-    // is the Born with gluon 0 polarised at (k1, k0, ..), and the plain Born is
-    // symmetric, so every lane then evaluates gluon 0 polarised (one code path).
-    const bool p0 = BPID == P_GG_TT && ab[3 % NBV] != 0.0, p1 = BPID == P_GG_TT && ab[4 % NBV] != 0.0;
-    const bool swap = p1 && !p0;
-#pragma unroll
-    for (int l = 0; l < 4; ++l) kb[0][l] = f.soft[l];
-    kb[1][0] = swap ? f.coll[1] : f.coll[0];
-    kb[1][1] = swap ? f.coll[0] : f.coll[1];
-    kb[1][2] = f.coll[2];
-    kb[1][3] = f.coll[3];
-    bx[1][0] = f.cphi;
-    bx[1][1] = f.sphi;
-    bx[1][2] = (double)((p0 ? 1 : 0) | (p1 ? 2 : 0) | (swap ? 4 : 0));
-  }
-  // the boundary of the FKS domain has measure zero and weight 0 (see real_sub_event)
-  const bool inside = act && xi > 0.0 && xi < 1.0 && 1.0 - y0 > 0.0 && 1.0 - y1 > 0.0;
-  const bool need_real = inside && cR > 0.0;
-  need[0] = need[0] && inside;
-  need[1] = need[1] && inside;
-  const bool rec = need_real || need[0] || need[1];
-  if (act && !rec) out[i] = 0.0;
-  const int slot = warp_reserve(tb.cnt + TC_REC, rec ? 1 : 0);
-  const int qr = warp_reserve(tb.cnt + TC_QR, need_real ? 1 : 0);
-  const int qb0 = warp_reserve(tb.cnt + TC_QB, need[0] ? 1 : 0);
-  const int qb1 = warp_reserve(tb.cnt + TC_QB1, need[1] ? 1 : 0);
-  if (!rec) return;
-  const long c = tb.cap, c2 = 2 * tb.cap;
-  tb.ev[slot] = (int)i;
-  tb.flags[slot] = near ? 1 : 0;
-  const float rho = fmaxf((float)fmin(1.0 - y0, 1.0 - y1), 1e-30f);
-  tb.grow[slot] = 1.0f + sqrtf(0.01f / rho);
-#pragma unroll
-  for (int b = 0; b < NB; ++b) {
-    tb.a[b * c + slot] = need_real ? a_R : 0.0;
-    tb.v[b * c + slot] = 0.0;
-  }
-#pragma unroll
-  for (int t = 0; t < NBV; ++t) {
-    tb.a[(NB + t) * c + slot] = ab[t];
-    tb.v[(NB + t) * c + slot] = 0.0;
-  }
-#pragma unroll
-  for (int r = 0; r < 6; ++r) tb.m[r * c + slot] = m[r];
-  if (need_real) tb.q_real[qr] = slot;
-#pragma unroll
-  for (int set = 0; set < 2; ++set) {
-    const int ci = set == 0 ? qb0 : (int)c + qb1;
-    tb.cfg[set * c + slot] = need[set] ? ci : -1;
-    if (!need[set]) continue;
-    tb.bslot[ci] = slot | (set << 30);
-#pragma unroll
-    for (int l = 0; l < 4; ++l) {
-      tb.bp[(0 * 4 + l) * c2 + ci] = kb[set][l].e;
-      tb.bp[(1 * 4 + l) * c2 + ci] = kb[set][l].x;
-      tb.bp[(2 * 4 + l) * c2 + ci] = kb[set][l].y;
-      tb.bp[(3 * 4 + l) * c2 + ci] = kb[set][l].z;
-    }
-    if constexpr (PID != P_EE_UUG) {
-      if (set == 0) {
-#pragma unroll
-        for (int q = 0; q < 4; ++q) tb.bx[q * c2 + ci] = E[q];
-      } else {
-        tb.bx[0 * c2 + ci] = bx[1][0];
-        tb.bx[1 * c2 + ci] = bx[1][1];
-        tb.bx[2 * c2 + ci] = bx[1][2];
-      }
+  const PointTerms t = point_terms<PID>(k, kp);
+  const bool rec = act && t.inside && t.a_R > 0.0;
+  const int slot = warp_reserve(tb.cnt, rec ? 1 : 0);
+  const RealSubOut r = combine_point(t, 0.0);
+  if (rec) {
+    const float g = (float)error_growth(r);
+    tb.ev[slot] = (int)i | (t.need[0] ? 1 << 29 : 0) | (t.need[1] ? 1 << 30 : 0);
+    tb.grow[slot] = t.near ? -g : g;
+    tb.a[slot] = t.a_R;
+    tb.a[tb.cap + slot] = t.w_born;
+    tb.a[2 * tb.cap + slot] = t.mag_b;
+  } else if (act) {
+    // no real matrix element: finished (a flagged one is float64 already)
+    out[i] = r.W == 0.0 ? 0.0 : (wgt ? wgt[i] : 1.0) * r.W;
+    if (kp.flag_unstable && t.inside && unstable_point(r, kp)) {
+      const double none[MAX_BLOCKS] = {};
+      append_flagged<PID>(counts, ib, i, 0.0, 0.0, t.need, none, 0);
     }
   }
 }
 
-// Every queued amplitude, one lane each, in precision T: reals (from the point's momenta;
-// all helicity blocks of a point in one lane, or one block per lane in the rescue queue)
-// and Born configurations (from the stored counter-event momenta), in one index space
-// (reals first).  RESCUE selects the float64 rescue queues.  PART: 0 every queue, 1 the
-// reals only, 2 the Born configurations only (the bulk launches the two kinds apart, so
-// that each kernel's code is smaller and its instruction fetch misses less).
-template <int PID, typename T, bool RESCUE, int PART = 0>
-__global__ void __launch_bounds__(128, ME_MINB) k_term_items(const double* __restrict__ p, long n, KParams kp,
-                                                             TermBufs tb) {
-  constexpr bool rescue = RESCUE;
+// The queued reals, one lane each, in precision T (grid-stride, their number read on the
+// device), W and the stability test.
+template <int PID, typename T>
+__global__ void __launch_bounds__(128, ME_MINB) k_term_reals(const double* __restrict__ p,
+                                                             const double* __restrict__ wgt, long n,
+                                                             double* __restrict__ out, KParams kp, TermBufs tb,
+                                                             int* __restrict__ counts, ItemBufs ib) {
   constexpr int NEXT = Proc<PID>::NEXT, NB = RealLayout<PID>::NB;
-  const int* qr = rescue ? tb.r_real : tb.q_real;
-  const long nr = PART == 2 ? 0 : tb.cnt[rescue ? TC_RR : TC_QR];
-  const long n0 = PART == 1 ? 0 : tb.cnt[rescue ? TC_RB : TC_QB];
-  const long nt = nr + n0 + (PART == 1 ? 0 : tb.cnt[rescue ? TC_RB1 : TC_QB1]);
-  const long c = tb.cap, c2 = 2 * tb.cap;
-  const unsigned self = 1u << (threadIdx.x & 31u);
-  for (long t = (long)blockIdx.x * blockDim.x + threadIdx.x; t < nt; t += (long)gridDim.x * blockDim.x) {
-    if (PART != 2 && t < nr) {
-      const int item = qr[t];
-      const int slot = rescue ? item >> 2 : item;
-      r4<double> k[NEXT];
-      load_event<NEXT>(p, n, tb.ev[slot], k);
-      const Kin<PID, T> K = prepare<PID, T>(k, kp.cp);
-      if constexpr (RESCUE) {
-        const int b = item & 3;
-        tb.v[b * c + slot] = real_block_value<PID, T>(K, b, kp);
-      } else {
+  const long nr = *tb.cnt;
+  for (long slot = (long)blockIdx.x * blockDim.x + threadIdx.x; slot < nr; slot += (long)gridDim.x * blockDim.x) {
+    const int code = tb.ev[slot], ev = code & 0x1fffffff;
+    r4<double> k[NEXT];
+    load_event<NEXT>(p, n, ev, k);
+    double v[NB], R = 0.0;
+    {
+      const Kin<PID, T> K = prepare<PID, T>(k, unit_couplings(kp.cp));
 #pragma unroll 1
-        for (int b = 0; b < NB; ++b) tb.v[b * c + slot] = real_block_value<PID, T>(K, b, kp);
-      }
-    } else if constexpr (PART != 1) {
-      // set-0 configurations, then set-1 ones (stored from index cap)
-      const long u = t - nr < n0 ? t - nr : c + (t - nr - n0);
-      const int ci = rescue ? tb.r_born[u] : (int)u;
-      const int bs = tb.bslot[ci], slot = bs & 0x3fffffff, set = bs >> 30;
-      r4<double> kb[4];
-#pragma unroll
-      for (int l = 0; l < 4; ++l)
-        kb[l] = r4<double>{tb.bp[(0 * 4 + l) * c2 + ci], tb.bp[(1 * 4 + l) * c2 + ci], tb.bp[(2 * 4 + l) * c2 + ci],
-                           tb.bp[(3 * 4 + l) * c2 + ci]};
-      if constexpr (PID == P_EE_UUG) {
-        tb.v[(NB + set) * c + slot] = fsr_born_one<T, 1>(kb, kp, 0, self);
-      } else {
-        constexpr int BPID = PID == P_GG_TTG ? P_GG_TT : P_UU_TT;
-        if (set == 0) {
-          const double E[4] = {tb.bx[0 * c2 + ci], tb.bx[1 * c2 + ci], tb.bx[2 * c2 + ci], tb.bx[3 * c2 + ci]};
-          double vE, vS;
-          isr_soft_pair<BPID, T, 1>(kb, E, kp, 0, self, vE, vS);
-          tb.v[NB * c + slot] = vE;
-          tb.v[(NB + 1) * c + slot] = vS;
-        } else {
-          double vc[3];
-          // only the spin-correlated Borns with a nonzero coefficient (flags from k_terms:
-          // 1 sector 1's, 2 sector 2's, 4 beams swapped so that sector 2's is gluon 0's)
-          const int fl = (int)tb.bx[2 * c2 + ci];
-          const bool sw = fl & 4;
-          isr_coll_set<BPID, T, 1>(kb, tb.bx[0 * c2 + ci], tb.bx[1 * c2 + ci], kp, 0, self, vc,
-                                   (fl & 1) || sw, (fl & 2) && !sw);
-          tb.v[(NB + 2) * c + slot] = vc[0];
-          if constexpr (BPID == P_GG_TT) {
-            if (fl & 1) tb.v[(NB + 3) * c + slot] = vc[1];
-            if (fl & 2) tb.v[(NB + 4) * c + slot] = sw ? vc[1] : vc[2];
-          }
-        }
-      }
+      for (int b = 0; b < NB; ++b) R += (v[b] = real_block_value<PID, T>(K, b, kp));
     }
-  }
-}
-
-// W of every record; in mixed precision (kp.flag_unstable) the stability test of
-// real_sub_event and the item selection of rescue_mask, with the flagged records' float64
-// items queued (whole warps iterate together for the aggregated appends).
-template <int PID>
-__global__ void __launch_bounds__(128) k_terms_combine(const double* __restrict__ wgt, double* __restrict__ out,
-                                                       KParams kp, TermBufs tb) {
-  constexpr int NB = RealLayout<PID>::NB, NI = RealLayout<PID>::NI;
-  const long nrec = tb.cnt[TC_REC];
-  const long c = tb.cap;
-  const int lane = threadIdx.x & 31;
-  const long stride = (long)gridDim.x * blockDim.x;
-  for (long t0 = (long)blockIdx.x * blockDim.x + (threadIdx.x & ~31); t0 < nrec; t0 += stride) {
-    const long slot = t0 + lane;
-    const bool act = slot < nrec;
-    double W = 0.0;
-    bool flag = false;
-    unsigned msk = 0;
-    int ev = 0;
-    if (act) {
-#pragma unroll
-      for (int q = 0; q < NI; ++q) W += tb.a[q * c + slot] * tb.v[q * c + slot];
-      ev = tb.ev[slot];
-      if (kp.flag_unstable) {
-        double R = 0.0;
-#pragma unroll
-        for (int b = 0; b < NB; ++b) R += tb.v[b * c + slot];
-        const double grow = (double)tb.grow[slot];
-        // the growth of the float32 error towards the collinear limit is the real's; the
-        // Born part enters unscaled (unstable_point)
-        const double bsc = term_born_scale<PID>(tb, slot) / grow;
-        const double mag = fabs(tb.a[slot] * R) + bsc;
-        const bool near = tb.flags[slot] & 1;
-        flag = near || !(mag * grow * kp.me_eps <= kp.tol * fabs(W));
-        if (flag) {
-          constexpr unsigned all = (1u << (NB + 1)) - 1u;
-          if (near) {
-            msk = all;
-          } else {
-            double e[NB + 1];
-            double rest = 0.0;
-#pragma unroll
-            for (int b = 0; b < NB; ++b) rest += (e[b] = fabs(tb.a[b * c + slot] * tb.v[b * c + slot]));
-            rest += (e[NB] = bsc);
-            const double budget = kp.item_budget * kp.tol * fabs(W) / (grow * kp.me_eps);
-#pragma unroll
-            for (int kk = 0; kk <= NB; ++kk) {
-              if (!(rest > budget)) break;
-              int pick = -1;
-              double best = -1.0;
-#pragma unroll
-              for (int b = 0; b <= NB; ++b)
-                if (!(msk >> b & 1u) && e[b] > best) {
-                  best = e[b];
-                  pick = b;
-                }
-              if (pick < 0) break;
-              msk |= 1u << pick;
-              rest -= best;
-            }
-            if (!msk) msk = all;
-          }
-          // real blocks with a zero coefficient (the real failed its cuts) stay as they are
-          if (tb.a[slot] == 0.0) msk &= ~((1u << NB) - 1u);
-        }
-      }
-      if (!flag) out[ev] = (wgt ? wgt[ev] : 1.0) * W;
-    }
-    // queue the flagged records' float64 items (every lane of the warp takes part)
-    const int nbl = __popc(msk & ((1u << NB) - 1u));
-    const bool born = msk >> NB & 1u;
-    const int ci0 = born ? tb.cfg[slot] : -1, ci1 = born ? tb.cfg[c + slot] : -1;
-    const int fb = warp_reserve(tb.cnt + TC_FLAG, flag ? 1 : 0);
-    const int rb = warp_reserve(tb.cnt + TC_RR, nbl);
-    const int cb0 = warp_reserve(tb.cnt + TC_RB, ci0 >= 0 ? 1 : 0);
-    const int cb1 = warp_reserve(tb.cnt + TC_RB1, ci1 >= 0 ? 1 : 0);
-    if (flag) {
-      tb.flagged[fb] = (int)slot;
-      int r = rb;
-#pragma unroll
-      for (int b = 0; b < NB; ++b)
-        if (msk >> b & 1u) tb.r_real[r++] = (int)slot * 4 + b;
-      if (ci0 >= 0) tb.r_born[cb0] = ci0;
-      if (ci1 >= 0) tb.r_born[c + cb1] = ci1;
-    }
-  }
-}
-
-// W of the flagged records after their float64 items; thread 0 of block 0 copies the
-// rescue counts to `counts` ([0] flagged points, [2] real blocks, [3] Born configurations,
-// [4] / [5] those of set 0 / set 1: the layout me_last_rescue_work and
-// me_last_rescue_configs read).
-template <int PID>
-__global__ void k_terms_final(const double* __restrict__ wgt, double* __restrict__ out, TermBufs tb,
-                              int* __restrict__ counts) {
-  constexpr int NI = RealLayout<PID>::NI;
-  const long nf = tb.cnt[TC_FLAG];
-  const long c = tb.cap;
-  if (blockIdx.x == 0 && threadIdx.x == 0 && counts) {
-    counts[0] = tb.cnt[TC_FLAG];
-    counts[2] = tb.cnt[TC_RR];
-    counts[3] = tb.cnt[TC_RB] + tb.cnt[TC_RB1];
-    counts[4] = tb.cnt[TC_RB];
-    counts[5] = tb.cnt[TC_RB1];
-  }
-  for (long t = (long)blockIdx.x * blockDim.x + threadIdx.x; t < nf; t += (long)gridDim.x * blockDim.x) {
-    const long slot = tb.flagged[t];
-    double W = 0.0;
-#pragma unroll
-    for (int q = 0; q < NI; ++q) W += tb.a[q * c + slot] * tb.v[q * c + slot];
-    const int ev = tb.ev[slot];
+    const double a_R = tb.a[slot], wb = tb.a[tb.cap + slot];
+    const double x = a_R * R, W = x + wb;
     out[ev] = (wgt ? wgt[ev] : 1.0) * W;
+    if (kp.flag_unstable) {
+      const float g = tb.grow[slot];
+      const RealSubOut r{W, fabs(x) + tb.a[2 * tb.cap + slot], fabs(x), {0.0, 0.0}, g < 0.0f};
+      if (unstable_point(r, kp, (double)fabsf(g))) {
+        const bool need[2] = {(code >> 29 & 1) != 0, (code >> 30 & 1) != 0};
+        append_flagged<PID>(counts, ib, ev, a_R, wb, need, v, rescue_mask<PID>(r, a_R, v, kp, (double)fabsf(g)));
+      }
+    }
   }
 }
 
@@ -1591,14 +1188,6 @@ __global__ void __launch_bounds__(128) k_cut_list(const double* __restrict__ p, 
   if (pass) list[at] = (int)i;
 }
 
-// ---------------------------------------------------------------- weight accumulation
-// Deterministic two-pass reduction: per-block partial (sum w, sum w^2) in a fixed tree
-// order, then one block adds the partials in block order.  No floating atomics.
-// `cnt` (optional, device): the number of points, read on the device (at most n).
-__global__ void k_partials(const double* __restrict__ w, long n, double* __restrict__ part, const int* __restrict__ cnt);
-__global__ void k_finish(const double* __restrict__ part, int nblk, double* __restrict__ acc, long n,
-                         const int* __restrict__ cnt);
-
 // ---------------------------------------------------------------- launch registry
 struct LaunchArgs {
   const double* p;
@@ -1609,7 +1198,7 @@ struct LaunchArgs {
   const int* idx;    // optional event list (rescue), length *count on the device
   const int* count;  // optional number of events, read on the device (events 0..*count-1 without idx)
   int* resc_list;    // real kernel in bulk precision: unstable points are appended here
-  int* resc_count;   // [0] flagged points, [1] queued kernel's tiles, [2] / [3] real-block / Born items
+  int* resc_count;   // counters: [1] the queued kernel's tiles, the others as in ItemBufs
   ItemBufs items;    // item rescue records and lists
   long groups;       // number of event groups to launch (n, or the list capacity)
   int* tiles;        // queued kernel: tile counter, zero at launch
@@ -1639,6 +1228,9 @@ cudaError_t launch_one(int kind, const LaunchArgs& a, cudaStream_t st) {
         const long tb = (total + TC4_THREADS - 1) / TC4_THREADS;
         k_tree_tc4<4><<<(unsigned)tb, TC4_THREADS, TC4_SMEM, st>>>(a.p, a.wgt, a.n, a.out, a.kp, a.idx, a.count);
       }
+    } else if constexpr (closed_tree<PID>()) {
+      if constexpr (LPE != 1) return launch_one<PID, T, 1>(kind, a, st);
+      else k_tree_closed<PID, T><<<(unsigned)((a.groups + 255) / 256), 256, 0, st>>>(a.p, a.wgt, a.n, a.out, a.kp, a.idx, a.count);
     } else {
       k_tree<PID, T, LPE><<<(unsigned)blocks, threads, 0, st>>>(a.p, a.wgt, a.n, a.out, a.kp, a.idx, a.count);
     }
@@ -1652,9 +1244,9 @@ cudaError_t launch_one(int kind, const LaunchArgs& a, cudaStream_t st) {
   return cudaGetLastError();
 }
 
-// The item rescue after a bulk-precision launch with kp.item_rescue: float64 items,
-// then the recombination.  Persistent grids (resident blocks x SMs, found once per
-// device) walk the lists, whose lengths are read on the device.
+// The item rescue after a bulk-precision launch: float64 items with their recombination.  A
+// persistent grid (resident blocks x SMs, found once per device) walks the list, whose
+// length is read on the device.
 template <int PID>
 cudaError_t launch_items_one(const LaunchArgs& a, cudaStream_t st) {
   (void)cudaGetLastError();
@@ -1675,10 +1267,7 @@ cudaError_t launch_items_one(const LaunchArgs& a, cudaStream_t st) {
   }
   const long cap_blocks = (a.items.cap * 4 + 127) / 128;
   const unsigned gx = (unsigned)std::max(1L, std::min<long>(g, cap_blocks));
-  k_rescue_items<PID><<<dim3(gx, 2), 128, 0, st>>>(a.p, a.n, a.kp, a.resc_count, a.items);
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  const unsigned gc = (unsigned)std::max(1L, std::min<long>(4 * g, (a.items.cap + 255) / 256));
-  k_rescue_combine<PID><<<gc, 256, 0, st>>>(a.wgt, a.out, a.resc_count, a.items);
+  k_rescue_items<PID><<<gx, 128, 0, st>>>(a.p_copy ? a.p_copy : a.p, a.wgt, a.n, a.out, a.kp, a.resc_count, a.items);
   return cudaGetLastError();
 }
 
@@ -1723,56 +1312,42 @@ cudaError_t launch_queued_one(const LaunchArgs& a, cudaStream_t st) {
   return cudaGetLastError();
 }
 
-// Per-term queues (k_terms ... k_terms_final): phase 0 enqueues the float64 pass, the
-// bulk-precision items and the recombination (with the stability test in mixed
-// precision); phase 1 the float64 rescue items and the flagged points' recombination
-// (mixed precision only), and copies the rescue counts to `counts`.
+// Per-term queues: the float64 pass, then the queued reals (in mixed precision the item
+// rescue follows, launch_items_*).
 template <int PID>
-cudaError_t launch_terms_one(int phase, bool mixed, const LaunchArgs& a, const TermBufs& tb, int* counts,
-                             cudaStream_t st) {
+cudaError_t launch_terms_one(bool mixed, const LaunchArgs& a, const TermBufs& tb, cudaStream_t st) {
   (void)cudaGetLastError();
   static std::atomic<int> resident[2][64];
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
   if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
-  const bool f64 = phase == 1 || !mixed;
-  int g = resident[f64][dev].load(std::memory_order_relaxed);
+  int g = resident[mixed][dev].load(std::memory_order_relaxed);
   if (g == 0) {
     int per = 0, sms = 0;
-    e = f64 ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_term_items<PID, double, true>, 128, 0)
-            : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_term_items<PID, float, false, 1>, 128, 0);
+    e = mixed ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_term_reals<PID, float>, 128, 0)
+              : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_term_reals<PID, double>, 128, 0);
     if (e != cudaSuccess) return e;
     e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
     g = (per > 0 ? per : 1) * (sms > 0 ? sms : 1);
-    resident[f64][dev].store(g, std::memory_order_relaxed);
+    resident[mixed][dev].store(g, std::memory_order_relaxed);
   }
-  const long items_cap = (RealLayout<PID>::NB + 2) * tb.cap;
-  const unsigned gi = (unsigned)std::max(1L, std::min<long>(g, (items_cap + 127) / 128));
-  const unsigned gc = (unsigned)std::max(1L, std::min<long>(4 * g, (tb.cap + 127) / 128));
-  if (phase == 0) {
-    if ((e = cudaMemsetAsync(tb.cnt, 0, 8 * sizeof(int), st)) != cudaSuccess) return e;
-    const long blocks = (a.groups + 127) / 128;
-    if (blocks <= 0) return cudaSuccess;
-    k_terms<PID><<<(unsigned)blocks, 128, 0, st>>>(a.p, a.n, a.out, a.kp, a.count, tb, a.p_copy);
-    const double* pi = a.p_copy ? a.p_copy : a.p;
-    if (mixed) {
-      k_term_items<PID, float, false, 1><<<gi, 128, 0, st>>>(pi, a.n, a.kp, tb);
-      k_term_items<PID, float, false, 2><<<gi, 128, 0, st>>>(pi, a.n, a.kp, tb);
-    } else {
-      k_term_items<PID, double, false><<<gi, 128, 0, st>>>(pi, a.n, a.kp, tb);
-    }
-    k_terms_combine<PID><<<gc, 128, 0, st>>>(a.wgt, a.out, a.kp, tb);
-  } else {
-    k_term_items<PID, double, true><<<gi, 128, 0, st>>>(a.p_copy ? a.p_copy : a.p, a.n, a.kp, tb);
-    k_terms_final<PID><<<gc, 128, 0, st>>>(a.wgt, a.out, tb, counts);
-  }
+  const long blocks = (a.groups + 127) / 128;
+  if (blocks <= 0) return cudaSuccess;
+  if ((e = cudaMemsetAsync(tb.cnt, 0, sizeof(int), st)) != cudaSuccess) return e;
+  k_terms<PID><<<(unsigned)blocks, 128, 0, st>>>(a.p, a.wgt, a.n, a.out, a.kp, a.count, tb, a.resc_count, a.items, a.p_copy);
+  const double* pi = a.p_copy ? a.p_copy : a.p;
+  const unsigned gr = (unsigned)std::min<long>(g, blocks);
+  if (mixed)
+    k_term_reals<PID, float><<<gr, 128, 0, st>>>(pi, a.wgt, a.n, a.out, a.kp, tb, a.resc_count, a.items);
+  else
+    k_term_reals<PID, double><<<gr, 128, 0, st>>>(pi, a.wgt, a.n, a.out, a.kp, tb, a.resc_count, a.items);
   return cudaGetLastError();
 }
-cudaError_t launch_terms_ee(int phase, bool mixed, const LaunchArgs& a, const TermBufs& tb, int* counts, cudaStream_t st);
-cudaError_t launch_terms_gg(int phase, bool mixed, const LaunchArgs& a, const TermBufs& tb, int* counts, cudaStream_t st);
-cudaError_t launch_terms_uu(int phase, bool mixed, const LaunchArgs& a, const TermBufs& tb, int* counts, cudaStream_t st);
+cudaError_t launch_terms_ee(bool mixed, const LaunchArgs& a, const TermBufs& tb, cudaStream_t st);
+cudaError_t launch_terms_gg(bool mixed, const LaunchArgs& a, const TermBufs& tb, cudaStream_t st);
+cudaError_t launch_terms_uu(bool mixed, const LaunchArgs& a, const TermBufs& tb, cudaStream_t st);
 // tree entries with per-term queues: list the points that pass the cuts (k_cut_list)
 cudaError_t launch_cut_list(int pid, const LaunchArgs& a, int* list, int* listed, cudaStream_t st);
 

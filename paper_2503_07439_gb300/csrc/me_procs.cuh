@@ -54,12 +54,36 @@ struct Couplings {
   __host__ __device__ Couplings(double g, double e, double m)
       : gs(g), ee(e), mt(m), gsf((float)g), eef((float)e), mtf((float)m) {}
 };
+// The same with both couplings at 1.  A tree amplitude is a fixed product of couplings times a
+// function of the momenta, so the kernels evaluate the function and multiply its square by
+// the couplings in float64 (tree_coupling): a float32 coupling, off by up to 3e-8, would
+// shift every matrix element by up to eight times that, and the subtraction would not
+// cancel the shift against the float64 counterterms.
+ME_HD Couplings unit_couplings(const Couplings& c) {
+  Couplings u = c;
+  u.gs = u.ee = 1.0;
+  u.gsf = u.eef = 1.0f;
+  return u;
+}
 template <typename T> ME_HD T gs_of(const Couplings& c) { return (T)c.gs; }
 template <> ME_HD float gs_of<float>(const Couplings& c) { return c.gsf; }
 template <typename T> ME_HD T ee_of(const Couplings& c) { return (T)c.ee; }
 template <> ME_HD float ee_of<float>(const Couplings& c) { return c.eef; }
 template <typename T> ME_HD T mt_of(const Couplings& c) { return (T)c.mt; }
 template <> ME_HD float mt_of<float>(const Couplings& c) { return c.mtf; }
+
+// the couplings of a process's tree |M|^2
+ME_HD double tree_coupling(int pid, const Couplings& c) {
+  const double g2 = c.gs * c.gs, e4 = c.ee * c.ee * c.ee * c.ee;
+  switch (pid) {
+    case P_EE_UU: return e4;
+    case P_EE_UUG: return e4 * g2;
+    case P_GG_TT:
+    case P_UU_TT: return g2 * g2;
+    case P_GG_TTGG: return g2 * g2 * g2 * g2;
+    default: return g2 * g2 * g2;
+  }
+}
 
 __host__ __device__ constexpr int factorial(int n) { return n <= 1 ? 1 : n * factorial(n - 1); }
 
@@ -208,11 +232,11 @@ ME_HD void amp_ttng(const KinTT<T, NG>& K, int hel, const Couplings& cp, cx<T>* 
 // and the amplitudes of all orderings then reuse them.  Orderings are numbered
 // lexicographically as in amp_ttng, so the colour basis is the same.
 template <typename T>
-ME_HD void amp_tt2_fast(const KinTT<T, 2>& K, int hel, const Couplings& cp, const c4<T>* ov, int ov_leg, cx<T>* A) {
+ME_HD void amp_tt2_fast(const KinTT<T, 2>& K, int hel, const Couplings& cp, cx<T>* A) {
   const T g = gs_of<T>(cp), mt = mt_of<T>(cp);
   const r4<T> k0 = K.q[0], k1 = K.q[1], kt = K.pl[2];
-  const c4<T> e0 = (ov != nullptr && ov_leg == 0) ? *ov : polvec(K.pl[0], hel_of(hel, 0), false);
-  const c4<T> e1 = (ov != nullptr && ov_leg == 1) ? *ov : polvec(K.pl[1], hel_of(hel, 1), false);
+  const c4<T> e0 = polvec(K.pl[0], hel_of(hel, 0), false);
+  const c4<T> e1 = polvec(K.pl[1], hel_of(hel, 1), false);
   const c4<T> ub = dbar(spinor_u(kt, mt, hel_of(hel, 2)));
   const c4<T> vb = spinor_v(K.pl[3], mt, hel_of(hel, 3));
   c4<T> J01 = vvv(e0, e1, -k0, -k1);
@@ -351,34 +375,6 @@ ME_HD void amp_tt3_fast(const KinTT<T, 3>& K, int hel, const Couplings& cp, cx<T
 // to 4737 operations and a g g -> t tbar g g block from 66751 to 49460.  GB300: 2^20
 // subtracted g g -> t tbar g points 5.55 -> 4.23 ms, 30011 in float64 1.385 -> 1.007 ms,
 // 8191 g g -> t tbar g g trees in float64 3.96 -> 3.04 ms.
-
-// g g -> t tbar.  A(01) = ubar [J01 + U0 e1] v,  A(10) = ubar [-J01 + U1 e0] v (no factor i g).
-template <typename T, class F>
-ME_HD void amp_tt2_block(const KinTT<T, 2>& K, int hb, const Couplings& cp, const c4<T>* ov, int ov_leg,
-                         F&& consume) {
-  const T g = gs_of<T>(cp), mt = mt_of<T>(cp);
-  const r4<T> k0 = K.q[0], k1 = K.q[1], kt = K.pl[2];
-  const c4<T> e0 = (ov != nullptr && ov_leg == 0) ? *ov : polvec_of(K.wg[0], hel_of(hb, 0), false);
-  const c4<T> e1 = (ov != nullptr && ov_leg == 1) ? *ov : polvec_of(K.wg[1], hel_of(hb, 1), false);
-  const c4<T> J01 = vvv(e0, e1, -k0, -k1, -g * K.ig[3]);
-  const sl4<T> s0 = slashed(e0), s1 = slashed(e1), s01 = slashed(J01);
-  const prop4<T> P0 = scaled_prop(kt + k0, mt, -g * K.iq[1]), P1 = scaled_prop(kt + k1, mt, -g * K.iq[2]);
-#pragma unroll
-  for (int ht = 0; ht < 2; ++ht) {
-    const c4<T> S = ubar_slash(K.wt, ht, s01);
-    const c4<T> U0 = row_prop(ubar_slash(K.wt, ht, s0), P0);
-    const c4<T> U1 = row_prop(ubar_slash(K.wt, ht, s1), P1);
-    c4<T> R0 = S;
-    row_slash_acc(R0, U0, s1);
-    c4<T> R1 = cneg(S);
-    row_slash_acc(R1, U1, s0);
-#pragma unroll
-    for (int hv = 0; hv < 2; ++hv) {
-      cx<T> A[2] = {dot_v(R0, K.wtb, hv), dot_v(R1, K.wtb, hv)};
-      consume(ht | (hv << 1), A);
-    }
-  }
-}
 
 // g g -> t tbar g: the three-gluon currents F(012) = F(210), F(021) = F(120),
 // F(102) = F(201) and the pair currents J(xy) are built once per block; per top spin the
@@ -666,14 +662,12 @@ ME_HD Kin<PID, T> prepare(const r4<double>* p, const Couplings& cp) {
   else return prep_uu<T, 5>(p, cp);
 }
 
-// partial amplitudes of one helicity; `eps_override` replaces the polarisation of gluon
-// leg `ov_leg` (g g -> t tbar only: the spin-correlated Born)
+// partial amplitudes of one helicity
 template <int PID, typename T>
-ME_HD void amplitude(const Kin<PID, T>& K, int hel, const Couplings& cp, cx<T>* A,
-                     const c4<T>* eps_override = nullptr, int ov_leg = -1) {
+ME_HD void amplitude(const Kin<PID, T>& K, int hel, const Couplings& cp, cx<T>* A) {
   if constexpr (PID == P_EE_UU) amp_ee_uu<T>(K, hel, cp, A);
   else if constexpr (PID == P_EE_UUG) amp_ee_uug<T>(K, hel, cp, A);
-  else if constexpr (PID == P_GG_TT) amp_tt2_fast<T>(K, hel, cp, eps_override, ov_leg, A);
+  else if constexpr (PID == P_GG_TT) amp_tt2_fast<T>(K, hel, cp, A);
   else if constexpr (PID == P_GG_TTG) amp_tt3_fast<T>(K, hel, cp, A);
   else if constexpr (PID == P_GG_TTGG) amp_ttng<T, 4>(K, hel, cp, A);
   else if constexpr (PID == P_UU_TT) amp_uu_tt<T>(K, hel, cp, A);
@@ -841,11 +835,8 @@ template <int PID> ME_HD int live_block_hel(int i) { return block_hel(massless_i
 // partial amplitudes of the four helicities hb | (r << 2) (see amp_tt2_block); processes
 // without a block routine evaluate them one at a time
 template <int PID, typename T, class F>
-ME_HD void amplitude_block(const Kin<PID, T>& K, int hb, const Couplings& cp, F&& consume,
-                           const c4<T>* eps_override = nullptr, int ov_leg = -1) {
-  if constexpr (PID == P_GG_TT) {
-    amp_tt2_block<T>(K, hb, cp, eps_override, ov_leg, consume);
-  } else if constexpr (PID == P_GG_TTG) {
+ME_HD void amplitude_block(const Kin<PID, T>& K, int hb, const Couplings& cp, F&& consume) {
+  if constexpr (PID == P_GG_TTG) {
     amp_tt3_block<T>(K, hb, cp, consume);
   } else if constexpr (PID == P_GG_TTGG) {
     amp_tt4_block<T>(K, hb, cp, consume);
@@ -855,8 +846,105 @@ ME_HD void amplitude_block(const Kin<PID, T>& K, int hb, const Couplings& cp, F&
         if (r == 0 || r == 3) continue;  // u, ubar with equal helicities: zero
       }
       cx<T> A[Proc<PID>::NFLOW];
-      amplitude<PID, T>(K, hb | (r << 2), cp, A, eps_override, ov_leg);
+      amplitude<PID, T>(K, hb | (r << 2), cp, A);
       consume(r, A);
+    }
+  }
+}
+
+// ----------------------------------------------------------------------------
+// Helicity- and colour-summed 2 -> 2 Borns in closed form.  With the massless beams p0, p1,
+// the quark p2 of mass m, tau_i = (p_i.p2) / (p0.p1) and rho = 4 m^2 / s:
+//   u ubar -> t tbar:  sum = 16 g^4 (tau_0^2 + tau_1^2 + rho / 2)   (one colour structure),
+//   e+e- -> u ubar:    sum = 24 e^4 Q_u^2 (tau_0^2 + tau_1^2),
+//   g g -> t tbar (Combridge 1979, by colour flow): the two orderings obey
+//     tau_0 A(01) = tau_1 A(10) =: X with sum |X|^2 = 8 g^4 tau_0 tau_1 F,
+//     F = tau_0^2 + tau_1^2 + rho - rho^2 / (4 tau_0 tau_1),
+//   so for any symmetric colour matrix M
+//     sum J^T M J = 8 g^4 F (M_00 tau_1 / tau_0 + 2 M_01 + M_11 tau_0 / tau_1);
+//   with one gluon polarised along a transverse unit vector e (either gluon: the value is
+//   symmetric), sum |X|^2 = 4 g^4 (tau_0 tau_1 F + rho (2 (e.p2)^2 / s - q)),
+//   q = tau_0 tau_1 - rho / 4 = pt^2 / s.
+// They take some 30 operations where the helicity amplitudes take 1400 to 3000, and stay
+// accurate at small tau; all terms but rho^2 are positive.
+template <typename T>
+struct Inv22 {
+  T c, t0, t1, rho;  // p0.p1, tau_0, tau_1, rho
+};
+template <typename T>
+ME_HD Inv22<T> inv22(const r4<double>* p, T m) {  // the products in float64
+  Inv22<T> k;
+  k.c = (T)mdot(p[0], p[1]);
+  const T ic = T(1) / k.c;
+  k.t0 = (T)mdot(p[0], p[2]) * ic;
+  k.t1 = (T)mdot(p[1], p[2]) * ic;
+  k.rho = T(2) * m * m * ic;
+  return k;
+}
+// u ubar -> t tbar and e+e- -> u ubar: the sum over everything but the couplings and colour
+template <typename T>
+ME_HD T born_qq(const Inv22<T>& k) {
+  return k.t0 * k.t0 + k.t1 * k.t1 + T(0.5) * k.rho;
+}
+// g g -> t tbar: sum J^T M J = f (M_00 r0 + 2 M_01 + M_11 r1)
+template <typename T>
+struct BornGG {
+  T f, r0, r1;
+};
+template <typename T>
+ME_HD BornGG<T> born_gg(const Inv22<T>& k, const Couplings& cp) {
+  const T i01 = T(1) / (k.t0 * k.t1), a = k.t0 * k.t0, b = k.t1 * k.t1;
+  const T g2 = gs_of<T>(cp) * gs_of<T>(cp);
+  const T F = a + b + k.rho * (T(1) - T(0.25) * k.rho * i01);
+  return BornGG<T>{T(8) * g2 * g2 * F, b * i01, a * i01};
+}
+constexpr double GG_C00 = 16.0 / 3.0, GG_C01 = -2.0 / 3.0;  // colour matrix of g g -> t tbar
+template <typename T>
+ME_HD T born_gg_colour(const BornGG<T>& b) {  // M = C
+  return b.f * (T(GG_C00) * (b.r0 + b.r1) + T(2.0 * GG_C01));
+}
+// the same with one gluon polarised along e, ep = e.p2 (either gluon)
+template <typename T>
+ME_HD T born_gg_polarised(const Inv22<T>& k, const BornGG<T>& b, T ep, const Couplings& cp) {
+  const T g2 = gs_of<T>(cp) * gs_of<T>(cp), t01 = k.t0 * k.t1;
+  const T col = T(0.5 * GG_C00) * (b.r0 + b.r1) + T(GG_C01);
+  return col * (b.f + T(8) * g2 * g2 * k.rho * (ep * ep / k.c - (t01 - T(0.25) * k.rho)) / t01);
+}
+// M the eikonal-weighted correlator matrix (row-major 2 x 2)
+template <typename T>
+ME_HD T born_gg_matrix(const BornGG<T>& b, const T* M) {
+  return b.f * (M[0] * b.r0 + (M[1] + M[2]) + M[3] * b.r1);
+}
+// u ubar -> t tbar with the matrix M: its amplitude in the basis (d_ik d_lj, d_ij d_lk) is
+// proportional to (1/2, -1/6), `sum` is the plain Born / 2
+template <typename T>
+ME_HD T born_uu_matrix(T sum, const T* M) {
+  return sum * (T(0.25) * M[0] - T(1.0 / 12.0) * (M[1] + M[2]) + T(1.0 / 36.0) * M[3]);
+}
+
+// Processes whose whole tree is one of these
+template <int PID> __host__ __device__ constexpr bool closed_tree() {
+  return PID == P_EE_UU || PID == P_GG_TT || PID == P_UU_TT;
+}
+// |M|^2 of one of them, summed over helicities and colours.  The quark pairs use the traces
+// of both lines, [(p0.p2)(p1.p3) + (p0.p3)(p1.p2) + m^2 p0.p1] / (p0.p1)^2 for born_qq, which
+// hold for momenta that do not add up exactly, as the sum over helicity amplitudes does.
+template <int PID, typename T>
+ME_HD T closed_sum(const r4<double>* p, const Couplings& cp) {
+  if constexpr (PID == P_GG_TT) {
+    return born_gg_colour(born_gg(inv22<T>(p, mt_of<T>(cp)), cp));
+  } else {
+    const T m = PID == P_EE_UU ? T(0) : mt_of<T>(cp);
+    const T c = (T)mdot(p[0], p[1]), ic = T(1) / c;
+    const T a = (T)mdot(p[0], p[2]) * ic, b = (T)mdot(p[1], p[3]) * ic;
+    const T d = (T)mdot(p[0], p[3]) * ic, e = (T)mdot(p[1], p[2]) * ic;
+    const T q = a * b + d * e + m * m * ic;
+    if constexpr (PID == P_EE_UU) {
+      const T e2 = ee_of<T>(cp) * ee_of<T>(cp);
+      return T(24.0 * 4.0 / 9.0) * e2 * e2 * q;
+    } else {
+      const T g2 = gs_of<T>(cp) * gs_of<T>(cp);
+      return T(16) * g2 * g2 * q;
     }
   }
 }
