@@ -45,6 +45,10 @@ static double block_ops(const r4<double>* p, int hb = 1) {
   const Kin<PID, Flop> K = prepare<PID, Flop>(p, cp);
   g_ops = 0;
   int calls = 0;
+  if constexpr (PID == P_EE_UUG) {
+    ee_uug_block(K, 0);
+    return (double)g_ops;
+  }
   amplitude_block<PID, Flop>(K, hb, cp, [&](int, const cx<Flop>*) { ++calls; });
   return (double)g_ops + calls * colour_flops(Proc<PID>::NFLOW);
 }

@@ -104,6 +104,19 @@ __device__ __forceinline__ T colour_sum(const ColourTables* tab, const cx<T>* J)
   return s;
 }
 
+// Live block b (K at unit couplings), summed over the four heavy-pair helicities and colours
+template <int PID, typename T, typename KP>
+__device__ __forceinline__ T block_sum(const Kin<PID, T>& K, int b, const KP& kp) {
+  if constexpr (PID == P_EE_UUG) {
+    return ee_uug_block(K, b);
+  } else {
+    T acc = T(0);
+    amplitude_block<PID, T>(K, live_block_hel<PID>(b), unit_couplings(kp.cp),
+                            [&](int, const cx<T>* J) { acc += colour_sum<PID, T>(kp.tab, J); });
+    return acc;
+  }
+}
+
 template <int LPE, typename T>
 __device__ __forceinline__ T group_sum(T v, unsigned mask) {
 #pragma unroll
@@ -189,12 +202,9 @@ __global__ void __launch_bounds__(128, ME_MINB) k_tree(const double* __restrict_
   load_event<NEXT>(p, n, ev, k);
   // Algorithm 2: every point is evaluated, and zeroed below where it fails the cuts
   const bool pass = !kp.cut.mask || pass_cuts<PID>(k, kp.cut);
-  const Couplings unit = unit_couplings(kp.cp);
-  const Kin<PID, T> K = prepare<PID, T>(k, unit);
+  const Kin<PID, T> K = prepare<PID, T>(k, unit_couplings(kp.cp));
   T acc = T(0);
-  for (int b = lane; b < n_live_blocks<PID>(); b += LPE)
-    amplitude_block<PID, T>(K, live_block_hel<PID>(b), unit,
-                            [&](int, const cx<T>* J) { acc += colour_sum<PID, T>(kp.tab, J); });
+  for (int b = lane; b < n_live_blocks<PID>(); b += LPE) acc += block_sum<PID, T>(K, b, kp);
   const double tot = 2.0 * (double)group_sum<LPE>(acc, group_mask<LPE>());
   if (lane == 0) {
     const double w = wgt ? wgt[ev] : 1.0;
@@ -759,10 +769,7 @@ __device__ __forceinline__ PointTerms point_terms(const r4<double>* k, const KPa
 // R = sum over the live blocks.
 template <int PID, typename T>
 __device__ __forceinline__ double real_block_value(const Kin<PID, T>& K, int b, const KParams& kp) {
-  T acc = T(0);
-  amplitude_block<PID, T>(K, live_block_hel<PID>(b), unit_couplings(kp.cp),
-                          [&](int, const cx<T>* J) { acc += colour_sum<PID, T>(kp.tab, J); });
-  return (double)acc * kp.real_scale;
+  return (double)block_sum<PID, T>(K, b, kp) * kp.real_scale;
 }
 
 // W and its error scale from a point's terms and R.

@@ -285,6 +285,14 @@ ME_HD wf_q<T> wf_quark(const r4<T>& p, T m) {
   const T s = msqrt(pp), is = T(1) / s;
   return wf_q<T>{s, m * is, {p.x * is, p.y * is}};
 }
+// Massless: the two nonzero components (a, b) of u or v of helicity + along p, up to a phase
+template <typename T>
+ME_HD void chi_massless(const r4<T>& p, cx<T>& a, cx<T>& b) {
+  const T s = msqrt(p.z >= T(0) ? p.e + p.z : p.e - p.z), is = T(1) / s;
+  const cx<T> t{p.x * is, p.y * is}, r{s, T(0)};
+  a = p.z >= T(0) ? r : conj(t);
+  b = p.z >= T(0) ? t : r;
+}
 template <typename T>
 ME_HD wf_q<T> scaled(const wf_q<T>& w, T f) {
   return wf_q<T>{f * w.s, f * w.m, f * w.t};
@@ -489,16 +497,6 @@ ME_HD void row_slash_acc(c4<T>& acc, const c4<T>& r, const spol<T>& S) {
   acc.v[2] = cmsb(rmac(acc.v[2], -S.z, r.v[0]), r.v[1], S.d);
   acc.v[3] = cmsb(rmac(acc.v[3], S.z, r.v[1]), r.v[0], S.c);
 }
-// eslash times column
-template <typename T>
-ME_HD c4<T> slash_col(const spol<T>& S, const c4<T>& s) {
-  c4<T> o;
-  o.v[0] = cmsb(-S.z * s.v[2], S.c, s.v[3]);
-  o.v[1] = cmsb(S.z * s.v[3], S.d, s.v[2]);
-  o.v[2] = cmac(S.z * s.v[0], S.c, s.v[1]);
-  o.v[3] = cmac(-S.z * s.v[1], S.d, s.v[0]);
-  return o;
-}
 // s (Qslash + m) times column, for the scaled propagator of row_prop
 template <typename T>
 ME_HD c4<T> col_prop(const prop4<T>& P, const c4<T>& s) {
@@ -565,11 +563,52 @@ ME_HD cx<T> dot_v(const c4<T>& r, const wf_q<T>& w, int h) {
   return h == 0 ? rmac(cmac(w.s * r.v[2], r.v[3], w.t), -w.m, r.v[0])
                 : rmac(cmsb(w.s * r.v[1], r.v[0], conj(w.t)), -w.m, r.v[3]);
 }
-// v of spin h as a column
+// eslash v of spin h
 template <typename T>
-ME_HD c4<T> v_column(const wf_q<T>& w, int h) {
-  const cx<T> z{T(0), T(0)};
-  return h == 0 ? c4<T>{{{-w.m, T(0)}, z, {w.s, T(0)}, w.t}} : c4<T>{{-conj(w.t), {w.s, T(0)}, z, {-w.m, T(0)}}};
+ME_HD c4<T> slash_v(const spol<T>& S, const wf_q<T>& w, int h) {
+  c4<T> o;
+  if (h == 0) {
+    o.v[0] = cmsb(cx<T>{-S.z * w.s, T(0)}, S.c, w.t);
+    o.v[1] = rmac(S.z * w.t, -w.s, S.d);
+    o.v[2] = cx<T>{-w.m * S.z, T(0)};
+    o.v[3] = -w.m * S.d;
+  } else {
+    o.v[0] = w.m * S.c;
+    o.v[1] = cx<T>{-w.m * S.z, T(0)};
+    o.v[2] = rmac(w.s * S.c, -S.z, conj(w.t));
+    o.v[3] = cmsb(cx<T>{-S.z * w.s, T(0)}, S.d, conj(w.t));
+  }
+  return o;
+}
+// A massless quark line of fixed helicity enters by two-component spinors: rho (the two
+// nonzero components of its row) and sigma (of its column), current 2 rho sigma.  A row R of
+// the heavy line contracted with it and with a column c gives 2 (X x + Y y):
+//   X = R0 rho1 - R1 rho0,  Y = R2 sigma0 + R3 sigma1  (row side),
+//   x = sigma1 c2 - sigma0 c3,  y = rho0 c0 + rho1 c1  (column side).
+template <typename T>
+struct c2 {
+  cx<T> a, b;
+};
+template <typename T> ME_HD cx<T> line_X(const c4<T>& R, const c2<T>& rho) { return cmsb(R.v[0] * rho.b, R.v[1], rho.a); }
+template <typename T> ME_HD cx<T> line_Y(const c4<T>& R, const c2<T>& sg) { return cmac(R.v[2] * sg.a, R.v[3], sg.b); }
+template <typename T> ME_HD cx<T> line_x(const c4<T>& c, const c2<T>& sg) { return cmsb(sg.b * c.v[2], sg.a, c.v[3]); }
+template <typename T> ME_HD cx<T> line_y(const c4<T>& c, const c2<T>& rho) { return cmac(rho.a * c.v[0], rho.b, c.v[1]); }
+// the same for ubar and v of spin h
+template <typename T>
+ME_HD cx<T> ubar_X(const wf_q<T>& w, int h, const c2<T>& rho) {
+  return h == 0 ? cmsb(w.s * rho.b, conj(w.t), rho.a) : -w.m * rho.a;
+}
+template <typename T>
+ME_HD cx<T> ubar_Y(const wf_q<T>& w, int h, const c2<T>& sg) {
+  return h == 0 ? w.m * sg.a : cmsb(w.s * sg.b, w.t, sg.a);
+}
+template <typename T>
+ME_HD cx<T> v_x(const wf_q<T>& w, int h, const c2<T>& sg) {
+  return h == 0 ? cmsb(w.s * sg.b, w.t, sg.a) : w.m * sg.a;
+}
+template <typename T>
+ME_HD cx<T> v_y(const wf_q<T>& w, int h, const c2<T>& rho) {
+  return h == 0 ? -w.m * rho.a : cmsb(w.s * rho.b, conj(w.t), rho.a);
 }
 template <typename T> ME_HD cx<T> cdot(const pol<T>& a, const pol<T>& b) {  // Minkowski product
   const cx<T> t = cmac(a.x * b.x, a.y, b.y);
