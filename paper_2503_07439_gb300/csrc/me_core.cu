@@ -455,6 +455,9 @@ struct me_handle {
   TermBufs tb{};
   size_t tcap = 0;
   double* d_part = nullptr;  // reduction partials
+  void* ws = nullptr;        // workspace of me_unweight, and its results in mapped host memory
+  size_t ws_bytes = 0;
+  void* ws_host = nullptr;
   double* d_acc = nullptr;   // accumulators (3)
   int lpe[2][2] = {{0, 0}, {0, 0}};  // [kind][fp64] chosen lanes per event
   int lpe_class[2][2] = {{-1, -1}, {-1, -1}};  // batch-size class they were chosen for
@@ -1066,6 +1069,8 @@ void me_destroy(me_handle* h) {
   free_terms(h);
   cudaFree(h->d_part);
   cudaFree(h->d_acc);
+  cudaFree(h->ws);
+  cudaFreeHost(h->ws_host);
   for (auto& ev : h->ev_used)
     for (auto e : ev) cudaEventDestroy(e);
   for (auto e : h->ev_pool) cudaEventDestroy(e);
@@ -1173,6 +1178,29 @@ int me_internal_final_masses(me_handle* h, double* masses, int* n_out, cudaStrea
   *n_out = nout;
   *stream = h->stream;
   ME_CUDA(cudaSetDevice(h->device));
+  return ME_OK;
+}
+
+int me_internal_workspace(me_handle* h, size_t bytes, void** dev, void** host, void** host_dev) {
+  if (!h || !dev || !host || !host_dev) return fail(ME_ERR_ARG, "NULL argument");
+  if (!h->ws_host && cudaHostAlloc(&h->ws_host, 64, cudaHostAllocMapped) != cudaSuccess) {
+    h->ws_host = nullptr;
+    return fail(ME_ERR_OOM, "workspace allocation failed");
+  }
+  if (bytes > h->ws_bytes) {
+    cudaFree(h->ws);
+    h->ws = nullptr;
+    h->ws_bytes = 0;
+    const size_t c = std::max(bytes, (size_t)1 << 16);
+    if (cudaMalloc(&h->ws, c) != cudaSuccess) {
+      h->ws = nullptr;
+      return fail(ME_ERR_OOM, "workspace allocation failed");
+    }
+    h->ws_bytes = c;
+  }
+  *dev = h->ws;
+  *host = h->ws_host;
+  ME_CUDA(cudaHostGetDevicePointer(host_dev, h->ws_host, 0));
   return ME_OK;
 }
 

@@ -19,6 +19,9 @@ int me_internal_launch_counted(me_handle* h, int me_kind, const double* d_p, con
 // Final-state masses of the handle's process (outgoing legs in order; at most 4), their
 // number, and the handle's stream.
 int me_internal_final_masses(me_handle* h, double* masses, int* n_out, cudaStream_t* stream);
+// Device workspace of at least `bytes` that the handle keeps between calls (grown on demand;
+// its contents do not survive growth), and 64 B of mapped host memory with its device address.
+int me_internal_workspace(me_handle* h, size_t bytes, void** dev, void** host, void** host_dev);
 // Process id (index into the library's process table) of a name, or -1.
 int me_internal_process_id(const char* name);
 // Process id of a handle, or -1 for NULL.
