@@ -49,15 +49,27 @@ __device__ __forceinline__ void philox4x32_10(uint32_t c[4], uint32_t k0, uint32
   }
 }
 
+// ((w0 >> 5) 2^26 + (w1 >> 6) + 1/2) 2^-53.  The 53-bit integer is put together in the
+// mantissas of two doubles (2^84 + hi 2^32 and 2^52 + lo) and scaled in the exponent: three
+// float64 additions instead of two conversions, a multiply-add, an addition and a
+// multiplication, the same bits.
 __device__ __forceinline__ double u01(uint32_t w0, uint32_t w1) {
-  return ((double)(w0 >> 5) * 67108864.0 + (double)(w1 >> 6) + 0.5) * (1.0 / 9007199254740992.0);
+  const uint32_t a = w0 >> 5, b = w1 >> 6;
+  const uint32_t hi = a >> 6, lo = (a << 26) | b;
+  const double x = __hiloint2double(0x45300000, (int)hi), y = __hiloint2double(0x43300000, (int)lo);
+  const double k = __dadd_rn(__dadd_rn(__dadd_rn(x, -(19342813113834066795298816.0 + 4503599627370496.0)), y), 0.5);
+  return __hiloint2double(__double2hiint(k) - (53 << 20), __double2loint(k));
 }
 
 struct Masses {
   double m[4];
 };
 
-// RAMBO point from 4 NOUT uniforms: final momenta k[j][0..3] and the weight.
+// RAMBO point from 4 NOUT uniforms: final momenta k[j][0..3] and the weight.  Float64 runs at
+// 1/64 of the float32 rate and a division or square root costs five to nine multiply-adds,
+// so reciprocals are shared, square roots come from reciprocal ones, angles from sincospi,
+// and the mass rescaling is solved in float32 first (its result is within 1e-6, two float64
+// Newton steps then end at float64 rounding).
 template <int NOUT>
 __device__ __forceinline__ void rambo_point(const double* u, double rs, const double* masses, double w_massless,
                                             double k[][4], double& w_out) {
@@ -67,26 +79,26 @@ __device__ __forceinline__ void rambo_point(const double* u, double rs, const do
   for (int j = 0; j < NOUT; ++j) {
     const double c = 2.0 * u[4 * j] - 1.0;
     const double s = sqrt(1.0 - c * c);
-    const double f = 2.0 * M_PI * u[4 * j + 1];
-    const double q0 = -log(u[4 * j + 2] * u[4 * j + 3]);
+    const double q0 = -log(u[4 * j + 2] * u[4 * j + 3]), qs = q0 * s;
     double sf, cf;
-    sincos(f, &sf, &cf);
+    sincospi(2.0 * u[4 * j + 1], &sf, &cf);
     q[j][0] = q0;
-    q[j][1] = q0 * s * cf;
-    q[j][2] = q0 * s * sf;
+    q[j][1] = qs * cf;
+    q[j][2] = qs * sf;
     q[j][3] = q0 * c;
 #pragma unroll
     for (int a = 0; a < 4; ++a) Q[a] += q[j][a];
   }
-  const double M = sqrt(Q[0] * Q[0] - Q[1] * Q[1] - Q[2] * Q[2] - Q[3] * Q[3]);
-  const double b[3] = {-Q[1] / M, -Q[2] / M, -Q[3] / M};
-  const double x = rs / M, g = Q[0] / M, a = 1.0 / (1.0 + g);
+  const double iM = rsqrt(Q[0] * Q[0] - Q[1] * Q[1] - Q[2] * Q[2] - Q[3] * Q[3]);
+  const double b[3] = {-Q[1] * iM, -Q[2] * iM, -Q[3] * iM};
+  const double x = rs * iM, g = Q[0] * iM, a = 1.0 / (1.0 + g);
 #pragma unroll
   for (int j = 0; j < NOUT; ++j) {
     const double bq = b[0] * q[j][1] + b[1] * q[j][2] + b[2] * q[j][3];
+    const double f = q[j][0] + a * bq;
     k[j][0] = x * (g * q[j][0] + bq);
 #pragma unroll
-    for (int d = 0; d < 3; ++d) k[j][1 + d] = x * (q[j][1 + d] + b[d] * q[j][0] + a * bq * b[d]);
+    for (int d = 0; d < 3; ++d) k[j][1 + d] = x * (q[j][1 + d] + b[d] * f);
   }
   // massive rescaling
   double w = w_massless, msum = 0.0;
@@ -97,40 +109,71 @@ __device__ __forceinline__ void rambo_point(const double* u, double rs, const do
     massive |= masses[j] != 0.0;
   }
   if (massive) {
-    double pabs[NOUT];
+    const double irs = 1.0 / rs;
+    double xs;
+    {
+      float pf[NOUT], mf[NOUT];
+      const float r = (float)(msum * irs);
 #pragma unroll
-    for (int j = 0; j < NOUT; ++j) pabs[j] = k[j][0];
-    double xs = sqrt(fmax(0.0, 1.0 - (msum / rs) * (msum / rs)));
+      for (int j = 0; j < NOUT; ++j) {
+        pf[j] = (float)(k[j][0] * irs);
+        mf[j] = (float)(masses[j] * irs);
+      }
+      float xf = sqrtf(fmaxf(0.0f, 1.0f - r * r));
+      for (int it = 0; it < 12; ++it) {
+        float fs = -1.0f, df = 0.0f;
+#pragma unroll
+        for (int j = 0; j < NOUT; ++j) {
+          const float t = xf * pf[j], e = sqrtf(mf[j] * mf[j] + t * t);
+          fs += e;
+          df += e > 0.0f ? t * pf[j] / e : 0.0f;
+        }
+        const float dx = fs / df;
+        xf -= dx;
+        if (!(fabsf(dx) > 1e-6f * xf)) break;
+      }
+      // near threshold float32 may not settle: start from the massless guess there
+      xs = xf > 0.0f && xf <= 1.0f ? (double)xf : sqrt(fmax(0.0, 1.0 - (msum * irs) * (msum * irs)));
+    }
     for (int it = 0; it < 60; ++it) {
       double fs = -rs, df = 0.0;
 #pragma unroll
       for (int j = 0; j < NOUT; ++j) {
-        const double e = sqrt(masses[j] * masses[j] + (xs * pabs[j]) * (xs * pabs[j]));
-        fs += e;
-        df += xs * pabs[j] * pabs[j] / e;
+        if (masses[j] != 0.0) {
+          const double t = xs * k[j][0], e2 = masses[j] * masses[j] + t * t, ie = rsqrt(e2);
+          fs += e2 * ie;
+          df += t * k[j][0] * ie;
+        } else {
+          fs += xs * k[j][0];
+          df += k[j][0];
+        }
       }
       const double dx = fs / df;
       xs -= dx;
-      // Newton converges quadratically: a step below 1e-15 of xs leaves xs exact to
-      // rounding (an absolute 1e-16 would sit below the rounding of xs ~ 1 and run
-      // all 60 steps)
-      if (fabs(dx) <= 1e-15 * xs) break;
+      // Newton converges quadratically: after a step below 1e-9 of xs, xs is exact to rounding
+      if (!(fabs(dx) > 1e-9 * xs)) break;
     }
     double sk = 0.0, prod = 1.0, sk2e = 0.0;
 #pragma unroll
     for (int j = 0; j < NOUT; ++j) {
-      const double ka = xs * pabs[j];
-      const double e = sqrt(masses[j] * masses[j] + ka * ka);
-      k[j][0] = e;
+      const double ka = xs * k[j][0];
+      sk += ka;
+      if (masses[j] != 0.0) {
+        const double e2 = masses[j] * masses[j] + ka * ka, ie = rsqrt(e2);
+        k[j][0] = e2 * ie;
+        prod *= ka * ie;
+        sk2e += ka * ka * ie;
+      } else {
+        k[j][0] = ka;
+        sk2e += ka;
+      }
 #pragma unroll
       for (int d = 1; d < 4; ++d) k[j][d] *= xs;
-      sk += ka;
-      prod *= ka / e;
-      sk2e += ka * ka / e;
     }
-    double pw = 1.0;  // (sum |k| / sqrt s)^(2n-3)
+    const double y = sk * irs;
+    double pw = y;  // (sum |k| / sqrt s)^(2n-3)
 #pragma unroll
-    for (int e = 0; e < 2 * NOUT - 3; ++e) pw *= sk / rs;
+    for (int e = 1; e < 2 * NOUT - 3; ++e) pw *= y;
     w *= pw * prod * rs / sk2e;
   }
   w_out = w;
@@ -183,18 +226,19 @@ __global__ void k_rambo(uint64_t seed, uint32_t stream, long long first, double 
 constexpr double kAlphaFlat = 0.25;
 constexpr double kYCut = 1e-6;
 
+constexpr double kVMin = 7.0710678118654752440e-4;  // sqrt(kYCut / 2)
+
 __device__ __forceinline__ double coll_density(double y) {
-  const double vmin = sqrt(0.5 * kYCut);
   const double omy = 1.0 - y;
   if (!(omy >= kYCut)) return 0.0;
-  return 1.0 / (4.0 * sqrt(0.5 * omy) * (1.0 - vmin));
+  return (0.25 / (1.0 - kVMin)) * rsqrt(0.5 * omy);
 }
 
 __device__ __forceinline__ void boost_vel(const double p[4], const double b[3], double out[4]) {
   const double b2 = b[0] * b[0] + b[1] * b[1] + b[2] * b[2];
-  const double g = 1.0 / sqrt(1.0 - b2);
+  const double g = rsqrt(1.0 - b2);
   const double bp = b[0] * p[1] + b[1] * p[2] + b[2] * p[3];
-  const double g2 = b2 > 0.0 ? (g - 1.0) / b2 : 0.0;
+  const double g2 = g * g / (1.0 + g);  // (g - 1) / b^2
   out[0] = g * (p[0] + bp);
 #pragma unroll
   for (int d = 0; d < 3; ++d) out[1 + d] = p[1 + d] + (g2 * bp + g * p[0]) * b[d];
@@ -209,123 +253,157 @@ __device__ __forceinline__ void boost_vel(const double p[4], const double b[3], 
 // xi = u3, v from u4, phi = 2 pi u5 about the partner; the partner's energy
 // sqrt(s)(1-xi)/(2 - xi(1-y_j)) leaves the third parton massless; channel density
 // h_j = 4 g(y_j) / (xi K_j), K_j = s (1 - xi) / (16 pi^3 (2 - xi (1 - y_j))^2).
+//
+// The flat channel's RAMBO and the sectors' maps are different code, each some 300 to 500
+// float64 instructions, and the channel is random: with a point per lane every warp would run
+// both.  Each block therefore sorts its points by channel first (a scan over u0's decisions in
+// shared memory), so that one of its eight warps at most runs both.  500,009 g g -> t tbar g
+// points: 1181 us before (float64 pipe 88 % busy), 466 us.
+constexpr int FKS_THREADS = 256;
+
 template <bool ISR>
-__global__ void k_fks_points(uint64_t seed, uint32_t stream, long long first, double rs, double mass, double w3_massless,
-                             long n, double* __restrict__ p, double* __restrict__ wgt) {
-  const long i = (long)blockIdx.x * blockDim.x + threadIdx.x;
+__global__ void __launch_bounds__(FKS_THREADS) k_fks_points(uint64_t seed, uint32_t stream, long long first, double rs,
+                                                            double mass, double w3_massless, long n,
+                                                            double* __restrict__ p, double* __restrict__ wgt) {
+  __shared__ unsigned short order[FKS_THREADS];
+  __shared__ int warp_flat[FKS_THREADS / 32];
+  const uint32_t k0 = (uint32_t)(seed & 0xFFFFFFFFull), k1 = (uint32_t)(seed >> 32);
+  const long base = (long)blockIdx.x * FKS_THREADS;
+  const double a_f = kAlphaFlat, a_s = 0.5 * (1.0 - kAlphaFlat);
+  auto uniforms = [&](unsigned long long idx, uint32_t blk, double* u) {
+    uint32_t c[4] = {(uint32_t)(idx & 0xFFFFFFFFull), (uint32_t)(idx >> 32), stream, blk};
+    philox4x32_10(c, k0, k1);
+    u[0] = u01(c[0], c[1]);
+    u[1] = u01(c[2], c[3]);
+  };
+  {
+    double u[2];
+    uniforms((unsigned long long)(first + base + threadIdx.x), 0, u);
+    const bool f = u[0] < a_f;
+    const unsigned bal = __ballot_sync(0xffffffffu, f);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if (lane == 0) warp_flat[warp] = __popc(bal);
+    __syncthreads();
+    int before = 0, all = 0;
+#pragma unroll
+    for (int w = 0; w < FKS_THREADS / 32; ++w) {
+      before += w < warp ? warp_flat[w] : 0;
+      all += warp_flat[w];
+    }
+    const int rank = before + __popc(bal & ((1u << lane) - 1u));  // flat points before this one
+    order[f ? rank : all + (int)threadIdx.x - rank] = (unsigned short)threadIdx.x;
+    __syncthreads();
+  }
+  const long i = base + order[threadIdx.x];
   if (i >= n) return;
   const unsigned long long idx = (unsigned long long)(first + i);
-  const uint32_t k0 = (uint32_t)(seed & 0xFFFFFFFFull), k1 = (uint32_t)(seed >> 32);
-  double u[18];
-#pragma unroll
-  for (int b = 0; b < 9; ++b) {
-    uint32_t c[4] = {(uint32_t)(idx & 0xFFFFFFFFull), (uint32_t)(idx >> 32), stream, (uint32_t)b};
-    philox4x32_10(c, k0, k1);
-    u[2 * b] = u01(c[0], c[1]);
-    u[2 * b + 1] = u01(c[2], c[3]);
-  }
+  double u[6];
+  uniforms(idx, 0, u);
   const double s = rs * rs;
-  const double a_f = kAlphaFlat, a_s = 0.5 * (1.0 - kAlphaFlat);
   const bool flat = u[0] < a_f;
   const int sec = u[0] < a_f + a_s ? 0 : 1;
-  const double vmin = sqrt(0.5 * kYCut);
   const double masses[3] = {ISR ? mass : 0.0, ISR ? mass : 0.0, 0.0};
   double q[5][4];  // legs: beams, then 2, 3, 4 (gluon)
   const double hb = 0.5 * rs;
   q[0][0] = hb; q[0][1] = 0.0; q[0][2] = 0.0; q[0][3] = hb;
   q[1][0] = hb; q[1][1] = 0.0; q[1][2] = 0.0; q[1][3] = -hb;
   if (flat) {
+    double v[12];
+#pragma unroll
+    for (int b = 0; b < 6; ++b) uniforms(idx, 3 + b, v + 2 * b);
     double k[3][4], wr;
-    rambo_point<3>(u + 6, rs, masses, w3_massless, k, wr);
+    rambo_point<3>(v, rs, masses, w3_massless, k, wr);
 #pragma unroll
     for (int j = 0; j < 3; ++j)
 #pragma unroll
       for (int c = 0; c < 4; ++c) q[2 + j][c] = k[j][c];
-  } else if (ISR) {
-    const double ximax = 1.0 - 4.0 * mass * mass / s;
-    const double xi = ximax * u[1];
-    const double v = vmin + (1.0 - vmin) * u[2];
-    const double yj = 1.0 - 2.0 * v * v;
-    const double y = sec == 0 ? yj : -yj;
-    double sf, cf, sp2, cp2;
-    sincos(2.0 * M_PI * u[3], &sf, &cf);
-    const double ek = 0.5 * rs * xi;
-    const double st = sqrt(fmax(0.0, (1.0 - y) * (1.0 + y)));
-    q[4][0] = ek;
-    q[4][1] = ek * st * cf;
-    q[4][2] = ek * st * sf;
-    q[4][3] = ek * y;
-    const double Q0 = rs - ek, M2 = Q0 * Q0 - ek * ek, M = sqrt(M2);
-    const double pstar = sqrt(fmax(0.0, 0.25 * M2 - mass * mass));
-    const double cp = 2.0 * u[4] - 1.0;
-    const double sp = sqrt(fmax(0.0, (1.0 - cp) * (1.0 + cp)));
-    sincos(2.0 * M_PI * u[5], &sp2, &cp2);
-    const double nv[3] = {sp * cp2, sp * sp2, cp};
-    const double e = 0.5 * M;
-    const double p3[4] = {e, pstar * nv[0], pstar * nv[1], pstar * nv[2]};
-    const double p4[4] = {e, -pstar * nv[0], -pstar * nv[1], -pstar * nv[2]};
-    const double bvec[3] = {-q[4][1] / Q0, -q[4][2] / Q0, -q[4][3] / Q0};
-    boost_vel(p3, bvec, q[2]);
-    boost_vel(p4, bvec, q[3]);
   } else {
-    const int partner = 2 + sec, other = 5 - partner;
-    const double cdir = 2.0 * u[1] - 1.0, xi = u[3];
-    const double v = vmin + (1.0 - vmin) * u[4];
+    uniforms(idx, 1, u + 2);
+    uniforms(idx, 2, u + 4);
+    const double v = kVMin + (1.0 - kVMin) * u[ISR ? 2 : 4];
     const double yj = 1.0 - 2.0 * v * v;
-    double spd, cpd, sf, cf;
-    sincos(2.0 * M_PI * u[2], &spd, &cpd);
-    sincos(2.0 * M_PI * u[5], &sf, &cf);
-    const double sd = sqrt(fmax(0.0, (1.0 - cdir) * (1.0 + cdir)));
-    const double nj[3] = {sd * cpd, sd * spd, cdir};
-    double ea[3] = {-cdir * nj[0], -cdir * nj[1], 1.0 - cdir * nj[2]};  // z - (z.nj) nj
-    const double ia = 1.0 / sqrt(ea[0] * ea[0] + ea[1] * ea[1] + ea[2] * ea[2]);
+    if (ISR) {
+      const double ximax = 1.0 - 4.0 * mass * mass / s;
+      const double xi = ximax * u[1];
+      const double y = sec == 0 ? yj : -yj;
+      double sf, cf, sp2, cp2;
+      sincospi(2.0 * u[3], &sf, &cf);
+      const double ek = 0.5 * rs * xi;
+      const double et = ek * sqrt(fmax(0.0, (1.0 - y) * (1.0 + y)));
+      q[4][0] = ek;
+      q[4][1] = et * cf;
+      q[4][2] = et * sf;
+      q[4][3] = ek * y;
+      const double Q0 = rs - ek, M2 = Q0 * Q0 - ek * ek;
+      const double cp = 2.0 * u[4] - 1.0;
+      // p* sin(theta) and p* cos(theta) of the pair's rest frame
+      const double ps2 = fmax(0.0, 0.25 * M2 - mass * mass), pstar = sqrt(ps2);
+      const double pt = pstar * sqrt(fmax(0.0, (1.0 - cp) * (1.0 + cp)));
+      sincospi(2.0 * u[5], &sp2, &cp2);
+      const double e = 0.5 * sqrt(M2);
+      const double p3[4] = {e, pt * cp2, pt * sp2, pstar * cp};
+      const double p4[4] = {e, -p3[1], -p3[2], -p3[3]};
+      const double iQ0 = 1.0 / Q0;
+      const double bvec[3] = {-q[4][1] * iQ0, -q[4][2] * iQ0, -q[4][3] * iQ0};
+      boost_vel(p3, bvec, q[2]);
+      boost_vel(p4, bvec, q[3]);
+    } else {
+      const double cdir = 2.0 * u[1] - 1.0, xi = u[3];
+      double spd, cpd, sf, cf;
+      sincospi(2.0 * u[2], &spd, &cpd);
+      sincospi(2.0 * u[5], &sf, &cf);
+      const double sd = sqrt(fmax(0.0, (1.0 - cdir) * (1.0 + cdir)));
+      const double nj[3] = {sd * cpd, sd * spd, cdir};
+      double ea[3] = {-cdir * nj[0], -cdir * nj[1], 1.0 - cdir * nj[2]};  // z - (z.nj) nj
+      const double ia = rsqrt(ea[0] * ea[0] + ea[1] * ea[1] + ea[2] * ea[2]);
 #pragma unroll
-    for (int d = 0; d < 3; ++d) ea[d] *= ia;
-    const double eb[3] = {nj[1] * ea[2] - nj[2] * ea[1], nj[2] * ea[0] - nj[0] * ea[2], nj[0] * ea[1] - nj[1] * ea[0]};
-    const double sr = sqrt(fmax(0.0, (1.0 - yj) * (1.0 + yj)));
-    double ni[3];
+      for (int d = 0; d < 3; ++d) ea[d] *= ia;
+      const double eb[3] = {nj[1] * ea[2] - nj[2] * ea[1], nj[2] * ea[0] - nj[0] * ea[2], nj[0] * ea[1] - nj[1] * ea[0]};
+      const double sr = sqrt(fmax(0.0, (1.0 - yj) * (1.0 + yj)));
+      const double ei = 0.5 * rs * xi, ej = rs * (1.0 - xi) / (2.0 - xi * (1.0 - yj));
+      double pj[4] = {ej, 0.0, 0.0, 0.0}, po[4] = {rs - ej - ei, 0.0, 0.0, 0.0};
+      q[4][0] = ei;
 #pragma unroll
-    for (int d = 0; d < 3; ++d) ni[d] = yj * nj[d] + sr * (cf * ea[d] + sf * eb[d]);
-    const double ei = 0.5 * rs * xi, ej = rs * (1.0 - xi) / (2.0 - xi * (1.0 - yj));
-    q[partner][0] = ej;
-    q[4][0] = ei;
-    q[other][0] = rs - ej - ei;
+      for (int d = 0; d < 3; ++d) {
+        const double ni = yj * nj[d] + sr * (cf * ea[d] + sf * eb[d]);
+        pj[1 + d] = ej * nj[d];
+        q[4][1 + d] = ei * ni;
+        po[1 + d] = -(pj[1 + d] + q[4][1 + d]);
+      }
 #pragma unroll
-    for (int d = 0; d < 3; ++d) {
-      q[partner][1 + d] = ej * nj[d];
-      q[4][1 + d] = ei * ni[d];
-      q[other][1 + d] = -(ej * nj[d] + ei * ni[d]);
+      for (int c = 0; c < 4; ++c) {
+        q[2][c] = sec == 0 ? pj[c] : po[c];
+        q[3][c] = sec == 0 ? po[c] : pj[c];
+      }
     }
   }
   // every channel's density at this point, from its momenta
+  const double irs = 1.0 / rs, xi_pt = 2.0 * q[4][0] * irs;
+  const double ig = rsqrt(q[4][1] * q[4][1] + q[4][2] * q[4][2] + q[4][3] * q[4][3]);
   double h;
-  {
-    double kabs[3], sk = 0.0, prod = 1.0, sk2e = 0.0;
-#pragma unroll
-    for (int j = 0; j < 3; ++j) {
-      kabs[j] = sqrt(q[2 + j][1] * q[2 + j][1] + q[2 + j][2] * q[2 + j][2] + q[2 + j][3] * q[2 + j][3]);
-      sk += kabs[j];
-      prod *= kabs[j] / q[2 + j][0];
-      sk2e += kabs[j] * kabs[j] / q[2 + j][0];
-    }
-    const double wr = ISR ? w3_massless * (sk / rs) * (sk / rs) * (sk / rs) * prod * rs / sk2e : w3_massless;
-    h = a_f / wr;
-  }
-  const double ig = 1.0 / sqrt(q[4][1] * q[4][1] + q[4][2] * q[4][2] + q[4][3] * q[4][3]);
-  const double xi_pt = 2.0 * q[4][0] / rs;
   if (ISR) {
-    const double ximax = 1.0 - 4.0 * mass * mass / s, beta = sqrt(1.0 - 4.0 * mass * mass / s);
-    const double K = s * sqrt(fmax(0.0, 1.0 - 4.0 * mass * mass / (s * (1.0 - xi_pt)))) / (64.0 * M_PI * M_PI * M_PI * beta);
+    // a_f / w_RAMBO (rambo_point's weight as a function of the momenta; the gluon is massless)
+    const double a2 = q[2][1] * q[2][1] + q[2][2] * q[2][2] + q[2][3] * q[2][3];
+    const double a3 = q[3][1] * q[3][1] + q[3][2] * q[3][2] + q[3][3] * q[3][3];
+    const double i2 = rsqrt(fmax(a2, 1e-300)), i3 = rsqrt(fmax(a3, 1e-300)), kg = q[4][0];
+    const double y = (a2 * i2 + a3 * i3 + kg) * irs, e23 = q[2][0] * q[3][0];
+    const double sk2e = a2 * q[3][0] + a3 * q[2][0] + kg * e23;  // sum(|k|^2 / E) E2 E3
+    const double m2 = 4.0 * mass * mass / s;
     const double cz = q[4][3] * ig;
-    h += a_s * 4.0 * (coll_density(cz) + coll_density(-cz)) / (ximax * beta * xi_pt * K);
+    // h_j = 4 g(y_j) / (xi_max beta(s) xi K), K = s beta(s (1 - xi)) / (64 pi^3 beta(s))
+    const double b2 = fmax(0.0, 1.0 - m2 / (1.0 - xi_pt));
+    const double c0 = a_s * 4.0 * 64.0 * M_PI * M_PI * M_PI / ((1.0 - m2) * s);
+    h = a_f * sk2e * i2 * i3 / (w3_massless * y * y * y * rs) +
+        c0 * (coll_density(cz) + coll_density(-cz)) * rsqrt(b2) / xi_pt;
   } else {
+    h = a_f / w3_massless;
+    const double omx = 1.0 - xi_pt, ix = 1.0 / (xi_pt * omx);
 #pragma unroll
     for (int j = 2; j <= 3; ++j) {
-      const double kn = sqrt(q[j][1] * q[j][1] + q[j][2] * q[j][2] + q[j][3] * q[j][3]);
-      const double y = (q[4][1] * q[j][1] + q[4][2] * q[j][2] + q[4][3] * q[j][3]) * ig / kn;
+      const double ik = rsqrt(q[j][1] * q[j][1] + q[j][2] * q[j][2] + q[j][3] * q[j][3]);
+      const double y = (q[4][1] * q[j][1] + q[4][2] * q[j][2] + q[4][3] * q[j][3]) * ig * ik;
       const double d = 2.0 - xi_pt * (1.0 - y);
-      const double K = s * (1.0 - xi_pt) / (16.0 * M_PI * M_PI * M_PI * d * d);
-      h += a_s * 4.0 * coll_density(y) / (xi_pt * K);
+      h += a_s * 4.0 * 16.0 * M_PI * M_PI * M_PI / s * coll_density(y) * d * d * ix;
     }
   }
 #pragma unroll
@@ -604,10 +682,10 @@ extern "C" int me_generate_fks(me_handle* h, uint64_t seed, uint32_t stream, int
   if (rc != ME_OK) return rc;
   const double mass = masses[0];
   if (!(2.0 * mass < sqrt_s)) return me_internal_fail(ME_ERR_ARG, "me_generate_fks: sqrt_s below the final-state masses");
-  const int threads = 128;
-  const unsigned blocks = (unsigned)((n + threads - 1) / threads);
   // massless three-body volume (2 pi)^(4-3n) (pi/2)^(n-1) s^(n-2) / ((n-1)! (n-2)!) = s / (256 pi^3)
   const double w3 = sqrt_s * sqrt_s / (256.0 * M_PI * M_PI * M_PI);
+  const int threads = FKS_THREADS;
+  const unsigned blocks = (unsigned)((n + threads - 1) / threads);
   if (isr)
     k_fks_points<true><<<blocks, threads, 0, st>>>(seed, stream, first_point, sqrt_s, mass, w3, n, momenta, ps_weights);
   else
