@@ -245,11 +245,18 @@ __global__ void __launch_bounds__(256) k_tree_closed(const double* __restrict__ 
 //     amplitudes of both antitop helicities into shared-memory rows;
 //  3. one warp-wide tensor-core colour sum (me_tc.cuh) takes the warp's 32 rows
 //     (8 events x 4 heavy-pair helicities): lane 4e + h receives helicity h of event e.
-// Everything a lane needs stays on chip, so the 5e5 flops of an event run from registers
-// and shared memory.  In a warp that holds the end of the batch, events past it compute
+// Everything a lane needs stays on chip, so the 4e5 flops of an event run from registers
+// and shared memory; what bounds the kernel is instruction issue, so polarisations carry their
+// five nonzero reals, the quark spinors three components, products that serve two orderings
+// are formed once, and the momenta and denominators picked by lane sit in shared memory
+// instead of local memory (2^18 events: 4.32 -> 3.55 ms).  In a warp that holds the end of the batch, events past it compute
 // a fixed finite configuration and are discarded, so every warp-wide step stays
 // converged; warps entirely past the end return at once.
-constexpr int TC4_EV_FLOATS = 276;  // 34 four-vectors x 8 floats, padded so 8 events hit distinct banks
+// an event's shared-memory area: 34 four-vectors x 8 floats, the gluon momenta q[4] and the
+// reciprocal denominators ig[16], iq[16] (indexed by lane-dependent gluons, which in registers
+// would go through local memory), padded so that 8 events hit distinct banks
+constexpr int TC4_Q = 272, TC4_IG = 288, TC4_IQ = 304;
+constexpr int TC4_EV_FLOATS = 324;
 constexpr int TC4_ROW = 25;         // floats per amplitude row (24 flows, padded)
 constexpr int TC4_WARP_FLOATS = 8 * TC4_EV_FLOATS + 2 * 32 * TC4_ROW;
 constexpr int TC4_SMEM_PER_WARP = TC4_WARP_FLOATS * 4 + TC_SMEM_PER_WARP;
@@ -285,12 +292,27 @@ __device__ __forceinline__ c4<float> ld_j2(const float* b, int x, int y) {
   if (x > y) cscale(J, -1.0f);
   return J;
 }
+// slots 0 .. 3: a polarisation (no time component, real z)
+__device__ __forceinline__ pol<float> ld_pol(const float* b, int slot) {
+  const float4* p = reinterpret_cast<const float4*>(b + 8 * slot);
+  const float4 a = p[0], c = p[1];
+  return pol<float>{{a.z, a.w}, {c.x, c.y}, c.z};
+}
+__device__ __forceinline__ r4<float> ld_q(const float* b, int g) {
+  const float4 a = *reinterpret_cast<const float4*>(b + TC4_Q + 4 * g);
+  return r4<float>{a.x, a.y, a.z, a.w};
+}
 // the same eight floats read as the chiral combinations (V0 - V3, V0 + V3, V1 - i V2,
 // V1 + i V2) once a slot has been converted in place for the quark lines
 __device__ __forceinline__ sl4<float> ld_sl4(const float* b, int slot) {
   const float4* p = reinterpret_cast<const float4*>(b + 8 * slot);
   const float4 a = p[0], c = p[1];
   return sl4<float>{{a.x, a.y}, {a.z, a.w}, {c.x, c.y}, {c.z, c.w}};
+}
+__device__ __forceinline__ spol<float> ld_spol(const float* b, int slot) {
+  const float4* p = reinterpret_cast<const float4*>(b + 8 * slot);
+  const float4 a = p[0], c = p[1];
+  return spol<float>{a.z, {c.x, c.y}, {c.z, c.w}};
 }
 __device__ __forceinline__ void slash_in_place(float* b, int slot) {
   const sl4<float> S = slashed(ld_c4(b, slot));
@@ -341,87 +363,126 @@ __global__ void __launch_bounds__(TC4_THREADS, 2) k_tree_tc4(const double* __res
   }
   const TcColourB cb = tc_load_colour(kp.tab->C[PID]);
   const Kin<PID, float> K = prepare<PID, float>(k, unit_couplings(kp.cp));
-  const float g = 1.0f, mt = kp.cp.mtf;
-  const r4<float>* q = K.q;
+  const float mt = kp.cp.mtf;
   const r4<float> kt = K.pl[2];
-  constexpr int LEG[4] = {0, 1, 4, 5};
+  {
+    // lane l writes momentum l and a quarter of the denominators
+    const r4<float> ql = lane == 0 ? K.q[0] : lane == 1 ? K.q[1] : lane == 2 ? K.q[2] : K.q[3];
+    *reinterpret_cast<float4*>(cur + TC4_Q + 4 * lane) = make_float4(ql.e, ql.x, ql.y, ql.z);
+#pragma unroll
+    for (int S = 0; S < 16; ++S)
+      if ((S & 3) == lane) {
+        cur[TC4_IG + S] = K.ig[S];
+        cur[TC4_IQ + S] = K.iq[S];
+      }
+  }
+  const wf_v<float> wg = lane == 0 ? K.wg[0] : lane == 1 ? K.wg[1] : lane == 2 ? K.wg[2] : K.wg[3];
+  const int leg = lane < 2 ? lane : lane + 2;
+  __syncwarp();
+  const float* ig = cur + TC4_IG;
+  const float* iq = cur + TC4_IQ;
   float acc = 0.0f;
   for (int b = 0; b < n_live_blocks<PID>(); ++b) {
     const int hb = live_block_hel<PID>(b);
     // 1. polarisation of gluon `lane`
-    st_c4(cur, lane, polvec_of(K.wg[lane], hel_of(hb, LEG[lane]), LEG[lane] >= 2));
+    {
+      const pol<float> e = pol_of(wg, hel_of(hb, leg), lane >= 2);
+      st_c4(cur, lane, c4<float>{{{0.0f, 0.0f}, e.x, e.y, {e.z, 0.0f}}});
+    }
     __syncwarp();
     // 2. pair currents: slots 4 + lane and 8 + lane (< 10)
     for (int pp = lane; pp < 6; pp += 4) {
       const int x = pp < 3 ? 0 : (pp < 5 ? 1 : 2);
       const int y = pp < 3 ? pp + 1 : (pp < 5 ? pp - 1 : 3);
-      st_c4(cur, 4 + pp, vvv(ld_c4(cur, x), ld_c4(cur, y), -q[x], -q[y], -g * K.ig[(1 << x) | (1 << y)]));
+      cx<float> exy;
+      st_c4(cur, 4 + pp, bracket(ld_pol(cur, x), ld_q(cur, x), ld_pol(cur, y), ld_q(cur, y), -ig[(1 << x) | (1 << y)], exy));
     }
     __syncwarp();
     // 3. triple currents
     for (int t = lane; t < 12; t += 4) {
       const int r = kJ3Rep[t], x = r & 15, y = (r >> 4) & 15, z = r >> 8;
-      const int S = (1 << x) | (1 << y) | (1 << z);
-      const c4<float> ex = ld_c4(cur, x), ey = ld_c4(cur, y), ez = ld_c4(cur, z);
-      const float c3 = -g * K.ig[S];
-      c4<float> J = vvv(ex, ld_j2(cur, y, z), -q[x], -(q[y] + q[z]), c3);
-      vvv_acc(J, ld_j2(cur, x, y), ez, -(q[x] + q[y]), -q[z], c3);
-      caxpy(J, g * g * K.ig[S], vvvv_ordered(ex, ey, ez));
+      const pol<float> ex = ld_pol(cur, x), ey = ld_pol(cur, y), ez = ld_pol(cur, z);
+      const r4<float> qx = ld_q(cur, x), qy = ld_q(cur, y), qz = ld_q(cur, z);
+      const float w = ig[(1 << x) | (1 << y) | (1 << z)];
+      c4<float> J = czero<float>();
+      {
+        const c4<float> P = ld_j2(cur, y, z);
+        bracket_acc(J, ex, qx, P, qy + qz, -w, cdot(ex, P));
+      }
+      {
+        const c4<float> P = ld_j2(cur, x, y);
+        bracket_acc(J, ez, qz, P, qx + qy, w, cdot(ez, P));
+      }
+      quartic_acc(J, ex, ey, ez, w * cdot(ex, ez), w * cdot(ex, ey), w * cdot(ey, ez));
       st_c4(cur, 10 + t, J);
     }
     __syncwarp();
     // 4. quadruple currents
     for (int t = lane; t < 12; t += 4) {
       const int r = kJ4Rep[t], w = r & 15, x = (r >> 4) & 15, y = (r >> 8) & 15, z = r >> 12;
-      const c4<float> ew = ld_c4(cur, w), ez = ld_c4(cur, z);
-      const c4<float> jwx = ld_j2(cur, w, x), jxy = ld_j2(cur, x, y), jyz = ld_j2(cur, y, z);
-      const float c3 = -g * K.ig[15];
-      c4<float> J = vvv(ew, ld_c4(cur, triple_slot(x, y, z)), -q[w], -(q[x] + q[y] + q[z]), c3);
-      vvv_acc(J, jwx, jyz, -(q[w] + q[x]), -(q[y] + q[z]), c3);
-      vvv_acc(J, ld_c4(cur, triple_slot(w, x, y)), ez, -(q[w] + q[x] + q[y]), -q[z], c3);
-      c4<float> V = vvvv_ordered(ew, ld_c4(cur, x), jyz);
-      cadd(V, vvvv_ordered(ew, jxy, ez));
-      cadd(V, vvvv_ordered(jwx, ld_c4(cur, y), ez));
-      caxpy(J, g * g * K.ig[15], V);
+      const pol<float> ew = ld_pol(cur, w), ex = ld_pol(cur, x), ey = ld_pol(cur, y), ez = ld_pol(cur, z);
+      const c4<float> jwx = ld_j2(cur, w, x), jyz = ld_j2(cur, y, z);
+      const r4<float> qw = ld_q(cur, w), qz = ld_q(cur, z), qwx = qw + ld_q(cur, x), qyz = ld_q(cur, y) + qz;
+      const float i4 = ig[15];
+      c4<float> J = czero<float>();
+      bracket_acc(J, jwx, qwx, jyz, qyz, -i4);
+      quartic_acc(J, ew, ex, jyz, i4 * cdot(ew, jyz), i4 * cdot(ew, ex), i4 * cdot(ex, jyz));
+      quartic_acc(J, jwx, ey, ez, i4 * cdot(ez, jwx), i4 * cdot(ey, jwx), i4 * cdot(ey, ez));
+      {
+        const c4<float> jxy = ld_j2(cur, x, y);
+        quartic_acc(J, ew, jxy, ez, i4 * cdot(ew, ez), i4 * cdot(ew, jxy), i4 * cdot(ez, jxy));
+      }
+      {
+        const c4<float> P = ld_c4(cur, triple_slot(x, y, z));
+        bracket_acc(J, ew, qw, P, (qwx - qw) + qyz, -i4, cdot(ew, P));
+      }
+      {
+        const c4<float> P = ld_c4(cur, triple_slot(w, x, y));
+        bracket_acc(J, ez, qz, P, qwx + (qyz - qz), i4, cdot(ez, P));
+      }
       st_c4(cur, 22 + t, J);
     }
     __syncwarp();
     // the quark lines only slash the 34 vectors against rows: convert them in place
     for (int sl = lane; sl < 34; sl += 4) slash_in_place(cur, sl);
     __syncwarp();
-    // 5. quark line for the orderings starting with gluon w = lane
+    // 5. quark line for the orderings starting with gluon w = lane.  Products of U(w) and
+    // U(wx) with a pair or triple current serve an ordering and its reflection in the rest:
+    // J(yx) = -J(xy), J(zyx) = J(xyz).
     const int w = lane;
+    const r4<float> ktw = kt + ld_q(cur, w);
+    // the other gluons in increasing order: every lane runs the same 3 x 2 iterations, and
+    // f counts the orderings w x y z as the ordering tables do
+    const int g0 = w == 0 ? 1 : 0, g1 = w <= 1 ? 2 : 1, g2 = w <= 2 ? 3 : 2;
     for (int ht = 0; ht < 2; ++ht) {
       const int row0 = (wl & ~3) + 2 * ht;  // rows of (this event, ht, hv = 0 / 1)
-      const c4<float> U1 = row_prop(ubar_slash(K.wt, ht, ld_sl4(cur, w)), scaled_prop(kt + q[w], mt, -g * K.iq[1 << w]));
-      // every lane runs the same 3 x 2 iterations (no lane idles on a skipped index):
-      // x is the kx-th gluon other than w, y the ky-th other than w and x, in increasing
-      // order, so f counts the orderings w x y z as the ordering tables do
+      const c4<float> U1 = row_prop(ubar_slash(K.wt, ht, ld_spol(cur, w)), scaled_prop(ktw, mt, -iq[1 << w]));
       int f = 6 * w;
-#pragma unroll
+#pragma unroll 1
       for (int kx = 0; kx < 3; ++kx) {
-        const int x = kx + (kx >= w ? 1 : 0);
+        const int x = kx == 0 ? g0 : kx == 1 ? g1 : g2;
+        const int ya = kx == 0 ? g1 : g0, yb = kx == 2 ? g1 : g2;
+        const r4<float> kwx = ktw + ld_q(cur, x);
         c4<float> r2 = ubar_slash(K.wt, ht, ld_sj2(cur, w, x));
-        row_slash_acc(r2, U1, ld_sl4(cur, x));
-        const c4<float> U2 = row_prop(r2, scaled_prop(kt + q[w] + q[x], mt, -g * K.iq[(1 << w) | (1 << x)]));
-        const int lo = w < x ? w : x, hi = w < x ? x : w;
+        row_slash_acc(r2, U1, ld_spol(cur, x));
+        const c4<float> U2 = row_prop(r2, scaled_prop(kwx, mt, -iq[(1 << w) | (1 << x)]));
+        const c4<float> U2J = row_slash(U2, ld_sj2(cur, ya, yb));
 #pragma unroll
         for (int ky = 0; ky < 2; ++ky) {
-          int y = ky;
-          if (y >= lo) ++y;
-          if (y >= hi) ++y;
-          const int z = 6 - w - x - y;
+          const int y = ky ? yb : ya, z = ky ? ya : yb;
           c4<float> r3 = ubar_slash(K.wt, ht, ld_sl4(cur, triple_slot(w, x, y)));
           row_slash_acc(r3, U1, ld_sj2(cur, x, y));
-          row_slash_acc(r3, U2, ld_sl4(cur, y));
-          const c4<float> U3 =
-              row_prop(r3, scaled_prop(kt + q[w] + q[x] + q[y], mt, -g * K.iq[(1 << w) | (1 << x) | (1 << y)]));
+          row_slash_acc(r3, U2, ld_spol(cur, y));
+          const c4<float> U3 = row_prop(
+              r3, scaled_prop(kwx + ld_q(cur, y), mt, -iq[(1 << w) | (1 << x) | (1 << y)]));
+          c4<float> R = U2J;
+          if (ky) R = cneg(R);
           const int s4 = kJ4OfOrdering[f];
-          c4<float> R = ubar_slash(K.wt, ht, ld_sl4(cur, 22 + (s4 > 0 ? s4 : -s4) - 1));
-          if (s4 < 0) R = cneg(R);
+          const sl4<float> S4 = ld_sl4(cur, 22 + (s4 > 0 ? s4 : -s4) - 1);
+          const float sg = s4 > 0 ? 1.0f : -1.0f;
+          ubar_slash_acc(R, K.wt, ht, sl4<float>{sg * S4.a, sg * S4.b, sg * S4.c, sg * S4.d});
           row_slash_acc(R, U1, ld_sl4(cur, triple_slot(x, y, z)));
-          row_slash_acc(R, U2, ld_sj2(cur, y, z));
-          row_slash_acc(R, U3, ld_sl4(cur, z));
+          row_slash_acc(R, U3, ld_spol(cur, z));
 #pragma unroll
           for (int hv = 0; hv < 2; ++hv) {
             const cx<float> a = dot_v(R, K.wtb, hv);
