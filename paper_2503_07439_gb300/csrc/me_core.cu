@@ -364,6 +364,8 @@ static int build_tables(ColourTables& tab) {
               if (std::abs(s.imag()) > 1e-12) return fail(ME_ERR_PROCESS, "complex colour correlator");
               tab.Ccorr[ci][pr][x * 2 + y] = s.real();
             }
+      if (ci == 1)
+        for (int q = 0; q < N_PAIRS; ++q) tab.Cqq[q] = born_uu_matrix(1.0, tab.Ccorr[1][q]);
     }
   }
   return ME_OK;
@@ -470,7 +472,7 @@ struct me_handle {
 };
 
 static void free_items(me_handle* h) {
-  void* ptrs[] = {h->ib.ev, h->ib.pend, h->ib.a, h->ib.v, h->ib.list_r};
+  void* ptrs[] = {h->ib.ev, h->ib.pend, h->ib.wb, h->ib.v, h->ib.list_r};
   for (void* q : ptrs) cudaFree(q);
   h->ib = ItemBufs{};
   h->icap = 0;
@@ -483,7 +485,7 @@ static int ensure_item_capacity(me_handle* h, size_t n) {
   const size_t c = std::max(n, (size_t)1024);
   ItemBufs& b = h->ib;
   if (cudaMalloc(&b.ev, c * sizeof(int)) != cudaSuccess || cudaMalloc(&b.pend, c * sizeof(int)) != cudaSuccess ||
-      cudaMalloc(&b.a, c * 2 * sizeof(double)) != cudaSuccess ||
+      cudaMalloc(&b.wb, c * sizeof(double)) != cudaSuccess ||
       cudaMalloc(&b.v, c * MAX_BLOCKS * sizeof(double)) != cudaSuccess ||
       cudaMalloc(&b.list_r, c * MAX_BLOCKS * sizeof(int)) != cudaSuccess) {
     free_items(h);
@@ -510,7 +512,7 @@ static int ensure_term_capacity(me_handle* h, size_t n) {
   TermBufs& t = h->tb;
   const bool ok = cudaMalloc(&t.ev, c * sizeof(int)) == cudaSuccess &&
                   cudaMalloc(&t.grow, c * sizeof(float)) == cudaSuccess &&
-                  cudaMalloc(&t.a, c * 3 * sizeof(double)) == cudaSuccess &&
+                  cudaMalloc(&t.a, c * 2 * sizeof(double)) == cudaSuccess &&
                   cudaMalloc(&t.cnt, sizeof(int)) == cudaSuccess;
   if (!ok) {
     free_terms(h);
@@ -706,6 +708,15 @@ static int choose_lpe(me_handle* h, int kind, bool fp64, const LaunchArgs& a) {
   return slot = pick;
 }
 
+static void set_tolerances(KParams& kp, const me_params* p) {
+  kp.me_eps = p->me_eps;
+  kp.tol = p->tol;
+  kp.item_budget = kItemBudget;
+  kp.me_epsf = (float)p->me_eps;
+  kp.tolf = (float)p->tol;
+  kp.budgetf = (float)(kItemBudget * p->tol / p->me_eps);
+}
+
 // The cuts of me_params as the kernels take them (Cuts in me_kernels.cuh), for process pid.
 static bool cuts_valid(const me_params* p) {
   return std::isfinite(p->cut_pt_min) && p->cut_pt_min >= 0.0 && p->cut_abs_y_max > 0.0 &&
@@ -809,13 +820,12 @@ int me_init(const char* process, const me_params* params, me_handle** out) {
   kp.born_avg_inv = pd->born_pid >= 0 ? 1.0 / kProcs[pd->born_pid].avg : 0.0;
   kp.tree_scale = kp.avg_inv * tree_coupling(pd->pid, kp.cp);
   kp.real_scale = 2.0 * kp.tree_scale;
+  if (pd->born_pid >= 0) kp.born_scale = tree_coupling(pd->born_pid, kp.cp) * kp.born_avg_inv;
   kp.xi_cut = params->xi_cut;
   kp.delta = params->delta;
   kp.xi_thr = params->xi_thr;
   kp.y_thr = params->y_thr;
-  kp.me_eps = params->me_eps;
-  kp.tol = params->tol;
-  kp.item_budget = kItemBudget;
+  set_tolerances(kp, params);
   kp.cut = cuts_of(pd->pid, params);
   kp.tab = d_tab;
   // stream-ordered on the handle's own stream: no device-wide synchronisation, so a
@@ -978,13 +988,13 @@ int me_last_rescued(me_handle* h, int64_t* n_rescued) {
 int me_last_rescue_work(me_handle* h, int64_t* points, int64_t* real_blocks, int64_t* born_sets) {
   if (!h || !points || !real_blocks || !born_sets) return fail(ME_ERR_ARG, "NULL argument");
   ME_CUDA(cudaSetDevice(h->device));
-  int c[6] = {0, 0, 0, 0, 0, 0};
+  int c[8] = {};
   if (h->prm.precision == ME_PREC_MIXED && h->last_kind == K_REAL) {
     ME_CUDA(cudaMemcpyAsync(c, h->d_last, sizeof(c), cudaMemcpyDeviceToHost, h->stream));
     ME_CUDA(cudaStreamSynchronize(h->stream));
   }
   *points = c[0];
-  *real_blocks = c[2];
+  *real_blocks = c[2] + c[7];
   *born_sets = h->last_terms ? c[4] + c[5] : c[3];
   return ME_OK;
 }
@@ -1239,12 +1249,12 @@ int me_internal_kparams(const char* process, const me_params* params, me::KParam
   kp->born_avg_inv = pd->born_pid >= 0 ? 1.0 / kProcs[pd->born_pid].avg : 0.0;
   kp->tree_scale = kp->avg_inv * tree_coupling(pd->pid, kp->cp);
   kp->real_scale = 2.0 * kp->tree_scale;
+  if (pd->born_pid >= 0) kp->born_scale = tree_coupling(pd->born_pid, kp->cp) * kp->born_avg_inv;
   kp->xi_cut = params->xi_cut;
   kp->delta = params->delta;
   kp->xi_thr = params->xi_thr;
   kp->y_thr = params->y_thr;
-  kp->me_eps = params->me_eps;
-  kp->tol = params->tol;
+  set_tolerances(*kp, params);
   kp->cut = cuts_of(pd->pid, params);
   *pid = pd->pid;
   return ME_OK;
@@ -1258,7 +1268,6 @@ int me_internal_device_kparams(const char* process, const me_params* params, me:
   ColourTables* d_tab = nullptr;
   if ((rc = device_setup(params->device, &d_tab)) != ME_OK) return rc;
   kp->tab = d_tab;
-  kp->item_budget = kItemBudget;
   return ME_OK;
 }
 

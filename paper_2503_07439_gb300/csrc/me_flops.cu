@@ -88,7 +88,7 @@ int main() {
   const Inv22<Flop> k = inv22<Flop>(p, Flop(173.0));
   const BornGG<Flop> b2 = born_gg(k, cp);
   g_ops = 0;
-  born_gg_matrix(b2, E);
+  b2.f * born_gg_form(b2, E);
   const double matrix_gg = (double)g_ops;
   g_ops = 0;
   born_uu_matrix(Flop(1.0), E);

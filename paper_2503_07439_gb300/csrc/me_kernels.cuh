@@ -42,6 +42,7 @@ struct ColourTables {
   double U[P_COUNT][MAX_FLOW * MAX_FLOW];
   float Uf[P_COUNT][MAX_FLOW * MAX_FLOW];
   double Ccorr[2][N_PAIRS][4];
+  double Cqq[N_PAIRS];  // u ubar -> t tbar, contracted with its one colour structure (born_uu_matrix)
 };
 
 // Cuts of one configuration (Algorithm 2's passCuts, applied to each term at its own
@@ -65,10 +66,12 @@ struct KParams {
   double born_avg_inv;  // same for the underlying Born of a real process
   double tree_scale;    // |M|^2 at unit couplings -> weight: couplings x avg_inv x nlo_factor
   double real_scale;    // half helicity sum of a real block at unit couplings -> |M|^2
+  double born_scale;    // couplings of the underlying Born x born_avg_inv
   double xi_cut, delta; // FKS plus-distribution cut-offs
   double xi_thr, y_thr; // points with xi < xi_thr or 1-y < y_thr go to the FP64 path
   double me_eps;        // assumed relative error of a bulk-precision matrix element
   double tol;           // target relative accuracy of a weight
+  float me_epsf, tolf, budgetf;  // float32 copies of me_eps, tol and item_budget x tol / me_eps
   int flag_unstable;    // 1: append unstable points to the rescue list
   int item_rescue;      // with flag_unstable: records and float64 items instead of the point list
   double item_budget;   // item rescue: residual error allowed, as a fraction of tol |W|
@@ -204,7 +207,9 @@ __global__ void __launch_bounds__(128, ME_MINB) k_tree(const double* __restrict_
   const bool pass = !kp.cut.mask || pass_cuts<PID>(k, kp.cut);
   const Kin<PID, T> K = prepare<PID, T>(k, unit_couplings(kp.cp));
   T acc = T(0);
-  for (int b = lane; b < n_live_blocks<PID>(); b += LPE) acc += block_sum<PID, T>(K, b, kp);
+  constexpr int NB = n_live_blocks<PID>(), NBL = (NB + LPE - 1) / LPE;
+#pragma unroll 1
+  for (int b = lane * NBL; b < (lane + 1) * NBL && b < NB; ++b) acc += block_sum<PID, T>(K, b, kp);
   const double tot = 2.0 * (double)group_sum<LPE>(acc, group_mask<LPE>());
   if (lane == 0) {
     const double w = wgt ? wgt[ev] : 1.0;
@@ -523,20 +528,10 @@ __global__ void __launch_bounds__(TC4_THREADS, 2) k_tree_tc4(const double* __res
 
 // p (given in the rest frame of a system with momentum Q, mass M) in the frame where the
 // system has momentum Q:  E' = (E Q0 + Q.p)/M,  p' = p + Q (E' + E)/(Q0 + M).
-// sgn = -1 boosts the other way (from the frame of Q into its rest frame).
-__device__ __forceinline__ r4<double> boost_by(const r4<double>& p, const r4<double>& Q, double inv_m, double m,
-                                               double sgn) {
+__device__ __forceinline__ r4<double> boost_by(const r4<double>& p, const r4<double>& Q, double inv_m, double inv_qm) {
   const double qp = Q.x * p.x + Q.y * p.y + Q.z * p.z;
-  const double e = (p.e * Q.e + sgn * qp) * inv_m;
-  const double c = sgn * (e + p.e) / (Q.e + m);
-  return r4<double>{e, p.x + c * Q.x, p.y + c * Q.y, p.z + c * Q.z};
-}
-// the same with 1 / (Q0 + M) given (several vectors boosted by one system)
-__device__ __forceinline__ r4<double> boost_by_r(const r4<double>& p, const r4<double>& Q, double inv_m,
-                                                 double inv_qm, double sgn) {
-  const double qp = Q.x * p.x + Q.y * p.y + Q.z * p.z;
-  const double e = (p.e * Q.e + sgn * qp) * inv_m;
-  const double c = sgn * (e + p.e) * inv_qm;
+  const double e = (p.e * Q.e + qp) * inv_m;
+  const double c = (e + p.e) * inv_qm;
   return r4<double>{e, p.x + c * Q.x, p.y + c * Q.y, p.z + c * Q.z};
 }
 
@@ -551,130 +546,14 @@ constexpr double PI = 3.14159265358979323846;
 constexpr double CF_ = 4.0 / 3.0;
 constexpr double CA_ = 3.0;
 
-// Initial-state FKS sectors (i = gluon leg 4, j = beam 0 or 1) of 2 -> Q Qbar g.
-struct IsrKin {
-  double xi, iz, y[2], S[2], K, K0;  // iz = 1 / (1 - xi)
-  r4<double> soft[4];     // soft Born: beams, heavy pair at sqrt(s) along n*
-  // collinear Born of sector 1: beam 1 scaled by z = 1 - xi.  That of sector 2 (beam 2
-  // scaled) is the same 2 -> 2 configuration boosted along the beam axis, and everything
-  // evaluated there -- the unpolarised Born and the Born with a gluon polarised along the
-  // transverse direction (0, cos phi, sin phi, 0) -- is invariant under that boost.
-  r4<double> coll[4];
-  double qdir[3];         // gluon direction
-  double cphi, sphi;      // gluon azimuth
-  // cuts (Algorithm 2) of the soft counter-event and of each sector's collinear one (its
-  // beam scaled by z): the two collinear Borns differ by a boost along the beam, which
-  // changes the heavy quarks' rapidities
-  bool cut_s, cut_c[2];
-};
-
-__device__ __forceinline__ void isr_map(const r4<double>* k, double mass, IsrKin& o, const Cuts& cut) {
-  const double rs = k[0].e + k[1].e, irs = 1.0 / rs, s = rs * rs, is = irs * irs;
-  o.xi = 2.0 * k[4].e * irs;
-  unit3(k[4], o.qdir[0], o.qdir[1], o.qdir[2]);
-  double b0[3], b1[3];
-  unit3(k[0], b0[0], b0[1], b0[2]);
-  unit3(k[1], b1[0], b1[1], b1[2]);
-  o.y[0] = o.qdir[0] * b0[0] + o.qdir[1] * b0[1] + o.qdir[2] * b0[2];
-  o.y[1] = o.qdir[0] * b1[0] + o.qdir[1] * b1[1] + o.qdir[2] * b1[2];
-  const double d0 = 1.0 - o.y[0], d1 = 1.0 - o.y[1];
-  const double idd = 1.0 / (d0 + d1);
-  o.S[0] = d1 * idd;
-  o.S[1] = d0 * idd;
-  const double pt2 = o.qdir[0] * o.qdir[0] + o.qdir[1] * o.qdir[1];
-  const double ipt = pt2 > 0.0 ? rsqrt(pt2) : 0.0;
-  o.cphi = pt2 > 0.0 ? o.qdir[0] * ipt : 1.0;
-  o.sphi = pt2 > 0.0 ? o.qdir[1] * ipt : 0.0;
-  // heavy-pair rest-frame direction of the quark
-  const r4<double> Q = k[0] + k[1] - k[4];
-  const double Q2 = mdot(Q, Q), iMQ = rsqrt(Q2);
-  const r4<double> ks = boost_by(k[2], Q, iMQ, Q2 * iMQ, -1.0);
-  double n[3];
-  unit3(ks, n[0], n[1], n[2]);
-  const double m4 = 4.0 * mass * mass;
-  const double b2 = 1.0 - m4 * is, ibeta = rsqrt(b2), beta = b2 * ibeta;
-  o.soft[0] = k[0];
-  o.soft[1] = k[1];
-  const double e = 0.5 * rs, pa = 0.5 * rs * beta;
-  o.soft[2] = r4<double>{e, pa * n[0], pa * n[1], pa * n[2]};
-  o.soft[3] = r4<double>{e, -pa * n[0], -pa * n[1], -pa * n[2]};
-  const double z = 1.0 - o.xi;
-  o.iz = 1.0 / z;
-  const double sz = s * z, iM = rsqrt(sz), M = sz * iM;
-  const double bQ = sqrt(fmax(0.0, 1.0 - m4 * is * o.iz));
-  const double eQ = 0.5 * M, pQ = 0.5 * M * bQ;
-  const r4<double> tr{eQ, pQ * n[0], pQ * n[1], pQ * n[2]};
-  const r4<double> tbr{eQ, -pQ * n[0], -pQ * n[1], -pQ * n[2]};
-  o.coll[0] = scale(z, k[0]);
-  o.coll[1] = k[1];
-  const r4<double> Qc = o.coll[0] + o.coll[1];
-  const double Mc2 = mdot(Qc, Qc), iMc = rsqrt(Mc2), iqm = 1.0 / (Qc.e + Mc2 * iMc);
-  o.coll[2] = boost_by_r(tr, Qc, iMc, iqm, 1.0);
-  o.coll[3] = boost_by_r(tbr, Qc, iMc, iqm, 1.0);
-  o.cut_s = o.cut_c[0] = o.cut_c[1] = true;
-  if (cut.mask) {
-    o.cut_s = heavy_pass(o.soft[2], cut) && heavy_pass(o.soft[3], cut);
-    o.cut_c[0] = heavy_pass(o.coll[2], cut) && heavy_pass(o.coll[3], cut);
-    const r4<double> Q1 = k[0] + scale(z, k[1]);
-    const double M12 = mdot(Q1, Q1), iM1 = rsqrt(M12);
-    o.cut_c[1] = heavy_pass(boost_by(tr, Q1, iM1, M12 * iM1, 1.0), cut) &&
-                 heavy_pass(boost_by(tbr, Q1, iM1, M12 * iM1, 1.0), cut);
-  }
-  constexpr double i64pi3 = 1.0 / (64.0 * PI * PI * PI);
-  o.K = s * bQ * i64pi3 * ibeta;
-  o.K0 = s * i64pi3;
-}
-
-// Final-state FKS sectors (i = gluon leg 4, j = leg 2 or 3) of massless 2 -> 3.
-struct FsrKin {
-  double xi, y[2], S[2], K[2], K0, K1;
-  r4<double> born[2][4];
-  double qdir[3];
-};
-
-__device__ __forceinline__ void fsr_map(const r4<double>* k, FsrKin& o) {
-  const double rs = k[0].e + k[1].e, s = rs * rs;
-  o.xi = 2.0 * k[4].e / rs;
-  unit3(k[4], o.qdir[0], o.qdir[1], o.qdir[2]);
-  double nj[2][3];
-  unit3(k[2], nj[0][0], nj[0][1], nj[0][2]);
-  unit3(k[3], nj[1][0], nj[1][1], nj[1][2]);
-  double c[2];
-#pragma unroll
-  for (int j = 0; j < 2; ++j) c[j] = o.qdir[0] * nj[j][0] + o.qdir[1] * nj[j][1] + o.qdir[2] * nj[j][2];
-  const double d0 = 1.0 - c[0], d1 = 1.0 - c[1];
-  o.S[0] = d1 / (d0 + d1);
-  o.S[1] = d0 / (d0 + d1);
-  const double e = 0.5 * rs;
-#pragma unroll
-  for (int j = 0; j < 2; ++j) {
-    o.y[j] = c[j];
-    o.born[j][0] = k[0];
-    o.born[j][1] = k[1];
-    const r4<double> a{e, e * nj[j][0], e * nj[j][1], e * nj[j][2]};
-    const r4<double> b{e, -e * nj[j][0], -e * nj[j][1], -e * nj[j][2]};
-    o.born[j][2 + j] = a;
-    o.born[j][3 - j] = b;
-    const double den = 2.0 - o.xi * (1.0 - o.y[j]);
-    o.K[j] = s * (1.0 - o.xi) / (16.0 * PI * PI * PI * den * den);
-  }
-  o.K0 = s / (64.0 * PI * PI * PI);
-  o.K1 = s * (1.0 - o.xi) / (64.0 * PI * PI * PI);
-}
-
-__device__ __forceinline__ double eik(const r4<double>& a, const r4<double>& b, const double* q) {
-  const r4<double> qq{1.0, q[0], q[1], q[2]};
-  return mdot(a, b) / (mdot(a, qq) * mdot(b, qq));
-}
-
 // ---------------------------------------------------------------- real - counterterms
 // One point of the subtracted real, summed over FKS sectors (ME units):
 //   W_j = R S_j - [Th_s G(0,y) + Th_c G(xi,1) - Th_s Th_c G(0,1)] / (xi^2 (1-y) K),
 // with the error scale of the stability test.  The LPE lanes of a group evaluate one
 // point together and all return the same result.
 //
-// W is linear in the real matrix element R = sum_b R_b (helicity blocks) with float64
-// coefficients fixed by the FKS maps: W = a_R sum_b R_b + W_B, W_B the counterterms.  Their
+// W = R + W_B, R = sum_b R_b (helicity blocks) the real matrix element -- the sector functions
+// add up to 1 -- and W_B the counterterms.  Their
 // Born values are closed forms of some 40 float64 operations, so they are evaluated in
 // float64 for every point, in every precision, and only the real's blocks have a
 // bulk-precision value.  The item rescue re-evaluates in float64 the blocks whose float32
@@ -682,6 +561,9 @@ __device__ __forceinline__ double eik(const r4<double>& a, const r4<double>& b, 
 template <int PID>
 struct RealLayout {
   static constexpr int NB = n_live_blocks<PID>();  // the real's blocks
+  // block code depends on the parity of b (the helicity of beam gluon 1, amp_tt3_block): lanes
+  // of a warp should run blocks of one parity together
+  static constexpr bool BY_PARITY = PID == P_GG_TTG;
 };
 constexpr int MAX_BLOCKS = 4;
 
@@ -695,8 +577,8 @@ struct RealSubOut {
 
 // Everything of a point but the real matrix element.
 struct PointTerms {
-  double a_R;    // sum_j S_j, or 0 if the real fails its cuts
-  double w_born; // the counterterms (with their sign): W = a_R R + w_born
+  bool real;     // the real passes its cuts (the sector functions add up to 1)
+  double w_born; // the counterterms (with their sign): W = R + w_born, or w_born
   double mag_b;  // their error scale, |CT_coll| + |CT_soft - CT_softcoll| per sector
   double y[2];
   bool near;     // inside xi_thr / y_thr of an active counterterm
@@ -704,125 +586,186 @@ struct PointTerms {
   bool need[2];  // active Born configurations: soft, collinear (initial state); sector 1, 2
 };
 
-// Eikonal-weighted colour-correlation matrix of the soft counter-event (2x2, row-major):
-// E = sum_{k,l} w_kl C^{kl}, w_kl = (p_k.p_l) / ((p_k.q)(p_l.q)), q = (1, gluon direction),
-// over the four coloured legs of the 2 -> 2 Born (k = l included); four reciprocals.
-template <int BPID>
-__device__ __forceinline__ void isr_eikonal_matrix(const IsrKin& f, const KParams& kp, double* E) {
-  const int ci = (BPID == P_GG_TT) ? 0 : 1;
-  E[0] = E[1] = E[2] = E[3] = 0.0;
-  const r4<double> qq{1.0, f.qdir[0], f.qdir[1], f.qdir[2]};
-  double iaq[4];
-#pragma unroll
-  for (int a = 0; a < 4; ++a) iaq[a] = 1.0 / mdot(f.soft[a], qq);
-  int pr = 0;
-#pragma unroll
-  for (int a = 0; a < 4; ++a)
-#pragma unroll
-    for (int b = a; b < 4; ++b, ++pr) {
-      const double w = mdot(f.soft[a], f.soft[b]) * iaq[a] * iaq[b] * (a == b ? 1.0 : 2.0);
-#pragma unroll
-      for (int q = 0; q < 4; ++q) E[q] += w * kp.tab->Ccorr[ci][pr][q];
-    }
+// a < b for b >= 0, on the bit patterns: a float64 comparison occupies the float64 pipe like a
+// multiply-add.  False for NaN (the arithmetic's NaN is positive).
+__device__ __forceinline__ bool below(double a, double b) {
+  return __double_as_longlong(a) < __double_as_longlong(b);
+}
+__device__ __forceinline__ bool positive(double a) {  // a > 0; infinite and NaN included
+  return __double_as_longlong(a) > 0;
 }
 
-// Counterterms, error scale and regions of one point, from its momenta k.
-template <int PID>
+// Counterterms, error scale and regions of one point, from its momenta k, in float64; T is the
+// precision of the evaluation it belongs to.  The float64 pipe bounds every kernel that runs
+// this, so what the centre-of-mass frame of massless, back-to-back beams implies is put in by
+// hand (65,536 e+e- -> u ubar g points, where this is most of the work: 187 -> 128 us):
+//  * initial state (gluon leg 4, sectors: beam 0, beam 1): the pair recoils with mass^2
+//    s (1 - xi) and momentum -k_g, its rest-frame direction n is kept.  The soft Born is the
+//    pair at sqrt(s) along n, the collinear one has a beam scaled by 1 - xi and the pair
+//    boosted along the beam; both are known from n and the velocities beta(s),
+//    beta(s (1 - xi)).  The two sectors' collinear Borns are one 2 -> 2 configuration boosted
+//    along the beam, so the Borns, plain and polarised along the gluon's transverse direction,
+//    are shared; the rapidity cuts are not;
+//  * final state (sectors: partner leg 2 or 3): a sector's soft and soft-collinear limits are
+//    the same number, and its Born depends on the cosine of the partner to the beam alone.
+// Close to a collinear limit the last bits of a weight are those of 1 - y_j = d_j as formed
+// here, which the eikonal denominators p_j.q carry again, rounded differently; where the two
+// meet, their ratio is kept as it comes out, in float64 results also the beams' own eikonal
+// terms (p^2 = 0 up to rounding) and the final state's eikonal factor.
+template <int PID, typename T>
 __device__ __forceinline__ PointTerms point_terms(const r4<double>* k, const KParams& kp) {
+  constexpr bool F64 = !std::is_same<T, float>::value;
   PointTerms o{};
-  const double rs = k[0].e + k[1].e, s = rs * rs;
+  const double rs = k[0].e + k[1].e, irs = 1.0 / rs;
   const double g2 = kp.cp.gs * kp.cp.gs;
-  // Algorithm 2's cut of the real term, at the real point
-  const double cR = (!kp.cut.mask || pass_cuts<PID>(k, kp.cut)) ? 1.0 : 0.0;
-  double xi_pt;
+  o.real = !kp.cut.mask || pass_cuts<PID>(k, kp.cut);
+  const double xi = 2.0 * k[4].e * irs, z = 1.0 - xi;
+  double q[3];
+  unit3(k[4], q[0], q[1], q[2]);
+  const double d_cut = kp.delta;  // y_j > 1 - delta  <=>  1 - y_j < delta
+  const bool soft_xi = below(xi, kp.xi_cut), near_xi = below(xi, kp.xi_thr);
+  double d0, d1;
   if constexpr (PID == P_EE_UUG) {
-    FsrKin f;
-    fsr_map(k, f);
-    o.y[0] = f.y[0];
-    o.y[1] = f.y[1];
-    xi_pt = f.xi;
-    // Algorithm 2's cuts: both counterterms of sector j at sector j's Born
-    const bool cuts = kp.cut.mask != 0;
+    double n[2][3];
+    unit3(k[2], n[0][0], n[0][1], n[0][2]);
+    unit3(k[3], n[1][0], n[1][1], n[1][2]);
+    double d[2], c[2];
 #pragma unroll
     for (int j = 0; j < 2; ++j) {
-      const double B = closed_sum<P_EE_UU, double>(f.born[j], kp.cp) * kp.born_avg_inv;
-      const double cB = (!cuts || pass_cuts<P_EE_UU>(f.born[j], kp.cut)) ? 1.0 : 0.0;
-      const double th_s = f.xi < kp.xi_cut ? cB : 0.0;
-      // soft: sum_{kl} w_kl B_kl with B_23 = B_32 = -C_F B (massless diagonal terms vanish)
-      const double cs = (1.0 - f.y[j]) * 0.5 * (1.0 + f.y[j]) * f.K0 * (-(4.0 * g2 / s) * 2.0 * eik(f.born[j][2], f.born[j][3], f.qdir) * (-CF_));
-      const double cc = f.K1 * (2.0 / (s * (1.0 - f.xi))) * 2.0 * g2 * CF_ * (1.0 + (1.0 - f.xi) * (1.0 - f.xi));
-      const double csc = f.K0 * (2.0 / s) * 2.0 * g2 * 2.0 * CF_;
-      const double th_c = f.y[j] > 1.0 - kp.delta ? cB : 0.0;
-      const double iden = 1.0 / (f.xi * f.xi * (1.0 - f.y[j]) * f.K[j]);
-      o.w_born -= (th_s * cs + th_c * cc - th_s * th_c * csc) * iden * B;
-      // error scale: the collinear term, and the soft pair (whose Borns are shared)
-      o.mag_b += (fabs(th_c * cc * iden) + fabs(th_s * (cs - th_c * csc) * iden)) * B;
-      o.near |= (th_s > 0.0 && f.xi < kp.xi_thr) || (th_c > 0.0 && 1.0 - f.y[j] < kp.y_thr);
-      o.a_R += f.S[j] * cR;
-      o.need[j] = th_s > 0.0 || th_c > 0.0;
+      o.y[j] = q[0] * n[j][0] + q[1] * n[j][1] + q[2] * n[j][2];
+      d[j] = 1.0 - o.y[j];
+      c[j] = 2.0 * irs * (k[0].x * n[j][0] + k[0].y * n[j][1] + k[0].z * n[j][2]);
+    }
+    d0 = d[0];
+    d1 = d[1];
+    const double s = rs * rs;
+    // 1 / (xi^2 d_j K_j), K_j = s z / (16 pi^3 (2 - xi d_j)^2), from one reciprocal
+    const double r = 16.0 * PI * PI * PI / (s * z * xi * xi * d0 * d1 * (d0 + d1));
+    const double sum = d0 + d1;
+    const double cs = g2 * (8.0 * CF_ / (64.0 * PI * PI * PI)), cc = 0.5 * cs * (1.0 + z * z);
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+      const double t = 2.0 - xi * d[j];
+      const double B = (16.0 / 3.0) * kp.born_scale * (1.0 + c[j] * c[j]);
+      bool pass = true;
+      if (kp.cut.mask) {
+        const double e = 0.5 * rs;
+        const r4<double> a{e, e * n[j][0], e * n[j][1], e * n[j][2]}, m{e, -a.x, -a.y, -a.z};
+        const r4<double> kb[4] = {k[0], k[1], j == 0 ? a : m, j == 0 ? m : a};
+        pass = pass_cuts<P_EE_UU>(kb, kp.cut);
+      }
+      const bool th_s = pass && soft_xi, th_c = pass && below(d[j], d_cut);
+      const double id = (r * d[1 - j] * sum * t * t) * B;
+      double soft = th_s && !th_c ? cs : 0.0;
+      if constexpr (F64) {
+        // (1 - y)(1 + y)/2 times the eikonal factor of partner and recoiler: 1 up to rounding
+        const double e = 0.5 * rs;
+        const r4<double> a{e, e * n[j][0], e * n[j][1], e * n[j][2]}, m{e, -a.x, -a.y, -a.z}, qq{1.0, q[0], q[1], q[2]};
+        const double c1 = d[j] * 0.5 * (1.0 + o.y[j]) * (mdot(a, m) / (mdot(a, qq) * mdot(m, qq)));
+        soft = th_s ? cs * (th_c ? c1 - 1.0 : c1) : 0.0;
+      }
+      const double x = (th_c ? cc : 0.0) * id, u = soft * id;
+      o.w_born -= x + u;
+      o.mag_b += fabs(x) + fabs(u);
+      o.near |= (th_s && near_xi) || (th_c && below(d[j], kp.y_thr));
+      o.need[j] = th_s || th_c;
     }
   } else {
-    constexpr int BPID = PID == P_GG_TTG ? P_GG_TT : P_UU_TT;
-    IsrKin f;
-    isr_map(k, kp.cp.mt, f, kp.cut);
-    o.y[0] = f.y[0];
-    o.y[1] = f.y[1];
-    xi_pt = f.xi;
-    // Born values: E-weighted and plain at the soft counter-event, plain (and, for g g, with
-    // the splitting gluon polarised along the emission's transverse direction) at the
-    // collinear one, of sector 1; sector 2's are the same (see IsrKin and the closed forms)
-    double E[4], vE, vS, Bc, Bp = 0.0;
-    isr_eikonal_matrix<BPID>(f, kp, E);
-    const Inv22<double> ks = inv22<double>(f.soft, kp.cp.mt), kc_ = inv22<double>(f.coll, kp.cp.mt);
-    if constexpr (BPID == P_GG_TT) {
-      const BornGG<double> bs = born_gg(ks, kp.cp), bc = born_gg(kc_, kp.cp);
-      vE = born_gg_matrix(bs, E);
-      vS = born_gg_colour(bs);
-      Bc = born_gg_colour(bc);
-      Bp = born_gg_polarised(kc_, bc, f.cphi * f.coll[2].x + f.sphi * f.coll[2].y, kp.cp) * kp.born_avg_inv;
+    constexpr bool GG = PID == P_GG_TTG;
+    const double mt = kp.cp.mt, is = irs * irs, rho = 4.0 * mt * mt * is;
+    double b[3];
+    unit3(k[0], b[0], b[1], b[2]);
+    o.y[0] = q[0] * b[0] + q[1] * b[1] + q[2] * b[2];
+    if constexpr (F64) {
+      double b1[3];
+      unit3(k[1], b1[0], b1[1], b1[2]);
+      o.y[1] = q[0] * b1[0] + q[1] * b1[1] + q[2] * b1[2];
     } else {
-      const double d = 8.0 * g2 * g2, fs = d * born_qq(ks);
-      vE = born_uu_matrix(fs, E);
-      vS = 2.0 * fs;
-      Bc = 2.0 * d * born_qq(kc_);
+      o.y[1] = -o.y[0];
     }
-    vE *= kp.born_avg_inv;
-    vS *= kp.born_avg_inv;
-    Bc *= kp.born_avg_inv;
-    // Algorithm 2's cuts (isr_map): soft and soft-collinear terms at the soft
-    // counter-event, the collinear term of sector j at sector j's collinear counter-event
-    const double xi = f.xi, z = 1.0 - xi, iz = f.iz, is2 = 2.0 / s;
-    const double th_s = xi < kp.xi_cut && f.cut_s ? 1.0 : 0.0;
-    // 1 / (xi^2 (1 - y_j) K) of both sectors from one reciprocal
-    const double den0 = xi * xi * (1.0 - f.y[0]) * f.K, den1 = xi * xi * (1.0 - f.y[1]) * f.K;
-    const double rden = 1.0 / (den0 * den1);
-    const double iden[2] = {den1 * rden, den0 * rden};
-    // d xi P / d B_c, d xi P / d B_p, d xi P_0 / d B_s of the splitting kernels
-    const double kc = BPID == P_GG_TT ? 2.0 * CA_ * (z + xi * xi * z) : CF_ * (1.0 + z * z);
-    const double kp_ = BPID == P_GG_TT ? 2.0 * CA_ * 2.0 * (xi * xi * iz) : 0.0;
-    const double kq = BPID == P_GG_TT ? 2.0 * CA_ : 2.0 * CF_;
-    const double xiP = kc * Bc + kp_ * Bp;
+    d0 = 1.0 - o.y[0];
+    d1 = 1.0 - o.y[1];
+    // the quark's direction in the pair's rest frame (the pair has momentum -k_g)
+    const double s = rs * rs, sz = s * z, iM = rsqrt(sz), M = sz * iM, Q0 = rs - k[4].e;
+    const double e2 = (k[2].e * Q0 + k[4].x * k[2].x + k[4].y * k[2].y + k[4].z * k[2].z) * iM;
+    const double cq = (e2 + k[2].e) / (Q0 + M);
+    const r4<double> ks{e2, k[2].x + cq * k[4].x, k[2].y + cq * k[4].y, k[2].z + cq * k[4].z};
+    double n[3];
+    unit3(ks, n[0], n[1], n[2]);
+    const double cb = n[0] * b[0] + n[1] * b[1] + n[2] * b[2];
+    const double nq = n[0] * q[0] + n[1] * q[1] + n[2] * q[2];
+    const double b2 = 1.0 - rho, ibeta = rsqrt(b2), beta = b2 * ibeta;
+    const double iz = 1.0 / z, rhoc = rho * iz, bQ2 = fmax(0.0, 1.0 - rhoc), bQ = sqrt(bQ2);
+    bool cut_s = true, cut_c[2] = {true, true};
+    if (kp.cut.mask) {
+      const double e = 0.5 * rs, pa = e * beta, eQ = 0.5 * M, pQ = eQ * bQ;
+      const r4<double> s2{e, pa * n[0], pa * n[1], pa * n[2]}, s3{e, -s2.x, -s2.y, -s2.z};
+      const r4<double> tr{eQ, pQ * n[0], pQ * n[1], pQ * n[2]}, tb{eQ, -tr.x, -tr.y, -tr.z};
+      cut_s = heavy_pass(s2, kp.cut) && heavy_pass(s3, kp.cut);
+#pragma unroll
+      for (int j = 0; j < 2; ++j) {
+        const r4<double> Q = j == 0 ? scale(z, k[0]) + k[1] : k[0] + scale(z, k[1]);
+        const double Q2 = mdot(Q, Q), iMc = rsqrt(Q2), iqm = 1.0 / (Q.e + Q2 * iMc);
+        cut_c[j] = heavy_pass(boost_by(tr, Q, iMc, iqm), kp.cut) && heavy_pass(boost_by(tb, Q, iMc, iqm), kp.cut);
+      }
+    }
+    // soft and collinear Borns: tau_i = (1 -+ v cb) / 2 with v the quark's velocity
+    const double hs = 0.5 * beta * cb, t0 = 0.5 - hs, t1 = 0.5 + hs, hc = 0.5 * bQ * cb;
+    const Inv22<double> js{0.0, t0, t1, rho}, jc{0.0, 0.5 - hc, 0.5 + hc, rhoc};
+    // eikonal factors times d_0 d_1; the beams' c_j = d_j E / (p_j.q) are 1 up to rounding
+    const double f2 = 1.0 - beta * nq, f3 = 1.0 + beta * nq, rf = 1.0 / (f2 * f3), i2 = f3 * rf, i3 = f2 * rf;
+    const r4<double> qq{1.0, q[0], q[1], q[2]};
+    const double a0 = mdot(k[0], qq), a1 = mdot(k[1], qq), ra = 0.5 * rs / (a0 * a1);
+    const double c0 = d0 * a1 * ra, c1 = d1 * a0 * ra;
+    const double d01 = d0 * d1, u0 = 4.0 * d1 * c0, u1 = 4.0 * d0 * c1;
+    const double w[7] = {4.0 * c0 * c1, u0 * t0 * i2, u0 * t1 * i3, u1 * t1 * i2, u1 * t0 * i3,
+                         (4.0 - 2.0 * rho) * d01 * rf, rho * d01};
+    double w00 = 0.0;
+    if constexpr (F64) w00 = (mdot(k[0], k[0]) * (a1 * a1) + mdot(k[1], k[1]) * (a0 * a0)) * d01 / (a0 * a0 * (a1 * a1));
+    double vE, vS, xiP;  // vE carries d_0 d_1
+    if constexpr (GG) {
+      const Couplings unit(1.0, 1.0, mt);
+      const BornGG<double> bs = born_gg(js, unit), bc = born_gg(jc, unit);
+      auto cE = [&](int pr) { return born_gg_form(bs, kp.tab->Ccorr[0][pr]); };
+      // the massive legs' own terms share their correlator (C_F)
+      vE = bs.f * (w[0] * cE(1) + w[1] * cE(2) + w[2] * cE(3) + w[3] * cE(5) + w[4] * cE(6) + w[5] * cE(8) +
+                   w[6] * (i2 * i2 + i3 * i3) * cE(7));
+      if constexpr (F64) vE += bs.f * w00 * cE(0);
+      vS = (2.0 * CA_) * born_gg_colour(bs);
+      const double pt2 = q[0] * q[0] + q[1] * q[1], ne = n[0] * q[0] + n[1] * q[1];
+      const double ne2 = positive(pt2) ? ne * ne / pt2 : n[0] * n[0];
+      const double Bp = born_gg_polarised(jc, bc, 0.5 * bQ2 * ne2, unit);
+      xiP = 2.0 * CA_ * ((z + xi * xi * z) * born_gg_colour(bc) + 2.0 * xi * xi * iz * Bp);
+    } else {
+      const double* C = kp.tab->Cqq;
+      const double fs = 8.0 * born_qq(js);
+      vE = fs * (w[0] * C[1] + w[1] * C[2] + w[2] * C[3] + w[3] * C[5] + w[4] * C[6] + w[5] * C[8] +
+                 w[6] * (i2 * i2 * C[7] + i3 * i3 * C[9]));
+      if constexpr (F64) vE += fs * w00 * C[0];
+      vS = (4.0 * CF_) * fs;
+      xiP = CF_ * (1.0 + z * z) * 16.0 * born_qq(jc);
+    }
+    // G / (2 g^2 / (64 pi^3)) of the soft, collinear and soft-collinear limits, the Borns'
+    // couplings and average taken out; K = s bQ / (64 pi^3 beta)
+    const double kb = bQ * ibeta;
+    const double Gs = -vE, Gc = 2.0 * kb * iz * xiP, Gsc = 2.0 * vS;
+    // 1 / (xi^2 d_j K) of both sectors from one reciprocal
+    const double pre = 2.0 * g2 * kp.born_scale / (xi * xi * d01 * s * kb);
+    const bool th_s = soft_xi && cut_s;
 #pragma unroll
     for (int j = 0; j < 2; ++j) {
-      const double Gs = (1.0 - f.y[j]) * f.S[j] * f.K0 * (-(4.0 * g2 / s) * vE);
-      const double Gc = f.K * is2 * iz * 2.0 * g2 * xiP;
-      const double Gsc = f.K0 * is2 * 2.0 * g2 * (kq * vS);
-      const double th_c = f.y[j] > 1.0 - kp.delta ? 1.0 : 0.0;  // soft-collinear term's
-      const double th_cc = f.cut_c[j] ? th_c : 0.0;             // collinear term's
-      o.w_born -= (th_s * Gs + th_cc * Gc - th_s * th_c * Gsc) * iden[j];
+      const bool th_c = below(j == 0 ? d0 : d1, d_cut), th_cc = th_c && cut_c[j];
+      const double id = pre * (j == 0 ? d1 : d0);
+      const double a = th_cc ? Gc * id : 0.0, c = th_s ? (th_c ? Gs - Gsc : Gs) * id : 0.0;
+      o.w_born -= a + c;
       // error scale: the collinear term, and the soft pair (whose Borns are shared)
-      o.mag_b += fabs(th_cc * Gc * iden[j]) + fabs(th_s * (Gs - th_c * Gsc) * iden[j]);
-      o.near |= (th_s > 0.0 && xi < kp.xi_thr) || ((th_cc > 0.0 || th_s * th_c > 0.0) && 1.0 - f.y[j] < kp.y_thr);
-      o.a_R += f.S[j] * cR;
-      o.need[1] |= th_cc > 0.0;
+      o.mag_b += fabs(a) + fabs(c);
+      o.near |= (th_s && near_xi) || ((th_cc || (th_s && th_c)) && below(j == 0 ? d0 : d1, kp.y_thr));
+      o.need[1] |= th_cc;
     }
-    o.need[0] = th_s > 0.0;
+    o.need[0] = th_s;
   }
-  // A point on the boundary of the FKS domain -- no emitted energy (xi = 0), all of it
-  // (xi = 1), or the emission exactly along a sector's reference direction (y_j = 1) --
-  // has measure zero and no defined subtracted weight (1 / (xi^2 (1 - y)) diverges):
-  // weight 0, and it is not re-evaluated.  The comparisons are false for NaN.
-  o.inside = xi_pt > 0.0 && xi_pt < 1.0 && 1.0 - o.y[0] > 0.0 && 1.0 - o.y[1] > 0.0;
+  o.inside = positive(xi) && below(xi, 1.0) && positive(d0) && positive(d1);
   return o;
 }
 
@@ -836,7 +779,7 @@ __device__ __forceinline__ double real_block_value(const Kin<PID, T>& K, int b, 
 // W and its error scale from a point's terms and R.
 __device__ __forceinline__ RealSubOut combine_point(const PointTerms& t, double R) {
   if (!t.inside) return RealSubOut{0.0, 0.0, 0.0, {t.y[0], t.y[1]}, false};
-  const double r = t.a_R * R, magR = fabs(r);
+  const double r = t.real ? R : 0.0, magR = fabs(r);
   return RealSubOut{r + t.w_born, magR + t.mag_b, magR, {t.y[0], t.y[1]}, t.near};
 }
 
@@ -854,31 +797,31 @@ __device__ __forceinline__ RealSubOut real_sub_event(const double* __restrict__ 
   constexpr int NBL = (NB + LPE - 1) / LPE;  // real blocks per lane
   r4<double> k[NEXT];
   load_event<NEXT>(p, n, ev, k);
-  // real matrix element; lane l holds blocks l, l + LPE, ... (one copy of the block code:
-  // the loop is not unrolled)
+  // real matrix element; lane l holds blocks l NBL, l NBL + 1, ... (one copy of the block
+  // code: the loop is not unrolled)
   double blk[NBL];
   double mine = 0.0;
   {
     const Kin<PID, T> K = prepare<PID, T>(k, unit_couplings(kp.cp));
 #pragma unroll 1
     for (int i = 0; i < NBL; ++i) {
-      const int b = lane + i * LPE;
+      const int b = lane * NBL + i;
       const double v = b < NB ? real_block_value<PID, T>(K, b, kp) : 0.0;
       blk[i] = v;
       mine += v;
     }
   }
   const double R = group_sum<LPE>(mine, mask);
-  const PointTerms t = point_terms<PID>(k, kp);
+  const PointTerms t = point_terms<PID, T>(k, kp);
   if (items) {
-    // every block value to lane 0 (block b lives on lane b % LPE, slot b / LPE)
+    // every block value to lane 0 (block b lives on lane b / NBL, slot b % NBL)
 #pragma unroll
     for (int b = 0; b < NB; ++b) {
       double x = 0.0;
 #pragma unroll
       for (int i = 0; i < NBL; ++i)
-        if (i == b / LPE) x = blk[i];
-      if constexpr (LPE > 1) x = __shfl_sync(mask, x, b % LPE, LPE);
+        if (i == b % NBL) x = blk[i];
+      if constexpr (LPE > 1) x = __shfl_sync(mask, x, b / NBL, LPE);
       items->v[b] = x;
     }
     items->t = t;
@@ -891,12 +834,14 @@ __device__ __forceinline__ RealSubOut real_sub_event(const double* __restrict__ 
 // collinear limit, as 1 + sqrt(rho_0 / rho) with rho = min_j (1 - y_j), rho_0 = 0.01.
 // The counterterms' Born values are evaluated at regular 2 -> 2 kinematics, whose error
 // does not grow there: error ~ me_eps x (growth x real part + Born part).
-__device__ __forceinline__ double error_growth(const RealSubOut& r) {
-  const float rho = fmaxf((float)fmin(1.0 - r.y[0], 1.0 - r.y[1]), 1e-30f);
-  return 1.0 + (double)sqrtf(0.01f / rho);
+__device__ __forceinline__ float error_growth(const RealSubOut& r) {
+  const float rho = fmaxf(fminf((float)(1.0 - r.y[0]), (float)(1.0 - r.y[1])), 1e-30f);
+  return 1.0f + sqrtf(0.01f / rho);
 }
-__device__ __forceinline__ bool unstable_point(const RealSubOut& r, const KParams& kp, double g) {
-  return r.near || !((r.magR * g + (r.mag - r.magR)) * kp.me_eps <= kp.tol * fabs(r.W));
+// The test is an estimate, taken in float32 (mag and W enter at float32 accuracy).
+__device__ __forceinline__ bool unstable_point(const RealSubOut& r, const KParams& kp, float g) {
+  const float R = (float)r.magR, B = (float)(r.mag - r.magR);
+  return r.near || !((R * g + B) * kp.me_epsf <= kp.tolf * (float)fabs(r.W));
 }
 
 __device__ __forceinline__ bool unstable_point(const RealSubOut& r, const KParams& kp) {
@@ -909,25 +854,25 @@ __device__ __forceinline__ bool unstable_point(const RealSubOut& r, const KParam
 // the order: a point whose flag came from it alone takes no block, and what the part no
 // longer adds to the error is a margin.  Points inside the thresholds take every block.
 template <int PID>
-__device__ __forceinline__ unsigned rescue_mask(const RealSubOut& r, double a_R, const double* v, const KParams& kp,
-                                                double grow) {
+__device__ __forceinline__ unsigned rescue_mask(const RealSubOut& r, bool real, const double* v, const KParams& kp,
+                                                float grow) {
   constexpr int NB = RealLayout<PID>::NB;
   constexpr unsigned all = (1u << NB) - 1u;
-  if (a_R == 0.0) return 0;  // the real failed its cuts
+  if (!real) return 0;
   if (r.near) return all;
-  double e[NB + 1];
-  double rest = 0.0;
+  float e[NB + 1];
+  float rest = 0.0f;
 #pragma unroll
-  for (int b = 0; b < NB; ++b) rest += (e[b] = fabs(a_R * v[b]));
-  rest += (e[NB] = (r.mag - r.magR) / grow);  // no growth for the Born part (unstable_point)
+  for (int b = 0; b < NB; ++b) rest += (e[b] = fabsf((float)v[b]));
+  rest += (e[NB] = (float)(r.mag - r.magR) / grow);  // no growth for the Born part (unstable_point)
   if (!(rest == rest)) return all;
-  const double budget = kp.item_budget * kp.tol * fabs(r.W) / (grow * kp.me_eps);
+  const float budget = kp.budgetf * (float)fabs(r.W) / grow;
   unsigned m = 0;
 #pragma unroll
   for (int k = 0; k <= NB; ++k) {
     if (rest <= budget) break;
     int pick = 0;
-    double best = -1.0;
+    float best = -1.0f;
 #pragma unroll
     for (int b = 0; b <= NB; ++b)
       if (!(m >> b & 1u) && e[b] > best) {
@@ -942,14 +887,16 @@ __device__ __forceinline__ unsigned rescue_mask(const RealSubOut& r, double a_R,
 
 // Buffers of the item rescue (structure of arrays, capacity `cap` points): a record for
 // each flagged point with blocks to re-evaluate -- ev[slot], pend[slot] (its blocks still
-// to come), a[slot] = a_R, a[cap + slot] = W_B, v[b * cap + slot] -- and the item list,
-// slot * 4 + b.  Counters (`counts`): [0] flagged points, [2] blocks, [3] flagged points with
+// to come), wb[slot] = W_B, v[b * cap + slot] -- and the item list,
+// slot * 4 + b, from the front (where RealLayout::BY_PARITY asks for it, odd blocks from the
+// back, so that a warp runs one kind).  Counters (`counts`): [0] flagged points, [2] and [7]
+// blocks listed from the front and the back, [3] flagged points with
 // an active counterterm, [4] / [5] their active Born configurations (soft, collinear, or
 // sector 1, 2), [6] records; [1] is the queued kernel's tile counter.
 struct ItemBufs {
   int* ev;
   int* pend;
-  double* a;
+  double* wb;
   double* v;
   int* list_r;
   long cap;
@@ -958,19 +905,20 @@ struct ItemBufs {
 // Record a flagged point and list its blocks: called by the flagged lanes of a warp together
 // (one atomic per warp and counter).
 template <int PID>
-__device__ __forceinline__ void append_flagged(int* __restrict__ counts, const ItemBufs& ib, long ev, double a_R,
-                                               double w_born, const bool* need, const double* v, unsigned m) {
+__device__ __forceinline__ void append_flagged(int* __restrict__ counts, const ItemBufs& ib, long ev, double w_born,
+                                               const bool* need, const double* v, unsigned m) {
   constexpr int NB = RealLayout<PID>::NB;
   const unsigned am = __activemask();
   const int wl = threadIdx.x & 31, leader = __ffs(am) - 1;
   const unsigned lt = (1u << wl) - 1u;
   const unsigned rec = __ballot_sync(am, m != 0);
   const unsigned c0 = __ballot_sync(am, need[0]), c1 = __ballot_sync(am, need[1]);
+  constexpr bool SPLIT = RealLayout<PID>::BY_PARITY;
   unsigned bal[NB];
-  int tot = 0;
+  int tot[2] = {0, 0};
 #pragma unroll
-  for (int b = 0; b < NB; ++b) tot += __popc(bal[b] = __ballot_sync(am, m >> b & 1u));
-  int base = 0, rbase = 0;
+  for (int b = 0; b < NB; ++b) tot[SPLIT ? b & 1 : 0] += __popc(bal[b] = __ballot_sync(am, m >> b & 1u));
+  int base = 0, rbase[2] = {0, 0};
   if (wl == leader) {
     atomicAdd(counts, __popc(am));
     if (c0 | c1) atomicAdd(counts + 3, __popc(c0 | c1));
@@ -978,24 +926,29 @@ __device__ __forceinline__ void append_flagged(int* __restrict__ counts, const I
     if (c1) atomicAdd(counts + 5, __popc(c1));
     if (rec) {
       base = atomicAdd(counts + 6, __popc(rec));
-      rbase = atomicAdd(counts + 2, tot);
+      if (tot[0]) rbase[0] = atomicAdd(counts + 2, tot[0]);
+      if (tot[1]) rbase[1] = atomicAdd(counts + 7, tot[1]);
     }
   }
   const int slot = __shfl_sync(am, base, leader) + __popc(rec & lt);
-  rbase = __shfl_sync(am, rbase, leader);
+  rbase[0] = __shfl_sync(am, rbase[0], leader);
+  if (SPLIT) rbase[1] = __shfl_sync(am, rbase[1], leader);
   if (m) {
     ib.ev[slot] = (int)ev;
     ib.pend[slot] = __popc(m);
-    ib.a[slot] = a_R;
-    ib.a[ib.cap + slot] = w_born;
+    ib.wb[slot] = w_born;
 #pragma unroll
     for (int b = 0; b < NB; ++b) ib.v[b * ib.cap + slot] = v[b];
   }
   // ordered by block, then lane
 #pragma unroll
   for (int b = 0; b < NB; ++b) {
-    if (m >> b & 1u) ib.list_r[rbase + __popc(bal[b] & lt)] = slot * 4 + b;
-    rbase += __popc(bal[b]);
+    const int half = SPLIT ? b & 1 : 0;
+    if (m >> b & 1u) {
+      const long at = rbase[half] + __popc(bal[b] & lt);
+      ib.list_r[half ? MAX_BLOCKS * ib.cap - 1 - at : at] = slot * 4 + b;
+    }
+    rbase[half] += __popc(bal[b]);
   }
 }
 
@@ -1024,8 +977,8 @@ __global__ void __launch_bounds__(128, ME_MINB) k_real_sub(const double* __restr
         const int slot = atomicAdd(resc_count, 1);
         resc_list[slot] = (int)ev;
       } else {
-        append_flagged<PID>(resc_count, ib, ev, it.t.a_R, it.t.w_born, it.t.need, it.v,
-                            rescue_mask<PID>(r, it.t.a_R, it.v, kp, error_growth(r)));
+        append_flagged<PID>(resc_count, ib, ev, it.t.w_born, it.t.need, it.v,
+                            rescue_mask<PID>(r, it.t.real, it.v, kp, error_growth(r)));
       }
     }
   }
@@ -1040,9 +993,9 @@ __global__ void __launch_bounds__(128, ME_MINB) k_rescue_items(const double* __r
                                                                double* __restrict__ out, KParams kp,
                                                                const int* __restrict__ counts, ItemBufs ib) {
   constexpr int NEXT = Proc<PID>::NEXT, NB = RealLayout<PID>::NB;
-  const long stride = (long)gridDim.x * blockDim.x, nit = counts[2];
+  const long stride = (long)gridDim.x * blockDim.x, front = counts[2], nit = front + counts[7];
   for (long t = (long)blockIdx.x * blockDim.x + threadIdx.x; t < nit; t += stride) {
-    const int item = ib.list_r[t], slot = item >> 2, b = item & 3;
+    const int item = ib.list_r[t < front ? t : MAX_BLOCKS * ib.cap - 1 - (t - front)], slot = item >> 2, b = item & 3;
     const int ev = ib.ev[slot];
     r4<double> k[NEXT];
     load_event<NEXT>(p, n, ev, k);
@@ -1054,7 +1007,7 @@ __global__ void __launch_bounds__(128, ME_MINB) k_rescue_items(const double* __r
       double R = 0.0;
 #pragma unroll
       for (int i = 0; i < NB; ++i) R += __ldcg(ib.v + i * ib.cap + slot);
-      out[ev] = (wgt ? wgt[ev] : 1.0) * (ib.a[slot] * R + ib.a[ib.cap + slot]);
+      out[ev] = (wgt ? wgt[ev] : 1.0) * (R + ib.wb[slot]);
     }
   }
 }
@@ -1127,12 +1080,12 @@ __global__ void __launch_bounds__(QT, ME_MINB) k_real_sub_queued(const double* _
 // its cuts; points without one are finished there.  k_term_reals evaluates the queued reals
 // one lane each and combines W, in mixed precision with the stability test and the records
 // and float64 items of the flagged points, as the masked evaluation (k_rescue_items follows).
-// A queued real carries 40 B: its point, a_R, W_B, the Born error scale, and the error
-// growth (negative for points inside the thresholds) with the active configurations.
+// A queued real carries 24 B: its point with the active configurations, W_B, the Born error
+// scale, and the error growth (negative for points inside the thresholds).
 struct TermBufs {
   int* ev;      // [cap] point of the record; bits 29, 30: active Born configurations
   float* grow;  // [cap] error growth factor of the stability test, negative: near
-  double* a;    // [3][cap] a_R, W_B, Born error scale
+  double* a;    // [2][cap] W_B, Born error scale
   int* cnt;     // records
   long cap;
 };
@@ -1157,7 +1110,7 @@ __device__ __forceinline__ int warp_reserve(int* ctr, int c) {
 // Float64 pass of the per-term queues: one thread per point.  `pc` (optional, device memory,
 // same layout as p): the momenta are copied there, so that the item kernels read device
 // memory when p is host memory read in place over the CPU-GPU link (p is then read once).
-template <int PID>
+template <int PID, typename T>
 __global__ void __launch_bounds__(128) k_terms(const double* __restrict__ p, const double* __restrict__ wgt, long n,
                                                double* __restrict__ out, KParams kp, const int* __restrict__ count,
                                                TermBufs tb, int* __restrict__ counts, ItemBufs ib,
@@ -1182,23 +1135,22 @@ __global__ void __launch_bounds__(128) k_terms(const double* __restrict__ p, con
 #pragma unroll
     for (int l = 0; l < NEXT; ++l) k[l] = r4<double>{1.0, 0.0, 0.0, 0.0};
   }
-  const PointTerms t = point_terms<PID>(k, kp);
-  const bool rec = act && t.inside && t.a_R > 0.0;
+  const PointTerms t = point_terms<PID, T>(k, kp);
+  const bool rec = act && t.inside && t.real;
   const int slot = warp_reserve(tb.cnt, rec ? 1 : 0);
   const RealSubOut r = combine_point(t, 0.0);
   if (rec) {
-    const float g = (float)error_growth(r);
+    const float g = error_growth(r);
     tb.ev[slot] = (int)i | (t.need[0] ? 1 << 29 : 0) | (t.need[1] ? 1 << 30 : 0);
     tb.grow[slot] = t.near ? -g : g;
-    tb.a[slot] = t.a_R;
-    tb.a[tb.cap + slot] = t.w_born;
-    tb.a[2 * tb.cap + slot] = t.mag_b;
+    tb.a[slot] = t.w_born;
+    tb.a[tb.cap + slot] = t.mag_b;
   } else if (act) {
     // no real matrix element: finished (a flagged one is float64 already)
     out[i] = r.W == 0.0 ? 0.0 : (wgt ? wgt[i] : 1.0) * r.W;
     if (kp.flag_unstable && t.inside && unstable_point(r, kp)) {
       const double none[MAX_BLOCKS] = {};
-      append_flagged<PID>(counts, ib, i, 0.0, 0.0, t.need, none, 0);
+      append_flagged<PID>(counts, ib, i, 0.0, t.need, none, 0);
     }
   }
 }
@@ -1222,15 +1174,14 @@ __global__ void __launch_bounds__(128, ME_MINB) k_term_reals(const double* __res
 #pragma unroll 1
       for (int b = 0; b < NB; ++b) R += (v[b] = real_block_value<PID, T>(K, b, kp));
     }
-    const double a_R = tb.a[slot], wb = tb.a[tb.cap + slot];
-    const double x = a_R * R, W = x + wb;
+    const double wb = tb.a[slot], W = R + wb;
     out[ev] = (wgt ? wgt[ev] : 1.0) * W;
     if (kp.flag_unstable) {
       const float g = tb.grow[slot];
-      const RealSubOut r{W, fabs(x) + tb.a[2 * tb.cap + slot], fabs(x), {0.0, 0.0}, g < 0.0f};
-      if (unstable_point(r, kp, (double)fabsf(g))) {
+      const RealSubOut r{W, fabs(R) + tb.a[tb.cap + slot], fabs(R), {0.0, 0.0}, g < 0.0f};
+      if (unstable_point(r, kp, fabsf(g))) {
         const bool need[2] = {(code >> 29 & 1) != 0, (code >> 30 & 1) != 0};
-        append_flagged<PID>(counts, ib, ev, a_R, wb, need, v, rescue_mask<PID>(r, a_R, v, kp, (double)fabsf(g)));
+        append_flagged<PID>(counts, ib, ev, wb, need, v, rescue_mask<PID>(r, true, v, kp, fabsf(g)));
       }
     }
   }
@@ -1404,13 +1355,15 @@ cudaError_t launch_terms_one(bool mixed, const LaunchArgs& a, const TermBufs& tb
   const long blocks = (a.groups + 127) / 128;
   if (blocks <= 0) return cudaSuccess;
   if ((e = cudaMemsetAsync(tb.cnt, 0, sizeof(int), st)) != cudaSuccess) return e;
-  k_terms<PID><<<(unsigned)blocks, 128, 0, st>>>(a.p, a.wgt, a.n, a.out, a.kp, a.count, tb, a.resc_count, a.items, a.p_copy);
   const double* pi = a.p_copy ? a.p_copy : a.p;
-  const unsigned gr = (unsigned)std::min<long>(g, blocks);
-  if (mixed)
+  const unsigned gr = (unsigned)std::min<long>(g, blocks), gt = (unsigned)blocks;
+  if (mixed) {
+    k_terms<PID, float><<<gt, 128, 0, st>>>(a.p, a.wgt, a.n, a.out, a.kp, a.count, tb, a.resc_count, a.items, a.p_copy);
     k_term_reals<PID, float><<<gr, 128, 0, st>>>(pi, a.wgt, a.n, a.out, a.kp, tb, a.resc_count, a.items);
-  else
+  } else {
+    k_terms<PID, double><<<gt, 128, 0, st>>>(a.p, a.wgt, a.n, a.out, a.kp, a.count, tb, a.resc_count, a.items, a.p_copy);
     k_term_reals<PID, double><<<gr, 128, 0, st>>>(pi, a.wgt, a.n, a.out, a.kp, tb, a.resc_count, a.items);
+  }
   return cudaGetLastError();
 }
 cudaError_t launch_terms_ee(bool mixed, const LaunchArgs& a, const TermBufs& tb, cudaStream_t st);

@@ -116,13 +116,24 @@ struct KinTT {
   T iq[1 << NG];
   wf_v<T> wg[NG];       // polarisation ingredients of the gluons (legs 0, 1, 4, 5)
   wf_q<T> wt, wtb;      // spinor ingredients of the top and, times g_s, of the antitop
+  bool axis;            // beams exactly along +z (leg 0) and -z (leg 1)
 };
+
+ME_HD bool zero_bits(double x) {  // x == 0, off the float64 pipe
+#ifdef __CUDA_ARCH__
+  return (__double_as_longlong(x) << 1) == 0;
+#else
+  return x == 0.0;
+#endif
+}
 
 template <typename T, int NG>
 ME_HD KinTT<T, NG> prep_tt(const r4<double>* p, const Couplings& cp) {
   KinTT<T, NG> K;
   const int NEXT = NG + 2;
   for (int l = 0; l < NEXT; ++l) K.pl[l] = cast4<T>(p[l]);
+  K.axis = zero_bits(p[0].x) && zero_bits(p[0].y) && zero_bits(p[1].x) && zero_bits(p[1].y) && K.pl[0].z > T(0) &&
+           T(0) > K.pl[1].z;
   r4<double> q[NG];
   for (int i = 0; i < NG; ++i) {
     const int l = i < 2 ? i : i + 2;
@@ -373,22 +384,22 @@ ME_HD void amp_tt3_fast(const KinTT<T, 3>& K, int hel, const Couplings& cp, cx<T
 // SM and cycle) and by instruction issue in float32, so what counts is the number of
 // operations.  Five-real polarisations (pol), light-cone quark spins (wf_q), brackets of
 // conserved currents without their vanishing terms, products e.J computed once and each
-// gluon-pair bracket used by both currents it enters take a g g -> t tbar g block from 7349
-// to 4737 operations and a g g -> t tbar g g block from 66751 to 49460.  GB300: 2^20
-// subtracted g g -> t tbar g points 5.55 -> 4.23 ms, 30011 in float64 1.385 -> 1.007 ms,
-// 8191 g g -> t tbar g g trees in float64 3.96 -> 3.04 ms.
+// gluon-pair bracket used by both currents it enters take a general g g -> t tbar g block from
+// 7349 to 4737 operations and a g g -> t tbar g g block from 66751 to 49460; beams on the z axis
+// take the former to about 3300.  GB300: 2^20 subtracted g g -> t tbar g points 5.55 -> 2.20 ms,
+// 30011 in float64 1.385 -> 0.552 ms (counterterms and rescue included).
 
 // g g -> t tbar g: the three-gluon currents F(012) = F(210), F(021) = F(120),
 // F(102) = F(201) and the pair currents J(xy) are built once per block; per top spin the
 // row R_s of ordering s collects ubar F(s), U(x) J(yz) and W(xy) e_z.
 // consume(r, A) receives the partial amplitudes of heavy spins r without the factor i g.
-template <typename T, class F>
-ME_HD void amp_tt3_block(const KinTT<T, 3>& K, int hb, const Couplings& cp, F&& consume) {
+// E0, E1: polarisations of the beam gluons, pol or axpol (on the axis the block takes about 1600
+// multiply-adds instead of 2500).
+template <typename T, class E0, class E1, class F>
+ME_HD void tt3_block(const KinTT<T, 3>& K, const E0& e0, const E1& e1, const pol<T>& e2, const Couplings& cp, F&& consume) {
+  constexpr bool PAIR = has_pair<E0, E1>::value;
   const T g = gs_of<T>(cp), mt = mt_of<T>(cp);
   const r4<T> k0 = K.q[0], k1 = K.q[1], k2 = K.q[2], kt = K.pl[2];
-  const pol<T> e0 = pol_of(K.wg[0], hel_of(hb, 0), false);
-  const pol<T> e1 = pol_of(K.wg[1], hel_of(hb, 1), false);
-  const pol<T> e2 = pol_of(K.wg[2], hel_of(hb, 4), true);
   const r4<T> k01 = k0 + k1, k02 = k0 + k2, k12 = k1 + k2;
   cx<T> e01, e02, e12;
   const c4<T> J01 = bracket(e0, k0, e1, k1, -g * K.ig[3], e01);
@@ -403,17 +414,30 @@ ME_HD void amp_tt3_block(const KinTT<T, 3>& K, int hb, const Couplings& cp, F&& 
   c4<T> F0 = czero<T>(), F2 = czero<T>(), B = czero<T>();
   bracket_acc(F0, e0, k0, J12, k12, c3, cdot(e0, J12));
   c4<T> F1 = cneg(F0);
-  bracket_acc(B, e2, k2, J01, k01, c3, cdot(e2, J01));  // J(2|01)
-  csub(F0, B);
-  cadd(F2, B);
-  B = czero<T>();
+  if constexpr (PAIR) {
+    bracket_acc(B, e2, k2, J01, k01, c3, cdot(e2, J01));  // J(2|01)
+    csub(F0, B);
+    cadd(F2, B);
+    B = czero<T>();
+  }
   bracket_acc(B, e1, k1, J02, k02, c3, cdot(e1, J02));  // J(1|02)
   csub(F1, B);
   cadd(F2, B);
-  quartic_acc(F0, e0, e1, e2, e02, e01, e12);
-  quartic_acc(F1, e0, e2, e1, e01, e02, e12);
-  quartic_acc(F2, e1, e0, e2, e12, e01, e02);
-  const spol<T> se0 = slashed(e0), se1 = slashed(e1), se2 = slashed(e2);
+  if constexpr (PAIR) {
+    quartic_acc(F0, e0, e1, e2, e02, e01, e12);
+    quartic_acc(F1, e0, e2, e1, e01, e02, e12);
+    quartic_acc(F2, e1, e0, e2, e12, e01, e02);
+  } else {  // e01 = 0
+    caxpy(F0, T(2) * e02, e1);
+    caxpy(F0, -e12, e0);
+    caxpy(F1, -e02, e1);
+    caxpy(F1, -e12, e0);
+    caxpy(F2, T(2) * e12, e0);
+    caxpy(F2, -e02, e1);
+  }
+  const auto se0 = slashed(e0);
+  const auto se1 = slashed(e1);
+  const spol<T> se2 = slashed(e2);
   const sl4<T> sJ01 = slashed(J01), sJ02 = slashed(J02), sJ12 = slashed(J12);
   const sl4<T> sF0 = slashed(F0), sF1 = slashed(F1), sF2 = slashed(F2);
   const r4<T> Q0 = kt + k0, Q1 = kt + k1, Q2 = kt + k2;
@@ -430,9 +454,11 @@ ME_HD void amp_tt3_block(const KinTT<T, 3>& K, int hb, const Couplings& cp, F&& 
     R[3] = R[1];
     R[4] = R[2];
     R[5] = R[0];
-    const c4<T> S01 = ubar_slash(K.wt, ht, sJ01), S02 = ubar_slash(K.wt, ht, sJ02), S12 = ubar_slash(K.wt, ht, sJ12);
+    const c4<T> S02 = ubar_slash(K.wt, ht, sJ02), S12 = ubar_slash(K.wt, ht, sJ12);
+    c4<T> S01 = czero<T>();
+    if constexpr (PAIR) S01 = ubar_slash(K.wt, ht, sJ01);
     {  // first gluon 0: orderings 012, 021
-      const c4<T> U = row_prop(ubar_slash(K.wt, ht, se0), P0);
+      const c4<T> U = gluon_line(K.wt, ht, se0, P0);
       const c4<T> t = row_slash(U, sJ12);
       cadd(R[0], t);
       csub(R[1], t);
@@ -444,7 +470,7 @@ ME_HD void amp_tt3_block(const KinTT<T, 3>& K, int hb, const Couplings& cp, F&& 
       row_slash_acc(R[1], row_prop(r, P02), se1);
     }
     {  // first gluon 1: orderings 102, 120
-      const c4<T> U = row_prop(ubar_slash(K.wt, ht, se1), P1);
+      const c4<T> U = gluon_line(K.wt, ht, se1, P1);
       const c4<T> t = row_slash(U, sJ02);
       cadd(R[2], t);
       csub(R[3], t);
@@ -456,10 +482,12 @@ ME_HD void amp_tt3_block(const KinTT<T, 3>& K, int hb, const Couplings& cp, F&& 
       row_slash_acc(R[3], row_prop(r, P12), se0);
     }
     {  // first gluon 2: orderings 201, 210
-      const c4<T> U = row_prop(ubar_slash(K.wt, ht, se2), P2);
-      const c4<T> t = row_slash(U, sJ01);
-      cadd(R[4], t);
-      csub(R[5], t);
+      const c4<T> U = gluon_line(K.wt, ht, se2, P2);
+      if constexpr (PAIR) {
+        const c4<T> t = row_slash(U, sJ01);
+        cadd(R[4], t);
+        csub(R[5], t);
+      }
       c4<T> r = cneg(S02);
       row_slash_acc(r, U, se0);
       row_slash_acc(R[4], row_prop(r, P02), se1);
@@ -474,6 +502,21 @@ ME_HD void amp_tt3_block(const KinTT<T, 3>& K, int hb, const Couplings& cp, F&& 
       for (int f = 0; f < 6; ++f) A[f] = dot_v(R[f], K.wtb, hv);
       consume(ht | (hv << 1), A);
     }
+  }
+}
+
+template <typename T, class F>
+ME_HD void amp_tt3_block(const KinTT<T, 3>& K, int hb, const Couplings& cp, F&& consume) {
+  const pol<T> e2 = pol_of(K.wg[2], hel_of(hb, 4), true);
+  if (K.axis) {
+    // leg 0 (helicity + in every block) is -(0, 1, i, 0) / sqrt 2, leg 1 the same for
+    // helicity - and (0, 1, -i, 0) / sqrt 2 for +
+    const T r2 = T(0.70710678118654752440);
+    const axpol<T, 1> e0{-r2};
+    if (hel_of(hb, 1) < 0) tt3_block(K, e0, axpol<T, 1>{-r2}, e2, cp, consume);
+    else tt3_block(K, e0, axpol<T, -1>{r2}, e2, cp, consume);
+  } else {
+    tt3_block(K, pol_of(K.wg[0], hel_of(hb, 0), false), pol_of(K.wg[1], hel_of(hb, 1), false), e2, cp, consume);
   }
 }
 
@@ -592,19 +635,32 @@ ME_HD KinUU<T> prep_uu(const r4<double>* p, const Couplings& cp) {
     q[l] = l < 2 ? -p[l] : p[l];
     K.q[l] = l < 2 ? -K.pl[l] : K.pl[l];
   }
-  const double m2 = cp.mt * cp.mt;
-  const r4<double> s01 = q[0] + q[1];
-  K.is = T(1) / (T)mdot(s01, s01);
   K.ia = K.ib = K.ic = K.id = K.is3 = K.it = T(0);
+  if constexpr (NEXT == 5 && std::is_same<T, float>::value) {
+    // on-shell legs: every denominator from five products (float64)
+    const double d01 = mdot(q[0], q[1]), d04 = mdot(q[0], q[4]), d14 = mdot(q[1], q[4]);
+    K.is = T(0.5) / (T)d01;
+    K.ia = T(0.5) / (T)mdot(q[2], q[4]);
+    K.ib = T(0.5) / (T)mdot(q[3], q[4]);
+    K.ic = T(0.5) / (T)d14;
+    K.id = T(0.5) / (T)d04;
+    K.is3 = K.it = T(0.5) / (T)(d01 + d04 + d14);
+  } else {
+    const double m2 = cp.mt * cp.mt;
+    const r4<double> s01 = q[0] + q[1];
+    K.is = T(1) / (T)mdot(s01, s01);
+    if (NEXT == 5) {
+      const r4<double> a = q[2] + q[4], b = q[3] + q[4], c = q[1] + q[4], d = q[0] + q[4];
+      const r4<double> s3 = s01 + q[4], t = q[2] + q[3];
+      K.ia = T(1) / (T)(mdot(a, a) - m2);
+      K.ib = T(1) / (T)(mdot(b, b) - m2);
+      K.ic = T(1) / (T)mdot(c, c);
+      K.id = T(1) / (T)mdot(d, d);
+      K.is3 = T(1) / (T)mdot(s3, s3);
+      K.it = T(1) / (T)mdot(t, t);
+    }
+  }
   if (NEXT == 5) {
-    const r4<double> a = q[2] + q[4], b = q[3] + q[4], c = q[1] + q[4], d = q[0] + q[4];
-    const r4<double> s3 = s01 + q[4], t = q[2] + q[3];
-    K.ia = T(1) / (T)(mdot(a, a) - m2);
-    K.ib = T(1) / (T)(mdot(b, b) - m2);
-    K.ic = T(1) / (T)mdot(c, c);
-    K.id = T(1) / (T)mdot(d, d);
-    K.is3 = T(1) / (T)mdot(s3, s3);
-    K.it = T(1) / (T)mdot(t, t);
     K.wt = wf_quark(K.pl[2], mt_of<T>(cp));
     K.wtb = wf_quark(K.pl[3], mt_of<T>(cp));
     K.wg = wf_vector(K.pl[4]);
@@ -1021,17 +1077,17 @@ template <typename T>
 ME_HD T born_gg_colour(const BornGG<T>& b) {  // M = C
   return b.f * (T(GG_C00) * (b.r0 + b.r1) + T(2.0 * GG_C01));
 }
-// the same with one gluon polarised along e, ep = e.p2 (either gluon)
+// the same with one gluon polarised along e, ep2 = (e.p2)^2 / (p0.p1) (either gluon)
 template <typename T>
-ME_HD T born_gg_polarised(const Inv22<T>& k, const BornGG<T>& b, T ep, const Couplings& cp) {
+ME_HD T born_gg_polarised(const Inv22<T>& k, const BornGG<T>& b, T ep2, const Couplings& cp) {
   const T g2 = gs_of<T>(cp) * gs_of<T>(cp), t01 = k.t0 * k.t1;
   const T col = T(0.5 * GG_C00) * (b.r0 + b.r1) + T(GG_C01);
-  return col * (b.f + T(8) * g2 * g2 * k.rho * (ep * ep / k.c - (t01 - T(0.25) * k.rho)) / t01);
+  return col * (b.f + T(8) * g2 * g2 * k.rho * (ep2 - (t01 - T(0.25) * k.rho)) / t01);
 }
-// M the eikonal-weighted correlator matrix (row-major 2 x 2)
+// (sum J^T M J) / f for a symmetric matrix M (row-major 2 x 2)
 template <typename T>
-ME_HD T born_gg_matrix(const BornGG<T>& b, const T* M) {
-  return b.f * (M[0] * b.r0 + (M[1] + M[2]) + M[3] * b.r1);
+ME_HD T born_gg_form(const BornGG<T>& b, const T* M) {
+  return M[0] * b.r0 + T(2) * M[1] + M[3] * b.r1;
 }
 // u ubar -> t tbar with the matrix M: its amplitude in the basis (d_ik d_lj, d_ij d_lk) is
 // proportional to (1/2, -1/6), `sum` is the plain Born / 2
