@@ -24,6 +24,16 @@ static double csum(const ColourTables& tab, const cx<T>* J) {
       t += C[a * NF + b] * ((double)J[a].re * (double)J[b].re + (double)J[a].im * (double)J[b].im);
   return t;
 }
+// the colour sum as the helicity blocks take it
+template <int PID, typename T>
+static double bsum(const ColourTables& tab, const cx<T>* J) {
+  if constexpr (PID == P_GG_TTGG) {
+    T coef[S4_COEF];
+    for (int i = 0; i < S4_COEF; ++i) coef[i] = (T)tab.S4[i];
+    return (double)s4_colour_sum(coef, J);
+  }
+  return csum<PID, T>(tab, J);
+}
 
 template <int PID, typename T>
 static void eval(const ColourTables& tab, const r4<double>* k, const Couplings& cp, double* blk, double* single) {
@@ -37,7 +47,7 @@ static void eval(const ColourTables& tab, const r4<double>* k, const Couplings& 
   }
   double b = 0;
   for (int i = 0; i < n_live_blocks<PID>(); ++i)
-    amplitude_block<PID, T>(K, live_block_hel<PID>(i), cp, [&](int, const cx<T>* A) { b += csum<PID, T>(tab, A); });
+    amplitude_block<PID, T>(K, live_block_hel<PID>(i), cp, [&](int, const cx<T>* A) { b += bsum<PID, T>(tab, A); });
   *blk = 2.0 * b;
   *single = s;
 }

@@ -350,6 +350,10 @@ static int build_tables(ColourTables& tab) {
         tab.U[it.pid][x * nf + y] = u;
         tab.Uf[it.pid][x * nf + y] = (float)u;
       }
+    if (it.pid == P_GG_TTGG) {
+      if (!s4_coefficients(tab.C[it.pid], tab.S4)) return fail(ME_ERR_PROCESS, "colour matrix lacks the gluon symmetry");
+      for (int i = 0; i < S4_COEF; ++i) tab.S4f[i] = (float)tab.S4[i];
+    }
     // Born colour correlators C^{kl}_{xy} = sum_a <T_k^a e_x | T_l^a e_y>
     if (it.pid == P_GG_TT || it.pid == P_UU_TT) {
       const int ci = it.pid == P_GG_TT ? 0 : 1;

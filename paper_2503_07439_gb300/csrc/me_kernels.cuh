@@ -42,6 +42,8 @@ struct ColourTables {
   double U[P_COUNT][MAX_FLOW * MAX_FLOW];
   float Uf[P_COUNT][MAX_FLOW * MAX_FLOW];
   double Ccorr[2][N_PAIRS][4];
+  double S4[S4_COEF];  // g g -> t tbar g g (s4_colour_sum)
+  float S4f[S4_COEF];
   double Cqq[N_PAIRS];  // u ubar -> t tbar, contracted with its one colour structure (born_uu_matrix)
 };
 
@@ -82,6 +84,9 @@ struct KParams {
 template <typename T> __device__ __forceinline__ const T* ctab(const ColourTables* t, int pid);
 template <> __device__ __forceinline__ const double* ctab<double>(const ColourTables* t, int pid) { return t->C[pid]; }
 template <> __device__ __forceinline__ const float* ctab<float>(const ColourTables* t, int pid) { return t->Cf[pid]; }
+template <typename T> __device__ __forceinline__ const T* s4tab(const ColourTables* t);
+template <> __device__ __forceinline__ const double* s4tab<double>(const ColourTables* t) { return t->S4; }
+template <> __device__ __forceinline__ const float* s4tab<float>(const ColourTables* t) { return t->S4f; }
 template <typename T> __device__ __forceinline__ const T* utab(const ColourTables* t, int pid);
 template <> __device__ __forceinline__ const double* utab<double>(const ColourTables* t, int pid) { return t->U[pid]; }
 template <> __device__ __forceinline__ const float* utab<float>(const ColourTables* t, int pid) { return t->Uf[pid]; }
@@ -89,14 +94,15 @@ template <> __device__ __forceinline__ const float* utab<float>(const ColourTabl
 template <int PID, typename T>
 __device__ __forceinline__ T colour_sum(const ColourTables* tab, const cx<T>* J) {
   constexpr int NF = Proc<PID>::NFLOW;
+  if constexpr (PID == P_GG_TTGG) return s4_colour_sum(s4tab<T>(tab), J);
   T s = T(0);
   // triangular form: NF (NF + 1) + 2 NF multiply-adds instead of 2 NF^2 + 2 NF
   const T* __restrict__ Um = utab<T>(tab, PID);
-#pragma unroll(NF <= 6 ? NF : 1)
+#pragma unroll
   for (int a = 0; a < NF; ++a) {
     const T d = Um[a * NF + a];
     T zr = d * J[a].re, zi = d * J[a].im;
-#pragma unroll(NF <= 6 ? NF : 4)
+#pragma unroll
     for (int b = a + 1; b < NF; ++b) {
       const T c = Um[a * NF + b];
       zr += c * J[b].re;
@@ -188,13 +194,13 @@ __device__ __forceinline__ bool pass_cuts(const r4<double>* k, const Cuts& c) {
 // ---------------------------------------------------------------- tree |M|^2
 // out[i] = wgt[i] * |M|^2(p_i) * nlo_factor.  `count` (optional): the number of events,
 // read on the device; `idx` (optional): the list of events to process (its length in
-// `count`).  Momenta have stride n either way.  (g g -> t tbar g g in float32 runs
-// k_tree_tc4 below instead.)
+// `count`).  Momenta have stride n either way.  (g g -> t tbar g g runs k_tree_tt4 and, in
+// float32, k_tree_tc4 below instead.)
 template <int PID, typename T, int LPE>
 __global__ void __launch_bounds__(128, ME_MINB) k_tree(const double* __restrict__ p, const double* __restrict__ wgt,
                                                        long n, double* __restrict__ out, KParams kp,
                                                        const int* __restrict__ idx, const int* __restrict__ count) {
-  static_assert(!(PID == P_GG_TTGG && std::is_same<T, float>::value), "float g g -> t tbar g g runs k_tree_tc4");
+  static_assert(PID != P_GG_TTGG, "g g -> t tbar g g runs k_tree_tt4 and k_tree_tc4");
   constexpr int NEXT = Proc<PID>::NEXT;
   const long gid = ((long)blockIdx.x * blockDim.x + threadIdx.x) / LPE;
   const int lane = threadIdx.x % LPE;
@@ -215,6 +221,38 @@ __global__ void __launch_bounds__(128, ME_MINB) k_tree(const double* __restrict_
     const double w = wgt ? wgt[ev] : 1.0;
     out[ev] = pass ? w * tot * kp.tree_scale : 0.0;
   }
+}
+
+// g g -> t tbar g g in float64: as k_tree, with the L = 2^lg lanes of an event in different warps
+// (half warps for L = 8), so that the beam gluons' helicities, which choose the form of a block,
+// are the same across a warp.  The float64 pipe bounds it.
+template <int PID>
+__global__ void __launch_bounds__(128, ME_MINB) k_tree_tt4(const double* __restrict__ p, const double* __restrict__ wgt,
+                                                           long n, double* __restrict__ out, KParams kp,
+                                                           const int* __restrict__ idx, const int* __restrict__ count, int lg) {
+  static_assert(PID == P_GG_TTGG, "eight blocks");
+  __shared__ double part[128];
+  const int slot = threadIdx.x & ((128 >> lg) - 1), lane = threadIdx.x >> (7 - lg);
+  const long gid = ((long)blockIdx.x << (7 - lg)) + slot;
+  const long nev = count ? (long)*count : n;
+  const bool live = gid < nev;
+  const long ev = live ? (idx ? (long)idx[gid] : gid) : 0;
+  double acc = 0.0;
+  bool pass = false;
+  if (live) {
+    r4<double> k[6];
+    load_event<6>(p, n, ev, k);
+    pass = !kp.cut.mask || pass_cuts<PID>(k, kp.cut);
+    const Kin<PID, double> K = prepare<PID, double>(k, unit_couplings(kp.cp));
+#pragma unroll 1
+    for (int b = lane << (3 - lg); b < (lane + 1) << (3 - lg); ++b)
+      acc += block_sum<PID, double>(K, ((b & 3) << 1) | (b >> 2), kp);  // leg 1 in the top bit
+  }
+  part[threadIdx.x] = acc;
+  __syncthreads();
+  if (!live || lane > 0) return;
+  for (int i = 1; i < 1 << lg; ++i) acc += part[(i << (7 - lg)) + slot];
+  out[ev] = pass ? (wgt ? wgt[ev] : 1.0) * (2.0 * acc) * kp.tree_scale : 0.0;
 }
 
 // The closed 2 -> 2 trees: one lane per event, bound by the momenta's DRAM traffic and, in
@@ -1234,22 +1272,22 @@ cudaError_t launch_one(int kind, const LaunchArgs& a, cudaStream_t st) {
   if (blocks <= 0) return cudaSuccess;
   if (kind == K_TREE) {
     if constexpr (PID == P_GG_TTGG && std::is_same<T, float>::value) {
-      if constexpr (LPE != 4) {
-        return cudaErrorInvalidValue;
-      } else {
-        static bool attr_set[64] = {};
-        int dev = 0;
-        cudaGetDevice(&dev);
-        if (dev < 64 && !attr_set[dev]) {
-          cudaFuncSetAttribute(k_tree_tc4<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, TC4_SMEM);
-          attr_set[dev] = true;
-        }
-        const long tb = (total + TC4_THREADS - 1) / TC4_THREADS;
-        k_tree_tc4<4><<<(unsigned)tb, TC4_THREADS, TC4_SMEM, st>>>(a.p, a.wgt, a.n, a.out, a.kp, a.idx, a.count);
+      static_assert(LPE == 4, "four lanes per event");
+      static bool attr_set[64] = {};
+      int dev = 0;
+      cudaGetDevice(&dev);
+      if (dev < 64 && !attr_set[dev]) {
+        cudaFuncSetAttribute(k_tree_tc4<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, TC4_SMEM);
+        attr_set[dev] = true;
       }
+      const long tb = (total + TC4_THREADS - 1) / TC4_THREADS;
+      k_tree_tc4<4><<<(unsigned)tb, TC4_THREADS, TC4_SMEM, st>>>(a.p, a.wgt, a.n, a.out, a.kp, a.idx, a.count);
     } else if constexpr (closed_tree<PID>()) {
       if constexpr (LPE != 1) return launch_one<PID, T, 1>(kind, a, st);
       else k_tree_closed<PID, T><<<(unsigned)((a.groups + 255) / 256), 256, 0, st>>>(a.p, a.wgt, a.n, a.out, a.kp, a.idx, a.count);
+    } else if constexpr (PID == P_GG_TTGG) {
+      constexpr int lg = LPE == 1 ? 0 : LPE == 2 ? 1 : LPE == 4 ? 2 : 3;
+      k_tree_tt4<PID><<<(unsigned)blocks, threads, 0, st>>>(a.p, a.wgt, a.n, a.out, a.kp, a.idx, a.count, lg);
     } else {
       k_tree<PID, T, LPE><<<(unsigned)blocks, threads, 0, st>>>(a.p, a.wgt, a.n, a.out, a.kp, a.idx, a.count);
     }

@@ -846,19 +846,56 @@ ME_HD void amplitude(const Kin<PID, T>& K, int hel, const Couplings& cp, cx<T>* 
   else amp_uu_ttg<T>(K, hel, cp, A);
 }
 
+// The four gluons of a block: beam gluons of type E0, E1 (pol or axpol), outgoing ones pol.  The
+// gluon index is a constant wherever these are called in unrolled code.
+template <typename T, class E0, class E1>
+struct FourGluons {
+  E0 e0;
+  E1 e1;
+  pol<T> e2, e3;
+  ME_HD cx<T> dot(int i, const c4<T>& J) const {
+    return i == 0 ? cdot(e0, J) : i == 1 ? cdot(e1, J) : i == 2 ? cdot(e2, J) : cdot(e3, J);
+  }
+  ME_HD void add(c4<T>& acc, cx<T> w, int i) const {
+    if (i == 0) caxpy(acc, w, e0);
+    else if (i == 1) caxpy(acc, w, e1);
+    else if (i == 2) caxpy(acc, w, e2);
+    else caxpy(acc, w, e3);
+  }
+  ME_HD void current(c4<T>& acc, int i, const r4<T>& q, const c4<T>& J, const r4<T>& Q, T s, cx<T> eJ) const {
+    if (i == 0) bracket_acc(acc, e0, q, J, Q, s, eJ);
+    else if (i == 1) bracket_acc(acc, e1, q, J, Q, s, eJ);
+    else if (i == 2) bracket_acc(acc, e2, q, J, Q, s, eJ);
+    else bracket_acc(acc, e3, q, J, Q, s, eJ);
+  }
+  ME_HD c4<T> pair(int x, int y, const r4<T>* q, T s, cx<T>& xy) const {  // x < y
+    return x == 0 ? (y == 1 ? bracket(e0, q[0], e1, q[1], s, xy) : y == 2 ? bracket(e0, q[0], e2, q[2], s, xy)
+                                                                          : bracket(e0, q[0], e3, q[3], s, xy))
+           : x == 1 ? (y == 2 ? bracket(e1, q[1], e2, q[2], s, xy) : bracket(e1, q[1], e3, q[3], s, xy))
+                    : bracket(e2, q[2], e3, q[3], s, xy);
+  }
+  ME_HD void row(c4<T>& acc, const c4<T>& r, int i) const {
+    if (i == 0) row_slash_acc(acc, r, slashed(e0));
+    else if (i == 1) row_slash_acc(acc, r, slashed(e1));
+    else if (i == 2) row_slash_acc(acc, r, slashed(e2));
+    else row_slash_acc(acc, r, slashed(e3));
+  }
+  ME_HD c4<T> line(const wf_q<T>& w, int h, int i, const prop4<T>& P) const {
+    return i == 0 ? gluon_line(w, h, slashed(e0), P) : i == 1 ? gluon_line(w, h, slashed(e1), P)
+           : i == 2 ? gluon_line(w, h, slashed(e2), P) : gluon_line(w, h, slashed(e3), P);
+  }
+};
+
 // g g -> t tbar g g.  The ordered gluon currents are built once per block with the
 // reflection identities: 6 pairs J(xy), x < y; 12 triples J(xyz) (one of each
 // reversed pair); 12 quadruples J(wxyz) with w < z.  Per top spin, the quark line
 // is extended ordering by ordering, U(w) -> U(wx) -> U(wxy), and the row of ordering
-// wxyz is ubar J(wxyz) + U(w) J(xyz) + U(wx) J(yz) + U(wxy) e_z.  Orderings are
+// wxyz is ubar J(wxyz) + U(w) J(xyz) + U(wx) J(yz) + U(wxy) e_z; a product of U(w) or U(wx)
+// with a current serves the ordering that has it reversed too.  Orderings are
 // numbered lexicographically, as in amp_ttng.
-template <typename T, class F>
-ME_HD void amp_tt4_block(const KinTT<T, 4>& K, int hb, const Couplings& cp, F&& consume) {
+template <typename T, class G, class F>
+ME_HD void tt4_block(const KinTT<T, 4>& K, const G& e, const Couplings& cp, F&& consume) {
   const T g = gs_of<T>(cp), mt = mt_of<T>(cp);
-  constexpr int LEG[4] = {0, 1, 4, 5};
-  pol<T> e[4];
-#pragma unroll
-  for (int i = 0; i < 4; ++i) e[i] = pol_of(K.wg[i], hel_of(hb, LEG[i]), LEG[i] >= 2);
   const r4<T>* q = K.q;
   // pair currents, index pidx(x, y) for x < y, and the products e_i . e_j, e_i . J(xy)
   c4<T> J2[6];
@@ -868,7 +905,7 @@ ME_HD void amp_tt4_block(const KinTT<T, 4>& K, int hb, const Couplings& cp, F&& 
   for (int x = 0; x < 4; ++x)
 #pragma unroll
     for (int y = x + 1; y < 4; ++y) {
-      J2[pidx(x, y)] = bracket(e[x], q[x], e[y], q[y], -g * K.ig[(1 << x) | (1 << y)], ee[pidx(x, y)]);
+      J2[pidx(x, y)] = e.pair(x, y, q, -g * K.ig[(1 << x) | (1 << y)], ee[pidx(x, y)]);
     }
 #pragma unroll
   for (int i = 0; i < 4; ++i)
@@ -876,7 +913,7 @@ ME_HD void amp_tt4_block(const KinTT<T, 4>& K, int hb, const Couplings& cp, F&& 
     for (int x = 0; x < 4; ++x)
 #pragma unroll
       for (int y = x + 1; y < 4; ++y)
-        if (i != x && i != y) eJ[i][pidx(x, y)] = cdot(e[i], J2[pidx(x, y)]);
+        if (i != x && i != y) eJ[i][pidx(x, y)] = e.dot(i, J2[pidx(x, y)]);
   auto e2 = [&](int x, int y) { return ee[x < y ? pidx(x, y) : pidx(y, x)]; };
   auto ej = [&](int i, int x, int y) {  // e_i . J(xy), J(yx) = -J(xy)
     return x < y ? eJ[i][pidx(x, y)] : -eJ[i][pidx(y, x)];
@@ -903,9 +940,11 @@ ME_HD void amp_tt4_block(const KinTT<T, 4>& K, int hb, const Couplings& cp, F&& 
         const int S = (1 << x) | (1 << y) | (1 << z);
         const T c3 = -g * K.ig[S], c4g = g * g * K.ig[S];
         c4<T> J = czero<T>();
-        bracket_acc(J, e[x], q[x], j2(y, z), q[y] + q[z], c3, ej(x, y, z));
-        bracket_acc(J, e[z], q[z], j2(x, y), q[x] + q[y], -c3, ej(z, x, y));
-        quartic_acc(J, e[x], e[y], e[z], c4g * e2(x, z), c4g * e2(x, y), c4g * e2(y, z));
+        e.current(J, x, q[x], j2(y, z), q[y] + q[z], c3, ej(x, y, z));
+        e.current(J, z, q[z], j2(x, y), q[x] + q[y], -c3, ej(z, x, y));
+        e.add(J, T(2) * c4g * e2(x, z), y);
+        e.add(J, -c4g * e2(x, y), z);
+        e.add(J, -c4g * e2(y, z), x);
         J3[tidx(x, y, z)] = J;
       }
   auto j3 = [&](int x, int y, int z) { return J3[tidx(x, y, z)]; };
@@ -925,12 +964,18 @@ ME_HD void amp_tt4_block(const KinTT<T, 4>& K, int hb, const Couplings& cp, F&& 
         const r4<T> qwx = q[w] + q[x], qyz = q[y] + q[z];
         const c4<T> Jxyz = j3(x, y, z), Jwxy = j3(w, x, y), Jwx = j2(w, x), Jxy = j2(x, y), Jyz = j2(y, z);
         c4<T> J = czero<T>();
-        bracket_acc(J, e[w], q[w], Jxyz, q[x] + qyz, c3, cdot(e[w], Jxyz));
+        e.current(J, w, q[w], Jxyz, q[x] + qyz, c3, e.dot(w, Jxyz));
         bracket_acc(J, Jwx, qwx, Jyz, qyz, c3);
-        bracket_acc(J, e[z], q[z], Jwxy, qwx + q[y], -c3, cdot(e[z], Jwxy));
-        quartic_acc(J, e[w], e[x], Jyz, c4g * ej(w, y, z), c4g * e2(w, x), c4g * ej(x, y, z));
-        quartic_acc(J, e[w], Jxy, e[z], c4g * e2(w, z), c4g * ej(w, x, y), c4g * ej(z, x, y));
-        quartic_acc(J, Jwx, e[y], e[z], c4g * ej(z, w, x), c4g * ej(y, w, x), c4g * e2(y, z));
+        e.current(J, z, q[z], Jwxy, qwx + q[y], -c3, e.dot(z, Jwxy));
+        // 2 (L.R) M - (L.M) R - (M.R) L for (e_w, e_x, J_yz), (e_w, J_xy, e_z), (J_wx, e_y, e_z),
+        // collected by vector
+        e.add(J, c4g * (T(2) * ej(w, y, z)), x);
+        e.add(J, c4g * (T(2) * ej(z, w, x)), y);
+        e.add(J, -c4g * (ej(x, y, z) + ej(z, x, y)), w);
+        e.add(J, -c4g * (ej(w, x, y) + ej(y, w, x)), z);
+        caxpy(J, -c4g * e2(w, x), Jyz);
+        caxpy(J, T(2) * c4g * e2(w, z), Jxy);
+        caxpy(J, -c4g * e2(y, z), Jwx);
         J4[n4++] = J;
       }
   // rank of the quadruple current of ordering wxyz among those with first < last
@@ -955,26 +1000,39 @@ ME_HD void amp_tt4_block(const KinTT<T, 4>& K, int hb, const Couplings& cp, F&& 
     int f = 0;
 #pragma unroll
     for (int w = 0; w < 4; ++w) {
-      const c4<T> U1 = row_prop(ubar_slash(K.wt, ht, slashed(e[w])), scaled_prop(kt + q[w], mt, -g * K.iq[1 << w]));
+      const c4<T> U1 = e.line(K.wt, ht, w, scaled_prop(kt + q[w], mt, -g * K.iq[1 << w]));
+      // U(w) J(xy), x < y, and U(w) J(xyz) by its middle gluon y
+      c4<T> P[6], Q[4];
+#pragma unroll
+      for (int x = 0; x < 4; ++x)
+#pragma unroll
+        for (int y = x + 1; y < 4; ++y)
+          if (x != w && y != w) {
+            P[pidx(x, y)] = row_slash(U1, slashed(J2[pidx(x, y)]));
+            Q[6 - w - x - y] = row_slash(U1, slashed(j3(x, 6 - w - x - y, y)));
+          }
 #pragma unroll
       for (int x = 0; x < 4; ++x) {
         if (x == w) continue;
         c4<T> r2 = ubar_slash(K.wt, ht, slashed(j2(w, x)));
-        row_slash_acc(r2, U1, slashed(e[x]));
+        e.row(r2, U1, x);
         const c4<T> U2 = row_prop(r2, scaled_prop(kt + q[w] + q[x], mt, -g * K.iq[(1 << w) | (1 << x)]));
+        c4<T> D = czero<T>();  // U(wx) J(yz), y < z
 #pragma unroll
         for (int y = 0; y < 4; ++y) {
           if (y == w || y == x) continue;
           const int z = 6 - w - x - y;
-          c4<T> r3 = ubar_slash(K.wt, ht, slashed(j3(w, x, y)));
-          row_slash_acc(r3, U1, j2(x, y));
-          row_slash_acc(r3, U2, slashed(e[y]));
+          if (y < z) D = row_slash(U2, slashed(J2[pidx(y, z)]));
+          c4<T> r3 = x < y ? P[pidx(x, y)] : cneg(P[pidx(y, x)]);
+          ubar_slash_acc(r3, K.wt, ht, slashed(j3(w, x, y)));
+          e.row(r3, U2, y);
           const c4<T> U3 =
               row_prop(r3, scaled_prop(kt + q[w] + q[x] + q[y], mt, -g * K.iq[(1 << w) | (1 << x) | (1 << y)]));
-          c4<T> R = ubar_slash(K.wt, ht, slashed(z > w ? J4[q4(w, x, y)] : cneg(J4[q4(z, y, x)])));
-          row_slash_acc(R, U1, j3(x, y, z));
-          row_slash_acc(R, U2, j2(y, z));
-          row_slash_acc(R, U3, slashed(e[z]));
+          c4<T> R = Q[y];
+          if (y < z) cadd(R, D);
+          else csub(R, D);
+          ubar_slash_acc(R, K.wt, ht, slashed(z > w ? J4[q4(w, x, y)] : cneg(J4[q4(z, y, x)])));
+          e.row(R, U3, z);
 #pragma unroll
           for (int hv = 0; hv < 2; ++hv) A[hv][f] = dot_v(R, K.wtb, hv);
           ++f;
@@ -984,6 +1042,92 @@ ME_HD void amp_tt4_block(const KinTT<T, 4>& K, int hb, const Couplings& cp, F&& 
 #pragma unroll
     for (int hv = 0; hv < 2; ++hv) consume(ht | (hv << 1), A[hv]);
   }
+}
+template <typename T, class F>
+ME_HD void amp_tt4_block(const KinTT<T, 4>& K, int hb, const Couplings& cp, F&& consume) {
+  const pol<T> e2 = pol_of(K.wg[2], hel_of(hb, 4), true), e3 = pol_of(K.wg[3], hel_of(hb, 5), true);
+  if (K.axis) {  // as amp_tt3_block
+    const T r2 = T(0.70710678118654752440);
+    using A = axpol<T, 1>;
+    using B = axpol<T, -1>;
+    if (hel_of(hb, 1) < 0) tt4_block(K, FourGluons<T, A, A>{{-r2}, {-r2}, e2, e3}, cp, consume);
+    else tt4_block(K, FourGluons<T, A, B>{{-r2}, {r2}, e2, e3}, cp, consume);
+  } else {
+    tt4_block(K, FourGluons<T, pol<T>, pol<T>>{pol_of(K.wg[0], hel_of(hb, 0), false), pol_of(K.wg[1], hel_of(hb, 1), false), e2, e3},
+              cp, consume);
+  }
+}
+
+// Colour sum of the 24 orderings of four gluons.  Relabelling the gluons changes no colour
+// factor, and l -> l ^ v, v = 0 .. 3, is a group of relabellings: in the sums
+//   S_k[a] = sum_v (-1)^|k & v| J(ordering v, v ^ x, v ^ y, v ^ z),
+// a numbering the arrangements xyz of 1, 2, 3 lexicographically, the matrix falls into one
+// 6 x 6 block for each k.  Nor does reversing an ordering, which takes S_k[a] to
+// (-1)^|k & z| S_k[a]: for k > 0 the two arrangements with sign + couple only to each other
+// and the four with - to each other.  That leaves 21 + 3 (3 + 10) coefficients (off-diagonal
+// ones doubled) and 264 operations, where the triangle of the 24 x 24 matrix takes 648.
+constexpr int S4_COEF = 60;
+// flow number (lexicographic) of the ordering v, v ^ x, v ^ y, v ^ z of arrangement a
+__host__ __device__ constexpr int s4_flow(int v, int a) {
+  const int x = 1 + (a >> 1), lo = x == 1 ? 2 : 1, hi = x == 3 ? 2 : 3;
+  const int w[4] = {v, v ^ x, v ^ ((a & 1) ? hi : lo), v ^ ((a & 1) ? lo : hi)};
+  int f = 0;
+  for (int i = 0; i < 3; ++i) {
+    int smaller = 0;
+    for (int j = i + 1; j < 4; ++j) smaller += w[j] < w[i];
+    f = f * (4 - i) + smaller;
+  }
+  return f;
+}
+// (-1)^|k & z| of arrangement a; 0 and the same for every a at k = 0
+__host__ __device__ constexpr int s4_parity(int k, int a) {
+  const int x = 1 + (a >> 1), lo = x == 1 ? 2 : 1, hi = x == 3 ? 2 : 3, z = k & ((a & 1) ? lo : hi);
+  return (z ^ (z >> 1)) & 1;
+}
+template <typename T>
+ME_HD T s4_colour_sum(const T* coef, const cx<T>* J) {
+  cx<T> S[4][6];
+#pragma unroll
+  for (int a = 0; a < 6; ++a) {
+    const cx<T> p = J[s4_flow(0, a)] + J[s4_flow(1, a)], m = J[s4_flow(0, a)] - J[s4_flow(1, a)];
+    const cx<T> q = J[s4_flow(2, a)] + J[s4_flow(3, a)], r = J[s4_flow(2, a)] - J[s4_flow(3, a)];
+    S[0][a] = p + q;
+    S[1][a] = m + r;
+    S[2][a] = p - q;
+    S[3][a] = m - r;
+  }
+  T s = T(0);
+  int i = 0;
+#pragma unroll
+  for (int k = 0; k < 4; ++k)
+#pragma unroll
+    for (int a = 0; a < 6; ++a) {
+      cx<T> z{T(0), T(0)};
+#pragma unroll
+      for (int b = a; b < 6; ++b)
+        if (s4_parity(k, a) == s4_parity(k, b)) z = rmac(z, coef[i++], S[k][b]);
+      s += S[k][a].re * z.re + S[k][a].im * z.im;
+    }
+  return s;
+}
+// the coefficients from the 24 x 24 matrix C; false if C lacks the symmetry
+inline bool s4_coefficients(const double* C, double* coef) {
+  auto c = [&](int v, int a, int u, int b) { return C[s4_flow(v, a) * 24 + s4_flow(u, b)]; };
+  int i = 0;
+  for (int k = 0; k < 4; ++k)
+    for (int a = 0; a < 6; ++a)
+      for (int b = a; b < 6; ++b) {
+        double t = 0;
+        for (int u = 0; u < 4; ++u) {
+          for (int v = 0; v < 4; ++v)
+            if (std::abs(c(v, a, v ^ u, b) - c(0, a, u, b)) > 1e-12) return false;
+          const int q = k & u;
+          t += ((q ^ (q >> 1)) & 1) ? -c(0, a, u, b) : c(0, a, u, b);
+        }
+        if (s4_parity(k, a) == s4_parity(k, b)) coef[i++] = (a == b ? 0.25 : 0.5) * t;
+        else if (std::abs(t) > 1e-12) return false;
+      }
+  return i == S4_COEF;
 }
 
 // Helicity blocks of one member of each flipped pair (leg 0 at +): NHEL / 8 blocks;
