@@ -92,10 +92,10 @@ WORKLOADS = {
            "workload": "gg -> t tbar LO, sqrt(s_hat) ~ U[400,2000] GeV, 2^20 points, float32 amplitudes",
            "kernels": {"gg_tt": "k_tree<gg_tt, float>"}, "l2": "inputs 134 MB per batch > 129 MB L2 (no flush)"},
     "c3": {"calls": [("gg_ttgg", "born", 6)], "n": 1 << 18,
-           "metric": "gg -> t tbar g g tree events/s (tensor-core colour sum, 1 GB300)",
+           "metric": "gg -> t tbar g g tree events/s (1 GB300)",
            "workload": "gg -> t tbar g g tree at sqrt(s)=2 TeV, 2^18 flat massive-RAMBO points, float32 "
-                       "amplitudes, 24-flow colour sum on tensor cores (bf16 x3 split, f32 accumulate)",
-           "kernels": {"gg_ttgg": "k_tree_tc4 (gg_ttgg, float; four lanes per event, mma.sync bf16 colour sum)"},
+                       "amplitudes and 24-flow colour sum",
+           "kernels": {"gg_ttgg": "k_tree_tt4f (gg_ttgg, float; four lanes per event)"},
            "l2": "inputs 50 MB (< L2; compute-bound kernel)"},
 }
 
@@ -772,7 +772,7 @@ def main():
                          "float64 over the compacted list)")
     ap.add_argument("--workload", default="c2", choices=["c0", "c1", "c2", "c3"],
                     help="c2 (default): gg->ttg real-minus-CT; c0: e+e- NLO (n-body + real-minus-CT); "
-                         "c1: gg->tt LO; c3: gg->ttgg tree with the tensor-core colour sum")
+                         "c1: gg->tt LO; c3: gg->ttgg tree")
     args = ap.parse_args()
     if args.impl == "reference":
         run_reference(args)

@@ -30,7 +30,7 @@ static double bsum(const ColourTables& tab, const cx<T>* J) {
   if constexpr (PID == P_GG_TTGG) {
     T coef[S4_COEF];
     for (int i = 0; i < S4_COEF; ++i) coef[i] = (T)tab.S4[i];
-    return (double)s4_colour_sum(coef, J);
+    return (double)s4_colour_sum(coef, [&](int v, int a) { return J[s4_flow(v, a)]; });
   }
   return csum<PID, T>(tab, J);
 }

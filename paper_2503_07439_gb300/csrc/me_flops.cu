@@ -33,10 +33,10 @@ inline Flop msqrt(Flop a) { ++g_ops; return Flop(std::sqrt(a.v)); }  // found by
 
 using namespace me;
 
-// J^dagger C J per helicity as the kernels evaluate it (me_kernels.cuh: colour_sum): for up
-// to 6 flows the triangular form over the doubled upper triangle, 2 NF^2 + 4 NF flops;
-// beyond, the full matrix, 4 NF^2 + 4 NF
-static double colour_flops(int nf) { return nf <= 6 ? 2.0 * nf * nf + 4.0 * nf : 4.0 * nf * nf + 4.0 * nf; }
+// J^dagger C J per helicity as the kernels evaluate it (me_kernels.cuh: colour_sum): the
+// triangular form over the doubled upper triangle, 2 NF^2 + 4 NF flops; for 24 flows
+// s4_colour_sum, 96 additions and 2 S4_COEF + 48 multiply-adds
+static double colour_flops(int nf) { return nf == 24 ? 96.0 + 4.0 * S4_COEF + 96.0 : 2.0 * nf * nf + 4.0 * nf; }
 
 // one helicity block (me_procs.cuh): amplitudes of four helicities plus their colour sums
 template <int PID>

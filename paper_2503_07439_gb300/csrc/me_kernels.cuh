@@ -16,7 +16,6 @@
 #include <atomic>
 
 #include "me_procs.cuh"
-#include "me_tc.cuh"
 
 // minimum resident 128-thread blocks per SM requested from the register allocator: 2
 // gives the subtracted-real kernels up to 255 registers (8 warps per SM, fewer spills);
@@ -94,7 +93,8 @@ template <> __device__ __forceinline__ const float* utab<float>(const ColourTabl
 template <int PID, typename T>
 __device__ __forceinline__ T colour_sum(const ColourTables* tab, const cx<T>* J) {
   constexpr int NF = Proc<PID>::NFLOW;
-  if constexpr (PID == P_GG_TTGG) return s4_colour_sum(s4tab<T>(tab), J);
+  if constexpr (PID == P_GG_TTGG)
+    return s4_colour_sum(s4tab<T>(tab), [&](int v, int a) { return J[s4_flow(v, a)]; });
   T s = T(0);
   // triangular form: NF (NF + 1) + 2 NF multiply-adds instead of 2 NF^2 + 2 NF
   const T* __restrict__ Um = utab<T>(tab, PID);
@@ -195,12 +195,12 @@ __device__ __forceinline__ bool pass_cuts(const r4<double>* k, const Cuts& c) {
 // out[i] = wgt[i] * |M|^2(p_i) * nlo_factor.  `count` (optional): the number of events,
 // read on the device; `idx` (optional): the list of events to process (its length in
 // `count`).  Momenta have stride n either way.  (g g -> t tbar g g runs k_tree_tt4 and, in
-// float32, k_tree_tc4 below instead.)
+// float32, k_tree_tt4f below instead.)
 template <int PID, typename T, int LPE>
 __global__ void __launch_bounds__(128, ME_MINB) k_tree(const double* __restrict__ p, const double* __restrict__ wgt,
                                                        long n, double* __restrict__ out, KParams kp,
                                                        const int* __restrict__ idx, const int* __restrict__ count) {
-  static_assert(PID != P_GG_TTGG, "g g -> t tbar g g runs k_tree_tt4 and k_tree_tc4");
+  static_assert(PID != P_GG_TTGG, "g g -> t tbar g g runs k_tree_tt4 and k_tree_tt4f");
   constexpr int NEXT = Proc<PID>::NEXT;
   const long gid = ((long)blockIdx.x * blockDim.x + threadIdx.x) / LPE;
   const int lane = threadIdx.x % LPE;
@@ -277,63 +277,46 @@ __global__ void __launch_bounds__(256) k_tree_closed(const double* __restrict__ 
   out[ev] = pass ? (wgt ? wgt[ev] * tot : tot) : 0.0;
 }
 
-// ---------------------------------------------------------------- g g -> t tbar g g, float32, tensor cores
+// ---------------------------------------------------------------- g g -> t tbar g g, float32
 // Four lanes share one event and one helicity block at a time (me_procs.cuh: the gluon
-// helicities fixed, the four (t, tbar) helicities open):
-//  1. the 34 gluon four-vectors of the block -- polarisations e[4], ordered currents
-//     J(xy) (6, x < y), J(xyz) (12, one of each reversed pair), J(wxyz) (12, w < z) --
-//     are built cooperatively (a quarter each) into the event's shared-memory area;
-//  2. lane w extends the quark line for the six orderings that start with gluon w,
-//     U(w) -> U(wx) -> U(wxy), for both top helicities, and writes the partial
-//     amplitudes of both antitop helicities into shared-memory rows;
-//  3. one warp-wide tensor-core colour sum (me_tc.cuh) takes the warp's 32 rows
-//     (8 events x 4 heavy-pair helicities): lane 4e + h receives helicity h of event e.
-// Everything a lane needs stays on chip, so the 4e5 flops of an event run from registers
-// and shared memory; what bounds the kernel is instruction issue, so polarisations carry their
-// five nonzero reals, the quark spinors three components, products that serve two orderings
-// are formed once, and the momenta and denominators picked by lane sit in shared memory
-// instead of local memory (2^18 events: 4.32 -> 3.55 ms).  In a warp that holds the end of the batch, events past it compute
-// a fixed finite configuration and are discarded, so every warp-wide step stays
-// converged; warps entirely past the end return at once.
-// an event's shared-memory area: 34 four-vectors x 8 floats, the gluon momenta q[4] and the
-// reciprocal denominators ig[16], iq[16] (indexed by lane-dependent gluons, which in registers
-// would go through local memory), padded so that 8 events hit distinct banks
-constexpr int TC4_Q = 272, TC4_IG = 288, TC4_IQ = 304;
-constexpr int TC4_EV_FLOATS = 324;
-constexpr int TC4_ROW = 25;         // floats per amplitude row (24 flows, padded)
-constexpr int TC4_WARP_FLOATS = 8 * TC4_EV_FLOATS + 2 * 32 * TC4_ROW;
-constexpr int TC4_SMEM_PER_WARP = TC4_WARP_FLOATS * 4 + TC_SMEM_PER_WARP;
-constexpr int TC4_THREADS = 128;
-constexpr int TC4_SMEM = (TC4_THREADS / 32) * TC4_SMEM_PER_WARP;
+// helicities fixed, the four (t, tbar) helicities open).  Lane w works on what belongs to
+// gluon w, the other gluons counted as w ^ 1, w ^ 2, w ^ 3, so that every index into the
+// event's shared-memory area is an exclusive or:
+//  1. polarisation w; pair currents J(xy) in both orders; the three triples J(xyz) of the
+//     gluons other than w; the quadruples J(wxyz), x < y, to the ends z = w ^ 1 and w ^ 2,
+//     and to w ^ 3 from decoupling, J(wxyz) = -J(xwyz) - J(xywz) - J(xyzw);
+//  2. the quark line of the six orderings that start with w, U(w) -> U(wx) -> U(wxy), for
+//     both top helicities, the partial amplitudes of both antitop helicities going to
+//     shared-memory rows;
+//  3. the colour sum of heavy-pair helicity w.
+// Everything a lane needs stays on chip, so the 3e5 flops of an event run from registers
+// and shared memory; instruction issue bounds the kernel.  2^18 events: 4.42 ms with four lanes
+// that picked currents from tables and a bf16 x 3 mma colour sum, 2.40 ms like this.  In a warp that holds the end of the
+// batch, events past it compute a fixed finite configuration and are discarded, so every
+// warp-wide step stays converged; warps entirely past the end return at once.
+// An event's shared-memory area: 40 four-vectors x 8 floats, the gluon momenta q[4], the
+// reciprocal denominators ig[16], iq[16], padded so that 8 events hit distinct banks.
+constexpr int TT4_Q = 320, TT4_IG = 336, TT4_IQ = 352, TT4_EV = 372;
+constexpr int TT4_ROW = 52;  // floats per amplitude row (24 complex, padded)
+constexpr int TT4_WARP = 8 * TT4_EV + 32 * TT4_ROW;
+constexpr int TT4_THREADS = 128;
+constexpr int TT4_SMEM = (TT4_THREADS / 32) * TT4_WARP * 4;
+// slots: polarisations 0 .. 3; ordered pairs J(xy); triples by missing and middle gluon;
+// quadruples J(w..z) by first and last gluon, the two in between in increasing order
+__device__ __forceinline__ int tt4_pair(int x, int y) { return 4 + 3 * x + (x ^ y) - 1; }
+__device__ __forceinline__ int tt4_triple(int miss, int mid) { return 16 + 3 * miss + (miss ^ mid) - 1; }
+__device__ __forceinline__ int tt4_quad(int w, int z) { return 28 + 3 * w + (w ^ z) - 1; }
 
-// J(xyz) representatives, slot t = 3 * (missing gluon) + (position of the middle gluon
-// among the three in increasing order); packed x | y << 4 | z << 8, x < z
-__constant__ short kJ3Rep[12] = {0x312, 0x321, 0x231, 0x302, 0x320, 0x230,
-                                 0x301, 0x310, 0x130, 0x201, 0x210, 0x120};
-// J(wxyz) representatives (w < z), enumerated by w, then x, then y: packed w | x<<4 | y<<8 | z<<12
-__constant__ short kJ4Rep[12] = {0x3210, 0x2310, 0x3120, 0x1320, 0x2130, 0x1230,
-                                 0x3201, 0x2301, 0x3021, 0x2031, 0x3102, 0x3012};
-// ordering f (lexicographic) -> +-(1 + representative of J(wxyz)); minus: reversed, J = -J(rep)
-__constant__ signed char kJ4OfOrdering[24] = {1,  2,  3,   4,  5,  6,  7,   8,  9,  -6, 10, -4,
-                                              11, -10, 12, -5, -8, -2, -12, -9, -11, -3, -7, -1};
-
-__device__ __forceinline__ void st_c4(float* b, int slot, const c4<float>& v) {
+__device__ __forceinline__ void st8(float* b, int slot, cx<float> a, cx<float> c, cx<float> d, cx<float> e) {
   float4* p = reinterpret_cast<float4*>(b + 8 * slot);
-  p[0] = make_float4(v.v[0].re, v.v[0].im, v.v[1].re, v.v[1].im);
-  p[1] = make_float4(v.v[2].re, v.v[2].im, v.v[3].re, v.v[3].im);
+  p[0] = make_float4(a.re, a.im, c.re, c.im);
+  p[1] = make_float4(d.re, d.im, e.re, e.im);
 }
+__device__ __forceinline__ void st_c4(float* b, int slot, const c4<float>& v) { st8(b, slot, v.v[0], v.v[1], v.v[2], v.v[3]); }
 __device__ __forceinline__ c4<float> ld_c4(const float* b, int slot) {
   const float4* p = reinterpret_cast<const float4*>(b + 8 * slot);
   const float4 a = p[0], c = p[1];
   return c4<float>{{{a.x, a.y}, {a.z, a.w}, {c.x, c.y}, {c.z, c.w}}};
-}
-__device__ __forceinline__ int pair_slot(int x, int y) {  // x < y
-  return 4 + (x == 0 ? y - 1 : (x == 1 ? y + 1 : 5));
-}
-__device__ __forceinline__ c4<float> ld_j2(const float* b, int x, int y) {
-  c4<float> J = ld_c4(b, pair_slot(x < y ? x : y, x < y ? y : x));
-  if (x > y) cscale(J, -1.0f);
-  return J;
 }
 // slots 0 .. 3: a polarisation (no time component, real z)
 __device__ __forceinline__ pol<float> ld_pol(const float* b, int slot) {
@@ -342,7 +325,7 @@ __device__ __forceinline__ pol<float> ld_pol(const float* b, int slot) {
   return pol<float>{{a.z, a.w}, {c.x, c.y}, c.z};
 }
 __device__ __forceinline__ r4<float> ld_q(const float* b, int g) {
-  const float4 a = *reinterpret_cast<const float4*>(b + TC4_Q + 4 * g);
+  const float4 a = *reinterpret_cast<const float4*>(b + TT4_Q + 4 * g);
   return r4<float>{a.x, a.y, a.z, a.w};
 }
 // the same eight floats read as the chiral combinations (V0 - V3, V0 + V3, V1 - i V2,
@@ -357,38 +340,20 @@ __device__ __forceinline__ spol<float> ld_spol(const float* b, int slot) {
   const float4 a = p[0], c = p[1];
   return spol<float>{a.z, {c.x, c.y}, {c.z, c.w}};
 }
-__device__ __forceinline__ void slash_in_place(float* b, int slot) {
-  const sl4<float> S = slashed(ld_c4(b, slot));
-  float4* p = reinterpret_cast<float4*>(b + 8 * slot);
-  p[0] = make_float4(S.a.re, S.a.im, S.b.re, S.b.im);
-  p[1] = make_float4(S.c.re, S.c.im, S.d.re, S.d.im);
-}
-__device__ __forceinline__ sl4<float> ld_sj2(const float* b, int x, int y) {
-  sl4<float> S = ld_sl4(b, pair_slot(x < y ? x : y, x < y ? y : x));
-  if (x > y) S = sl4<float>{-S.a, -S.b, -S.c, -S.d};
-  return S;
-}
-__device__ __forceinline__ int triple_slot(int x, int y, int z) {  // any order: J(zyx) = J(xyz)
-  const int miss = 6 - x - y - z;
-  const int a = miss == 0 ? 1 : 0, c = miss == 3 ? 2 : 3;
-  return 10 + 3 * miss + (y == a ? 0 : (y == c ? 2 : 1));
-}
+__device__ __forceinline__ void st_sl4(float* b, int slot, const sl4<float>& S) { st8(b, slot, S.a, S.b, S.c, S.d); }
 
-template <int LPE>
-__global__ void __launch_bounds__(TC4_THREADS, 2) k_tree_tc4(const double* __restrict__ p, const double* __restrict__ wgt,
-                                                             long n, double* __restrict__ out, KParams kp,
-                                                             const int* __restrict__ idx, const int* __restrict__ count) {
-  static_assert(LPE == 4, "four lanes per event");
-  constexpr int PID = P_GG_TTGG;
-  extern __shared__ __align__(16) float tc4_smem[];
+template <int PID>
+__global__ void __launch_bounds__(TT4_THREADS, 2) k_tree_tt4f(const double* __restrict__ p, const double* __restrict__ wgt,
+                                                              long n, double* __restrict__ out, KParams kp,
+                                                              const int* __restrict__ idx, const int* __restrict__ count) {
+  static_assert(PID == P_GG_TTGG, "eight blocks");
+  extern __shared__ __align__(16) float tt4_smem[];
   const int warp = threadIdx.x >> 5, wl = threadIdx.x & 31;
-  float* wsm = tc4_smem + warp * (TC4_SMEM_PER_WARP / 4);
-  float* cur = wsm + (wl >> 2) * TC4_EV_FLOATS;         // this event's four-vectors
-  float* are = wsm + 8 * TC4_EV_FLOATS;                 // amplitude rows, real parts [32][TC4_ROW]
-  float* aim = are + 32 * TC4_ROW;                      // imaginary parts
-  unsigned char* stage = reinterpret_cast<unsigned char*>(wsm + TC4_WARP_FLOATS);
+  float* wsm = tt4_smem + warp * TT4_WARP;
+  float* cur = wsm + (wl >> 2) * TT4_EV;  // this event's area
+  float* rows = wsm + 8 * TT4_EV;         // amplitude rows [32][TT4_ROW]: 4 event + helicity
   const long gid = ((long)blockIdx.x * blockDim.x + threadIdx.x) / 4;
-  const int lane = threadIdx.x & 3;
+  const int w = threadIdx.x & 3;
   const long nev = count ? (long)*count : n;
   // a warp whose eight events all lie past the batch leaves together (every
   // synchronisation below is warp-wide), so a grid sized for a capacity costs little
@@ -404,149 +369,175 @@ __global__ void __launch_bounds__(TC4_THREADS, 2) k_tree_tc4(const double* __res
 #pragma unroll
     for (int l = 0; l < 6; ++l) k[l] = r4<double>{d[l][0], d[l][1], d[l][2], d[l][3]};
   }
-  const TcColourB cb = tc_load_colour(kp.tab->C[PID]);
   const Kin<PID, float> K = prepare<PID, float>(k, unit_couplings(kp.cp));
   const float mt = kp.cp.mtf;
   const r4<float> kt = K.pl[2];
   {
     // lane l writes momentum l and a quarter of the denominators
-    const r4<float> ql = lane == 0 ? K.q[0] : lane == 1 ? K.q[1] : lane == 2 ? K.q[2] : K.q[3];
-    *reinterpret_cast<float4*>(cur + TC4_Q + 4 * lane) = make_float4(ql.e, ql.x, ql.y, ql.z);
+    const r4<float> ql = w == 0 ? K.q[0] : w == 1 ? K.q[1] : w == 2 ? K.q[2] : K.q[3];
+    *reinterpret_cast<float4*>(cur + TT4_Q + 4 * w) = make_float4(ql.e, ql.x, ql.y, ql.z);
 #pragma unroll
     for (int S = 0; S < 16; ++S)
-      if ((S & 3) == lane) {
-        cur[TC4_IG + S] = K.ig[S];
-        cur[TC4_IQ + S] = K.iq[S];
+      if ((S & 3) == w) {
+        cur[TT4_IG + S] = K.ig[S];
+        cur[TT4_IQ + S] = K.iq[S];
       }
   }
-  const wf_v<float> wg = lane == 0 ? K.wg[0] : lane == 1 ? K.wg[1] : lane == 2 ? K.wg[2] : K.wg[3];
-  const int leg = lane < 2 ? lane : lane + 2;
+  const wf_v<float> wg = w == 0 ? K.wg[0] : w == 1 ? K.wg[1] : w == 2 ? K.wg[2] : K.wg[3];
+  const int leg = w < 2 ? w : w + 2;
   __syncwarp();
-  const float* ig = cur + TC4_IG;
-  const float* iq = cur + TC4_IQ;
+  const float* ig = cur + TT4_IG;
+  const float* iq = cur + TT4_IQ;
+  const float* coef = kp.tab->S4f;
   float acc = 0.0f;
+#pragma unroll 1
   for (int b = 0; b < n_live_blocks<PID>(); ++b) {
     const int hb = live_block_hel<PID>(b);
-    // 1. polarisation of gluon `lane`
     {
-      const pol<float> e = pol_of(wg, hel_of(hb, leg), lane >= 2);
-      st_c4(cur, lane, c4<float>{{{0.0f, 0.0f}, e.x, e.y, {e.z, 0.0f}}});
+      const pol<float> e = pol_of(wg, hel_of(hb, leg), w >= 2);
+      st_c4(cur, w, c4<float>{{{0.0f, 0.0f}, e.x, e.y, {e.z, 0.0f}}});
     }
     __syncwarp();
-    // 2. pair currents: slots 4 + lane and 8 + lane (< 10)
-    for (int pp = lane; pp < 6; pp += 4) {
-      const int x = pp < 3 ? 0 : (pp < 5 ? 1 : 2);
-      const int y = pp < 3 ? pp + 1 : (pp < 5 ? pp - 1 : 3);
+    // pairs (0, 1), (2, 3), (0, 2), (1, 3), then (0, 3), (1, 2)
+#pragma unroll
+    for (int r = 0; r < 2; ++r) {
+      if (r == 1 && w >= 2) break;
+      const int x = r == 0 ? (w < 2 ? 2 * w : w - 2) : w;
+      const int y = r == 0 ? (w < 2 ? x + 1 : w) : 3 - w;
       cx<float> exy;
-      st_c4(cur, 4 + pp, bracket(ld_pol(cur, x), ld_q(cur, x), ld_pol(cur, y), ld_q(cur, y), -ig[(1 << x) | (1 << y)], exy));
+      const c4<float> J = bracket(ld_pol(cur, x), ld_q(cur, x), ld_pol(cur, y), ld_q(cur, y), -ig[(1 << x) | (1 << y)], exy);
+      st_c4(cur, tt4_pair(x, y), J);
+      st_c4(cur, tt4_pair(y, x), cneg(J));
     }
     __syncwarp();
-    // 3. triple currents
-    for (int t = lane; t < 12; t += 4) {
-      const int r = kJ3Rep[t], x = r & 15, y = (r >> 4) & 15, z = r >> 8;
+    // triples of x, y, z = w ^ 1, w ^ 2, w ^ 3: each bracket of a gluon and a pair enters two of
+    // the three currents, and the three add up to zero
+    {
+      const int x = w ^ 1, y = w ^ 2, z = w ^ 3;
       const pol<float> ex = ld_pol(cur, x), ey = ld_pol(cur, y), ez = ld_pol(cur, z);
       const r4<float> qx = ld_q(cur, x), qy = ld_q(cur, y), qz = ld_q(cur, z);
-      const float w = ig[(1 << x) | (1 << y) | (1 << z)];
-      c4<float> J = czero<float>();
+      const float i3 = ig[15 ^ (1 << w)];
+      const cx<float> exy = i3 * cdot(ex, ey), eyz = i3 * cdot(ey, ez), exz = i3 * cdot(ex, ez);
+      c4<float> Jy = czero<float>(), Jx = czero<float>();
       {
-        const c4<float> P = ld_j2(cur, y, z);
-        bracket_acc(J, ex, qx, P, qy + qz, -w, cdot(ex, P));
+        const c4<float> P = ld_c4(cur, tt4_pair(y, z));
+        bracket_acc(Jy, ex, qx, P, qy + qz, -i3, cdot(ex, P));  // x (yz)
       }
       {
-        const c4<float> P = ld_j2(cur, x, y);
-        bracket_acc(J, ez, qz, P, qx + qy, w, cdot(ez, P));
+        const c4<float> P = ld_c4(cur, tt4_pair(x, z));
+        bracket_acc(Jx, ey, qy, P, qx + qz, -i3, cdot(ey, P));  // y (xz)
       }
-      quartic_acc(J, ex, ey, ez, w * cdot(ex, ez), w * cdot(ex, ey), w * cdot(ey, ez));
-      st_c4(cur, 10 + t, J);
+      {
+        const c4<float> P = ld_c4(cur, tt4_pair(x, y));
+        c4<float> Bz = czero<float>();
+        bracket_acc(Bz, ez, qz, P, qx + qy, -i3, cdot(ez, P));  // z (xy)
+        csub(Jy, Bz);
+        cadd(Jx, Bz);
+      }
+      quartic_acc(Jy, ex, ey, ez, exz, exy, eyz);  // J(xyz)
+      quartic_acc(Jx, ey, ex, ez, eyz, exy, exz);  // J(yxz)
+      st_c4(cur, tt4_triple(w, y), Jy);
+      st_c4(cur, tt4_triple(w, x), Jx);
+      cadd(Jx, Jy);
+      st_c4(cur, tt4_triple(w, z), cneg(Jx));
     }
     __syncwarp();
-    // 4. quadruple currents
-    for (int t = lane; t < 12; t += 4) {
-      const int r = kJ4Rep[t], w = r & 15, x = (r >> 4) & 15, y = (r >> 8) & 15, z = r >> 12;
-      const pol<float> ew = ld_pol(cur, w), ex = ld_pol(cur, x), ey = ld_pol(cur, y), ez = ld_pol(cur, z);
-      const c4<float> jwx = ld_j2(cur, w, x), jyz = ld_j2(cur, y, z);
-      const r4<float> qw = ld_q(cur, w), qz = ld_q(cur, z), qwx = qw + ld_q(cur, x), qyz = ld_q(cur, y) + qz;
-      const float i4 = ig[15];
+    // quadruples J(w x y z), z = w ^ 1, w ^ 2, slashed as they are stored
+    const pol<float> ew = ld_pol(cur, w);
+    const r4<float> qw = ld_q(cur, w);
+    const float i4 = ig[15];
+#pragma unroll
+    for (int pz = 1; pz < 3; ++pz) {
+      const int z = w ^ pz, o = w ^ (3 - pz), o3 = w ^ 3, x = min(o, o3), y = max(o, o3);
+      const pol<float> ex = ld_pol(cur, x), ey = ld_pol(cur, y), ez = ld_pol(cur, z);
+      const c4<float> jwx = ld_c4(cur, tt4_pair(w, x)), jyz = ld_c4(cur, tt4_pair(y, z));
+      const r4<float> qz = ld_q(cur, z), qwx = qw + ld_q(cur, x), qyz = ld_q(cur, y) + qz;
       c4<float> J = czero<float>();
       bracket_acc(J, jwx, qwx, jyz, qyz, -i4);
       quartic_acc(J, ew, ex, jyz, i4 * cdot(ew, jyz), i4 * cdot(ew, ex), i4 * cdot(ex, jyz));
       quartic_acc(J, jwx, ey, ez, i4 * cdot(ez, jwx), i4 * cdot(ey, jwx), i4 * cdot(ey, ez));
       {
-        const c4<float> jxy = ld_j2(cur, x, y);
+        const c4<float> jxy = ld_c4(cur, tt4_pair(x, y));
         quartic_acc(J, ew, jxy, ez, i4 * cdot(ew, ez), i4 * cdot(ew, jxy), i4 * cdot(ez, jxy));
       }
       {
-        const c4<float> P = ld_c4(cur, triple_slot(x, y, z));
+        const c4<float> P = ld_c4(cur, tt4_triple(w, y));
         bracket_acc(J, ew, qw, P, (qwx - qw) + qyz, -i4, cdot(ew, P));
       }
       {
-        const c4<float> P = ld_c4(cur, triple_slot(w, x, y));
+        const c4<float> P = ld_c4(cur, tt4_triple(z, x));
         bracket_acc(J, ez, qz, P, qwx + (qyz - qz), i4, cdot(ez, P));
       }
-      st_c4(cur, 22 + t, J);
+      st_sl4(cur, tt4_quad(w, z), slashed(J));
     }
     __syncwarp();
-    // the quark lines only slash the 34 vectors against rows: convert them in place
-    for (int sl = lane; sl < 34; sl += 4) slash_in_place(cur, sl);
+    // the quark lines only slash the other vectors too: convert them in place; and the
+    // quadruples to z = w ^ 3, x < y: J(xwyz) + J(xywz) = J(x..z) - J(z..x) of increasing middles
+#pragma unroll
+    for (int i = 0; i < 7; ++i) st_sl4(cur, 4 * i + w, slashed(ld_c4(cur, 4 * i + w)));
+    {
+      const int z = w ^ 3, x = min(w ^ 1, w ^ 2), y = max(w ^ 1, w ^ 2);
+      const sl4<float> A = ld_sl4(cur, tt4_quad(x, z)), B = ld_sl4(cur, tt4_quad(z, x));
+      const sl4<float> C = ld_sl4(cur, y < z ? tt4_quad(x, w) : tt4_quad(w, x));
+      const float s = y < z ? -1.0f : 1.0f;
+      auto f = [&](cx<float> a, cx<float> b, cx<float> c) { return rmac(b - a, s, c); };
+      st8(cur, tt4_quad(w, z), f(A.a, B.a, C.a), f(A.b, B.b, C.b), f(A.c, B.c, C.c), f(A.d, B.d, C.d));
+    }
     __syncwarp();
-    // 5. quark line for the orderings starting with gluon w = lane.  Products of U(w) and
-    // U(wx) with a pair or triple current serve an ordering and its reflection in the rest:
-    // J(yx) = -J(xy), J(zyx) = J(xyz).
-    const int w = lane;
-    const r4<float> ktw = kt + ld_q(cur, w);
-    // the other gluons in increasing order: every lane runs the same 3 x 2 iterations, and
-    // f counts the orderings w x y z as the ordering tables do
-    const int g0 = w == 0 ? 1 : 0, g1 = w <= 1 ? 2 : 1, g2 = w <= 2 ? 3 : 2;
+    // quark lines.  Products of U(w) and U(wx) with a pair or triple current serve an
+    // ordering and its reflection in the rest: J(yx) = -J(xy), J(zyx) = J(xyz).
+    const r4<float> ktw = kt + qw;
+#pragma unroll
     for (int ht = 0; ht < 2; ++ht) {
-      const int row0 = (wl & ~3) + 2 * ht;  // rows of (this event, ht, hv = 0 / 1)
+      float2* row = reinterpret_cast<float2*>(rows + ((wl & ~3) + 2 * ht) * TT4_ROW) + 6 * w;  // hv = 0; hv = 1 in the next
       const c4<float> U1 = row_prop(ubar_slash(K.wt, ht, ld_spol(cur, w)), scaled_prop(ktw, mt, -iq[1 << w]));
-      int f = 6 * w;
-#pragma unroll 1
-      for (int kx = 0; kx < 3; ++kx) {
-        const int x = kx == 0 ? g0 : kx == 1 ? g1 : g2;
-        const int ya = kx == 0 ? g1 : g0, yb = kx == 2 ? g1 : g2;
+      c4<float> P[3], Q[3];  // by the gluon left out of the pair, the middle of the triple
+#pragma unroll
+      for (int i = 0; i < 3; ++i) {
+        P[i] = row_slash(U1, ld_sl4(cur, tt4_pair(w ^ (i == 0 ? 2 : 1), w ^ (i == 2 ? 2 : 3))));
+        Q[i] = row_slash(U1, ld_sl4(cur, tt4_triple(w, w ^ (i + 1))));
+      }
+#pragma unroll
+      for (int px = 1; px < 4; ++px) {
+        const int x = w ^ px;
         const r4<float> kwx = ktw + ld_q(cur, x);
-        c4<float> r2 = ubar_slash(K.wt, ht, ld_sj2(cur, w, x));
+        c4<float> r2 = ubar_slash(K.wt, ht, ld_sl4(cur, tt4_pair(w, x)));
         row_slash_acc(r2, U1, ld_spol(cur, x));
         const c4<float> U2 = row_prop(r2, scaled_prop(kwx, mt, -iq[(1 << w) | (1 << x)]));
-        const c4<float> U2J = row_slash(U2, ld_sj2(cur, ya, yb));
+        const int pl = px == 1 ? 2 : 1, ph = px == 3 ? 2 : 3;
+        const c4<float> D = row_slash(U2, ld_sl4(cur, tt4_pair(w ^ pl, w ^ ph)));
 #pragma unroll
         for (int ky = 0; ky < 2; ++ky) {
-          const int y = ky ? yb : ya, z = ky ? ya : yb;
-          c4<float> r3 = ubar_slash(K.wt, ht, ld_sl4(cur, triple_slot(w, x, y)));
-          row_slash_acc(r3, U1, ld_sj2(cur, x, y));
+          const int py = ky ? ph : pl, pz = ky ? pl : ph, y = w ^ py, z = w ^ pz;
+          c4<float> r3 = px < py ? P[pz - 1] : cneg(P[pz - 1]);
+          ubar_slash_acc(r3, K.wt, ht, ld_sl4(cur, tt4_triple(z, x)));
           row_slash_acc(r3, U2, ld_spol(cur, y));
-          const c4<float> U3 = row_prop(
-              r3, scaled_prop(kwx + ld_q(cur, y), mt, -iq[(1 << w) | (1 << x) | (1 << y)]));
-          c4<float> R = U2J;
-          if (ky) R = cneg(R);
-          const int s4 = kJ4OfOrdering[f];
-          const sl4<float> S4 = ld_sl4(cur, 22 + (s4 > 0 ? s4 : -s4) - 1);
-          const float sg = s4 > 0 ? 1.0f : -1.0f;
-          ubar_slash_acc(R, K.wt, ht, sl4<float>{sg * S4.a, sg * S4.b, sg * S4.c, sg * S4.d});
-          row_slash_acc(R, U1, ld_sl4(cur, triple_slot(x, y, z)));
+          const c4<float> U3 = row_prop(r3, scaled_prop(kwx + ld_q(cur, y), mt, -iq[15 ^ (1 << z)]));
+          c4<float> R = Q[py - 1];
+          if (ky) csub(R, D);
+          else cadd(R, D);
+          const bool up = x < y;  // J(wxyz), or -J(zyxw)
+          ubar_slash_acc(R, scaled(K.wt, up ? 1.0f : -1.0f), ht, ld_sl4(cur, up ? tt4_quad(w, z) : tt4_quad(z, w)));
           row_slash_acc(R, U3, ld_spol(cur, z));
-#pragma unroll
-          for (int hv = 0; hv < 2; ++hv) {
-            const cx<float> a = dot_v(R, K.wtb, hv);
-            are[(row0 + hv) * TC4_ROW + f] = a.re;
-            aim[(row0 + hv) * TC4_ROW + f] = a.im;
-          }
-          ++f;
+          const cx<float> a0 = dot_v(R, K.wtb, 0), a1 = dot_v(R, K.wtb, 1);
+          const int a = 2 * (px - 1) + ky;
+          row[a] = make_float2(a0.re, a0.im);
+          row[TT4_ROW / 2 + a] = make_float2(a1.re, a1.im);
         }
       }
     }
     __syncwarp();
-    // 6. colour sum of row wl (this event, heavy-pair helicity lane) on the tensor cores
-    cx<float> J[TC_NF];
-#pragma unroll
-    for (int fl = 0; fl < TC_NF; ++fl) J[fl] = cx<float>{are[wl * TC4_ROW + fl], aim[wl * TC4_ROW + fl]};
-    const float sres = tc_colour_sum(J, cb, stage);
+    // colour sum of row wl: this event, heavy-pair helicity w
+    const float2* mine = reinterpret_cast<const float2*>(rows + wl * TT4_ROW);
+    const float sres = s4_colour_sum(coef, [&](int v, int a) {
+      const float2 z = mine[6 * v + a];
+      return cx<float>{z.x, z.y};
+    });
     if (active) acc += sres;
-    __syncwarp();
+    // the next block's writes to the rows come after its __syncwarp calls
   }
   const double tot = 2.0 * (double)group_sum<4>(acc, group_mask<4>());
-  if (active && lane == 0) {
+  if (active && w == 0) {
     const double w8 = wgt ? wgt[ev] : 1.0;
     bool pass = true;
     if (kp.cut.mask) {
@@ -1277,11 +1268,11 @@ cudaError_t launch_one(int kind, const LaunchArgs& a, cudaStream_t st) {
       int dev = 0;
       cudaGetDevice(&dev);
       if (dev < 64 && !attr_set[dev]) {
-        cudaFuncSetAttribute(k_tree_tc4<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, TC4_SMEM);
+        cudaFuncSetAttribute(k_tree_tt4f<PID>, cudaFuncAttributeMaxDynamicSharedMemorySize, TT4_SMEM);
         attr_set[dev] = true;
       }
-      const long tb = (total + TC4_THREADS - 1) / TC4_THREADS;
-      k_tree_tc4<4><<<(unsigned)tb, TC4_THREADS, TC4_SMEM, st>>>(a.p, a.wgt, a.n, a.out, a.kp, a.idx, a.count);
+      const long tb = (total + TT4_THREADS - 1) / TT4_THREADS;
+      k_tree_tt4f<PID><<<(unsigned)tb, TT4_THREADS, TT4_SMEM, st>>>(a.p, a.wgt, a.n, a.out, a.kp, a.idx, a.count);
     } else if constexpr (closed_tree<PID>()) {
       if constexpr (LPE != 1) return launch_one<PID, T, 1>(kind, a, st);
       else k_tree_closed<PID, T><<<(unsigned)((a.groups + 255) / 256), 256, 0, st>>>(a.p, a.wgt, a.n, a.out, a.kp, a.idx, a.count);

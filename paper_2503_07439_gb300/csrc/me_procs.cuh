@@ -1067,10 +1067,14 @@ ME_HD void amp_tt4_block(const KinTT<T, 4>& K, int hb, const Couplings& cp, F&& 
 // and the four with - to each other.  That leaves 21 + 3 (3 + 10) coefficients (off-diagonal
 // ones doubled) and 264 operations, where the triangle of the 24 x 24 matrix takes 648.
 constexpr int S4_COEF = 60;
+// gluon i = 0, 1, 2 of arrangement a
+__host__ __device__ constexpr int s4_at(int a, int i) {
+  const int x = 1 + (a >> 1), lo = x == 1 ? 2 : 1, hi = x == 3 ? 2 : 3;
+  return i == 0 ? x : (i == 1) == ((a & 1) == 0) ? lo : hi;
+}
 // flow number (lexicographic) of the ordering v, v ^ x, v ^ y, v ^ z of arrangement a
 __host__ __device__ constexpr int s4_flow(int v, int a) {
-  const int x = 1 + (a >> 1), lo = x == 1 ? 2 : 1, hi = x == 3 ? 2 : 3;
-  const int w[4] = {v, v ^ x, v ^ ((a & 1) ? hi : lo), v ^ ((a & 1) ? lo : hi)};
+  const int w[4] = {v, v ^ s4_at(a, 0), v ^ s4_at(a, 1), v ^ s4_at(a, 2)};
   int f = 0;
   for (int i = 0; i < 3; ++i) {
     int smaller = 0;
@@ -1079,18 +1083,19 @@ __host__ __device__ constexpr int s4_flow(int v, int a) {
   }
   return f;
 }
-// (-1)^|k & z| of arrangement a; 0 and the same for every a at k = 0
+// 0 if (-1)^|k & z| of arrangement a is +, 1 if -
 __host__ __device__ constexpr int s4_parity(int k, int a) {
-  const int x = 1 + (a >> 1), lo = x == 1 ? 2 : 1, hi = x == 3 ? 2 : 3, z = k & ((a & 1) ? lo : hi);
+  const int z = k & s4_at(a, 2);
   return (z ^ (z >> 1)) & 1;
 }
-template <typename T>
-ME_HD T s4_colour_sum(const T* coef, const cx<T>* J) {
+// J(v, a): the amplitude of the ordering v, v ^ x, v ^ y, v ^ z
+template <typename T, class A>
+ME_HD T s4_colour_sum(const T* coef, const A& J) {
   cx<T> S[4][6];
 #pragma unroll
   for (int a = 0; a < 6; ++a) {
-    const cx<T> p = J[s4_flow(0, a)] + J[s4_flow(1, a)], m = J[s4_flow(0, a)] - J[s4_flow(1, a)];
-    const cx<T> q = J[s4_flow(2, a)] + J[s4_flow(3, a)], r = J[s4_flow(2, a)] - J[s4_flow(3, a)];
+    const cx<T> j0 = J(0, a), j1 = J(1, a), j2 = J(2, a), j3 = J(3, a);
+    const cx<T> p = j0 + j1, m = j0 - j1, q = j2 + j3, r = j2 - j3;
     S[0][a] = p + q;
     S[1][a] = m + r;
     S[2][a] = p - q;
