@@ -888,7 +888,8 @@ struct FourGluons {
 
 // g g -> t tbar g g.  The ordered gluon currents are built once per block with the
 // reflection identities: 6 pairs J(xy), x < y; 12 triples J(xyz) (one of each
-// reversed pair); 12 quadruples J(wxyz) with w < z.  Per top spin, the quark line
+// reversed pair), for each left-out gluon from three brackets and J(xyz) + J(yxz) + J(xzy) = 0;
+// 6 quadruples J(0xyz), which give the others by sums.  Per top spin, the quark line
 // is extended ordering by ordering, U(w) -> U(wx) -> U(wxy), and the row of ordering
 // wxyz is ubar J(wxyz) + U(w) J(xyz) + U(wx) J(yz) + U(wxy) e_z; a product of U(w) or U(wx)
 // with a current serves the ordering that has it reversed too.  Orderings are
@@ -931,67 +932,67 @@ ME_HD void tt4_block(const KinTT<T, 4>& K, const G& e, const Couplings& cp, F&& 
     return 3 * miss + (y == a ? 0 : (y == c ? 2 : 1));
   };
 #pragma unroll
-  for (int x = 0; x < 4; ++x)
-#pragma unroll
-    for (int y = 0; y < 4; ++y)
-#pragma unroll
-      for (int z = x + 1; z < 4; ++z) {
-        if (y == x || y == z) continue;
-        const int S = (1 << x) | (1 << y) | (1 << z);
-        const T c3 = -g * K.ig[S], c4g = g * g * K.ig[S];
-        c4<T> J = czero<T>();
-        e.current(J, x, q[x], j2(y, z), q[y] + q[z], c3, ej(x, y, z));
-        e.current(J, z, q[z], j2(x, y), q[x] + q[y], -c3, ej(z, x, y));
-        e.add(J, T(2) * c4g * e2(x, z), y);
-        e.add(J, -c4g * e2(x, y), z);
-        e.add(J, -c4g * e2(y, z), x);
-        J3[tidx(x, y, z)] = J;
-      }
+  for (int w = 0; w < 4; ++w) {  // x < y < z: the gluons other than w
+    const int x = w == 0 ? 1 : 0, y = w <= 1 ? 2 : 1, z = w <= 2 ? 3 : 2;
+    const T c3 = -g * K.ig[15 ^ (1 << w)], c4g = g * g * K.ig[15 ^ (1 << w)];
+    const cx<T> exy = c4g * e2(x, y), eyz = c4g * e2(y, z), exz = c4g * e2(x, z);
+    c4<T> Jy = czero<T>(), Jx = czero<T>(), B = czero<T>();
+    e.current(Jy, x, q[x], J2[pidx(y, z)], q[y] + q[z], c3, ej(x, y, z));  // x (yz)
+    e.current(Jx, y, q[y], J2[pidx(x, z)], q[x] + q[z], c3, ej(y, x, z));  // y (xz)
+    e.current(B, z, q[z], J2[pidx(x, y)], q[x] + q[y], c3, ej(z, x, y));   // z (xy)
+    csub(Jy, B);
+    cadd(Jx, B);
+    e.add(Jy, T(2) * exz, y);
+    e.add(Jy, -exy, z);
+    e.add(Jy, -eyz, x);
+    e.add(Jx, T(2) * eyz, x);
+    e.add(Jx, -exy, z);
+    e.add(Jx, -exz, y);
+    J3[tidx(x, y, z)] = Jy;
+    J3[tidx(y, x, z)] = Jx;
+    cadd(Jx, Jy);
+    J3[tidx(x, z, y)] = cneg(Jx);
+  }
   auto j3 = [&](int x, int y, int z) { return J3[tidx(x, y, z)]; };
-  // quadruple currents J(wxyz) for w < z (J(zyxw) = -J(wxyz)); index by ordering rank
-  c4<T> J4[12];
-  int n4 = 0;
+  // quadruple currents J(0xyz)
+  c4<T> J4[6];
+  auto q0 = [](int x, int y) { return 2 * (x - 1) + (y > (x == 1 ? 2 : 1) ? 1 : 0); };
 #pragma unroll
-  for (int w = 0; w < 4; ++w)
+  for (int x = 1; x < 4; ++x)
 #pragma unroll
-    for (int x = 0; x < 4; ++x)
-#pragma unroll
-      for (int y = 0; y < 4; ++y) {
-        if (x == w || y == w || y == x) continue;
-        const int z = 6 - w - x - y;
-        if (z < w) continue;
-        const T c3 = -g * K.ig[15], c4g = g * g * K.ig[15];
-        const r4<T> qwx = q[w] + q[x], qyz = q[y] + q[z];
-        const c4<T> Jxyz = j3(x, y, z), Jwxy = j3(w, x, y), Jwx = j2(w, x), Jxy = j2(x, y), Jyz = j2(y, z);
-        c4<T> J = czero<T>();
-        e.current(J, w, q[w], Jxyz, q[x] + qyz, c3, e.dot(w, Jxyz));
-        bracket_acc(J, Jwx, qwx, Jyz, qyz, c3);
-        e.current(J, z, q[z], Jwxy, qwx + q[y], -c3, e.dot(z, Jwxy));
-        // 2 (L.R) M - (L.M) R - (M.R) L for (e_w, e_x, J_yz), (e_w, J_xy, e_z), (J_wx, e_y, e_z),
-        // collected by vector
-        e.add(J, c4g * (T(2) * ej(w, y, z)), x);
-        e.add(J, c4g * (T(2) * ej(z, w, x)), y);
-        e.add(J, -c4g * (ej(x, y, z) + ej(z, x, y)), w);
-        e.add(J, -c4g * (ej(w, x, y) + ej(y, w, x)), z);
-        caxpy(J, -c4g * e2(w, x), Jyz);
-        caxpy(J, T(2) * c4g * e2(w, z), Jxy);
-        caxpy(J, -c4g * e2(y, z), Jwx);
-        J4[n4++] = J;
-      }
-  // rank of the quadruple current of ordering wxyz among those with first < last
-  auto q4 = [](int w, int x, int y) {
-    // enumeration order above: w ascending, then x, then y, keeping z > w
-    int r = 0;
-    for (int a = 0; a < 4; ++a)
-      for (int b = 0; b < 4; ++b)
-        for (int c = 0; c < 4; ++c) {
-          if (b == a || c == a || c == b) continue;
-          const int d = 6 - a - b - c;
-          if (d < a) continue;
-          if (a == w && b == x && c == y) return r;
-          ++r;
-        }
-    return -1;
+    for (int y = 1; y < 4; ++y) {
+      if (y == x) continue;
+      const int w = 0, z = 6 - x - y;
+      const T c3 = -g * K.ig[15], c4g = g * g * K.ig[15];
+      const r4<T> qwx = q[w] + q[x], qyz = q[y] + q[z];
+      const c4<T> Jxyz = j3(x, y, z), Jwxy = j3(w, x, y), Jwx = j2(w, x), Jxy = j2(x, y), Jyz = j2(y, z);
+      c4<T> J = czero<T>();
+      e.current(J, w, q[w], Jxyz, q[x] + qyz, c3, e.dot(w, Jxyz));
+      bracket_acc(J, Jwx, qwx, Jyz, qyz, c3);
+      e.current(J, z, q[z], Jwxy, qwx + q[y], -c3, e.dot(z, Jwxy));
+      // 2 (L.R) M - (L.M) R - (M.R) L for (e_w, e_x, J_yz), (e_w, J_xy, e_z), (J_wx, e_y, e_z),
+      // collected by vector
+      e.add(J, c4g * (T(2) * ej(w, y, z)), x);
+      e.add(J, c4g * (T(2) * ej(z, w, x)), y);
+      e.add(J, -c4g * (ej(x, y, z) + ej(z, x, y)), w);
+      e.add(J, -c4g * (ej(w, x, y) + ej(y, w, x)), z);
+      caxpy(J, -c4g * e2(w, x), Jyz);
+      caxpy(J, T(2) * c4g * e2(w, z), Jxy);
+      caxpy(J, -c4g * e2(y, z), Jwx);
+      J4[q0(x, y)] = J;
+    }
+  // the others by reflection and decoupling: 0 second in x 0 y z, with J(x 0 y z) + J(0 x y z)
+  // + J(0 y x z) + J(0 y z x) = 0
+  auto quad = [&](int w, int x, int y) {
+    const int z = 6 - w - x - y;
+    if (w == 0) return J4[q0(x, y)];
+    if (z == 0) return cneg(J4[q0(y, x)]);
+    const bool second = x == 0;
+    const int a = second ? w : z, b = second ? y : x, c = second ? z : w;
+    c4<T> J = J4[q0(a, b)];
+    cadd(J, J4[q0(b, a)]);
+    cadd(J, J4[q0(b, c)]);
+    return second ? cneg(J) : J;
   };
   const r4<T> kt = K.pl[2];
 #pragma unroll 1
@@ -1031,7 +1032,7 @@ ME_HD void tt4_block(const KinTT<T, 4>& K, const G& e, const Couplings& cp, F&& 
           c4<T> R = Q[y];
           if (y < z) cadd(R, D);
           else csub(R, D);
-          ubar_slash_acc(R, K.wt, ht, slashed(z > w ? J4[q4(w, x, y)] : cneg(J4[q4(z, y, x)])));
+          ubar_slash_acc(R, K.wt, ht, slashed(quad(w, x, y)));
           e.row(R, U3, z);
 #pragma unroll
           for (int hv = 0; hv < 2; ++hv) A[hv][f] = dot_v(R, K.wtb, hv);
