@@ -291,7 +291,8 @@ __global__ void __launch_bounds__(256) k_tree_closed(const double* __restrict__ 
 //  3. the colour sum of heavy-pair helicity w.
 // Everything a lane needs stays on chip, so the 3e5 flops of an event run from registers
 // and shared memory; instruction issue bounds the kernel.  2^18 events: 4.42 ms with four lanes
-// that picked currents from tables and a bf16 x 3 mma colour sum, 2.40 ms like this.  In a warp that holds the end of the
+// that picked currents from tables and a bf16 x 3 mma colour sum, 2.15 ms like this; three
+// blocks per SM (168 registers) 2.47 ms.  In a warp that holds the end of the
 // batch, events past it compute a fixed finite configuration and are discarded, so every
 // warp-wide step stays converged; warps entirely past the end return at once.
 // An event's shared-memory area: 40 four-vectors x 8 floats, the gluon momenta q[4], the
@@ -388,7 +389,6 @@ __global__ void __launch_bounds__(TT4_THREADS, 2) k_tree_tt4f(const double* __re
   __syncwarp();
   const float* ig = cur + TT4_IG;
   const float* iq = cur + TT4_IQ;
-  const float* coef = kp.tab->S4f;
   float acc = 0.0f;
 #pragma unroll 1
   for (int b = 0; b < n_live_blocks<PID>(); ++b) {
@@ -489,6 +489,7 @@ __global__ void __launch_bounds__(TT4_THREADS, 2) k_tree_tt4f(const double* __re
     const r4<float> ktw = kt + qw;
 #pragma unroll
     for (int ht = 0; ht < 2; ++ht) {
+      asm volatile("" ::: "memory");  // currents are read again: held for both spins, or for all x, they spill
       float2* row = reinterpret_cast<float2*>(rows + ((wl & ~3) + 2 * ht) * TT4_ROW) + 6 * w;  // hv = 0; hv = 1 in the next
       const c4<float> U1 = row_prop(ubar_slash(K.wt, ht, ld_spol(cur, w)), scaled_prop(ktw, mt, -iq[1 << w]));
       c4<float> P[3], Q[3];  // by the gluon left out of the pair, the middle of the triple
@@ -500,6 +501,7 @@ __global__ void __launch_bounds__(TT4_THREADS, 2) k_tree_tt4f(const double* __re
 #pragma unroll
       for (int px = 1; px < 4; ++px) {
         const int x = w ^ px;
+        asm volatile("" ::: "memory");
         const r4<float> kwx = ktw + ld_q(cur, x);
         c4<float> r2 = ubar_slash(K.wt, ht, ld_sl4(cur, tt4_pair(w, x)));
         row_slash_acc(r2, U1, ld_spol(cur, x));
@@ -529,6 +531,8 @@ __global__ void __launch_bounds__(TT4_THREADS, 2) k_tree_tt4f(const double* __re
     __syncwarp();
     // colour sum of row wl: this event, heavy-pair helicity w
     const float2* mine = reinterpret_cast<const float2*>(rows + wl * TT4_ROW);
+    const float* coef = kp.tab->S4f;
+    asm volatile("" : "+l"(coef));  // 60 coefficients from L1 for each block, not from registers across blocks
     const float sres = s4_colour_sum(coef, [&](int v, int a) {
       const float2 z = mine[6 * v + a];
       return cx<float>{z.x, z.y};
