@@ -589,27 +589,40 @@ __global__ void __launch_bounds__(UW_THREADS) k_uw_decide(UwArgs a, UwResult* __
   }
 }
 
+// Each warp places the kept points of UW_ITEMS neighbouring words: the popcounts of the block's
+// words are scanned by every warp, and the weights of its words load before the first store.
+// The overweight test compares bits (a kept weight is no NaN), which stays off the float64 pipe.
 __global__ void __launch_bounds__(UW_THREADS) k_uw_write(UwArgs a, int* __restrict__ kept, double* __restrict__ kept_w) {
-  __shared__ unsigned words[UW_WORDS];
+  static_assert(UW_WORDS == 64 && UW_WORDS == UW_ITEMS * (UW_THREADS / 32), "two words per lane, UW_ITEMS per warp");
+  const int lane = threadIdx.x & 31, first = (threadIdx.x >> 5) * UW_ITEMS;
   const long w0 = (long)blockIdx.x * UW_WORDS, nw = (a.n + 31) / 32;
+  const unsigned lo = w0 + 2 * lane < nw ? a.bits[w0 + 2 * lane] : 0u;
+  const unsigned hi = w0 + 2 * lane + 1 < nw ? a.bits[w0 + 2 * lane + 1] : 0u;
+  const int own = __popc(lo) + __popc(hi);
+  int incl = own;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int y = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += y;
+  }
   const double wmax = uw_wmax(a);
-  if (threadIdx.x < UW_WORDS) words[threadIdx.x] = w0 + threadIdx.x < nw ? a.bits[w0 + threadIdx.x] : 0u;
-  __syncthreads();
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  int pos = a.counts[blockIdx.x];
-#pragma unroll 1
-  for (int k = 0; k < UW_WORDS; ++k) {
-    const unsigned m = words[k];
-    if (k % (UW_THREADS / 32) == warp && (m >> lane & 1u)) {
-      const long i = (w0 + k) * 32 + lane;
-      const int at = pos + __popc(m & ((1u << lane) - 1u));
-      kept[at] = (int)i;
-      if (kept_w) {
-        const double w = a.w[i];
-        kept_w[at] = fabs(w) > wmax ? w : copysign(wmax, w);
-      }
+  const unsigned long long mb = abs_bits(wmax);
+  int pos = a.counts[blockIdx.x] + __shfl_sync(0xffffffffu, incl - own, first / 2);
+  double w[UW_ITEMS];
+  unsigned m[UW_ITEMS];
+#pragma unroll
+  for (int k = 0; k < UW_ITEMS; ++k) {
+    m[k] = __shfl_sync(0xffffffffu, k & 1 ? hi : lo, (first + k) / 2);
+    w[k] = kept_w && (m[k] >> lane & 1u) ? a.w[(w0 + first + k) * 32 + lane] : 0.0;
+  }
+#pragma unroll
+  for (int k = 0; k < UW_ITEMS; ++k) {
+    if (m[k] >> lane & 1u) {
+      const int at = pos + __popc(m[k] & ((1u << lane) - 1u));
+      kept[at] = (int)((w0 + first + k) * 32 + lane);
+      if (kept_w) kept_w[at] = abs_bits(w[k]) > mb ? w[k] : copysign(wmax, w[k]);
     }
-    pos += __popc(m);
+    pos += __popc(m[k]);
   }
 }
 
