@@ -605,14 +605,20 @@ static cudaError_t launch_rescue(me_handle* h, const LaunchArgs& a, int lpe64) {
   return dispatch(h->proc->pid, K_REAL, true, lpe64, r, h->stream);
 }
 
-// Whether a subtracted-real call of n points runs the per-term queues.
+// Whether a subtracted-real call of n points runs the per-term queues.  The automatic choice
+// takes them where they are the faster path: from 2^19 points (flat 2^20: g g -> t tbar g 2.36
+// against 2.41 ms masked, with cuts 2.03 and 2.29; u ubar -> t tbar g 1.30 and 1.30, with cuts 1.27
+// and 1.33), except for e+e- -> u ubar g without cuts, whose amplitude costs less than queueing it
+// (2^20: 0.565 ms queued, 0.461 masked; with cuts 0.389 and 0.430).
 constexpr int64_t kTermsAutoMin = (int64_t)1 << 19;
+static Cuts cuts_of(int pid, const me_params* p);
 static bool use_terms(const me_handle* h, int64_t n) {
   const int t = h->prm.term_queues;
   // the automatic choice leaves the masked path's own rescue options (whole points, the
   // per-block queue) to the masked path
-  return t == ME_TERMS_QUEUED || (t == ME_TERMS_AUTO && h->prm.precision == ME_PREC_MIXED && n >= kTermsAutoMin &&
-                                  h->prm.queued_rescue == 0 && h->prm.rescue == ME_RESCUE_ITEMS);
+  return t == ME_TERMS_QUEUED ||
+         (t == ME_TERMS_AUTO && h->prm.precision == ME_PREC_MIXED && n >= kTermsAutoMin && h->prm.queued_rescue == 0 &&
+          h->prm.rescue == ME_RESCUE_ITEMS && (h->proc->pid != P_EE_UUG || cuts_of(h->proc->pid, &h->prm).mask));
 }
 
 // Per-term queues of the subtracted real: float64 pass, reals and recombination.
