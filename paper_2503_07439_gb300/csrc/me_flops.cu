@@ -120,6 +120,6 @@ int main() {
   // sector's Born
   std::printf(" \"term_config_per_event\": {\"ee_uug\": [%.0f, %.0f], \"gg_ttg\": [%.0f, %.0f], "
               "\"uu_ttg\": [%.0f, %.0f]},\n", b[0], b[0], soft_gg, coll_gg, soft_uu, coll_uu);
-  std::printf(" \"colour_sum_per_event\": {\"gg_ttgg\": %.0f}}\n", 32 * (4.0 * 24 * 24 + 4.0 * 24));
+  std::printf(" \"colour_sum_per_event\": {\"gg_ttgg\": %.0f}}\n", 32 * colour_flops(24));
   return 0;
 }

@@ -9,8 +9,10 @@
 // colour-summed squared amplitude (and every colour/spin-correlated one) unchanged for
 // these tree amplitudes with real couplings (pinned against the oracle).  A helicity
 // block (me_procs.cuh) is one configuration of the other legs with the four helicities
-// of the heavy pair, evaluated with shared gluon currents and quark-line rows.  Born, real, soft and collinear terms are evaluated for every point and
-// masked afterwards (Sec. 4.3, Algorithm 2), so a warp never diverges on cuts.
+// of the heavy pair, evaluated with shared gluon currents and quark-line rows; the 2 -> 2
+// trees and the counterterms' Borns are closed forms in float64.  Born, real, soft and
+// collinear terms are evaluated for every point and masked afterwards (Sec. 4.3, Algorithm 2),
+// so a warp never diverges on cuts, or through the per-term queues below.
 #pragma once
 #include <algorithm>
 #include <atomic>
@@ -225,7 +227,9 @@ __global__ void __launch_bounds__(128, ME_MINB) k_tree(const double* __restrict_
 
 // g g -> t tbar g g in float64: as k_tree, with the L = 2^lg lanes of an event in different warps
 // (half warps for L = 8), so that the beam gluons' helicities, which choose the form of a block,
-// are the same across a warp.  The float64 pipe bounds it.
+// are the same across a warp.  The float64 pipe bounds it (85 % at 8191 events, whose 2048 warps
+// fill the schedulers unevenly): 3.96 ms with general polarisations, every current and product
+// built on its own and the triangle of the colour matrix, 2.13 ms like this.
 template <int PID>
 __global__ void __launch_bounds__(128, ME_MINB) k_tree_tt4(const double* __restrict__ p, const double* __restrict__ wgt,
                                                            long n, double* __restrict__ out, KParams kp,
@@ -1020,20 +1024,51 @@ __global__ void __launch_bounds__(128, ME_MINB) k_real_sub(const double* __restr
 // Float64 evaluation of the listed blocks (grid-stride over the list, its length read on the
 // device).  The lane that delivers a record's last block recombines its W: the values are
 // published with a fence before the count, and read from L2 after it.
+// A list that leaves half the lanes idle takes the time of one block's serial float64 chain
+// (a warp's float64 instruction holds its scheduler's pipe for 64 cycles, however few lanes it
+// has): g g -> t tbar g then gives the two top spins of a block to lanes of different warps,
+// which repeat the currents (calls of 4099 points, 68 -> 50 us each with several in flight).  The
+// line is where both halves of every block still have lanes of their own; past it the repeated
+// work would cost a second round.  Both ways add the spins' sums in the same order.
 template <int PID>
 __global__ void __launch_bounds__(128, ME_MINB) k_rescue_items(const double* __restrict__ p,
                                                                const double* __restrict__ wgt, long n,
                                                                double* __restrict__ out, KParams kp,
                                                                const int* __restrict__ counts, ItemBufs ib) {
   constexpr int NEXT = Proc<PID>::NEXT, NB = RealLayout<PID>::NB;
+  __shared__ double part[64];
   const long stride = (long)gridDim.x * blockDim.x, front = counts[2], nit = front + counts[7];
-  for (long t = (long)blockIdx.x * blockDim.x + threadIdx.x; t < nit; t += stride) {
-    const int item = ib.list_r[t < front ? t : MAX_BLOCKS * ib.cap - 1 - (t - front)], slot = item >> 2, b = item & 3;
-    const int ev = ib.ev[slot];
-    r4<double> k[NEXT];
-    load_event<NEXT>(p, n, ev, k);
-    const Kin<PID, double> K = prepare<PID, double>(k, unit_couplings(kp.cp));
-    __stcg(ib.v + b * ib.cap + slot, real_block_value<PID, double>(K, b, kp));
+  const bool split = PID == P_GG_TTG && 2 * nit <= stride;  // the same in every block
+  const int half = split ? threadIdx.x >> 6 : 0, lane = split ? threadIdx.x & 63 : threadIdx.x;
+  for (long t = split ? (long)blockIdx.x * 64 + lane : (long)blockIdx.x * blockDim.x + lane;; t += stride) {
+    const bool live = t < nit;
+    if (!split && !live) break;
+    int slot = 0, b = 0, ev = 0;
+    double s[2] = {0.0, 0.0};
+    if (live) {
+      const int item = ib.list_r[t < front ? t : MAX_BLOCKS * ib.cap - 1 - (t - front)];
+      slot = item >> 2;
+      b = item & 3;
+      ev = ib.ev[slot];
+      r4<double> k[NEXT];
+      load_event<NEXT>(p, n, ev, k);
+      const Kin<PID, double> K = prepare<PID, double>(k, unit_couplings(kp.cp));
+      if constexpr (PID == P_GG_TTG) {
+        amplitude_block<PID, double>(
+            K, live_block_hel<PID>(b), unit_couplings(kp.cp),
+            [&](int r, const cx<double>* J) { s[r & 1] += colour_sum<PID, double>(kp.tab, J); },
+            split ? 1u << half : 3u);
+      } else {
+        s[0] = block_sum<PID, double>(K, b, kp);
+      }
+    }
+    if (split) {
+      if (half) part[lane] = s[1];
+      __syncthreads();
+      if (half || !live) return;
+      s[1] = part[lane];
+    }
+    __stcg(ib.v + b * ib.cap + slot, (s[0] + s[1]) * kp.real_scale);
     __threadfence();
     if (atomicSub(ib.pend + slot, 1) == 1) {
       __threadfence();
@@ -1042,6 +1077,7 @@ __global__ void __launch_bounds__(128, ME_MINB) k_rescue_items(const double* __r
       for (int i = 0; i < NB; ++i) R += __ldcg(ib.v + i * ib.cap + slot);
       out[ev] = (wgt ? wgt[ev] : 1.0) * (R + ib.wb[slot]);
     }
+    if (split) return;
   }
 }
 

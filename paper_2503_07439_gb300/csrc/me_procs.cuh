@@ -385,7 +385,8 @@ ME_HD void amp_tt3_fast(const KinTT<T, 3>& K, int hel, const Couplings& cp, cx<T
 // operations.  Five-real polarisations (pol), light-cone quark spins (wf_q), brackets of
 // conserved currents without their vanishing terms, products e.J computed once and each
 // gluon-pair bracket used by both currents it enters take a general g g -> t tbar g block from
-// 7349 to 4737 operations and a g g -> t tbar g g block from 66751 to 49460; beams on the z axis
+// 7349 to 4737 operations and a g g -> t tbar g g block from 66751 to 49460 (28044 with the products,
+// currents and colour sums shared as in tt4_block and s4_colour_sum); beams on the z axis
 // take the former to about 3300.  GB300: 2^20 subtracted g g -> t tbar g points 5.55 -> 2.20 ms,
 // 30011 in float64 1.385 -> 0.552 ms (counterterms and rescue included).
 
@@ -394,9 +395,10 @@ ME_HD void amp_tt3_fast(const KinTT<T, 3>& K, int hel, const Couplings& cp, cx<T
 // row R_s of ordering s collects ubar F(s), U(x) J(yz) and W(xy) e_z.
 // consume(r, A) receives the partial amplitudes of heavy spins r without the factor i g.
 // E0, E1: polarisations of the beam gluons, pol or axpol (on the axis the block takes about 1600
-// multiply-adds instead of 2500).
+// multiply-adds instead of 2500).  spins: the top spins evaluated, bit ht.
 template <typename T, class E0, class E1, class F>
-ME_HD void tt3_block(const KinTT<T, 3>& K, const E0& e0, const E1& e1, const pol<T>& e2, const Couplings& cp, F&& consume) {
+ME_HD void tt3_block(const KinTT<T, 3>& K, const E0& e0, const E1& e1, const pol<T>& e2, const Couplings& cp, unsigned spins,
+                     F&& consume) {
   constexpr bool PAIR = has_pair<E0, E1>::value;
   const T g = gs_of<T>(cp), mt = mt_of<T>(cp);
   const r4<T> k0 = K.q[0], k1 = K.q[1], k2 = K.q[2], kt = K.pl[2];
@@ -447,6 +449,7 @@ ME_HD void tt3_block(const KinTT<T, 3>& K, const E0& e0, const E1& e1, const pol
                  P12 = scaled_prop(kt + k12, mt, -g * K.iq[6]);
 #pragma unroll
   for (int ht = 0; ht < 2; ++ht) {
+    if (!(spins >> ht & 1u)) continue;
     c4<T> R[6];
     R[0] = ubar_slash(K.wt, ht, sF0);  // orderings 012, 021, 102, 120, 201, 210
     R[1] = ubar_slash(K.wt, ht, sF1);
@@ -506,17 +509,18 @@ ME_HD void tt3_block(const KinTT<T, 3>& K, const E0& e0, const E1& e1, const pol
 }
 
 template <typename T, class F>
-ME_HD void amp_tt3_block(const KinTT<T, 3>& K, int hb, const Couplings& cp, F&& consume) {
+ME_HD void amp_tt3_block(const KinTT<T, 3>& K, int hb, const Couplings& cp, unsigned spins, F&& consume) {
   const pol<T> e2 = pol_of(K.wg[2], hel_of(hb, 4), true);
   if (K.axis) {
     // leg 0 (helicity + in every block) is -(0, 1, i, 0) / sqrt 2, leg 1 the same for
     // helicity - and (0, 1, -i, 0) / sqrt 2 for +
     const T r2 = T(0.70710678118654752440);
     const axpol<T, 1> e0{-r2};
-    if (hel_of(hb, 1) < 0) tt3_block(K, e0, axpol<T, 1>{-r2}, e2, cp, consume);
-    else tt3_block(K, e0, axpol<T, -1>{r2}, e2, cp, consume);
+    if (hel_of(hb, 1) < 0) tt3_block(K, e0, axpol<T, 1>{-r2}, e2, cp, spins, consume);
+    else tt3_block(K, e0, axpol<T, -1>{r2}, e2, cp, spins, consume);
   } else {
-    tt3_block(K, pol_of(K.wg[0], hel_of(hb, 0), false), pol_of(K.wg[1], hel_of(hb, 1), false), e2, cp, consume);
+    tt3_block(K, pol_of(K.wg[0], hel_of(hb, 0), false), pol_of(K.wg[1], hel_of(hb, 1), false), e2, cp, spins,
+              consume);
   }
 }
 
@@ -1154,12 +1158,13 @@ template <int PID> __host__ __device__ constexpr int n_live_blocks() {
 }
 template <int PID> ME_HD int live_block_hel(int i) { return block_hel(massless_initial_pair<PID>() ? 2 * i : i); }
 
-// partial amplitudes of the four helicities hb | (r << 2) (see amp_tt2_block); processes
+// partial amplitudes of the four helicities hb | (r << 2) (see amp_tt2_block), of g g -> t tbar g
+// those whose top spin r & 1 is among `spins`; processes
 // without a block routine evaluate them one at a time
 template <int PID, typename T, class F>
-ME_HD void amplitude_block(const Kin<PID, T>& K, int hb, const Couplings& cp, F&& consume) {
+ME_HD void amplitude_block(const Kin<PID, T>& K, int hb, const Couplings& cp, F&& consume, unsigned spins = 3u) {
   if constexpr (PID == P_GG_TTG) {
-    amp_tt3_block<T>(K, hb, cp, consume);
+    amp_tt3_block<T>(K, hb, cp, spins, consume);
   } else if constexpr (PID == P_GG_TTGG) {
     amp_tt4_block<T>(K, hb, cp, consume);
   } else if constexpr (PID == P_UU_TTG) {
