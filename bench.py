@@ -39,8 +39,8 @@ METRIC = "NLO real-minus-counterterm events/s (gg->ttg, FKS, 1 GB300)"
 UNIT = "events/s"
 CUT_PT_MIN, CUT_ABS_Y_MAX = 100.0, 1.0  # heavy-quark cuts of the per-term queue comparison
 WORKLOAD = ("gg->ttg real-emission minus FKS soft/collinear counterterms, sqrt(s)=1 TeV, m_t=173, "
-            "2^20 flat massive-RAMBO points, mixed precision (fp32 amplitudes; fp64 re-evaluation of the "
-            "flagged points' real-emission blocks and counterterm Borns that their tolerance needs)")
+            "2^20 flat massive-RAMBO points, mixed precision (fp32 real emission; fp64 counterterms and "
+            "re-evaluation of the flagged points' real-emission blocks that their tolerance needs)")
 SM_COUNT, FP32_LANES, SM_MAX_MHZ = 152, 128, 2070.0
 NB_REAL = {"gg_ttg": 4, "uu_ttg": 2, "ee_uug": 2}  # live helicity blocks of the real emission
 FP64_PER_SM_CLK = 2  # DFMA thread-ops per SM per clock (ncu: ..._op_dfma_pred_on.avg.peak_sustained)
@@ -85,12 +85,12 @@ WORKLOADS = {
            "metric": "e+e- -> u ubar NLO events/s (n-body + real-minus-counterterm, 1 GB300)",
            "workload": "e+e- -> u ubar (g) at sqrt(s)=100 GeV: 65536 Born points (n-body NLO weight) + 65536 "
                        "real points (FKS final-state sectors), mixed precision",
-           "kernels": {"ee_uu": "k_tree<ee_uu, float>", "ee_uug": "k_real_sub<ee_uug, float>"},
+           "kernels": {"ee_uu": "k_tree_closed<ee_uu, float>", "ee_uug": "k_real_sub<ee_uug, float>"},
            "l2": "inputs 15 MB (< L2; compute-bound kernels)"},
     "c1": {"calls": [("gg_tt", "born", 3)], "n": N_POINTS,
            "metric": "gg -> t tbar LO events/s (1 GB300)",
            "workload": "gg -> t tbar LO, sqrt(s_hat) ~ U[400,2000] GeV, 2^20 points, float32 amplitudes",
-           "kernels": {"gg_tt": "k_tree<gg_tt, float>"}, "l2": "inputs 134 MB per batch > 129 MB L2 (no flush)"},
+           "kernels": {"gg_tt": "k_tree_closed<gg_tt, float>"}, "l2": "inputs 134 MB per batch > 129 MB L2 (no flush)"},
     "c3": {"calls": [("gg_ttgg", "born", 6)], "n": 1 << 18,
            "metric": "gg -> t tbar g g tree events/s (1 GB300)",
            "workload": "gg -> t tbar g g tree at sqrt(s)=2 TeV, 2^18 flat massive-RAMBO points, float32 "
@@ -446,45 +446,26 @@ def _stage_roofline(ops, calls, stages, n, workload, queued=False):
         per = max(1, ncalls)
         flops = ops["real_subtracted_per_event" if entry == "real_subtracted" else "born_per_event"][proc]
         kname = WORKLOADS[workload]["kernels"][proc]
-        if entry == "real_subtracted" and (cfg[0] or cfg[1]) and t_resc > 0:
-            # per-term queues (the default for large mixed-precision batches): the float64
-            # rescue queues hold real blocks and Born configurations of two kinds
-            real = ops["born_per_event"][proc]
-            per_block = real / NB_REAL[proc]
-            c_soft, c_coll = ops["term_config_per_event"][proc]
-            item_flops = work[1] * per_block + cfg[0] * c_soft + cfg[1] * c_coll
-            cands.append({"bound": "alu", "achieved": item_flops / (t_resc / per * 1e-3) / 1e12, "peak": peak64,
-                          "unit": "TFLOP/s", "traffic": traffic_per_launch(workload, "term_items", resc_pts),
-                          "kernel": f"k_term_items<{proc}, double> + k_terms_final (float64 rescue queues of "
-                                    "the per-term path: real-emission helicity blocks and counterterm Born "
-                                    "configurations of the flagged points)",
-                          "peak_note": note64, "flops_per_block": per_block,
-                          "flops_per_config": [c_soft, c_coll], "points": resc_pts, "real_blocks": work[1],
-                          "born_configs": list(cfg), "ms_per_launch": t_resc / per})
-            cands.append({"bound": "alu", "achieved": flops * n / (t_main / per * 1e-3) / 1e12 if t_main else 0.0,
-                          "peak": peak32, "unit": "TFLOP/s", "traffic": None,
-                          "kernel": f"k_terms<{proc}> + k_term_items<{proc}, float> + k_terms_combine (float64 "
-                                    "maps and queues, bulk amplitudes, recombination)",
-                          "peak_note": note32, "flops_per_event": flops, "points_per_launch": n,
-                          "ms_per_launch": t_main / per,
-                          "note": "flops counted as for the masked evaluation (every Born set); the queues "
-                                  "evaluate only the active ones"})
-            continue
-        if entry == "real_subtracted" and (work[1] or work[2]) and t_resc > 0:
-            # item rescue: the float64 work is the real's helicity blocks and the counterterm
-            # Born sets actually re-evaluated (op counts: real = born_per_event[proc] over
-            # its live blocks; Born set = the rest of the subtracted real)
-            real = ops["born_per_event"][proc]
-            per_block = real / NB_REAL[proc]
-            born_set = flops - real
-            item_flops = work[1] * per_block + work[2] * born_set
-            cands.append({"bound": "alu", "achieved": item_flops / (t_resc / per * 1e-3) / 1e12, "peak": peak64,
-                          "unit": "TFLOP/s", "traffic": traffic_per_launch(workload, "items", resc_pts),
-                          "kernel": f"k_rescue_items<{proc}> + k_rescue_combine (float64 items of the flagged "
-                                    "points: real-emission helicity blocks and counterterm Born sets)",
-                          "peak_note": note64, "flops_per_block": per_block, "flops_per_born_set": born_set,
-                          "points": resc_pts, "real_blocks": work[1], "born_sets": work[2],
-                          "ms_per_launch": t_resc / per})
+        if entry == "real_subtracted" and work[1] and t_resc > 0:
+            # item rescue: the float64 work is the real's helicity blocks re-evaluated (the
+            # counterterms' Borns are float64 at every point of the main stage)
+            terms = bool(cfg[0] or cfg[1])  # per-term queues, the default for large mixed-precision batches
+            per_block = ops["born_per_event"][proc] / NB_REAL[proc]
+            cands.append({"bound": "alu", "achieved": work[1] * per_block / (t_resc / per * 1e-3) / 1e12,
+                          "peak": peak64, "unit": "TFLOP/s", "traffic": traffic_per_launch(workload, "items", resc_pts),
+                          "kernel": f"k_rescue_items<{proc}> (float64 helicity blocks of the flagged points and "
+                                    "their recombination)",
+                          "peak_note": note64, "flops_per_block": per_block, "points": resc_pts,
+                          "real_blocks": work[1], "ms_per_launch": t_resc / per})
+            if terms:
+                cands.append({"bound": "alu", "achieved": flops * n / (t_main / per * 1e-3) / 1e12 if t_main else 0.0,
+                              "peak": peak32, "unit": "TFLOP/s", "traffic": None,
+                              "kernel": f"k_terms<{proc}> + k_term_reals<{proc}, float> (float64 maps, Borns and "
+                                        "queues; bulk amplitudes, recombination)",
+                              "peak_note": note32, "flops_per_event": flops, "points_per_launch": n,
+                              "ms_per_launch": t_main / per,
+                              "note": "amplitude flops only; the first kernel's float64 maps are not counted"})
+                continue
             resc_pts = 0  # accounted for above
         if queued and entry == "real_subtracted" and resc_pts > 0:
             cands.append({"bound": "alu", "achieved": flops * resc_pts / (t_main / per * 1e-3) / 1e12,
@@ -716,15 +697,13 @@ def measure(me, mebuild, workload, args, n, rank, world, local, dist, full):
     link = _link_rate(hosts[0][1], torch)
     ops = mebuild.op_counts()
     roofline, other = _stage_roofline(ops, calls, stages, n, workload, queued=args.queued_rescue)
-    # per call: the main kernel, the float64 work of the two-launch subtracted real (item
-    # rescue: items + recombination; whole points: one launch) and the two reduction kernels
-    # per-term queues (mixed precision): k_terms, the reals' and the Born configurations'
-    # float32 items, k_terms_combine, the float64 items, k_terms_final
+    # per call: the main kernel, the subtracted real's float64 launch (items with their
+    # recombination, or whole points) and the reduction
+    # per-term queues (mixed precision): k_terms, k_term_reals, k_rescue_items, the reduction
     def call_launches(entry, st):
         if entry == "real_subtracted" and (st[6][0] or st[6][1]):
-            return 6 + 2
-        return 1 + ((2 if st[5][1] or st[5][2] else 1) if entry == "real_subtracted" and
-                    not args.queued_rescue else 0) + 2
+            return 3 + 1
+        return 1 + (1 if entry == "real_subtracted" and not args.queued_rescue else 0) + 1
     launches_per_step = sum(call_launches(entry, st) for (_, entry, _), st in zip(calls, stages))
     return {
         "metric": wl["metric"], "value": value, "unit": UNIT, "ms_per_step": ms / args.steps, "steps": args.steps,
