@@ -44,19 +44,15 @@ WORKLOAD = ("gg->ttg real-emission minus FKS soft/collinear counterterms, sqrt(s
 SM_COUNT, FP32_LANES, SM_MAX_MHZ = 152, 128, 2070.0
 NB_REAL = {"gg_ttg": 4, "uu_ttg": 2, "ee_uug": 2}  # live helicity blocks of the real emission
 FP64_PER_SM_CLK = 2  # DFMA thread-ops per SM per clock (ncu: ..._op_dfma_pred_on.avg.peak_sustained)
-# DRAM bytes per launch (dram__bytes_read.sum + dram__bytes_write.sum) from one ncu --set full
+# DRAM bytes per launch (dram__bytes_read.sum + dram__bytes_write.sum) from one ncu
 # capture of each kernel (summaries in profiles/), with the hash of the kernel sources they
 # were taken on; reported only while the sources still hash the same.
-KERNEL_SOURCES_SHA = "160a62aeb5ea1b7f"
+KERNEL_SOURCES_SHA = "9b0f5d272d7d44b3"
 TRAFFIC = {
     # DRAM bytes per launch from one ncu capture of each kernel (the profile named), and the
     # points of that launch; traffic_per_launch scales them to the launch measured
-    ("c2", "term_items"): {"bytes": 0.401756e9 + 0.498245e9, "points": 172941,
-                           "profile": "profiles/k_term_items_double_gg_ttg_2p20.md"},
-    ("c1", "main"): {"bytes": 4489728 + 0, "points": 32768,
-                     "profile": "profiles/k_tree_gg_tt_float_2p20.md"},
-    ("c3", "main"): {"bytes": 6718208 + 2575872, "points": 32768,
-                     "profile": "profiles/k_tree_gg_ttgg_float_tc_2p18.md"},
+    ("c1", "main"): {"bytes": 100676096 + 3108608, "points": 1 << 20, "profile": "profiles/cases_ncu.md"},
+    ("c3", "main"): {"bytes": 52536832 + 835584, "points": 1 << 18, "profile": "profiles/cases_ncu.md"},
 }
 
 

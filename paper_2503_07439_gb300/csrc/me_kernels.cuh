@@ -1027,7 +1027,7 @@ __global__ void __launch_bounds__(128, ME_MINB) k_real_sub(const double* __restr
 // A list that leaves half the lanes idle takes the time of one block's serial float64 chain
 // (a warp's float64 instruction holds its scheduler's pipe for 64 cycles, however few lanes it
 // has): g g -> t tbar g then gives the two top spins of a block to lanes of different warps,
-// which repeat the currents (calls of 4099 points, 68 -> 50 us each with several in flight).  The
+// which repeat the currents (calls of 4099 points, 68 -> 53 us each with several in flight).  The
 // line is where both halves of every block still have lanes of their own; past it the repeated
 // work would cost a second round.  Both ways add the spins' sums in the same order.
 template <int PID>

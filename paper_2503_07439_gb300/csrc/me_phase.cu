@@ -427,7 +427,7 @@ __global__ void __launch_bounds__(FKS_THREADS) k_fks_points(uint64_t seed, uint3
 // u) of each other, or not ordinary numbers: the same decisions.  The
 // workspace stays with the handle (allocating and freeing it from the pool took most of a
 // call).  2^20 weights against their maximum, the events filled in by the caller: 365 us
-// before, 100 us.
+// before, 105 us.
 constexpr int UW_THREADS = 256;
 constexpr int UW_ITEMS = 8;                       // points per thread
 constexpr int UW_TILE = UW_THREADS * UW_ITEMS;    // points per block
