@@ -47,7 +47,7 @@ FP64_PER_SM_CLK = 2  # DFMA thread-ops per SM per clock (ncu: ..._op_dfma_pred_o
 # DRAM bytes per launch (dram__bytes_read.sum + dram__bytes_write.sum) from one ncu
 # capture of each kernel (summaries in profiles/), with the hash of the kernel sources they
 # were taken on; reported only while the sources still hash the same.
-KERNEL_SOURCES_SHA = "9b0f5d272d7d44b3"
+KERNEL_SOURCES_SHA = "ed3b884972d024c9"
 TRAFFIC = {
     # DRAM bytes per launch from one ncu capture of each kernel (the profile named), and the
     # points of that launch; traffic_per_launch scales them to the launch measured

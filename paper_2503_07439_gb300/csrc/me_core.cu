@@ -340,7 +340,6 @@ static int build_tables(ColourTables& tab) {
         const cd c = inner(B[x], B[y]);
         if (std::abs(c.imag()) > 1e-12) return fail(ME_ERR_PROCESS, "complex colour matrix");
         tab.C[it.pid][x * nf + y] = c.real();
-        tab.Cf[it.pid][x * nf + y] = (float)c.real();
       }
     }
     for (int x = 0; x < nf; ++x)

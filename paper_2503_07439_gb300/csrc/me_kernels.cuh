@@ -32,14 +32,13 @@ constexpr int MAX_FLOW = 24;
 constexpr int N_PAIRS = 10;  // unordered pairs (k<=l) of the 4 coloured legs of a 2->2 Born
 
 // Device-resident process constants (written once per device at set-up):
-// colour matrices (row-major NFLOW x NFLOW, in double and float) and the 2->2 Born
+// colour matrices (row-major NFLOW x NFLOW) and the 2->2 Born
 // colour correlators C^{kl} (pair order (0,0),(0,1),..,(3,3); [0] gg->tt, [1] uu->tt).
 // U holds the upper triangle of the symmetric C with the off-diagonal entries doubled
 // (U_aa = C_aa, U_ab = 2 C_ab for b > a, zero below), so that
 // J^dagger C J = sum_a Re(J_a^* sum_{b >= a} U_ab J_b).
 struct ColourTables {
   double C[P_COUNT][MAX_FLOW * MAX_FLOW];
-  float Cf[P_COUNT][MAX_FLOW * MAX_FLOW];
   double U[P_COUNT][MAX_FLOW * MAX_FLOW];
   float Uf[P_COUNT][MAX_FLOW * MAX_FLOW];
   double Ccorr[2][N_PAIRS][4];
@@ -82,9 +81,6 @@ struct KParams {
   const ColourTables* tab;
 };
 
-template <typename T> __device__ __forceinline__ const T* ctab(const ColourTables* t, int pid);
-template <> __device__ __forceinline__ const double* ctab<double>(const ColourTables* t, int pid) { return t->C[pid]; }
-template <> __device__ __forceinline__ const float* ctab<float>(const ColourTables* t, int pid) { return t->Cf[pid]; }
 template <typename T> __device__ __forceinline__ const T* s4tab(const ColourTables* t);
 template <> __device__ __forceinline__ const double* s4tab<double>(const ColourTables* t) { return t->S4; }
 template <> __device__ __forceinline__ const float* s4tab<float>(const ColourTables* t) { return t->S4f; }

@@ -229,56 +229,7 @@ ME_HD c4<T> polvec(const r4<T>& k, int lam, bool outgoing) {
 }
 
 // Helicity-independent ingredients of the wavefunctions, computed once per event and
-// shared by all helicities (the same operations, in the same order, as the routines above).
-// Fermion: omega_+, omega_- and the two-spinor chi_+ = (a, bx + i by), chi_- = (-bx + i by, a).
-template <typename T>
-struct wf_f {
-  T wp, wm, a, bx, by;
-};
-template <typename T>
-ME_HD wf_f<T> wf_fermion(const r4<T>& p, T m) {
-  wf_f<T> w;
-  omegas(p, m, w.wp, w.wm);
-  T pt2 = p.x * p.x + p.y * p.y;
-  T pa = msqrt(pt2 + p.z * p.z);
-  T s = (p.z >= T(0)) ? pa + p.z : pt2 / (pa - p.z);
-  if (s > T(0)) {
-    T rden = T(1) / msqrt(T(2) * pa * s);
-    w.a = s * rden;
-    w.bx = p.x * rden;
-    w.by = p.y * rden;
-  } else {  // exactly along -z
-    w.a = T(0);
-    w.bx = T(1);
-    w.by = T(0);
-  }
-  return w;
-}
-template <typename T>
-ME_HD void chi_of(const wf_f<T>& w, int lam, cx<T>& c0, cx<T>& c1) {
-  if (lam > 0) {
-    c0 = cx<T>{w.a, T(0)};
-    c1 = cx<T>{w.bx, w.by};
-  } else {
-    c0 = cx<T>{-w.bx, w.by};
-    c1 = cx<T>{w.a, T(0)};
-  }
-}
-template <typename T>
-ME_HD c4<T> spinor_u_of(const wf_f<T>& w, int lam) {
-  cx<T> a, b;
-  chi_of(w, lam, a, b);
-  T top = lam > 0 ? w.wm : w.wp, bot = lam > 0 ? w.wp : w.wm;
-  return c4<T>{{top * a, top * b, bot * a, bot * b}};
-}
-template <typename T>
-ME_HD c4<T> spinor_v_of(const wf_f<T>& w, int lam) {
-  cx<T> a, b;
-  chi_of(w, -lam, a, b);
-  T top = lam > 0 ? -w.wp : w.wm;
-  T bot = lam > 0 ? w.wm : -w.wp;
-  return c4<T>{{top * a, top * b, bot * a, bot * b}};
-}
+// shared by all helicities.
 // Massive quark with spins along the light cone instead of the helicity axis (a sum over
 // both spins does not depend on the axis): of the four components one is zero and two are
 // real, with p+ = E + pz, s = sqrt(p+), m' = m / s, t = (px + i py) / s,
@@ -322,20 +273,6 @@ ME_HD wf_v<T> wf_vector(const r4<T>& k) {
   if (!(pt2 > T(0))) return wf_v<T>{ct, T(0), T(0), T(0), r2};
   const T ipt = mrsqrt(pt2), cp = k.x * ipt, sp = k.y * ipt;
   return wf_v<T>{ct * cp, ct * sp, pt2 * ipt * ika * r2, sp * r2, cp * r2};
-}
-template <typename T>
-ME_HD c4<T> polvec_of(const wf_v<T>& w, int lam, bool outgoing) {
-  // eps = (-lam e1 - i e2)/sqrt(2), as polvec
-  c4<T> e;
-  e.v[0] = cx<T>{T(0), T(0)};
-  e.v[1] = cx<T>{lam > 0 ? -w.ccp : w.ccp, w.sp};
-  e.v[2] = cx<T>{lam > 0 ? -w.csp : w.csp, -w.cp};
-  e.v[3] = cx<T>{lam > 0 ? w.st : -w.st, T(0)};
-  if (outgoing) {
-#pragma unroll
-    for (int i = 1; i < 4; ++i) e.v[i] = conj(e.v[i]);
-  }
-  return e;
 }
 
 // ---------------------------------------------------------------- Dirac algebra
@@ -469,7 +406,7 @@ struct pol {
   T z;
 };
 template <typename T>
-ME_HD pol<T> pol_of(const wf_v<T>& w, int lam, bool outgoing) {  // as polvec_of
+ME_HD pol<T> pol_of(const wf_v<T>& w, int lam, bool outgoing) {  // as polvec
   const T s = outgoing ? T(-1) : T(1);
   return pol<T>{{lam > 0 ? -w.ccp : w.ccp, s * w.sp}, {lam > 0 ? -w.csp : w.csp, -s * w.cp}, lam > 0 ? w.st : -w.st};
 }
@@ -788,20 +725,6 @@ ME_HD c4<T> vvv(const c4<T>& J1, const c4<T>& J2, const r4<T>& k1, const r4<T>& 
   W.v[2] = cmac(cmac(d.y * j12, a, J2.v[2]), b, J1.v[2]);
   W.v[3] = cmac(cmac(d.z * j12, a, J2.v[3]), b, J1.v[3]);
   return W;
-}
-template <typename T>
-ME_HD void vvv_acc(c4<T>& acc, const c4<T>& J1, const c4<T>& J2, const r4<T>& k1, const r4<T>& k2, T s) {
-  r4<T> k3 = -(k1 + k2);
-  const cx<T> j12 = s * cdot(J1, J2);
-  const cx<T> a = s * rdot(k2 - k3, J1);
-  const cx<T> b = s * rdot(k3 - k1, J2);
-  r4<T> d = k1 - k2;
-  const T dd[4] = {d.e, d.x, d.y, d.z};
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const cx<T> t{acc.v[i].re + dd[i] * j12.re, acc.v[i].im + dd[i] * j12.im};
-    acc.v[i] = cmac(cmac(t, a, J2.v[i]), b, J1.v[i]);
-  }
 }
 // colour-ordered four-gluon structure: 2(L.R) M - (L.M) R - (M.R) L
 template <typename T>
