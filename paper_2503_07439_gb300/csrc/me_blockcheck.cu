@@ -4,9 +4,15 @@
 // helicity one at a time, and over the blocks of one member of each flipped pair
 // (doubled), in float64 and in float32.  It prints one line per point:
 //   <block fp64> <single fp64> <block fp32> <single fp32>
+// With the arguments "kernels <mt>" it prints what the kernels evaluate instead -- block_sum over
+// the live blocks, or the closed form of a 2 -> 2 tree, at unit couplings and scaled in
+// float64 -- with mt the top mass:
+//   <fp64> <fp32>
 // Input: "<pid> <n> <n_ext>" then the momenta [4][n_ext][n] (float64, SoA).
 #include <cmath>
 #include <cstdio>
+#include <cstdlib>
+#include <cstring>
 #include <vector>
 
 #include "me_internal.h"
@@ -52,13 +58,31 @@ static void eval(const ColourTables& tab, const r4<double>* k, const Couplings& 
   *single = s;
 }
 
+template <int PID, typename T>
+static double kernel_value(const ColourTables& tab, const r4<double>* k, const Couplings& cp) {
+  if constexpr (closed_tree<PID>()) return (double)closed_sum<PID, T>(k, unit_couplings(cp)) * tree_coupling(PID, cp);
+  KParams kp{};
+  kp.cp = cp;
+  kp.tab = &tab;
+  const Kin<PID, T> K = prepare<PID, T>(k, unit_couplings(cp));
+  T acc = T(0);
+  for (int b = 0; b < n_live_blocks<PID>(); ++b) acc += block_sum<PID, T>(K, b, kp);
+  return 2.0 * (double)acc * tree_coupling(PID, cp);
+}
+
+static double g_mt = 0.0;  // > 0: the kernels' values with this top mass
+
 template <int PID>
 static void run(const ColourTables& tab, const std::vector<double>& p, int n, int next) {
-  const Couplings cp{std::sqrt(4 * M_PI * 0.118), std::sqrt(4 * M_PI / 132.507), 173.0};
+  const Couplings cp{std::sqrt(4 * M_PI * 0.118), std::sqrt(4 * M_PI / 132.507), g_mt > 0.0 ? g_mt : 173.0};
   for (int i = 0; i < n; ++i) {
     r4<double> k[6];
     for (int l = 0; l < next; ++l)
       k[l] = {p[(0 * next + l) * n + i], p[(1 * next + l) * n + i], p[(2 * next + l) * n + i], p[(3 * next + l) * n + i]};
+    if (g_mt > 0.0) {
+      std::printf("%.17g %.17g\n", kernel_value<PID, double>(tab, k, cp), kernel_value<PID, float>(tab, k, cp));
+      continue;
+    }
     double b64, s64, b32, s32;
     eval<PID, double>(tab, k, cp, &b64, &s64);
     eval<PID, float>(tab, k, cp, &b32, &s32);
@@ -66,7 +90,8 @@ static void run(const ColourTables& tab, const std::vector<double>& p, int n, in
   }
 }
 
-int main() {
+int main(int argc, char** argv) {
+  if (argc == 3 && std::strcmp(argv[1], "kernels") == 0) g_mt = std::atof(argv[2]);
   static ColourTables tab;
   if (me_internal_build_tables(&tab) != ME_OK) return 1;
   int pid, n, next;

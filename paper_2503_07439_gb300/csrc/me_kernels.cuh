@@ -81,15 +81,15 @@ struct KParams {
   const ColourTables* tab;
 };
 
-template <typename T> __device__ __forceinline__ const T* s4tab(const ColourTables* t);
-template <> __device__ __forceinline__ const double* s4tab<double>(const ColourTables* t) { return t->S4; }
-template <> __device__ __forceinline__ const float* s4tab<float>(const ColourTables* t) { return t->S4f; }
-template <typename T> __device__ __forceinline__ const T* utab(const ColourTables* t, int pid);
-template <> __device__ __forceinline__ const double* utab<double>(const ColourTables* t, int pid) { return t->U[pid]; }
-template <> __device__ __forceinline__ const float* utab<float>(const ColourTables* t, int pid) { return t->Uf[pid]; }
+template <typename T> ME_HD const T* s4tab(const ColourTables* t);
+template <> ME_HD const double* s4tab<double>(const ColourTables* t) { return t->S4; }
+template <> ME_HD const float* s4tab<float>(const ColourTables* t) { return t->S4f; }
+template <typename T> ME_HD const T* utab(const ColourTables* t, int pid);
+template <> ME_HD const double* utab<double>(const ColourTables* t, int pid) { return t->U[pid]; }
+template <> ME_HD const float* utab<float>(const ColourTables* t, int pid) { return t->Uf[pid]; }
 
 template <int PID, typename T>
-__device__ __forceinline__ T colour_sum(const ColourTables* tab, const cx<T>* J) {
+ME_HD T colour_sum(const ColourTables* tab, const cx<T>* J) {
   constexpr int NF = Proc<PID>::NFLOW;
   if constexpr (PID == P_GG_TTGG)
     return s4_colour_sum(s4tab<T>(tab), [&](int v, int a) { return J[s4_flow(v, a)]; });
@@ -113,7 +113,7 @@ __device__ __forceinline__ T colour_sum(const ColourTables* tab, const cx<T>* J)
 
 // Live block b (K at unit couplings), summed over the four heavy-pair helicities and colours
 template <int PID, typename T, typename KP>
-__device__ __forceinline__ T block_sum(const Kin<PID, T>& K, int b, const KP& kp) {
+ME_HD T block_sum(const Kin<PID, T>& K, int b, const KP& kp) {
   if constexpr (PID == P_EE_UUG) {
     return ee_uug_block(K, b);
   } else {
