@@ -712,17 +712,18 @@ ME_HD void amp_uu_block(const KinUU<T>& K, int hb, const Couplings& cp, F&& cons
     sp.a = cmac(b * o0, c, o1);
     sp.b = cmac(a * o1, conj(c), o0);
   }
-  const T fu = T(2) * g * g * K.is, f3 = T(2) * g * g * K.is3, fw = T(2) * g * K.it * fu;
-  // the light current (without its factor 2) slashed, and the vertex's vector
-  // Z = (q4.J) e - (J.e) q4
+  const T fu = T(2) * g * g * K.is, f3 = T(2) * g * g * K.is3, fw = T(2) * g * fu, it = K.it, ih = T(0.5) * it;
+  // the light current (without its factor 2) slashed, and the vertex's vector times 1 / (q2 + q3)^2,
+  // Z = (q4.J) e - (J.e) q4 (1 / (q2 + q3)^2 times the other propagator, of order s^-2, would
+  // leave float32 from sqrt(s) = 1e10 on)
   const cx<T> ja = rho.b * sg.b, jb = rho.a * sg.a, jc = rho.b * sg.a, jd = rho.a * sg.b;
   const T qa = q[4].e - q[4].z, qb = q[4].e + q[4].z;
   const cx<T> qc{q[4].x, -q[4].y};
-  const cx<T> qJ = T(0.5) * cmsb(cmsb(rmac(qa * jb, qb, ja), qc, jd), conj(qc), jc);
-  const cx<T> eJ = T(0.5) * cmsb(cmsb(se.z * (ja - jb), se.c, jd), se.d, jc);
+  const cx<T> qJ = ih * cmsb(cmsb(rmac(qa * jb, qb, ja), qc, jd), conj(qc), jc);
+  const cx<T> eJ = ih * cmsb(cmsb(se.z * (ja - jb), se.c, jd), se.d, jc);
   const sl4<T> Z{rmac(-se.z * qJ, -qa, eJ), rmac(se.z * qJ, -qb, eJ), cmsb(qJ * se.c, eJ, qc),
                  cmsb(qJ * se.d, eJ, conj(qc))};
-  const cx<T> ke = rdot(K.pl[0] + K.pl[1], e);
+  const cx<T> ke = it * rdot(K.pl[0] + K.pl[1], e);
   const prop4<T> P1 = scaled_prop(q[2] + q[4], mt, -g * K.ia), P2 = scaled_prop(-(q[3] + q[4]), mt, -g * K.ib);
   cx<T> xs[2], xsp[2], yr[2], yrp[2], cx1[2], cy1[2];
 #pragma unroll

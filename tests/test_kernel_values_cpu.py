@@ -59,7 +59,7 @@ def test_kernel_values_equal_single_helicities(tool, name):
 # with 4, 5 and 6 legs, the ends come from single reciprocal invariants, of order E^-2, and, with
 # colour flows, from squares of amplitudes.
 RANGE = {"ee_uu": (-50, 50), "ee_uug": (-50, 50), "gg_tt": (-50, 50), "gg_ttg": (-48, 34), "gg_ttgg": (-34, 23),
-         "uu_tt": (-50, 50)}
+         "uu_tt": (-50, 50), "uu_ttg": (-50, 50)}
 
 
 @pytest.mark.parametrize("name,shift", [(n, s) for n, r in RANGE.items() for s in (r[0], -10, 10, r[1])])
