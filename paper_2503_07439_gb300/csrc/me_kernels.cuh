@@ -615,17 +615,25 @@ struct PointTerms {
   double mag_b;  // their error scale, |CT_coll| + |CT_soft - CT_softcoll| per sector
   double y[2];
   bool near;     // inside xi_thr / y_thr of an active counterterm
-  bool inside;   // inside the FKS domain
+  bool inside;   // inside the FKS domain (false where a direction is NaN)
   bool need[2];  // active Born configurations: soft, collinear (initial state); sector 1, 2
 };
 
 // a < b for b >= 0, on the bit patterns: a float64 comparison occupies the float64 pipe like a
-// multiply-add.  False for NaN (the arithmetic's NaN is positive).
+// multiply-add.  For a NaN the answer follows its sign bit; the domain test (PointTerms::inside)
+// then discards the point.
 __device__ __forceinline__ bool below(double a, double b) {
   return __double_as_longlong(a) < __double_as_longlong(b);
 }
-__device__ __forceinline__ bool positive(double a) {  // a > 0; infinite and NaN included
-  return __double_as_longlong(a) > 0;
+// a > 0, infinity included; false for a NaN of either sign
+__device__ __forceinline__ bool positive(double a) {
+  return (unsigned long long)(__double_as_longlong(a) - 1) < 0x7ff0000000000000ull;
+}
+// Whether unit3 gives p a direction: no component infinite or NaN, and the largest at least
+// 2^-537, whose square does not underflow.  From the exponents.
+__device__ __forceinline__ bool has_direction(const r4<double>& p) {
+  const int m = max(max(__double2hiint(p.x) & 0x7fffffff, __double2hiint(p.y) & 0x7fffffff), __double2hiint(p.z) & 0x7fffffff);
+  return m >= 486 << 20 && m < 2047 << 20;
 }
 
 // Counterterms, error scale and regions of one point, from its momenta k, in float64; T is the
@@ -658,6 +666,7 @@ __device__ __forceinline__ PointTerms point_terms(const r4<double>* k, const KPa
   const double d_cut = kp.delta;  // y_j > 1 - delta  <=>  1 - y_j < delta
   const bool soft_xi = below(xi, kp.xi_cut), near_xi = below(xi, kp.xi_thr);
   double d0, d1;
+  bool beams = true;  // both have a direction (known from d0 and d1 unless said otherwise)
   if constexpr (PID == P_EE_UUG) {
     double n[2][3];
     unit3(k[2], n[0][0], n[0][1], n[0][2]);
@@ -715,6 +724,7 @@ __device__ __forceinline__ PointTerms point_terms(const r4<double>* k, const KPa
       o.y[1] = q[0] * b1[0] + q[1] * b1[1] + q[2] * b1[2];
     } else {
       o.y[1] = -o.y[0];
+      beams = has_direction(k[1]);
     }
     d0 = 1.0 - o.y[0];
     d1 = 1.0 - o.y[1];
@@ -798,7 +808,7 @@ __device__ __forceinline__ PointTerms point_terms(const r4<double>* k, const KPa
     }
     o.need[0] = th_s;
   }
-  o.inside = positive(xi) && below(xi, 1.0) && positive(d0) && positive(d1);
+  o.inside = positive(xi) && below(xi, 1.0) && positive(d0) && positive(d1) && beams;
   return o;
 }
 
