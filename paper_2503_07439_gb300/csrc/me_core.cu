@@ -4,6 +4,7 @@
 
 #include <algorithm>
 #include <array>
+#include <cfloat>
 #include <chrono>
 #include <cmath>
 #include <complex>
@@ -114,17 +115,6 @@ __global__ void __launch_bounds__(256) k_reduce(const double* __restrict__ w, lo
   }
 }
 constexpr int RED_BLOCKS = 304;  // 2 x 152 SMs
-// Item rescue: a flagged point re-evaluates items in float64, largest error scale first,
-// until the float32 error left is at most this fraction of tol |W| -- half the budget of
-// an unflagged point, so that flagged points add little to the tail that the calibration
-// of me_eps bounds (2^20 flat points: the 99.9th percentile of the error stays at 8.2e-6
-// (g g -> t tbar g), 8.0e-6 (u ubar -> t tbar g) and 7.3e-6 (e+e- -> u ubar g) of tol =
-// 1e-5; at 1 it reaches 1.5e-5).  A compile-time setting, like ME_MINB, for calibration
-// studies: -DME_ITEM_BUDGET=x.
-#ifndef ME_ITEM_BUDGET
-#define ME_ITEM_BUDGET 0.5
-#endif
-constexpr double kItemBudget = ME_ITEM_BUDGET;
 
 // ---------------------------------------------------------------- colour algebra (host)
 using cd = std::complex<double>;
@@ -718,12 +708,8 @@ static int choose_lpe(me_handle* h, int kind, bool fp64, const LaunchArgs& a) {
 }
 
 static void set_tolerances(KParams& kp, const me_params* p) {
-  kp.me_eps = p->me_eps;
-  kp.tol = p->tol;
-  kp.item_budget = kItemBudget;
-  kp.me_epsf = (float)p->me_eps;
-  kp.tolf = (float)p->tol;
-  kp.budgetf = (float)(kItemBudget * p->tol / p->me_eps);
+  // tol <= 0 flags every point that has an error scale, me_eps <= 0 none
+  kp.tol_eps = p->me_eps <= 0.0 ? DBL_MAX : p->tol > 0.0 && p->me_eps > 0.0 ? p->tol / p->me_eps : 0.0;
 }
 
 // The cuts of me_params as the kernels take them (Cuts in me_kernels.cuh), for process pid.

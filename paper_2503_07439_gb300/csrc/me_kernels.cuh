@@ -71,12 +71,10 @@ struct KParams {
   double born_scale;    // couplings of the underlying Born x born_avg_inv
   double xi_cut, delta; // FKS plus-distribution cut-offs
   double xi_thr, y_thr; // points with xi < xi_thr or 1-y < y_thr go to the FP64 path
-  double me_eps;        // assumed relative error of a bulk-precision matrix element
-  double tol;           // target relative accuracy of a weight
-  float me_epsf, tolf, budgetf;  // float32 copies of me_eps, tol and item_budget x tol / me_eps
+  double tol_eps;       // tol / me_eps: target accuracy of a weight over the assumed error of a
+                        // bulk-precision matrix element
   int flag_unstable;    // 1: append unstable points to the rescue list
   int item_rescue;      // with flag_unstable: records and float64 items instead of the point list
-  double item_budget;   // item rescue: residual error allowed, as a fraction of tol |W|
   Cuts cut;             // cuts of every term (mask 0: none)
   const ColourTables* tab;
 };
@@ -602,8 +600,8 @@ constexpr int MAX_BLOCKS = 4;
 
 struct RealSubOut {
   double W;     // subtracted real, summed over sectors
-  double mag;   // error scale: |R S| + |CT_coll| + |CT_soft - CT_softcoll| per sector
-  double magR;  // its real part, sum_j |R S_j|
+  double magR;  // error scale: sum_j |R S_j|
+  double magB;  // and |CT_coll| + |CT_soft - CT_softcoll| per sector
   double y[2];  // y_j of both sectors (collinear resolution of the test)
   bool near;    // inside xi_thr / y_thr of an active counterterm
 };
@@ -628,6 +626,9 @@ __device__ __forceinline__ bool below(double a, double b) {
 // a > 0, infinity included; false for a NaN of either sign
 __device__ __forceinline__ bool positive(double a) {
   return (unsigned long long)(__double_as_longlong(a) - 1) < 0x7ff0000000000000ull;
+}
+__device__ __forceinline__ bool is_nan(double a) {
+  return (unsigned long long)__double_as_longlong(a) << 1 > 0xffe0000000000000ull;
 }
 // Whether unit3 gives p a direction: no component infinite or NaN, and the largest at least
 // 2^-537, whose square does not underflow.  From the exponents.
@@ -823,7 +824,7 @@ __device__ __forceinline__ double real_block_value(const Kin<PID, T>& K, int b, 
 __device__ __forceinline__ RealSubOut combine_point(const PointTerms& t, double R) {
   if (!t.inside) return RealSubOut{0.0, 0.0, 0.0, {t.y[0], t.y[1]}, false};
   const double r = t.real ? R : 0.0, magR = fabs(r);
-  return RealSubOut{r + t.w_born, magR + t.mag_b, magR, {t.y[0], t.y[1]}, t.near};
+  return RealSubOut{r + t.w_born, magR, t.mag_b, {t.y[0], t.y[1]}, t.near};
 }
 
 // `items` (optional): filled with the terms and block values on group lane 0 (every lane of
@@ -872,19 +873,33 @@ __device__ __forceinline__ RealSubOut real_sub_event(const double* __restrict__ 
   return combine_point(t, R);
 }
 
+// Item rescue: a flagged point re-evaluates items in float64, largest error scale first,
+// until the float32 error left is at most this fraction of tol |W| -- half the budget of
+// an unflagged point, so that flagged points add little to the tail that the calibration
+// of me_eps bounds (2^20 flat points: the 99.9th percentile of the error stays at 8.2e-6
+// (g g -> t tbar g), 8.0e-6 (u ubar -> t tbar g) and 7.3e-6 (e+e- -> u ubar g) of tol =
+// 1e-5; at 1 it reaches 1.5e-5).  A compile-time setting, like ME_MINB, for calibration
+// studies: -DME_ITEM_BUDGET=x.
+#ifndef ME_ITEM_BUDGET
+#define ME_ITEM_BUDGET 0.5
+#endif
+constexpr double kItemBudget = ME_ITEM_BUDGET;
+
 // Stability test of a bulk-precision result: the error of W is ~ me_eps x (error
 // scale); the float32 error of the real's amplitudes per unit scale grows towards the
 // collinear limit, as 1 + sqrt(rho_0 / rho) with rho = min_j (1 - y_j), rho_0 = 0.01.
 // The counterterms' Born values are evaluated at regular 2 -> 2 kinematics, whose error
 // does not grow there: error ~ me_eps x (growth x real part + Born part).
-__device__ __forceinline__ float error_growth(const RealSubOut& r) {
+__device__ __forceinline__ double error_growth(const RealSubOut& r) {
   const float rho = fmaxf(fminf((float)(1.0 - r.y[0]), (float)(1.0 - r.y[1])), 1e-30f);
-  return 1.0f + sqrtf(0.01f / rho);
+  return 1.0 + (double)sqrtf(0.01f / rho);
 }
-// The test is an estimate, taken in float32 (mag and W enter at float32 accuracy).
-__device__ __forceinline__ bool unstable_point(const RealSubOut& r, const KParams& kp, float g) {
-  const float R = (float)r.magR, B = (float)(r.mag - r.magR);
-  return r.near || !((R * g + B) * kp.me_epsf <= kp.tolf * (float)fabs(r.W));
+// The test itself in float64 (two operations; magnitudes compare like their bits, off the
+// float64 pipe): weights have no fixed scale, and float32 would compare 0 <= 0 or inf <= inf
+// where they leave its range, and call such a point stable.  A NaN is unstable.
+__device__ __forceinline__ bool unstable_point(const RealSubOut& r, const KParams& kp, double g) {
+  const double s = r.magR * g + r.magB;
+  return r.near || below(kp.tol_eps * fabs(r.W), s) || is_nan(s);
 }
 
 __device__ __forceinline__ bool unstable_point(const RealSubOut& r, const KParams& kp) {
@@ -892,33 +907,32 @@ __device__ __forceinline__ bool unstable_point(const RealSubOut& r, const KParam
 }
 
 // Blocks of a flagged point to re-evaluate in float64 (bit b: block b).  Largest error scale
-// first, until the scale of what is left, times the bulk-precision error per unit scale, is
-// within kp.item_budget x tol |W|.  The Born part is float64 already but keeps its place in
-// the order: a point whose flag came from it alone takes no block, and what the part no
-// longer adds to the error is a margin.  Points inside the thresholds take every block.
+// first, until the scale of what is left is within kItemBudget of what the test allows.  The
+// Born part is float64 already but keeps its place in the order (without growth): what it no
+// longer adds to the error is a margin.  Points inside the thresholds take every block, and so
+// do those with a NaN.
 template <int PID>
 __device__ __forceinline__ unsigned rescue_mask(const RealSubOut& r, bool real, const double* v, const KParams& kp,
-                                                float grow) {
+                                                double g) {
   constexpr int NB = RealLayout<PID>::NB;
   constexpr unsigned all = (1u << NB) - 1u;
   if (!real) return 0;
-  if (r.near) return all;
-  float e[NB + 1];
-  float rest = 0.0f;
+  double rest = r.magR * g + r.magB;
+  if (r.near || is_nan(rest)) return all;
+  double e[NB + 1];
 #pragma unroll
-  for (int b = 0; b < NB; ++b) rest += (e[b] = fabsf((float)v[b]));
-  rest += (e[NB] = (float)(r.mag - r.magR) / grow);  // no growth for the Born part (unstable_point)
-  if (!(rest == rest)) return all;
-  const float budget = kp.budgetf * (float)fabs(r.W) / grow;
+  for (int b = 0; b < NB; ++b) e[b] = g * fabs(v[b]);
+  e[NB] = r.magB;
+  const double budget = kItemBudget * (kp.tol_eps * fabs(r.W));
   unsigned m = 0;
 #pragma unroll
   for (int k = 0; k <= NB; ++k) {
-    if (rest <= budget) break;
+    if (!below(budget, rest)) break;
     int pick = 0;
-    float best = -1.0f;
+    double best = -1.0;
 #pragma unroll
     for (int b = 0; b <= NB; ++b)
-      if (!(m >> b & 1u) && e[b] > best) {
+      if (!(m >> b & 1u) && below(best, e[b])) {
         best = e[b];
         pick = b;
       }
@@ -1215,7 +1229,7 @@ __global__ void __launch_bounds__(128) k_terms(const double* __restrict__ p, con
   const int slot = warp_reserve(tb.cnt, rec ? 1 : 0);
   const RealSubOut r = combine_point(t, 0.0);
   if (rec) {
-    const float g = error_growth(r);
+    const float g = (float)error_growth(r);
     tb.ev[slot] = (int)i | (t.need[0] ? 1 << 29 : 0) | (t.need[1] ? 1 << 30 : 0);
     tb.grow[slot] = t.near ? -g : g;
     tb.a[slot] = t.w_born;
@@ -1252,11 +1266,11 @@ __global__ void __launch_bounds__(128, ME_MINB) k_term_reals(const double* __res
     const double wb = tb.a[slot], W = R + wb;
     out[ev] = (wgt ? wgt[ev] : 1.0) * W;
     if (kp.flag_unstable) {
-      const float g = tb.grow[slot];
-      const RealSubOut r{W, fabs(R) + tb.a[tb.cap + slot], fabs(R), {0.0, 0.0}, g < 0.0f};
-      if (unstable_point(r, kp, fabsf(g))) {
+      const double g = tb.grow[slot];
+      const RealSubOut r{W, fabs(R), tb.a[tb.cap + slot], {0.0, 0.0}, g < 0.0};
+      if (unstable_point(r, kp, fabs(g))) {
         const bool need[2] = {(code >> 29 & 1) != 0, (code >> 30 & 1) != 0};
-        append_flagged<PID>(counts, ib, ev, wb, need, v, rescue_mask<PID>(r, true, v, kp, fabsf(g)));
+        append_flagged<PID>(counts, ib, ev, wb, need, v, rescue_mask<PID>(r, true, v, kp, fabs(g)));
       }
     }
   }
