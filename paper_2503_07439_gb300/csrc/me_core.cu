@@ -61,16 +61,18 @@ __device__ __forceinline__ void block_sum2(double& a, double& b, double (*sm)[8]
 
 // Weight accumulation and the end of a call: (sum w, sum w^2) by blocks in a fixed order,
 // then the block that finishes last adds the blocks' partials in block order (no floating
-// atomics: the result is reproducible) and hands the call's counters over, `live` to `last`,
-// leaving `live` zero for the next call.  One launch instead of three (a memset of the
-// counters, the partials, their sum), each mostly launch and drain latency: with the closed
-// form, a call with 999 e+e- n-body points went from 56 to 33 us.  `cnt` (optional, device):
-// the number of points, at most n.
-constexpr int CNT_LIVE = 12;    // counters handed over
-constexpr int CNT_TICKET = 12;  // blocks finished
+// atomics: the result is reproducible).  One launch instead of two (the partials, their sum),
+// each mostly launch and drain latency.  `ticket`, the number of blocks finished, is set to zero
+// earlier in the same call (clear_counters, or the tree kernels): a call relies on nothing
+// that an earlier one left behind, so one that failed half way, or that overlapped with
+// another stream's, spoils no later call and no replay of a captured one.  `cnt` (optional,
+// device): the number of points, at most n.
+constexpr int CNT_RECORDS = 11;  // counters besides those of ItemBufs: records of the per-term queues,
+constexpr int CNT_TICKET = 12;   // blocks of the reduction finished,
+constexpr int CNT_LISTED = 13;   // points passing the cuts (tree entries with per-term queues)
 __global__ void __launch_bounds__(256) k_reduce(const double* __restrict__ w, long n, const int* __restrict__ cnt,
                                                 double* __restrict__ part, double* __restrict__ acc,
-                                                int* __restrict__ live, int* __restrict__ last) {
+                                                int* __restrict__ ticket) {
   __shared__ double sm[2][8];
   __shared__ bool final_block;
   double a = 0.0, b = 0.0;
@@ -92,7 +94,7 @@ __global__ void __launch_bounds__(256) k_reduce(const double* __restrict__ w, lo
     __stcg(part + 2 * blockIdx.x, a);
     __stcg(part + 2 * blockIdx.x + 1, b);
     __threadfence();
-    final_block = atomicAdd(live + CNT_TICKET, 1) == (int)gridDim.x - 1;
+    final_block = atomicAdd(ticket, 1) == (int)gridDim.x - 1;
   }
   __syncthreads();
   if (!final_block) return;
@@ -107,11 +109,6 @@ __global__ void __launch_bounds__(256) k_reduce(const double* __restrict__ w, lo
     acc[0] += a;
     acc[1] += b;
     acc[2] += (double)n;
-    live[CNT_TICKET] = 0;
-  }
-  if (threadIdx.x < CNT_LIVE) {
-    last[threadIdx.x] = live[threadIdx.x];
-    live[threadIdx.x] = 0;
   }
 }
 constexpr int RED_BLOCKS = 304;  // 2 x 152 SMs
@@ -436,12 +433,7 @@ struct me_handle {
   double* d_out = nullptr;
   size_t cap = 0;
   int* d_resc = nullptr;     // rescue index list (capacity cap)
-  // counters of the running call (ItemBufs, the reduction's ticket; zero between calls) and,
-  // from d_last, those of the last finished one; [13]: points passing the cuts (tree entries
-  // with per-term queues)
-  int* d_nresc = nullptr;
-  int* d_last = nullptr;
-  bool dirty = false;       // a call failed half way: the counters have to be cleared
+  int* d_nresc = nullptr;    // counters of the last call (ItemBufs, CNT_*)
   bool last_terms = false;  // the last subtracted-real call ran the per-term queues
   // item rescue (mixed-precision subtracted real): records and item lists, capacity icap
   ItemBufs ib{};
@@ -491,7 +483,7 @@ static int ensure_item_capacity(me_handle* h, size_t n) {
 
 static void free_terms(me_handle* h) {
   TermBufs& t = h->tb;
-  void* ptrs[] = {t.ev, t.grow, t.a, t.cnt};
+  void* ptrs[] = {t.ev, t.grow, t.a};
   for (void* q : ptrs) cudaFree(q);
   h->tb = TermBufs{};
   h->tcap = 0;
@@ -505,12 +497,12 @@ static int ensure_term_capacity(me_handle* h, size_t n) {
   TermBufs& t = h->tb;
   const bool ok = cudaMalloc(&t.ev, c * sizeof(int)) == cudaSuccess &&
                   cudaMalloc(&t.grow, c * sizeof(float)) == cudaSuccess &&
-                  cudaMalloc(&t.a, c * 2 * sizeof(double)) == cudaSuccess &&
-                  cudaMalloc(&t.cnt, sizeof(int)) == cudaSuccess;
+                  cudaMalloc(&t.a, c * 2 * sizeof(double)) == cudaSuccess;
   if (!ok) {
     free_terms(h);
     return fail(ME_ERR_OOM, "per-term queue scratch allocation failed");
   }
+  t.cnt = h->d_nresc + CNT_RECORDS;
   t.cap = (long)c;
   h->tcap = c;
   return ME_OK;
@@ -620,21 +612,68 @@ static cudaError_t launch_terms(me_handle* h, bool mixed, const LaunchArgs& a) {
   return cudaErrorInvalidValue;
 }
 
-// Weight accumulation of n results (or *cnt) and hand-over of the call's counters.
+// Weight accumulation of n results (or *cnt).
 static cudaError_t launch_reduce(me_handle* h, const double* out, long n, const int* cnt) {
   const long blocks = std::min<long>(RED_BLOCKS, (n + 1023) / 1024);
-  k_reduce<<<(unsigned)std::max(1L, blocks), 256, 0, h->stream>>>(out, n, cnt, h->d_part, h->d_acc, h->d_nresc, h->d_last);
+  k_reduce<<<(unsigned)std::max(1L, blocks), 256, 0, h->stream>>>(out, n, cnt, h->d_part, h->d_acc, h->d_nresc + CNT_TICKET);
   return cudaGetLastError();
 }
 
-// Counters of the running call at zero: the reduction leaves them so, unless a call failed.
-static cudaError_t begin_call(me_handle* h) {
-  if (h->dirty) {
-    const cudaError_t e = cudaMemsetAsync(h->d_nresc, 0, 16 * sizeof(int), h->stream);
-    if (e != cudaSuccess) return e;
+// The counters of a subtracted-real call (ItemBufs, the queues' records and tiles, the reduction's
+// ticket) at zero, in stream order, and so inside a captured call too.  (A tree call counts
+// only the reduction's blocks; its kernels clear that themselves, LaunchArgs::ticket.)
+static cudaError_t clear_counters(me_handle* h) { return cudaMemsetAsync(h->d_nresc, 0, 16 * sizeof(int), h->stream); }
+
+// Failure injection on the host, for tests (me_internal.h).
+static thread_local int g_fail_stage = 0;
+static cudaError_t injected(int stage) {
+  if (g_fail_stage != stage) return cudaSuccess;
+  g_fail_stage = 0;
+  return cudaErrorLaunchOutOfResources;
+}
+
+// The launches of one call: main kernel(s), float64 rescue, reduction; `ev` (optional): events
+// recorded around the three.
+struct CallPlan {
+  int kind;
+  bool mixed, terms, queued, cut_list;
+  int lpe, lpe64;
+};
+static cudaError_t launch_call(me_handle* h, const CallPlan& c, LaunchArgs a, const cudaEvent_t* ev) {
+  cudaError_t e = cudaSuccess;
+  auto run = [&](auto&& f) {
+    if (e == cudaSuccess) e = f();
+  };
+  auto mark = [&](int i) {
+    if (ev) run([&] { return cudaEventRecord(ev[i], h->stream); });
+  };
+  const long n = a.n;
+  const int* count = a.count;
+  mark(0);
+  run([&] { return injected(1); });
+  if (c.kind == K_REAL) run([&] { return clear_counters(h); });
+  if (c.terms) {
+    run([&] { return launch_terms(h, c.mixed, a); });
+  } else if (c.queued) {
+    run([&] { return launch_queued(h->proc->pid, a, h->stream); });
+  } else {
+    if (c.cut_list) {
+      // per-term queues of a tree entry: only the points that pass the cuts are evaluated
+      run([&] { return launch_cut_list(h->proc->pid, a, h->d_resc, h->d_nresc + CNT_LISTED, h->stream); });
+      a.idx = h->d_resc;
+      a.count = h->d_nresc + CNT_LISTED;
+    }
+    run([&] { return dispatch(h->proc->pid, c.kind, !c.mixed, c.lpe, a, h->stream); });
   }
-  h->dirty = true;
-  return cudaSuccess;
+  mark(1);
+  run([&] { return injected(2); });
+  if (c.kind == K_REAL && c.mixed && !c.queued)
+    run([&] { return c.terms ? launch_items(h, a) : launch_rescue(h, a, c.lpe64); });
+  mark(2);
+  run([&] { return injected(3); });
+  run([&] { return launch_reduce(h, a.out, n, count); });
+  mark(3);
+  return e;
 }
 
 // pick lanes-per-event by timing each candidate once on the caller's batch (first use)
@@ -802,12 +841,11 @@ int me_init(const char* process, const me_params* params, me_handle** out) {
     return fail(ME_ERR_CUDA, "me_init: stream creation failed");
   }
   h->stream = h->own_stream;
-  if (cudaMalloc(&h->d_nresc, 32 * sizeof(int)) != cudaSuccess || cudaMalloc(&h->d_part, 2 * RED_BLOCKS * sizeof(double)) != cudaSuccess ||
+  if (cudaMalloc(&h->d_nresc, 16 * sizeof(int)) != cudaSuccess || cudaMalloc(&h->d_part, 2 * RED_BLOCKS * sizeof(double)) != cudaSuccess ||
       cudaMalloc(&h->d_acc, 3 * sizeof(double)) != cudaSuccess) {
     me_destroy(h);
     return fail(ME_ERR_OOM, "me_init: allocation failed");
   }
-  h->d_last = h->d_nresc + 16;
   KParams& kp = h->kp;
   kp = KParams{};
   kp.cp = Couplings(std::sqrt(4.0 * M_PI * params->alpha_s), std::sqrt(4.0 * M_PI * params->alpha), params->mt);
@@ -826,7 +864,7 @@ int me_init(const char* process, const me_params* params, me_handle** out) {
   // stream-ordered on the handle's own stream: no device-wide synchronisation, so a
   // handle can be created while other threads capture CUDA graphs
   if (cudaMemsetAsync(h->d_acc, 0, 3 * sizeof(double), h->own_stream) != cudaSuccess ||
-      cudaMemsetAsync(h->d_nresc, 0, 32 * sizeof(int), h->own_stream) != cudaSuccess ||
+      cudaMemsetAsync(h->d_nresc, 0, 16 * sizeof(int), h->own_stream) != cudaSuccess ||
       cudaStreamSynchronize(h->own_stream) != cudaSuccess) {
     me_destroy(h);
     return fail(ME_ERR_CUDA, "me_init: device error");
@@ -878,6 +916,7 @@ static int run(me_handle* h, int kind, double nlo_factor, const double* momenta,
   a.resc_list = h->d_resc;
   a.resc_count = h->d_nresc;
   a.tiles = h->d_nresc + 1;
+  a.ticket = h->d_nresc + CNT_TICKET;
   const bool terms = kind == K_REAL && use_terms(h, n);
   const bool cut_list = kind == K_TREE && h->prm.term_queues == ME_TERMS_QUEUED && a.kp.cut.mask;
   const bool queued = kind == K_REAL && mixed && h->prm.queued_rescue && !terms;
@@ -917,29 +956,8 @@ static int run(me_handle* h, int kind, double nlo_factor, const double* momenta,
       h->ev_pool.pop_back();
     }
     h->ev_used.push_back(ev);
-    ME_CUDA(cudaEventRecord(ev[0], h->stream));
   }
-  ME_CUDA(begin_call(h));
-  if (terms) {
-    ME_CUDA(launch_terms(h, mixed, a));
-  } else if (queued) {
-    ME_CUDA(launch_queued(h->proc->pid, a, h->stream));
-  } else {
-    if (cut_list) {
-      // per-term queues of a tree entry: only the points that pass the cuts are evaluated
-      ME_CUDA(launch_cut_list(h->proc->pid, a, h->d_resc, h->d_nresc + 13, h->stream));
-      a.idx = h->d_resc;
-      a.count = h->d_nresc + 13;
-    }
-    ME_CUDA(dispatch(h->proc->pid, kind, !mixed, lpe, a, h->stream));
-  }
-  if (timed) ME_CUDA(cudaEventRecord(ev[1], h->stream));
-  if (terms && mixed) ME_CUDA(launch_items(h, a));
-  if (kind == K_REAL && mixed && !queued && !terms) ME_CUDA(launch_rescue(h, a, lpe64));
-  if (timed) ME_CUDA(cudaEventRecord(ev[2], h->stream));
-  ME_CUDA(launch_reduce(h, O, n, nullptr));
-  h->dirty = false;
-  if (timed) ME_CUDA(cudaEventRecord(ev[3], h->stream));
+  ME_CUDA(launch_call(h, CallPlan{kind, mixed, terms, queued, cut_list, lpe, lpe64}, a, timed ? ev.data() : nullptr));
   if (!vo) ME_CUDA(cudaMemcpyAsync(out, O, (size_t)n * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
   if (on_host) ME_CUDA(cudaStreamSynchronize(h->stream));
   return ME_OK;
@@ -973,7 +991,7 @@ int me_last_rescued(me_handle* h, int64_t* n_rescued) {
   ME_CUDA(cudaSetDevice(h->device));
   int c = 0;
   if (h->prm.precision == ME_PREC_MIXED && h->last_kind == K_REAL) {
-    ME_CUDA(cudaMemcpyAsync(&c, h->d_last, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
+    ME_CUDA(cudaMemcpyAsync(&c, h->d_nresc, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
     ME_CUDA(cudaStreamSynchronize(h->stream));
   }
   *n_rescued = c;
@@ -985,7 +1003,7 @@ int me_last_rescue_work(me_handle* h, int64_t* points, int64_t* real_blocks, int
   ME_CUDA(cudaSetDevice(h->device));
   int c[8] = {};
   if (h->prm.precision == ME_PREC_MIXED && h->last_kind == K_REAL) {
-    ME_CUDA(cudaMemcpyAsync(c, h->d_last, sizeof(c), cudaMemcpyDeviceToHost, h->stream));
+    ME_CUDA(cudaMemcpyAsync(c, h->d_nresc, sizeof(c), cudaMemcpyDeviceToHost, h->stream));
     ME_CUDA(cudaStreamSynchronize(h->stream));
   }
   *points = c[0];
@@ -999,7 +1017,7 @@ int me_last_rescue_configs(me_handle* h, int64_t* set0, int64_t* set1) {
   ME_CUDA(cudaSetDevice(h->device));
   int c[6] = {0, 0, 0, 0, 0, 0};
   if (h->prm.precision == ME_PREC_MIXED && h->last_kind == K_REAL && h->last_terms) {
-    ME_CUDA(cudaMemcpyAsync(c, h->d_last, sizeof(c), cudaMemcpyDeviceToHost, h->stream));
+    ME_CUDA(cudaMemcpyAsync(c, h->d_nresc, sizeof(c), cudaMemcpyDeviceToHost, h->stream));
     ME_CUDA(cudaStreamSynchronize(h->stream));
   }
   *set0 = c[4];
@@ -1139,6 +1157,7 @@ int me_internal_launch_counted(me_handle* h, int me_kind, const double* d_p, con
   a.resc_list = h->d_resc;
   a.resc_count = h->d_nresc;
   a.tiles = h->d_nresc + 1;
+  a.ticket = h->d_nresc + CNT_TICKET;
   const bool terms = kind == K_REAL && use_terms(h, cap);
   const bool cut_list = kind == K_TREE && h->prm.term_queues == ME_TERMS_QUEUED && a.kp.cut.mask;
   const bool queued = kind == K_REAL && mixed && h->prm.queued_rescue && !terms;
@@ -1154,25 +1173,11 @@ int me_internal_launch_counted(me_handle* h, int me_kind, const double* d_p, con
     h->last_kind = K_REAL;
     h->last_terms = terms;
   }
-  ME_CUDA(begin_call(h));
-  if (terms) {
-    ME_CUDA(launch_terms(h, mixed, a));
-    if (mixed) ME_CUDA(launch_items(h, a));
-  } else if (queued) {
-    ME_CUDA(launch_queued(h->proc->pid, a, h->stream));
-  } else {
-    if (cut_list) {
-      ME_CUDA(launch_cut_list(h->proc->pid, a, h->d_resc, h->d_nresc + 13, h->stream));
-      a.idx = h->d_resc;
-      a.count = h->d_nresc + 13;
-    }
-    ME_CUDA(dispatch(h->proc->pid, kind, !mixed, lpe, a, h->stream));
-  }
-  if (kind == K_REAL && mixed && !queued && !terms) ME_CUDA(launch_rescue(h, a, lpe64));
-  ME_CUDA(launch_reduce(h, d_out, cap, d_n));
-  h->dirty = false;
+  ME_CUDA(launch_call(h, CallPlan{kind, mixed, terms, queued, cut_list, lpe, lpe64}, a, nullptr));
   return ME_OK;
 }
+
+void me_internal_fail_stage(int stage) { g_fail_stage = stage; }
 
 int me_internal_final_masses(me_handle* h, double* masses, int* n_out, cudaStream_t* stream) {
   if (!h || !masses || !n_out || !stream) return fail(ME_ERR_ARG, "NULL argument");
@@ -1215,7 +1220,7 @@ int me_internal_rescued_async(me_handle* h, int* dst) {
     *dst = 0;
     return ME_OK;
   }
-  ME_CUDA(cudaMemcpyAsync(dst, h->d_last, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
+  ME_CUDA(cudaMemcpyAsync(dst, h->d_nresc, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
   return ME_OK;
 }
 

@@ -16,6 +16,10 @@ int me_internal_rescued_async(me_handle* h, int* dst);
 int me_internal_prepare_counted(me_handle* h, int me_kind, int64_t cap);
 int me_internal_launch_counted(me_handle* h, int me_kind, const double* d_p, const double* d_w, int64_t cap,
                                const int* d_n, double* d_out);
+// Failure injection on the host, for tests: the calling thread's next evaluation of a handle
+// reports a launch failure in place of its main kernel (stage 1), its float64 rescue (2) or its
+// reduction (3), with what comes before launched and nothing after.
+extern "C" void me_internal_fail_stage(int stage);
 // Final-state masses of the handle's process (outgoing legs in order; at most 4), their
 // number, and the handle's stream.
 int me_internal_final_masses(me_handle* h, double* masses, int* n_out, cudaStream_t* stream);

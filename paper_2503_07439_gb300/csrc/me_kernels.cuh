@@ -188,6 +188,11 @@ __device__ __forceinline__ bool pass_cuts(const r4<double>* k, const Cuts& c) {
 }
 
 // ---------------------------------------------------------------- tree |M|^2
+// The tree kernels clear the ticket of the reduction that follows them.
+__device__ __forceinline__ void clear_ticket(int* ticket) {
+  if (blockIdx.x == 0 && threadIdx.x == 0 && ticket) *ticket = 0;
+}
+
 // out[i] = wgt[i] * |M|^2(p_i) * nlo_factor.  `count` (optional): the number of events,
 // read on the device; `idx` (optional): the list of events to process (its length in
 // `count`).  Momenta have stride n either way.  (g g -> t tbar g g runs k_tree_tt4 and, in
@@ -195,8 +200,10 @@ __device__ __forceinline__ bool pass_cuts(const r4<double>* k, const Cuts& c) {
 template <int PID, typename T, int LPE>
 __global__ void __launch_bounds__(128, ME_MINB) k_tree(const double* __restrict__ p, const double* __restrict__ wgt,
                                                        long n, double* __restrict__ out, KParams kp,
-                                                       const int* __restrict__ idx, const int* __restrict__ count) {
+                                                       const int* __restrict__ idx, const int* __restrict__ count,
+                                                       int* __restrict__ ticket) {
   static_assert(PID != P_GG_TTGG, "g g -> t tbar g g runs k_tree_tt4 and k_tree_tt4f");
+  clear_ticket(ticket);
   constexpr int NEXT = Proc<PID>::NEXT;
   const long gid = ((long)blockIdx.x * blockDim.x + threadIdx.x) / LPE;
   const int lane = threadIdx.x % LPE;
@@ -227,8 +234,10 @@ __global__ void __launch_bounds__(128, ME_MINB) k_tree(const double* __restrict_
 template <int PID>
 __global__ void __launch_bounds__(128, ME_MINB) k_tree_tt4(const double* __restrict__ p, const double* __restrict__ wgt,
                                                            long n, double* __restrict__ out, KParams kp,
-                                                           const int* __restrict__ idx, const int* __restrict__ count, int lg) {
+                                                           const int* __restrict__ idx, const int* __restrict__ count,
+                                                           int* __restrict__ ticket, int lg) {
   static_assert(PID == P_GG_TTGG, "eight blocks");
+  clear_ticket(ticket);
   __shared__ double part[128];
   const int slot = threadIdx.x & ((128 >> lg) - 1), lane = threadIdx.x >> (7 - lg);
   const long gid = ((long)blockIdx.x << (7 - lg)) + slot;
@@ -259,7 +268,9 @@ __global__ void __launch_bounds__(128, ME_MINB) k_tree_tt4(const double* __restr
 template <int PID, typename T>
 __global__ void __launch_bounds__(256) k_tree_closed(const double* __restrict__ p, const double* __restrict__ wgt,
                                                      long n, double* __restrict__ out, KParams kp,
-                                                     const int* __restrict__ idx, const int* __restrict__ count) {
+                                                     const int* __restrict__ idx, const int* __restrict__ count,
+                                                     int* __restrict__ ticket) {
+  clear_ticket(ticket);
   const long gid = (long)blockIdx.x * blockDim.x + threadIdx.x;
   const long nev = count ? (long)*count : n;
   if (gid >= nev) return;
@@ -344,8 +355,10 @@ __device__ __forceinline__ void st_sl4(float* b, int slot, const sl4<float>& S) 
 template <int PID>
 __global__ void __launch_bounds__(TT4_THREADS, 2) k_tree_tt4f(const double* __restrict__ p, const double* __restrict__ wgt,
                                                               long n, double* __restrict__ out, KParams kp,
-                                                              const int* __restrict__ idx, const int* __restrict__ count) {
+                                                              const int* __restrict__ idx, const int* __restrict__ count,
+                                                              int* __restrict__ ticket) {
   static_assert(PID == P_GG_TTGG, "eight blocks");
+  clear_ticket(ticket);
   extern __shared__ __align__(16) float tt4_smem[];
   const int warp = threadIdx.x >> 5, wl = threadIdx.x & 31;
   float* wsm = tt4_smem + warp * TT4_WARP;
@@ -1175,7 +1188,7 @@ struct TermBufs {
   int* ev;      // [cap] point of the record; bits 29, 30: active Born configurations
   float* grow;  // [cap] error growth factor of the stability test, negative: near
   double* a;    // [2][cap] W_B, Born error scale
-  int* cnt;     // records
+  int* cnt;     // records, zero at launch
   long cap;
 };
 
@@ -1310,6 +1323,7 @@ struct LaunchArgs {
   ItemBufs items;    // item rescue records and lists
   long groups;       // number of event groups to launch (n, or the list capacity)
   int* tiles;        // queued kernel: tile counter, zero at launch
+  int* ticket;       // tree kernels: counter that they set to zero (the reduction's), or null
   double* p_copy;    // per-term queues: device copy of p made by k_terms (p in host memory), or null
 };
 enum KernelKind : int { K_TREE = 0, K_REAL = 1 };
@@ -1332,15 +1346,15 @@ cudaError_t launch_one(int kind, const LaunchArgs& a, cudaStream_t st) {
         attr_set[dev] = true;
       }
       const long tb = (total + TT4_THREADS - 1) / TT4_THREADS;
-      k_tree_tt4f<PID><<<(unsigned)tb, TT4_THREADS, TT4_SMEM, st>>>(a.p, a.wgt, a.n, a.out, a.kp, a.idx, a.count);
+      k_tree_tt4f<PID><<<(unsigned)tb, TT4_THREADS, TT4_SMEM, st>>>(a.p, a.wgt, a.n, a.out, a.kp, a.idx, a.count, a.ticket);
     } else if constexpr (closed_tree<PID>()) {
       if constexpr (LPE != 1) return launch_one<PID, T, 1>(kind, a, st);
-      else k_tree_closed<PID, T><<<(unsigned)((a.groups + 255) / 256), 256, 0, st>>>(a.p, a.wgt, a.n, a.out, a.kp, a.idx, a.count);
+      else k_tree_closed<PID, T><<<(unsigned)((a.groups + 255) / 256), 256, 0, st>>>(a.p, a.wgt, a.n, a.out, a.kp, a.idx, a.count, a.ticket);
     } else if constexpr (PID == P_GG_TTGG) {
       constexpr int lg = LPE == 1 ? 0 : LPE == 2 ? 1 : LPE == 4 ? 2 : 3;
-      k_tree_tt4<PID><<<(unsigned)blocks, threads, 0, st>>>(a.p, a.wgt, a.n, a.out, a.kp, a.idx, a.count, lg);
+      k_tree_tt4<PID><<<(unsigned)blocks, threads, 0, st>>>(a.p, a.wgt, a.n, a.out, a.kp, a.idx, a.count, a.ticket, lg);
     } else {
-      k_tree<PID, T, LPE><<<(unsigned)blocks, threads, 0, st>>>(a.p, a.wgt, a.n, a.out, a.kp, a.idx, a.count);
+      k_tree<PID, T, LPE><<<(unsigned)blocks, threads, 0, st>>>(a.p, a.wgt, a.n, a.out, a.kp, a.idx, a.count, a.ticket);
     }
   } else {
     if constexpr (PID == P_EE_UUG || PID == P_GG_TTG || PID == P_UU_TTG)
@@ -1443,7 +1457,6 @@ cudaError_t launch_terms_one(bool mixed, const LaunchArgs& a, const TermBufs& tb
   }
   const long blocks = (a.groups + 127) / 128;
   if (blocks <= 0) return cudaSuccess;
-  if ((e = cudaMemsetAsync(tb.cnt, 0, sizeof(int), st)) != cudaSuccess) return e;
   const double* pi = a.p_copy ? a.p_copy : a.p;
   const unsigned gr = (unsigned)std::min<long>(g, blocks), gt = (unsigned)blocks;
   if (mixed) {
