@@ -307,7 +307,9 @@ int me_generate_fks(me_handle* h, uint64_t seed, uint32_t stream, int64_t first_
  *   n_kept        host: number of kept points (entries written to kept, kept_weights)
  *   w_max_used    host or NULL: the w_max applied
  *   n_over        host or NULL: number of overweight points (all kept)
- * Runs on the handle's stream and returns when the results are in place.  ME_ERR_ARG for
+ * Runs on the handle's stream and returns when the results are in place; several threads may
+ * call it through one handle.  The handle keeps up to four workspaces of n / 8 bytes, of at most
+ * 16 MiB each, for later calls.  ME_ERR_ARG for
  * host buffers, n outside [0, 2^31), first_point < 0 or a NaN w_max.
  */
 int me_unweight(me_handle* h, const double* weights, int64_t n, double w_max, uint64_t seed, uint32_t stream,

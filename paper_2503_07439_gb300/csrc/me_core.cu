@@ -442,9 +442,8 @@ struct me_handle {
   TermBufs tb{};
   size_t tcap = 0;
   double* d_part = nullptr;  // reduction partials
-  void* ws = nullptr;        // workspace of me_unweight, and its results in mapped host memory
-  size_t ws_bytes = 0;
-  void* ws_host = nullptr;
+  std::mutex ws_mu;
+  std::vector<Workspace> ws;  // idle workspaces of me_unweight
   double* d_acc = nullptr;   // accumulators (3)
   int lpe[2][2] = {{0, 0}, {0, 0}};  // [kind][fp64] chosen lanes per event
   int lpe_class[2][2] = {{-1, -1}, {-1, -1}};  // batch-size class they were chosen for
@@ -1092,8 +1091,10 @@ void me_destroy(me_handle* h) {
   free_terms(h);
   cudaFree(h->d_part);
   cudaFree(h->d_acc);
-  cudaFree(h->ws);
-  cudaFreeHost(h->ws_host);
+  for (auto& w : h->ws) {
+    cudaFree(w.dev);
+    cudaFreeHost(w.host);
+  }
   for (auto& ev : h->ev_used)
     for (auto e : ev) cudaEventDestroy(e);
   for (auto e : h->ev_pool) cudaEventDestroy(e);
@@ -1191,27 +1192,63 @@ int me_internal_final_masses(me_handle* h, double* masses, int* n_out, cudaStrea
   return ME_OK;
 }
 
-int me_internal_workspace(me_handle* h, size_t bytes, void** dev, void** host, void** host_dev) {
-  if (!h || !dev || !host || !host_dev) return fail(ME_ERR_ARG, "NULL argument");
-  if (!h->ws_host && cudaHostAlloc(&h->ws_host, 64, cudaHostAllocMapped) != cudaSuccess) {
-    h->ws_host = nullptr;
-    return fail(ME_ERR_OOM, "workspace allocation failed");
-  }
-  if (bytes > h->ws_bytes) {
-    cudaFree(h->ws);
-    h->ws = nullptr;
-    h->ws_bytes = 0;
-    const size_t c = std::max(bytes, (size_t)1 << 16);
-    if (cudaMalloc(&h->ws, c) != cudaSuccess) {
-      h->ws = nullptr;
-      return fail(ME_ERR_OOM, "workspace allocation failed");
+// Idle workspaces kept by a handle: at most four, each of at most 16 MiB (2^27 points).
+constexpr size_t kWorkspaces = 4, kWorkspaceBytes = (size_t)16 << 20;
+
+int me_internal_workspace_take(me_handle* h, size_t bytes, cudaStream_t st, Workspace* out) {
+  if (!h || !out) return fail(ME_ERR_ARG, "NULL argument");
+  Workspace w{};
+  {
+    std::lock_guard<std::mutex> lk(h->ws_mu);
+    if (!h->ws.empty()) {
+      // the last one given back that is large enough, else the last one
+      size_t i = h->ws.size() - 1;
+      for (size_t k = i + 1; k-- > 0;)
+        if (h->ws[k].bytes >= bytes) {
+          i = k;
+          break;
+        }
+      w = h->ws[i];
+      h->ws.erase(h->ws.begin() + (long)i);
     }
-    h->ws_bytes = c;
   }
-  *dev = h->ws;
-  *host = h->ws_host;
-  ME_CUDA(cudaHostGetDevicePointer(host_dev, h->ws_host, 0));
+  cudaError_t e = cudaSuccess;
+  if (!w.host) {
+    e = cudaHostAlloc(&w.host, 64, cudaHostAllocMapped);
+    if (e == cudaSuccess) e = cudaHostGetDevicePointer(&w.host_dev, w.host, 0);
+  }
+  if (e == cudaSuccess && w.bytes < bytes) {
+    const size_t c = std::max(bytes, (size_t)1 << 16);
+    if (w.dev) cudaFreeAsync(w.dev, st);
+    w.dev = nullptr;
+    w.bytes = 0;
+    e = cudaMallocAsync(&w.dev, c, st);
+    if (e == cudaSuccess) w.bytes = c;
+    else w.dev = nullptr;
+  }
+  if (e != cudaSuccess) {
+    me_internal_workspace_give(h, w, st);
+    return fail(ME_ERR_OOM, std::string("workspace allocation failed: ") + cudaGetErrorString(e));
+  }
+  *out = w;
   return ME_OK;
+}
+
+void me_internal_workspace_give(me_handle* h, Workspace w, cudaStream_t st) {
+  if (w.bytes > kWorkspaceBytes) {
+    cudaFreeAsync(w.dev, st);
+    w.dev = nullptr;
+    w.bytes = 0;
+  }
+  if (w.host) {
+    std::lock_guard<std::mutex> lk(h->ws_mu);
+    if (h->ws.size() < kWorkspaces) {
+      h->ws.push_back(w);
+      return;
+    }
+  }
+  if (w.dev) cudaFreeAsync(w.dev, st);
+  if (w.host) cudaFreeHost(w.host);
 }
 
 int me_internal_rescued_async(me_handle* h, int* dst) {

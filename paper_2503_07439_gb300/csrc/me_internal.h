@@ -23,9 +23,18 @@ extern "C" void me_internal_fail_stage(int stage);
 // Final-state masses of the handle's process (outgoing legs in order; at most 4), their
 // number, and the handle's stream.
 int me_internal_final_masses(me_handle* h, double* masses, int* n_out, cudaStream_t* stream);
-// Device workspace of at least `bytes` that the handle keeps between calls (grown on demand;
-// its contents do not survive growth), and 64 B of mapped host memory with its device address.
-int me_internal_workspace(me_handle* h, size_t bytes, void** dev, void** host, void** host_dev);
+// A workspace for one call: device memory of at least `bytes` (stream-ordered on `st`) and 64 B of
+// mapped host memory with its device address.  Each call takes its own, so that several
+// threads can use one handle, and gives it back once `st` has finished with it; the handle keeps
+// a few for later calls and releases the others.
+struct Workspace {
+  void* dev;
+  size_t bytes;
+  void* host;
+  void* host_dev;
+};
+int me_internal_workspace_take(me_handle* h, size_t bytes, cudaStream_t st, Workspace* out);
+void me_internal_workspace_give(me_handle* h, Workspace w, cudaStream_t st);
 // Process id (index into the library's process table) of a name, or -1.
 int me_internal_process_id(const char* name);
 // Process id of a handle, or -1 for NULL.

@@ -424,9 +424,9 @@ __global__ void __launch_bounds__(FKS_THREADS) k_fks_points(uint64_t seed, uint3
 // The decision is u w_max < |w| in float64, but float64 instructions run at 1/64 of the
 // float32 rate, so it is taken in float32 first, from the leading bits of u and |w|, and in
 // float64 only where the two sides are within 1e-6 relative or 1e-8 (the leading 27 bits of
-// u) of each other, or not ordinary numbers: the same decisions.  The
-// workspace stays with the handle (allocating and freeing it from the pool took most of a
-// call).  2^20 weights against their maximum, the events filled in by the caller: 365 us
+// u) of each other, or not ordinary numbers: the same decisions.  A call
+// takes its workspace from those that the handle keeps (allocating and freeing it from the pool
+// took most of a call).  2^20 weights against their maximum, the events filled in by the caller: 365 us
 // before, 105 us.
 constexpr int UW_THREADS = 256;
 constexpr int UW_ITEMS = 8;                       // points per thread
@@ -725,14 +725,24 @@ extern "C" int me_unweight(me_handle* h, const double* weights, int64_t n, doubl
   cudaStream_t st = nullptr;
   const int rc = me_internal_final_masses(h, masses, &nout, &st);  // the handle's device and stream
   if (rc != ME_OK) return rc;
-  // workspace kept by the handle: counters, per-block counts, one bit per point, and the
-  // result in mapped host memory
+  // allocation and the wait below are allowed while another thread captures a stream, in any mode
+  struct Relaxed {
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    Relaxed() { cudaThreadExchangeStreamCaptureMode(&mode); }
+    ~Relaxed() { cudaThreadExchangeStreamCaptureMode(&mode); }
+  } relaxed;
+  cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(st, &capturing) != cudaSuccess || capturing != cudaStreamCaptureStatusNone) {
+    cudaGetLastError();
+    return me_internal_fail(ME_ERR_CUDA, "me_unweight: the handle's stream is being captured");
+  }
+  // workspace: counters, per-block counts, one bit per point, and the result in mapped host memory
   const long nb = (long)((n + UW_TILE - 1) / UW_TILE), nw = (long)((n + 31) / 32);
-  char* ws = nullptr;
-  void *host = nullptr, *host_dev = nullptr;
   const size_t counts_at = 64, bits_at = counts_at + ((size_t)nb * sizeof(int) + 63) / 64 * 64;
-  int rcw = me_internal_workspace(h, bits_at + (size_t)nw * sizeof(unsigned), (void**)&ws, &host, &host_dev);
+  Workspace space{};
+  const int rcw = me_internal_workspace_take(h, bits_at + (size_t)nw * sizeof(unsigned), st, &space);
   if (rcw != ME_OK) return rcw;
+  char* ws = (char*)space.dev;
   UwArgs a{weights, (long)n, w_max, seed, stream, (long long)first_point, (UwCounters*)ws, (int*)(ws + counts_at),
            (unsigned*)(ws + bits_at)};
   cudaError_t e = cudaMemsetAsync(ws, 0, sizeof(UwCounters), st);
@@ -741,19 +751,21 @@ extern "C" int me_unweight(me_handle* h, const double* weights, int64_t n, doubl
     k_uw_absmax<<<g, UW_THREADS, 0, st>>>(weights, (long)n, &a.ctr->max_bits);
   }
   if (e == cudaSuccess) {
-    k_uw_decide<<<(unsigned)nb, UW_THREADS, 0, st>>>(a, (UwResult*)host_dev);
+    k_uw_decide<<<(unsigned)nb, UW_THREADS, 0, st>>>(a, (UwResult*)space.host_dev);
     k_uw_write<<<(unsigned)nb, UW_THREADS, 0, st>>>(a, kept, kept_weights);
     e = cudaGetLastError();
   }
-  if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+  const cudaError_t es = cudaStreamSynchronize(st);
+  if (e == cudaSuccess) e = es;
+  const UwResult res = *(const UwResult*)space.host;
+  me_internal_workspace_give(h, space, st);
   if (e != cudaSuccess)
     return me_internal_fail(ME_ERR_CUDA, (std::string("me_unweight: ") + cudaGetErrorString(e)).c_str());
-  const UwResult* r = (const UwResult*)host;
-  *n_kept = (int64_t)r->n_kept;
-  if (n_over) *n_over = (int64_t)r->n_over;
+  *n_kept = (int64_t)res.n_kept;
+  if (n_over) *n_over = (int64_t)res.n_over;
   if (w_max_used) {
     double wm = w_max;
-    if (!(w_max > 0.0)) std::memcpy(&wm, &r->max_bits, sizeof wm);
+    if (!(w_max > 0.0)) std::memcpy(&wm, &res.max_bits, sizeof wm);
     *w_max_used = wm;
   }
   return ME_OK;
