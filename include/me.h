@@ -115,13 +115,14 @@ extern "C" {
  *                    stability test and float64 item rescue).  Tree-level entries
  *                    (me_eval_born, me_eval_nbody_nlo) queue the points that pass the cuts.
  *                    Results agree with ME_TERMS_MASKED to rounding.  ME_TERMS_AUTO
- *                    (default) takes the queues for mixed-precision batches of at least
- *                    2^19 points, for e+e- -> u ubar g only if cuts are set (on GB300 they
- *                    are faster there, and slower on small batches, whose extra launches
- *                    do not amortise), and the masked evaluation otherwise; queued_rescue 1 or rescue
- *                    ME_RESCUE_POINTS, options of the masked evaluation, select it.  With
- *                    ME_TERMS_QUEUED the queues always run their item rescue.  The allocation-free entry and the
- *                    persistent serving kernels always run the masked evaluation.
+ *                    (default) takes the queues for mixed-precision batches of 2^19 to
+ *                    2^29 - 1 points (their limit), for e+e- -> u ubar g only if cuts are
+ *                    set (on GB300 they are faster there, and slower on small batches, whose
+ *                    extra launches do not amortise), and the masked evaluation otherwise;
+ *                    queued_rescue 1 or rescue ME_RESCUE_POINTS, options of the masked
+ *                    evaluation, select it.  With ME_TERMS_QUEUED the queues always run their
+ *                    item rescue.  The allocation-free entry and the persistent serving kernels
+ *                    always run the masked evaluation.
  *   cut_pt_min, cut_abs_y_max
  *                    cuts on both heavy quarks (legs 2, 3 of the t tbar processes and of
  *                    their Born counter-events): p_T >= cut_pt_min [GeV] and |rapidity

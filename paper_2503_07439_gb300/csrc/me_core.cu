@@ -590,15 +590,16 @@ static cudaError_t launch_rescue(me_handle* h, const LaunchArgs& a, int lpe64) {
 // against 2.41 ms masked, with cuts 2.03 and 2.29; u ubar -> t tbar g 1.30 and 1.30, with cuts 1.27
 // and 1.33), except for e+e- -> u ubar g without cuts, whose amplitude costs less than queueing it
 // (2^20: 0.565 ms queued, 0.461 masked; with cuts 0.389 and 0.430).
-constexpr int64_t kTermsAutoMin = (int64_t)1 << 19;
+// Their records encode slot * 4 + block in 32 bits: larger calls stay on the masked evaluation, and
+// are refused where the queues are asked for.
+constexpr int64_t kTermsAutoMin = (int64_t)1 << 19, kTermsEnd = (int64_t)1 << 29;
 static Cuts cuts_of(int pid, const me_params* p);
-static bool use_terms(const me_handle* h, int64_t n) {
-  const int t = h->prm.term_queues;
+static bool use_terms(int pid, const me_params* p, int64_t n) {
   // the automatic choice leaves the masked path's own rescue options (whole points, the
   // per-block queue) to the masked path
-  return t == ME_TERMS_QUEUED ||
-         (t == ME_TERMS_AUTO && h->prm.precision == ME_PREC_MIXED && n >= kTermsAutoMin && h->prm.queued_rescue == 0 &&
-          h->prm.rescue == ME_RESCUE_ITEMS && (h->proc->pid != P_EE_UUG || cuts_of(h->proc->pid, &h->prm).mask));
+  return p->term_queues == ME_TERMS_QUEUED ||
+         (p->term_queues == ME_TERMS_AUTO && p->precision == ME_PREC_MIXED && n >= kTermsAutoMin && n < kTermsEnd &&
+          p->queued_rescue == 0 && p->rescue == ME_RESCUE_ITEMS && (pid != P_EE_UUG || cuts_of(pid, p).mask));
 }
 
 // Per-term queues of the subtracted real: float64 pass, reals and recombination.
@@ -916,11 +917,10 @@ static int run(me_handle* h, int kind, double nlo_factor, const double* momenta,
   a.resc_count = h->d_nresc;
   a.tiles = h->d_nresc + 1;
   a.ticket = h->d_nresc + CNT_TICKET;
-  const bool terms = kind == K_REAL && use_terms(h, n);
+  const bool terms = kind == K_REAL && use_terms(h->proc->pid, &h->prm, n);
   const bool cut_list = kind == K_TREE && h->prm.term_queues == ME_TERMS_QUEUED && a.kp.cut.mask;
   const bool queued = kind == K_REAL && mixed && h->prm.queued_rescue && !terms;
-  // the queues encode slot * 4 + block in 32 bits
-  if (terms && n >= (int64_t)1 << 29) return fail(ME_ERR_ARG, "term_queues: at most 2^29 - 1 points per call");
+  if (terms && n >= kTermsEnd) return fail(ME_ERR_ARG, "term_queues: at most 2^29 - 1 points per call");
   if (terms && (rc = ensure_term_capacity(h, (size_t)n)) != ME_OK) return rc;
   // host momenta read in place: the float64 pass copies them to the device for the item
   // kernels, so that they cross the CPU-GPU link once
@@ -1127,8 +1127,8 @@ int me_internal_prepare_counted(me_handle* h, int me_kind, int64_t cap) {
     return fail(ME_ERR_ARG, "counted launch: run one ordinary call of this kind first");
   ME_CUDA(cudaSetDevice(h->device));
   int rc = ensure_capacity(h, (size_t)cap);
-  if (rc == ME_OK && kind == K_REAL && use_terms(h, cap)) {
-    if (cap >= (int64_t)1 << 29) return fail(ME_ERR_ARG, "term_queues: at most 2^29 - 1 points per call");
+  if (rc == ME_OK && kind == K_REAL && use_terms(h->proc->pid, &h->prm, cap)) {
+    if (cap >= kTermsEnd) return fail(ME_ERR_ARG, "term_queues: at most 2^29 - 1 points per call");
     rc = ensure_term_capacity(h, (size_t)cap);
     if (rc == ME_OK && mixed) rc = ensure_item_capacity(h, (size_t)cap);
     return rc;
@@ -1159,7 +1159,7 @@ int me_internal_launch_counted(me_handle* h, int me_kind, const double* d_p, con
   a.resc_count = h->d_nresc;
   a.tiles = h->d_nresc + 1;
   a.ticket = h->d_nresc + CNT_TICKET;
-  const bool terms = kind == K_REAL && use_terms(h, cap);
+  const bool terms = kind == K_REAL && use_terms(h->proc->pid, &h->prm, cap);
   const bool cut_list = kind == K_TREE && h->prm.term_queues == ME_TERMS_QUEUED && a.kp.cut.mask;
   const bool queued = kind == K_REAL && mixed && h->prm.queued_rescue && !terms;
   h->last_kind = K_TREE;
@@ -1176,6 +1176,12 @@ int me_internal_launch_counted(me_handle* h, int me_kind, const double* d_p, con
   }
   ME_CUDA(launch_call(h, CallPlan{kind, mixed, terms, queued, cut_list, lpe, lpe64}, a, nullptr));
   return ME_OK;
+}
+
+int me_internal_term_queues(const char* process, const me_params* params, int64_t n) {
+  const int pid = process ? me_internal_process_id(process) : -1;
+  if (!params || (pid != P_EE_UUG && pid != P_GG_TTG && pid != P_UU_TTG)) return -1;
+  return use_terms(pid, params, n) ? 1 : 0;
 }
 
 void me_internal_fail_stage(int stage) { g_fail_stage = stage; }

@@ -16,6 +16,9 @@ int me_internal_rescued_async(me_handle* h, int* dst);
 int me_internal_prepare_counted(me_handle* h, int me_kind, int64_t cap);
 int me_internal_launch_counted(me_handle* h, int me_kind, const double* d_p, const double* d_w, int64_t cap,
                                const int* d_n, double* d_out);
+// Whether a subtracted-real call of n points runs the per-term queues (1), the masked evaluation (0),
+// or is not defined (-1); a rule on the arguments alone.
+extern "C" int me_internal_term_queues(const char* process, const me_params* params, int64_t n);
 // Failure injection on the host, for tests: the calling thread's next evaluation of a handle
 // reports a launch failure in place of its main kernel (stage 1), its float64 rescue (2) or its
 // reduction (3), with what comes before launched and nothing after.
