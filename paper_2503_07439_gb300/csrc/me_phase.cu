@@ -257,11 +257,16 @@ __device__ __forceinline__ void boost_vel(const double p[4], const double b[3], 
 // The flat channel's RAMBO and the sectors' maps are different code, each some 300 to 500
 // float64 instructions, and the channel is random: with a point per lane every warp would run
 // both.  Each block therefore sorts its points by channel first (a scan over u0's decisions in
-// shared memory), so that one of its eight warps at most runs both.  500,009 g g -> t tbar g
-// points: 1181 us before (float64 pipe 88 % busy), 466 us.
-constexpr int FKS_THREADS = 256;
+// shared memory), so that one of its warps at most runs both.  500,009 g g -> t tbar g
+// points: 1181 us before (float64 pipe 88 % busy), 466 us with eight warps in a block.
+// While blocks of four warps fit on the SMs one each (19,456 points), every scheduler's float64
+// pipe has a single warp, and a call takes one warp's serial chain: 8192 points 24.6 us for
+// e+e- -> u ubar g and 31 us for g g -> t tbar g.  With eight warps two share each pipe: 32.8 and
+// 43 us (30.7 and 49 us without the sort).
+constexpr int FKS_WIDE = 256, FKS_NARROW = 128;
+constexpr int64_t FKS_NARROW_POINTS = 152 * FKS_NARROW;
 
-template <bool ISR>
+template <bool ISR, int FKS_THREADS>
 __global__ void __launch_bounds__(FKS_THREADS) k_fks_points(uint64_t seed, uint32_t stream, long long first, double rs,
                                                             double mass, double w3_massless, long n,
                                                             double* __restrict__ p, double* __restrict__ wgt) {
@@ -697,12 +702,14 @@ extern "C" int me_generate_fks(me_handle* h, uint64_t seed, uint32_t stream, int
   if (!(2.0 * mass < sqrt_s)) return me_internal_fail(ME_ERR_ARG, "me_generate_fks: sqrt_s below the final-state masses");
   // massless three-body volume (2 pi)^(4-3n) (pi/2)^(n-1) s^(n-2) / ((n-1)! (n-2)!) = s / (256 pi^3)
   const double w3 = sqrt_s * sqrt_s / (256.0 * M_PI * M_PI * M_PI);
-  const int threads = FKS_THREADS;
+  const bool narrow = n <= FKS_NARROW_POINTS;
+  const int threads = narrow ? FKS_NARROW : FKS_WIDE;
   const unsigned blocks = (unsigned)((n + threads - 1) / threads);
-  if (isr)
-    k_fks_points<true><<<blocks, threads, 0, st>>>(seed, stream, first_point, sqrt_s, mass, w3, n, momenta, ps_weights);
-  else
-    k_fks_points<false><<<blocks, threads, 0, st>>>(seed, stream, first_point, sqrt_s, mass, w3, n, momenta, ps_weights);
+  auto launch = [&](auto kernel) {
+    kernel<<<blocks, threads, 0, st>>>(seed, stream, first_point, sqrt_s, mass, w3, n, momenta, ps_weights);
+  };
+  if (narrow) launch(isr ? k_fks_points<true, FKS_NARROW> : k_fks_points<false, FKS_NARROW>);
+  else launch(isr ? k_fks_points<true, FKS_WIDE> : k_fks_points<false, FKS_WIDE>);
   const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return me_internal_fail(ME_ERR_CUDA, (std::string("me_generate_fks: ") + cudaGetErrorString(e)).c_str());
   return ME_OK;
