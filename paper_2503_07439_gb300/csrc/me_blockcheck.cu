@@ -2,7 +2,8 @@
 // test suite; no GPU needed).  For every point read from stdin it evaluates the
 // colour-summed |M|^2 twice with the same templates the kernels use: over every
 // helicity one at a time, and over the blocks of one member of each flipped pair
-// (doubled), in float64 and in float32.  It prints one line per point:
+// (doubled; for processes without a block routine, the helicities of those blocks), in float64 and
+// in float32.  It prints one line per point:
 //   <block fp64> <single fp64> <block fp32> <single fp32>
 // With the arguments "kernels <mt>" it prints what the kernels evaluate instead -- block_sum over
 // the live blocks, or the closed form of a 2 -> 2 tree, at unit couplings and scaled in
@@ -17,6 +18,7 @@
 
 #include "me_internal.h"
 #include "me_kernels.cuh"
+#include "me_single.cuh"
 
 using namespace me;
 
@@ -52,22 +54,28 @@ static void eval(const ColourTables& tab, const r4<double>* k, const Couplings& 
     s += csum<PID, T>(tab, J);
   }
   double b = 0;
-  for (int i = 0; i < n_live_blocks<PID>(); ++i)
-    amplitude_block<PID, T>(K, live_block_hel<PID>(i), cp, [&](int, const cx<T>* A) { b += bsum<PID, T>(tab, A); });
+  for (int i = 0; i < n_live_blocks<PID>(); ++i) {
+    auto add = [&](int, const cx<T>* A) { b += bsum<PID, T>(tab, A); };
+    if constexpr (closed_tree<PID>() || PID == P_EE_UUG) single_block<PID, T>(K, live_block_hel<PID>(i), cp, add);
+    else amplitude_block<PID, T>(K, live_block_hel<PID>(i), cp, add);
+  }
   *blk = 2.0 * b;
   *single = s;
 }
 
 template <int PID, typename T>
 static double kernel_value(const ColourTables& tab, const r4<double>* k, const Couplings& cp) {
-  if constexpr (closed_tree<PID>()) return (double)closed_sum<PID, T>(k, unit_couplings(cp)) * tree_coupling(PID, cp);
-  KParams kp{};
-  kp.cp = cp;
-  kp.tab = &tab;
-  const Kin<PID, T> K = prepare<PID, T>(k, unit_couplings(cp));
-  T acc = T(0);
-  for (int b = 0; b < n_live_blocks<PID>(); ++b) acc += block_sum<PID, T>(K, b, kp);
-  return 2.0 * (double)acc * tree_coupling(PID, cp);
+  if constexpr (closed_tree<PID>()) {
+    return (double)closed_sum<PID, T>(k, unit_couplings(cp)) * tree_coupling(PID, cp);
+  } else {
+    KParams kp{};
+    kp.cp = cp;
+    kp.tab = &tab;
+    const Kin<PID, T> K = prepare<PID, T>(k, unit_couplings(cp));
+    T acc = T(0);
+    for (int b = 0; b < n_live_blocks<PID>(); ++b) acc += block_sum<PID, T>(K, b, kp);
+    return 2.0 * (double)acc * tree_coupling(PID, cp);
+  }
 }
 
 static double g_mt = 0.0;  // > 0: the kernels' values with this top mass

@@ -746,11 +746,6 @@ static int choose_lpe(me_handle* h, int kind, bool fp64, const LaunchArgs& a) {
   return slot = pick;
 }
 
-static void set_tolerances(KParams& kp, const me_params* p) {
-  // tol <= 0 flags every point that has an error scale, me_eps <= 0 none
-  kp.tol_eps = p->me_eps <= 0.0 ? DBL_MAX : p->tol > 0.0 && p->me_eps > 0.0 ? p->tol / p->me_eps : 0.0;
-}
-
 // The cuts of me_params as the kernels take them (Cuts in me_kernels.cuh), for process pid.
 static bool cuts_valid(const me_params* p) {
   return std::isfinite(p->cut_pt_min) && p->cut_pt_min >= 0.0 && p->cut_abs_y_max > 0.0 &&
@@ -781,6 +776,23 @@ static Cuts cuts_of(int pid, const me_params* p) {
     }
   }
   return c;
+}
+
+// Kernel parameters of a process (table pointer unset).
+static KParams kernel_params(const ProcDesc& pd, const me_params* p) {
+  KParams kp{};
+  kp.cp = Couplings(std::sqrt(4.0 * M_PI * p->alpha_s), std::sqrt(4.0 * M_PI * p->alpha), p->mt);
+  kp.tree_scale = 1.0 / pd.avg * tree_coupling(pd.pid, kp.cp);
+  kp.real_scale = 2.0 * kp.tree_scale;
+  if (pd.born_pid >= 0) kp.born_scale = tree_coupling(pd.born_pid, kp.cp) * (1.0 / kProcs[pd.born_pid].avg);
+  kp.xi_cut = p->xi_cut;
+  kp.delta = p->delta;
+  kp.xi_thr = p->xi_thr;
+  kp.y_thr = p->y_thr;
+  // tol <= 0 flags every point that has an error scale, me_eps <= 0 none
+  kp.tol_eps = p->me_eps <= 0.0 ? DBL_MAX : p->tol > 0.0 && p->me_eps > 0.0 ? p->tol / p->me_eps : 0.0;
+  kp.cut = cuts_of(pd.pid, p);
+  return kp;
 }
 
 extern "C" {
@@ -846,21 +858,8 @@ int me_init(const char* process, const me_params* params, me_handle** out) {
     me_destroy(h);
     return fail(ME_ERR_OOM, "me_init: allocation failed");
   }
-  KParams& kp = h->kp;
-  kp = KParams{};
-  kp.cp = Couplings(std::sqrt(4.0 * M_PI * params->alpha_s), std::sqrt(4.0 * M_PI * params->alpha), params->mt);
-  kp.avg_inv = 1.0 / pd->avg;
-  kp.born_avg_inv = pd->born_pid >= 0 ? 1.0 / kProcs[pd->born_pid].avg : 0.0;
-  kp.tree_scale = kp.avg_inv * tree_coupling(pd->pid, kp.cp);
-  kp.real_scale = 2.0 * kp.tree_scale;
-  if (pd->born_pid >= 0) kp.born_scale = tree_coupling(pd->born_pid, kp.cp) * kp.born_avg_inv;
-  kp.xi_cut = params->xi_cut;
-  kp.delta = params->delta;
-  kp.xi_thr = params->xi_thr;
-  kp.y_thr = params->y_thr;
-  set_tolerances(kp, params);
-  kp.cut = cuts_of(pd->pid, params);
-  kp.tab = d_tab;
+  h->kp = kernel_params(*pd, params);
+  h->kp.tab = d_tab;
   // stream-ordered on the handle's own stream: no device-wide synchronisation, so a
   // handle can be created while other threads capture CUDA graphs
   if (cudaMemsetAsync(h->d_acc, 0, 3 * sizeof(double), h->own_stream) != cudaSuccess ||
@@ -1286,19 +1285,7 @@ int me_internal_kparams(const char* process, const me_params* params, me::KParam
   for (const auto& d : kProcs)
     if (std::strcmp(d.name, process) == 0) pd = &d;
   if (!pd) return fail(ME_ERR_PROCESS, std::string("unknown process ") + process);
-  *kp = KParams{};
-  kp->cp = Couplings(std::sqrt(4.0 * M_PI * params->alpha_s), std::sqrt(4.0 * M_PI * params->alpha), params->mt);
-  kp->avg_inv = 1.0 / pd->avg;
-  kp->born_avg_inv = pd->born_pid >= 0 ? 1.0 / kProcs[pd->born_pid].avg : 0.0;
-  kp->tree_scale = kp->avg_inv * tree_coupling(pd->pid, kp->cp);
-  kp->real_scale = 2.0 * kp->tree_scale;
-  if (pd->born_pid >= 0) kp->born_scale = tree_coupling(pd->born_pid, kp->cp) * kp->born_avg_inv;
-  kp->xi_cut = params->xi_cut;
-  kp->delta = params->delta;
-  kp->xi_thr = params->xi_thr;
-  kp->y_thr = params->y_thr;
-  set_tolerances(*kp, params);
-  kp->cut = cuts_of(pd->pid, params);
+  *kp = kernel_params(*pd, params);
   *pid = pd->pid;
   return ME_OK;
 }

@@ -45,11 +45,8 @@ static double block_ops(const r4<double>* p, int hb = 1) {
   const Kin<PID, Flop> K = prepare<PID, Flop>(p, cp);
   g_ops = 0;
   int calls = 0;
-  if constexpr (PID == P_EE_UUG) {
-    ee_uug_block(K, 0);
-    return (double)g_ops;
-  }
-  amplitude_block<PID, Flop>(K, hb, cp, [&](int, const cx<Flop>*) { ++calls; });
+  if constexpr (PID == P_EE_UUG) ee_uug_block(K, 0);
+  else amplitude_block<PID, Flop>(K, hb, cp, [&](int, const cx<Flop>*) { ++calls; });
   return (double)g_ops + calls * colour_flops(Proc<PID>::NFLOW);
 }
 
@@ -71,10 +68,11 @@ static double born_ops(const r4<double>* p) {
     g_ops = 0;
     closed_sum<PID, Flop>(p, Couplings{1.2, 0.3, 173.0});
     return (double)g_ops;
+  } else {
+    double t = prep_ops<PID>(p);
+    for (int b = 0; b < n_live_blocks<PID>(); ++b) t += block_ops<PID>(p, live_block_hel<PID>(b));
+    return t;
   }
-  double t = prep_ops<PID>(p);
-  for (int b = 0; b < n_live_blocks<PID>(); ++b) t += block_ops<PID>(p, live_block_hel<PID>(b));
-  return t;
 }
 
 int main() {

@@ -10,7 +10,8 @@
 // these tree amplitudes with real couplings (pinned against the oracle).  A helicity
 // block (me_procs.cuh) is one configuration of the other legs with the four helicities
 // of the heavy pair, evaluated with shared gluon currents and quark-line rows; the 2 -> 2
-// trees and the counterterms' Borns are closed forms in float64.  Born, real, soft and
+// trees are closed forms (their invariants in float64), and so are the counterterms' Borns, in
+// float64 throughout.  Born, real, soft and
 // collinear terms are evaluated for every point and masked afterwards (Sec. 4.3, Algorithm 2),
 // so a warp never diverges on cuts, or through the per-term queues below.
 #pragma once
@@ -64,11 +65,10 @@ struct Cuts {
 
 struct KParams {
   Couplings cp;
-  double avg_inv;       // 1 / (initial spin x colour average), x identical-particle factor
-  double born_avg_inv;  // same for the underlying Born of a real process
-  double tree_scale;    // |M|^2 at unit couplings -> weight: couplings x avg_inv x nlo_factor
+  double tree_scale;    // |M|^2 at unit couplings -> weight: couplings / (initial spin x colour average and
+                        // identical-particle factor), x the n-body NLO factor
   double real_scale;    // half helicity sum of a real block at unit couplings -> |M|^2
-  double born_scale;    // couplings of the underlying Born x born_avg_inv
+  double born_scale;    // couplings of the underlying Born / its average
   double xi_cut, delta; // FKS plus-distribution cut-offs
   double xi_thr, y_thr; // points with xi < xi_thr or 1-y < y_thr go to the FP64 path
   double tol_eps;       // tol / me_eps: target accuracy of a weight over the assumed error of a

@@ -4,7 +4,7 @@
 // Conventions (standard QFT; the paper fixes none): metric (+,-,-,-); chiral
 // gamma matrices gamma^0 = [[0,1],[1,0]], gamma^k = [[0,s^k],[-s^k,0]], so that
 //   Vslash = [[0, V0 - s.V], [V0 + s.V, 0]];
-// helicity spinors u(p,l) = (w_{-l} chi_l, w_{+l} chi_l),
+// helicity spinors (me_single.cuh) u(p,l) = (w_{-l} chi_l, w_{+l} chi_l),
 //   v(p,l) = (-l w_{+l} chi_{-l}, l w_{-l} chi_{-l}), w_+- = sqrt(E +- |p|);
 // polarisation vectors eps(k,l) = (-l e1 - i e2)/sqrt(2).
 // Everything is templated on the arithmetic type T (float for the bulk path,
@@ -41,7 +41,6 @@ struct cx {
   T re, im;
 };
 
-template <typename T> ME_HD cx<T> mk(T r, T i) { return cx<T>{r, i}; }
 template <typename T> ME_HD cx<T> operator+(cx<T> a, cx<T> b) { return {a.re + b.re, a.im + b.im}; }
 template <typename T> ME_HD cx<T> operator-(cx<T> a, cx<T> b) { return {a.re - b.re, a.im - b.im}; }
 template <typename T> ME_HD cx<T> operator-(cx<T> a) { return {-a.re, -a.im}; }
@@ -123,16 +122,6 @@ ME_HD c4<T> cneg(const c4<T>& x) {
   return o;
 }
 template <typename T>
-ME_HD void cscale(c4<T>& x, cx<T> a) {
-#pragma unroll
-  for (int i = 0; i < 4; ++i) x.v[i] = a * x.v[i];
-}
-template <typename T>
-ME_HD void cscale(c4<T>& x, T a) {
-#pragma unroll
-  for (int i = 0; i < 4; ++i) x.v[i] = a * x.v[i];
-}
-template <typename T>
 ME_HD c4<T> czero() {
   c4<T> z;
 #pragma unroll
@@ -141,93 +130,6 @@ ME_HD c4<T> czero() {
 }
 
 // ---------------------------------------------------------------- wavefunctions
-// two-component helicity eigenstate chi_lam along p/|p|; |p|+pz is formed without
-// cancellation as pt^2/(|p|-pz) when pz < 0.
-template <typename T>
-ME_HD void chi(const r4<T>& p, int lam, cx<T>& c0, cx<T>& c1) {
-  T pt2 = p.x * p.x + p.y * p.y;
-  T pa = msqrt(pt2 + p.z * p.z);
-  T s = (p.z >= T(0)) ? pa + p.z : pt2 / (pa - p.z);
-  if (s > T(0)) {
-    T rden = T(1) / msqrt(T(2) * pa * s);
-    if (lam > 0) {
-      c0 = cx<T>{s * rden, T(0)};
-      c1 = cx<T>{p.x * rden, p.y * rden};
-    } else {
-      c0 = cx<T>{-p.x * rden, p.y * rden};
-      c1 = cx<T>{s * rden, T(0)};
-    }
-  } else {  // exactly along -z
-    if (lam > 0) {
-      c0 = cx<T>{T(0), T(0)};
-      c1 = cx<T>{T(1), T(0)};
-    } else {
-      c0 = cx<T>{T(-1), T(0)};
-      c1 = cx<T>{T(0), T(0)};
-    }
-  }
-}
-
-template <typename T>
-ME_HD void omegas(const r4<T>& p, T m, T& wp, T& wm) {
-  T pa = msqrt(p.x * p.x + p.y * p.y + p.z * p.z);
-  wp = msqrt(p.e + pa);
-  wm = (m == T(0)) ? T(0) : m / wp;
-}
-
-template <typename T>
-ME_HD c4<T> spinor_u(const r4<T>& p, T m, int lam) {
-  T wp, wm;
-  omegas(p, m, wp, wm);
-  cx<T> a, b;
-  chi(p, lam, a, b);
-  T top = lam > 0 ? wm : wp, bot = lam > 0 ? wp : wm;
-  return c4<T>{{top * a, top * b, bot * a, bot * b}};
-}
-
-template <typename T>
-ME_HD c4<T> spinor_v(const r4<T>& p, T m, int lam) {
-  T wp, wm;
-  omegas(p, m, wp, wm);
-  cx<T> a, b;
-  chi(p, -lam, a, b);
-  T top = lam > 0 ? -wp : wm;   // -lam * w_{+lam}
-  T bot = lam > 0 ? wm : -wp;   //  lam * w_{-lam}
-  return c4<T>{{top * a, top * b, bot * a, bot * b}};
-}
-
-// Dirac adjoint psi^dagger gamma^0 (chiral rep: swap blocks, conjugate)
-template <typename T>
-ME_HD c4<T> dbar(const c4<T>& s) {
-  return c4<T>{{conj(s.v[2]), conj(s.v[3]), conj(s.v[0]), conj(s.v[1])}};
-}
-
-template <typename T>
-ME_HD c4<T> polvec(const r4<T>& k, int lam, bool outgoing) {
-  T pt2 = k.x * k.x + k.y * k.y;
-  T pt = msqrt(pt2);
-  T ka = msqrt(pt2 + k.z * k.z);
-  T ct = k.z / ka, st = pt / ka;
-  T cp = T(1), sp = T(0);
-  if (pt > T(0)) {
-    cp = k.x / pt;
-    sp = k.y / pt;
-  }
-  const T r2 = T(0.70710678118654752440);
-  // eps = (-lam e1 - i e2)/sqrt(2), e1 = (0, ct cp, ct sp, -st), e2 = (0, -sp, cp, 0)
-  T l = (T)lam;
-  c4<T> e;
-  e.v[0] = cx<T>{T(0), T(0)};
-  e.v[1] = cx<T>{-l * ct * cp * r2, sp * r2};
-  e.v[2] = cx<T>{-l * ct * sp * r2, -cp * r2};
-  e.v[3] = cx<T>{l * st * r2, T(0)};
-  if (outgoing) {
-#pragma unroll
-    for (int i = 1; i < 4; ++i) e.v[i] = conj(e.v[i]);
-  }
-  return e;
-}
-
 // Helicity-independent ingredients of the wavefunctions, computed once per event and
 // shared by all helicities.
 // Massive quark with spins along the light cone instead of the helicity axis (a sum over
@@ -321,31 +223,6 @@ template <typename T>
 ME_HD void row_slash_acc(c4<T>& acc, const c4<T>& r, const c4<T>& V) {
   row_slash_acc(acc, r, slashed(V));
 }
-// Vslash times column spinor
-template <typename T>
-ME_HD c4<T> slash_col(const c4<T>& V, const c4<T>& s) {
-  cx<T> a = V.v[0] - V.v[3], b = V.v[0] + V.v[3];
-  cx<T> c = V.v[1] - times_i(V.v[2]);
-  cx<T> d = V.v[1] + times_i(V.v[2]);
-  c4<T> o;
-  o.v[0] = cmsb(a * s.v[2], c, s.v[3]);
-  o.v[1] = cmsb(b * s.v[3], d, s.v[2]);
-  o.v[2] = cmac(b * s.v[0], c, s.v[1]);
-  o.v[3] = cmac(d * s.v[0], a, s.v[1]);
-  return o;
-}
-// row spinor times (Qslash + m), Q real
-template <typename T>
-ME_HD c4<T> row_prop(const c4<T>& r, const r4<T>& Q, T m) {
-  T a = Q.e - Q.z, b = Q.e + Q.z;
-  cx<T> c = cx<T>{Q.x, -Q.y}, d = cx<T>{Q.x, Q.y};
-  c4<T> o;
-  o.v[0] = cmac(b * r.v[2] + m * r.v[0], r.v[3], d);
-  o.v[1] = cmac(a * r.v[3] + m * r.v[1], r.v[2], c);
-  o.v[2] = cmsb(a * r.v[0] + m * r.v[2], r.v[1], d);
-  o.v[3] = cmsb(b * r.v[1] + m * r.v[3], r.v[0], c);
-  return o;
-}
 // s (Qslash + m) for rows, Q real: the combinations row_prop uses, formed once for a
 // propagator that closes several rows (the scale s, a coupling times the reciprocal
 // denominator, is folded in here instead of into every row)
@@ -368,33 +245,6 @@ ME_HD c4<T> row_prop(const c4<T>& r, const prop4<T>& P) {
   o.v[3] = cmsb(P.b * r.v[1] + P.m * r.v[3], r.v[0], P.c);
   return o;
 }
-// (-Qslash + m) times column spinor, Q real
-template <typename T>
-ME_HD c4<T> col_prop(const r4<T>& Q, T m, const c4<T>& s) {
-  T a = Q.e - Q.z, b = Q.e + Q.z;
-  cx<T> c = cx<T>{Q.x, -Q.y}, d = cx<T>{Q.x, Q.y};
-  c4<T> o;
-  o.v[0] = cmac(m * s.v[0] - a * s.v[2], c, s.v[3]);
-  o.v[1] = cmac(m * s.v[1] - b * s.v[3], d, s.v[2]);
-  o.v[2] = cmsb(m * s.v[2] - b * s.v[0], c, s.v[1]);
-  o.v[3] = cmsb(m * s.v[3] - a * s.v[1], d, s.v[0]);
-  return o;
-}
-// vector current J^mu = r gamma^mu s
-template <typename T>
-ME_HD c4<T> vcurrent(const c4<T>& r, const c4<T>& s) {
-  c4<T> J;
-  J.v[0] = cmac(cmac(cmac(r.v[0] * s.v[2], r.v[1], s.v[3]), r.v[2], s.v[0]), r.v[3], s.v[1]);
-  J.v[1] = cmsb(cmsb(cmac(r.v[0] * s.v[3], r.v[1], s.v[2]), r.v[2], s.v[1]), r.v[3], s.v[0]);
-  J.v[2] = times_i(cmac(cmsb(cmsb(r.v[1] * s.v[2], r.v[0], s.v[3]), r.v[3], s.v[0]), r.v[2], s.v[1]));
-  J.v[3] = cmac(cmsb(cmsb(r.v[0] * s.v[2], r.v[1], s.v[3]), r.v[2], s.v[0]), r.v[3], s.v[1]);
-  return J;
-}
-template <typename T>
-ME_HD cx<T> spdot(const c4<T>& r, const c4<T>& s) {
-  return cmac(cmac(cmac(r.v[0] * s.v[0], r.v[1], s.v[1]), r.v[2], s.v[2]), r.v[3], s.v[3]);
-}
-
 // ---------------------------------------------------------------- polarisation vectors
 // A transverse polarisation vector in the frame of the momenta has no time component and a
 // real z component: 5 reals instead of 8.  Contractions and slashes against it skip the
@@ -406,7 +256,7 @@ struct pol {
   T z;
 };
 template <typename T>
-ME_HD pol<T> pol_of(const wf_v<T>& w, int lam, bool outgoing) {  // as polvec
+ME_HD pol<T> pol_of(const wf_v<T>& w, int lam, bool outgoing) {  // as polvec (me_single.cuh)
   const T s = outgoing ? T(-1) : T(1);
   return pol<T>{{lam > 0 ? -w.ccp : w.ccp, s * w.sp}, {lam > 0 ? -w.csp : w.csp, -s * w.cp}, lam > 0 ? w.st : -w.st};
 }
@@ -655,7 +505,7 @@ template <typename T, int H> struct has_pair<axpol<T, H>, axpol<T, H>> { static 
 // ---------------------------------------------------------------- gluon vertices
 // The three-gluon bracket of two conserved currents (Q_i . J_i = 0) with outgoing momenta,
 //   s [(J1.J2)(Q2 - Q1) - 2 (Q2.J1) J2 + 2 (Q1.J2) J1],
-// which is vvv(J1, J2, -Q1, -Q2, s) with the vanishing products Q1.J1 and Q2.J2 left out.
+// which is s vvv(J1, J2, -Q1, -Q2) (me_single.cuh) with the vanishing products Q1.J1 and Q2.J2 left out.
 // `j12` receives J1.J2 of two polarisations (the four-gluon vertex needs it again).
 template <typename T, class E1, class E2>
 ME_HD c4<T> bracket(const E1& e1, const r4<T>& q1, const E2& e2, const r4<T>& q2, T s, cx<T>& j12) {
@@ -693,48 +543,6 @@ ME_HD void quartic_acc(c4<T>& acc, const L& l, const M& m, const R& r, cx<T> lr,
   caxpy(acc, T(2) * lr, m);
   caxpy(acc, -lm, r);
   caxpy(acc, -mr, l);
-}
-
-// three-gluon Lorentz structure contracted with J1_mu J2_nu, momenta k1,k2,k3 incoming:
-// W^rho = (J1.J2)(k1-k2)^rho + J2^rho (k2-k3).J1 + J1^rho (k3-k1).J2
-template <typename T>
-ME_HD c4<T> vvv(const c4<T>& J1, const c4<T>& J2, const r4<T>& k1, const r4<T>& k2) {
-  r4<T> k3 = -(k1 + k2);
-  cx<T> j12 = cdot(J1, J2);
-  cx<T> a = rdot(k2 - k3, J1);
-  cx<T> b = rdot(k3 - k1, J2);
-  r4<T> d = k1 - k2;
-  c4<T> W;
-  W.v[0] = cmac(cmac(d.e * j12, a, J2.v[0]), b, J1.v[0]);
-  W.v[1] = cmac(cmac(d.x * j12, a, J2.v[1]), b, J1.v[1]);
-  W.v[2] = cmac(cmac(d.y * j12, a, J2.v[2]), b, J1.v[2]);
-  W.v[3] = cmac(cmac(d.z * j12, a, J2.v[3]), b, J1.v[3]);
-  return W;
-}
-// s W(J1, J2), and acc + s W(J1, J2): the scale goes into the three scalar coefficients
-template <typename T>
-ME_HD c4<T> vvv(const c4<T>& J1, const c4<T>& J2, const r4<T>& k1, const r4<T>& k2, T s) {
-  r4<T> k3 = -(k1 + k2);
-  const cx<T> j12 = s * cdot(J1, J2);
-  const cx<T> a = s * rdot(k2 - k3, J1);
-  const cx<T> b = s * rdot(k3 - k1, J2);
-  r4<T> d = k1 - k2;
-  c4<T> W;
-  W.v[0] = cmac(cmac(d.e * j12, a, J2.v[0]), b, J1.v[0]);
-  W.v[1] = cmac(cmac(d.x * j12, a, J2.v[1]), b, J1.v[1]);
-  W.v[2] = cmac(cmac(d.y * j12, a, J2.v[2]), b, J1.v[2]);
-  W.v[3] = cmac(cmac(d.z * j12, a, J2.v[3]), b, J1.v[3]);
-  return W;
-}
-// colour-ordered four-gluon structure: 2(L.R) M - (L.M) R - (M.R) L
-template <typename T>
-ME_HD c4<T> vvvv_ordered(const c4<T>& L, const c4<T>& M, const c4<T>& R) {
-  cx<T> lr = cdot(L, R), lm = cdot(L, M), mr = cdot(M, R);
-  cx<T> two_lr = lr + lr;
-  c4<T> o;
-#pragma unroll
-  for (int i = 0; i < 4; ++i) o.v[i] = cmsb(cmsb(two_lr * M.v[i], lm, R.v[i]), mr, L.v[i]);
-  return o;
 }
 
 }  // namespace me

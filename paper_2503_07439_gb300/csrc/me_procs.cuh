@@ -1,7 +1,7 @@
 // Per-process colour-decomposed helicity amplitudes (device).
 //
-// Each routine returns, for one helicity configuration, the partial amplitudes
-// J_c of the process in its colour-flow basis, so that the colour-summed squared
+// Each block routine returns, for one helicity configuration after another, the partial
+// amplitudes J_c of the process in its colour-flow basis, so that the colour-summed squared
 // amplitude is J^dagger C J (Sec. 2.1, Eq. (born): |sum of diagrams|^2; Sec. 4.2:
 // Born, real and counterterms are all tree-level amplitudes).
 //
@@ -17,7 +17,9 @@
 // Momenta: all-outgoing (q = -p for incoming legs).  Everything that does not depend
 // on the helicities -- momenta in T and the reciprocal propagator denominators, whose
 // invariants are formed in float64 to avoid cancellation -- is prepared once per event
-// (prepare<PID,T>) and shared by all helicities; spinors and currents are in T.
+// (prepare<PID,T>) and shared by all helicities; spinors and currents are in T.  The 2 -> 2 processes
+// and e+e- -> u ubar g have closed forms; me_single.cuh has every process one helicity at a time, for
+// the host check.
 #pragma once
 #include <type_traits>
 
@@ -87,22 +89,6 @@ ME_HD double tree_coupling(int pid, const Couplings& c) {
   }
 }
 
-__host__ __device__ constexpr int factorial(int n) { return n <= 1 ? 1 : n * factorial(n - 1); }
-
-// permutation number `idx` (lexicographic) of {0..n-1}
-ME_HD void nth_perm(int n, int idx, int* out) {
-  int pool[4] = {0, 1, 2, 3};
-  int m = n;
-  for (int i = 0; i < n; ++i) {
-    int f = factorial(m - 1);
-    int k = idx / f;
-    idx -= k * f;
-    out[i] = pool[k];
-    for (int j = k; j < m - 1; ++j) pool[j] = pool[j + 1];
-    --m;
-  }
-}
-
 ME_HD int hel_of(int hel, int leg) { return ((hel >> leg) & 1) ? 1 : -1; }
 
 // ----------------------------------------------------------------------------
@@ -166,208 +152,6 @@ ME_HD KinTT<T, NG> prep_tt(const r4<double>* p, const Couplings& cp) {
   }
   K.ig[0] = K.iq[0] = T(0);
   return K;
-}
-
-// Generic colour-ordered recursion (used for 4 gluons): for every ordering, contiguous
-// gluon currents J[i][j] and the top line U[k]; denominators from the per-event table.
-template <typename T, int NG>
-ME_HD void amp_ttng(const KinTT<T, NG>& K, int hel, const Couplings& cp, cx<T>* A) {
-  constexpr int NF = factorial(NG);
-  const T g = gs_of<T>(cp);
-  const T mt = mt_of<T>(cp);
-  c4<T> eps[NG];
-#pragma unroll
-  for (int i = 0; i < NG; ++i) {
-    const int l = i < 2 ? i : i + 2;
-    eps[i] = polvec(K.pl[l], hel_of(hel, l), l >= 2);
-  }
-  const c4<T> ub = dbar(spinor_u(K.pl[2], mt, hel_of(hel, 2)));
-  const c4<T> vb = spinor_v(K.pl[3], mt, hel_of(hel, 3));
-  for (int f = 0; f < NF; ++f) {
-    int s[NG];
-    nth_perm(NG, f, s);
-    c4<T> J[NG][NG];
-    r4<T> Q[NG][NG];
-    int M[NG][NG];
-#pragma unroll
-    for (int i = 0; i < NG; ++i) {
-      J[i][i] = eps[s[i]];
-      Q[i][i] = K.q[s[i]];
-      M[i][i] = 1 << s[i];
-    }
-#pragma unroll
-    for (int len = 2; len <= NG; ++len) {
-#pragma unroll
-      for (int i = 0; i + len - 1 < NG; ++i) {
-        const int j = i + len - 1;
-        Q[i][j] = Q[i][j - 1] + K.q[s[j]];
-        M[i][j] = M[i][j - 1] | (1 << s[j]);
-        const T inv = K.ig[M[i][j]];
-        c4<T> acc = czero<T>();
-#pragma unroll
-        for (int k = i; k < j; ++k) cadd(acc, vvv(J[i][k], J[k + 1][j], -Q[i][k], -Q[k + 1][j]));
-        cscale(acc, -g * inv);
-        if (len >= 3) {
-          c4<T> acc4 = czero<T>();
-#pragma unroll
-          for (int k = i; k < j - 1; ++k)
-#pragma unroll
-            for (int l = k + 1; l < j; ++l) cadd(acc4, vvvv_ordered(J[i][k], J[k + 1][l], J[l + 1][j]));
-          caxpy(acc, cx<T>{g * g * inv, T(0)}, acc4);
-        }
-        J[i][j] = acc;
-      }
-    }
-    c4<T> U[NG];
-    U[0] = ub;
-    r4<T> Qu = K.pl[2];
-#pragma unroll
-    for (int k = 1; k < NG; ++k) {
-      Qu = Qu + K.q[s[k - 1]];
-      c4<T> acc = czero<T>();
-#pragma unroll
-      for (int j = 0; j < k; ++j) cadd(acc, row_slash(U[j], J[j][k - 1]));
-      c4<T> pr = row_prop(acc, Qu, mt);
-      cscale(pr, -g * K.iq[M[0][k - 1]]);
-      U[k] = pr;
-    }
-    cx<T> a = cx<T>{T(0), T(0)};
-#pragma unroll
-    for (int j = 0; j < NG; ++j) a = a + spdot(row_slash(U[j], J[j][NG - 1]), vb);
-    A[f] = times_i(a) * g;
-  }
-}
-
-// t tbar + 2 or 3 gluons with every sub-current computed once per helicity.
-// Colour-ordered currents obey the reflection identity J(s reversed) = (-1)^(k+1) J(s)
-// for k gluons (V3 is antisymmetric in its two legs, the ordered V4 symmetric in its
-// outer legs), so J(yx) = -J(xy) and J(zyx) = J(xyz); the quark currents U(x), U(xy)
-// and the amplitudes of all orderings then reuse them.  Orderings are numbered
-// lexicographically as in amp_ttng, so the colour basis is the same.
-template <typename T>
-ME_HD void amp_tt2_fast(const KinTT<T, 2>& K, int hel, const Couplings& cp, cx<T>* A) {
-  const T g = gs_of<T>(cp), mt = mt_of<T>(cp);
-  const r4<T> k0 = K.q[0], k1 = K.q[1], kt = K.pl[2];
-  const c4<T> e0 = polvec(K.pl[0], hel_of(hel, 0), false);
-  const c4<T> e1 = polvec(K.pl[1], hel_of(hel, 1), false);
-  const c4<T> ub = dbar(spinor_u(kt, mt, hel_of(hel, 2)));
-  const c4<T> vb = spinor_v(K.pl[3], mt, hel_of(hel, 3));
-  c4<T> J01 = vvv(e0, e1, -k0, -k1);
-  cscale(J01, -g * K.ig[3]);
-  const cx<T> s01 = spdot(row_slash(ub, J01), vb);
-  c4<T> U0 = row_prop(row_slash(ub, e0), kt + k0, mt);
-  cscale(U0, -g * K.iq[1]);
-  c4<T> U1 = row_prop(row_slash(ub, e1), kt + k1, mt);
-  cscale(U1, -g * K.iq[2]);
-  // A(01) = ig[ub J01 v + U0 e1 v],  A(10) = ig[-ub J01 v + U1 e0 v]
-  A[0] = times_i(s01 + spdot(row_slash(U0, e1), vb)) * g;
-  A[1] = times_i(spdot(row_slash(U1, e0), vb) - s01) * g;
-}
-
-template <typename T>
-ME_HD void amp_tt3_fast(const KinTT<T, 3>& K, int hel, const Couplings& cp, cx<T>* A) {
-  const T g = gs_of<T>(cp), mt = mt_of<T>(cp);
-  const r4<T> k0 = K.q[0], k1 = K.q[1], k2 = K.q[2], kt = K.pl[2];
-  const c4<T> e0 = polvec(K.pl[0], hel_of(hel, 0), false);
-  const c4<T> e1 = polvec(K.pl[1], hel_of(hel, 1), false);
-  const c4<T> e2 = polvec(K.pl[4], hel_of(hel, 4), true);
-  const c4<T> ub = dbar(spinor_u(kt, mt, hel_of(hel, 2)));
-  const c4<T> vb = spinor_v(K.pl[3], mt, hel_of(hel, 3));
-  // pair currents J(xy), x<y; J(yx) = -J(xy)
-  c4<T> J01 = vvv(e0, e1, -k0, -k1);
-  cscale(J01, -g * K.ig[3]);
-  c4<T> J02 = vvv(e0, e2, -k0, -k2);
-  cscale(J02, -g * K.ig[5]);
-  c4<T> J12 = vvv(e1, e2, -k1, -k2);
-  cscale(J12, -g * K.ig[6]);
-  // three-gluon currents F(abc) = F(cba): -(g/Q^2)[V3(a, bc) + V3(ab, c)] + (g^2/Q^2) V4(a,b,c)
-  const T c3 = -g * K.ig[7], c4g = g * g * K.ig[7];
-  cx<T> a[6];
-  {
-    c4<T> F = vvv(e0, J12, -k0, -(k1 + k2));
-    cadd(F, vvv(J01, e2, -(k0 + k1), -k2));
-    cscale(F, c3);
-    caxpy(F, cx<T>{c4g, T(0)}, vvvv_ordered(e0, e1, e2));
-    a[0] = a[5] = spdot(row_slash(ub, F), vb);  // 012, 210
-  }
-  {
-    c4<T> mJ12 = J12;
-    cscale(mJ12, T(-1));
-    c4<T> F = vvv(e0, mJ12, -k0, -(k1 + k2));
-    cadd(F, vvv(J02, e1, -(k0 + k2), -k1));
-    cscale(F, c3);
-    caxpy(F, cx<T>{c4g, T(0)}, vvvv_ordered(e0, e2, e1));
-    a[1] = a[3] = spdot(row_slash(ub, F), vb);  // 021, 120
-  }
-  {
-    c4<T> mJ01 = J01;
-    cscale(mJ01, T(-1));
-    c4<T> F = vvv(e1, J02, -k1, -(k0 + k2));
-    cadd(F, vvv(mJ01, e2, -(k0 + k1), -k2));
-    cscale(F, c3);
-    caxpy(F, cx<T>{c4g, T(0)}, vvvv_ordered(e1, e0, e2));
-    a[2] = a[4] = spdot(row_slash(ub, F), vb);  // 102, 201
-  }
-  // orderings grouped by the gluon next to the top: U(x), then U(x y) = U(x) e_y + ubar J(xy)
-  {  // x = 0: orderings 012 (a0), 021 (a1)
-    c4<T> U = row_prop(row_slash(ub, e0), kt + k0, mt);
-    cscale(U, -g * K.iq[1]);
-    const cx<T> t = spdot(row_slash(U, J12), vb);
-    a[0] = a[0] + t;
-    a[1] = a[1] - t;
-    c4<T> r = row_slash(U, e1);
-    cadd(r, row_slash(ub, J01));
-    c4<T> W = row_prop(r, kt + k0 + k1, mt);
-    cscale(W, -g * K.iq[3]);
-    a[0] = a[0] + spdot(row_slash(W, e2), vb);
-    r = row_slash(U, e2);
-    cadd(r, row_slash(ub, J02));
-    W = row_prop(r, kt + k0 + k2, mt);
-    cscale(W, -g * K.iq[5]);
-    a[1] = a[1] + spdot(row_slash(W, e1), vb);
-  }
-  {  // x = 1: orderings 102 (a2), 120 (a3)
-    c4<T> U = row_prop(row_slash(ub, e1), kt + k1, mt);
-    cscale(U, -g * K.iq[2]);
-    const cx<T> t = spdot(row_slash(U, J02), vb);
-    a[2] = a[2] + t;
-    a[3] = a[3] - t;
-    c4<T> r = row_slash(U, e0);
-    c4<T> b = row_slash(ub, J01);
-    cscale(b, T(-1));
-    cadd(r, b);
-    c4<T> W = row_prop(r, kt + k0 + k1, mt);
-    cscale(W, -g * K.iq[3]);
-    a[2] = a[2] + spdot(row_slash(W, e2), vb);
-    r = row_slash(U, e2);
-    cadd(r, row_slash(ub, J12));
-    W = row_prop(r, kt + k1 + k2, mt);
-    cscale(W, -g * K.iq[6]);
-    a[3] = a[3] + spdot(row_slash(W, e0), vb);
-  }
-  {  // x = 2: orderings 201 (a4), 210 (a5)
-    c4<T> U = row_prop(row_slash(ub, e2), kt + k2, mt);
-    cscale(U, -g * K.iq[4]);
-    const cx<T> t = spdot(row_slash(U, J01), vb);
-    a[4] = a[4] + t;
-    a[5] = a[5] - t;
-    c4<T> r = row_slash(U, e0);
-    c4<T> b = row_slash(ub, J02);
-    cscale(b, T(-1));
-    cadd(r, b);
-    c4<T> W = row_prop(r, kt + k0 + k2, mt);
-    cscale(W, -g * K.iq[5]);
-    a[4] = a[4] + spdot(row_slash(W, e1), vb);
-    r = row_slash(U, e1);
-    b = row_slash(ub, J12);
-    cscale(b, T(-1));
-    cadd(r, b);
-    W = row_prop(r, kt + k1 + k2, mt);
-    cscale(W, -g * K.iq[6]);
-    a[5] = a[5] + spdot(row_slash(W, e0), vb);
-  }
-#pragma unroll
-  for (int f = 0; f < 6; ++f) A[f] = times_i(a[f]) * g;
 }
 
 // ----------------------------------------------------------------------------
@@ -578,43 +362,6 @@ ME_HD T ee_uug_block(const KinEE<T>& K, int b) {
   return T(512.0 / 9.0) * K.is * ((x * K.n1) * (x * K.n2) + (y * K.n1) * (y * K.n2));
 }
 
-template <typename T>
-ME_HD c4<T> lepton_current(const KinEE<T>& K, int hel, const Couplings& cp) {
-  // vbar(e+) gamma^mu u(e-) with the photon propagator: (e Q_e / s) vbar gamma u
-  c4<T> vb = dbar(spinor_v(K.pl[0], T(0), hel_of(hel, 0)));
-  c4<T> u = spinor_u(K.pl[1], T(0), hel_of(hel, 1));
-  c4<T> L = vcurrent(vb, u);
-  cscale(L, -ee_of<T>(cp) * K.is);
-  return L;
-}
-
-template <typename T>
-ME_HD void amp_ee_uu(const KinEE<T>& K, int hel, const Couplings& cp, cx<T>* A) {
-  c4<T> L = lepton_current<T>(K, hel, cp);
-  c4<T> ub = dbar(spinor_u(K.pl[2], T(0), hel_of(hel, 2)));
-  c4<T> v = spinor_v(K.pl[3], T(0), hel_of(hel, 3));
-  const T equ = (T)(cp.ee * (2.0 / 3.0));
-  A[0] = times_i(spdot(row_slash(ub, L), v)) * equ;
-}
-
-template <typename T>
-ME_HD void amp_ee_uug(const KinEE<T>& K, int hel, const Couplings& cp, cx<T>* A) {
-  c4<T> L = lepton_current<T>(K, hel, cp);
-  c4<T> ub = dbar(spinor_u(K.pl[2], T(0), hel_of(hel, 2)));
-  c4<T> v = spinor_v(K.pl[3], T(0), hel_of(hel, 3));
-  c4<T> eps = polvec(K.pl[4], hel_of(hel, 4), true);
-  const T g = gs_of<T>(cp);
-  const T equ = (T)(cp.ee * (2.0 / 3.0));
-  // gluon on the quark side: ubar (i g eps) i(Q1slash)/Q1^2, Q1 = p_u + p_g
-  c4<T> u1 = row_prop(row_slash(ub, eps), K.pl[2] + K.pl[4], T(0));
-  cscale(u1, -g * K.i1);
-  // gluon on the antiquark side: i(-Q2slash)/Q2^2 (i g eps) v, Q2 = p_ubar + p_g
-  c4<T> v1 = col_prop(K.pl[3] + K.pl[4], T(0), slash_col(eps, v));
-  cscale(v1, -g * K.i2);
-  cx<T> a = spdot(row_slash(u1, L), v) + spdot(row_slash(ub, L), v1);
-  A[0] = times_i(a) * equ;
-}
-
 // ----------------------------------------------------------------------------
 // u(0) ubar(1) -> t(2) tbar(3) [g(4)].  Colour basis (i=t, j=tbar, k=u, l=ubar):
 //   Born: e1 = d_ik d_lj, e2 = d_ij d_lk;  (T^b)_ij (T^b)_lk = (e1 - e2/N)/2.
@@ -755,69 +502,6 @@ ME_HD void amp_uu_block(const KinUU<T>& K, int hb, const Couplings& cp, F&& cons
   }
 }
 
-template <typename T>
-ME_HD c4<T> light_current(const c4<T>& vbar_ub, const c4<T>& u_u, T inv, T g) {
-  // (g/Q^2) vbar gamma u  (vertex i g gamma, propagator -i/Q^2)
-  c4<T> J = vcurrent(vbar_ub, u_u);
-  cscale(J, g * inv);
-  return J;
-}
-
-template <typename T>
-ME_HD void amp_uu_tt(const KinUU<T>& K, int hel, const Couplings& cp, cx<T>* A) {
-  const T g = gs_of<T>(cp), mt = mt_of<T>(cp);
-  c4<T> uu = spinor_u(K.pl[0], T(0), hel_of(hel, 0));
-  c4<T> vbu = dbar(spinor_v(K.pl[1], T(0), hel_of(hel, 1)));
-  c4<T> ub = dbar(spinor_u(K.pl[2], mt, hel_of(hel, 2)));
-  c4<T> vt = spinor_v(K.pl[3], mt, hel_of(hel, 3));
-  c4<T> Ju = light_current(vbu, uu, K.is, g);
-  cx<T> d = times_i(spdot(row_slash(ub, Ju), vt)) * g;
-  A[0] = d * T(0.5);
-  A[1] = d * (T)(-1.0 / 6.0);
-}
-
-template <typename T>
-ME_HD void amp_uu_ttg(const KinUU<T>& K, int hel, const Couplings& cp, cx<T>* A) {
-  const T g = gs_of<T>(cp), mt = mt_of<T>(cp);
-  c4<T> uu = spinor_u(K.pl[0], T(0), hel_of(hel, 0));
-  c4<T> vbu = dbar(spinor_v(K.pl[1], T(0), hel_of(hel, 1)));
-  c4<T> ub = dbar(spinor_u(K.pl[2], mt, hel_of(hel, 2)));
-  c4<T> vt = spinor_v(K.pl[3], mt, hel_of(hel, 3));
-  c4<T> eps = polvec(K.pl[4], hel_of(hel, 4), true);
-  const r4<T>* q = K.q;
-  // u-line current without emission
-  c4<T> Ju = light_current(vbu, uu, K.is, g);
-  // D1: gluon off the top: ubar (ig eps) S_F(q2+q4) (ig Ju) v
-  c4<T> r1 = row_prop(row_slash(ub, eps), q[2] + q[4], mt);
-  cscale(r1, -g * K.ia);
-  cx<T> D1 = times_i(spdot(row_slash(r1, Ju), vt)) * g;
-  // D2: gluon off the antitop: ubar (ig Ju) S_F(-(q3+q4)) (ig eps) v
-  c4<T> c1 = col_prop(q[3] + q[4], mt, slash_col(eps, vt));
-  cscale(c1, -g * K.ib);
-  cx<T> D2 = times_i(spdot(row_slash(ub, Ju), c1)) * g;
-  // D3: gluon off the incoming antiquark (row side of the light line)
-  c4<T> r3 = row_prop(row_slash(vbu, eps), q[1] + q[4], T(0));
-  cscale(r3, -g * K.ic);
-  c4<T> J3 = light_current(r3, uu, K.is3, g);
-  cx<T> D3 = times_i(spdot(row_slash(ub, J3), vt)) * g;
-  // D4: gluon off the incoming quark (column side)
-  c4<T> c4u = col_prop(q[0] + q[4], T(0), slash_col(eps, uu));
-  cscale(c4u, -g * K.id);
-  c4<T> J4 = light_current(vbu, c4u, K.is3, g);
-  cx<T> D4 = times_i(spdot(row_slash(ub, J4), vt)) * g;
-  // D5: three-gluon vertex joining the light current, the heavy current and the gluon
-  c4<T> Jt = vcurrent(ub, vt);
-  cscale(Jt, g * K.it);
-  c4<T> W = vvv(Ju, Jt, -(q[0] + q[1]), -(q[2] + q[3]));
-  cx<T> D5 = cdot(W, eps) * g;
-  const T h = T(0.5), hn = (T)(-1.0 / 6.0);
-  cx<T> iD5 = times_i(D5);
-  A[0] = (D1 + D4) * h - iD5 * h;
-  A[1] = (D2 + D3) * h + iD5 * h;
-  A[2] = (D1 + D2) * hn;
-  A[3] = (D3 + D4) * hn;
-}
-
 // ----------------------------------------------------------------------------
 template <int PID, typename T> struct KinOf;
 template <typename T> struct KinOf<P_EE_UU, T> { using type = KinEE<T>; };
@@ -839,18 +523,6 @@ ME_HD Kin<PID, T> prepare(const r4<double>* p, const Couplings& cp) {
   else if constexpr (PID == P_GG_TTGG) return prep_tt<T, 4>(p, cp);
   else if constexpr (PID == P_UU_TT) return prep_uu<T, 4>(p, cp);
   else return prep_uu<T, 5>(p, cp);
-}
-
-// partial amplitudes of one helicity
-template <int PID, typename T>
-ME_HD void amplitude(const Kin<PID, T>& K, int hel, const Couplings& cp, cx<T>* A) {
-  if constexpr (PID == P_EE_UU) amp_ee_uu<T>(K, hel, cp, A);
-  else if constexpr (PID == P_EE_UUG) amp_ee_uug<T>(K, hel, cp, A);
-  else if constexpr (PID == P_GG_TT) amp_tt2_fast<T>(K, hel, cp, A);
-  else if constexpr (PID == P_GG_TTG) amp_tt3_fast<T>(K, hel, cp, A);
-  else if constexpr (PID == P_GG_TTGG) amp_ttng<T, 4>(K, hel, cp, A);
-  else if constexpr (PID == P_UU_TT) amp_uu_tt<T>(K, hel, cp, A);
-  else amp_uu_ttg<T>(K, hel, cp, A);
 }
 
 // The four gluons of a block: beam gluons of type E0, E1 (pol or axpol), outgoing ones pol.  The
@@ -1161,27 +833,14 @@ template <int PID> __host__ __device__ constexpr int n_live_blocks() {
 }
 template <int PID> ME_HD int live_block_hel(int i) { return block_hel(massless_initial_pair<PID>() ? 2 * i : i); }
 
-// partial amplitudes of the four helicities hb | (r << 2) (see amp_tt2_block), of g g -> t tbar g
-// those whose top spin r & 1 is among `spins`; processes
-// without a block routine evaluate them one at a time
+// Partial amplitudes of the four helicities hb | (r << 2), of g g -> t tbar g those whose top spin
+// r & 1 is among `spins`.  (e+e- -> u ubar g has ee_uug_block, the 2 -> 2 processes closed_sum.)
 template <int PID, typename T, class F>
 ME_HD void amplitude_block(const Kin<PID, T>& K, int hb, const Couplings& cp, F&& consume, unsigned spins = 3u) {
-  if constexpr (PID == P_GG_TTG) {
-    amp_tt3_block<T>(K, hb, cp, spins, consume);
-  } else if constexpr (PID == P_GG_TTGG) {
-    amp_tt4_block<T>(K, hb, cp, consume);
-  } else if constexpr (PID == P_UU_TTG) {
-    amp_uu_block<T>(K, hb, cp, consume);
-  } else {
-    for (int r = 0; r < 4; ++r) {
-      if constexpr (PID == P_EE_UU || PID == P_EE_UUG) {
-        if (r == 0 || r == 3) continue;  // u, ubar with equal helicities: zero
-      }
-      cx<T> A[Proc<PID>::NFLOW];
-      amplitude<PID, T>(K, hb | (r << 2), cp, A);
-      consume(r, A);
-    }
-  }
+  static_assert(PID == P_GG_TTG || PID == P_GG_TTGG || PID == P_UU_TTG, "processes with block routines");
+  if constexpr (PID == P_GG_TTG) amp_tt3_block<T>(K, hb, cp, spins, consume);
+  else if constexpr (PID == P_GG_TTGG) amp_tt4_block<T>(K, hb, cp, consume);
+  else amp_uu_block<T>(K, hb, cp, consume);
 }
 
 // ----------------------------------------------------------------------------
