@@ -665,8 +665,10 @@ __device__ __forceinline__ bool has_direction(const r4<double>& p) {
 //    the same number, and its Born depends on the cosine of the partner to the beam alone.
 // Close to a collinear limit the last bits of a weight are those of 1 - y_j = d_j as formed
 // here, which the eikonal denominators p_j.q carry again, rounded differently; where the two
-// meet, their ratio is kept as it comes out, in float64 results also the beams' own eikonal
-// terms (p^2 = 0 up to rounding) and the final state's eikonal factor.
+// meet, their ratio is kept as it comes out.  A float64 handle also keeps the beams' own eikonal
+// terms (p^2 = 0 up to rounding) and the final state's eikonal factor (1 up to rounding): its weights
+// serve as the reference for others and are held, to 1e-12 where the inputs fix them, to a
+// term-by-term evaluation in float64, which carries these factors.  A mixed handle leaves them out.
 template <int PID, typename T>
 __device__ __forceinline__ PointTerms point_terms(const r4<double>* k, const KParams& kp) {
   constexpr bool F64 = !std::is_same<T, float>::value;

@@ -352,8 +352,8 @@ ME_HD KinEE<T> prep_ee(const r4<double>* p) {
 // momenta, and a numerator that goes like the angle, formed from the spinors: where the gluon
 // is nearly collinear the two round differently.  In float64 the block keeps that form,
 // |<24>|^2 / (2 p2.p4)^2 for 1 / (2 p2.p4), so that it stays the float64 value of the
-// amplitude; float32 takes the closed form as it is (99 % of the errors within 2.0e-7 instead
-// of 6.9e-7).  65,536 subtracted points: 286 us with the helicity amplitudes, 187 us here.
+// amplitude, to which float64 results are held where their inputs fix them; float32 takes the
+// closed form as it is (99 % of the errors within 2.1e-7 instead of 6.9e-7).  65,536 subtracted points: 286 us with the helicity amplitudes, 187 us here.
 // The products with 1 / (2 p2.p4) and 1 / (2 p3.p4) come first, as ratios without a dimension:
 // the three reciprocal invariants alone, of order s^-3, would leave float32 from sqrt(s) = 1e7 on.
 template <typename T>
