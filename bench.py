@@ -47,12 +47,12 @@ FP64_PER_SM_CLK = 2  # DFMA thread-ops per SM per clock (ncu: ..._op_dfma_pred_o
 # DRAM bytes per launch (dram__bytes_read.sum + dram__bytes_write.sum) from one ncu
 # capture of each kernel (summaries in profiles/), with the hash of the kernel sources they
 # were taken on; reported only while the sources still hash the same.
-KERNEL_SOURCES_SHA = "ed3b884972d024c9"
+KERNEL_SOURCES_SHA = "176f70cf4be9ce6e"
 TRAFFIC = {
     # DRAM bytes per launch from one ncu capture of each kernel (the profile named), and the
     # points of that launch; traffic_per_launch scales them to the launch measured
-    ("c1", "main"): {"bytes": 100676096 + 3108608, "points": 1 << 20, "profile": "profiles/cases_ncu.md"},
-    ("c3", "main"): {"bytes": 52536832 + 835584, "points": 1 << 18, "profile": "profiles/cases_ncu.md"},
+    ("c1", "main"): {"bytes": 100674560 + 3044096, "points": 1 << 20, "profile": "profiles/cases_ncu.md"},
+    ("c3", "main"): {"bytes": 52537088 + 800512, "points": 1 << 18, "profile": "profiles/cases_ncu.md"},
 }
 
 

@@ -230,11 +230,11 @@ int me_last_rescued(me_handle* h, int64_t* n_rescued);
  * configurations, soft and collinear separately.  Synchronises the handle's stream. */
 int me_last_rescue_work(me_handle* h, int64_t* points, int64_t* real_blocks, int64_t* born_sets);
 
-/* The float64 Born configurations of the last mixed-precision me_eval_real_subtracted
- * call that ran the per-term queues (Sec. 4.3), by kind: set0 = soft counter-events
- * (initial state) or sector-1 Borns (final state), set1 = collinear counter-events or
- * sector-2 Borns.  Both 0 after a call that ran the masked evaluation.  Synchronises
- * the handle's stream. */
+/* The active Born configurations of the points that the last mixed-precision
+ * me_eval_real_subtracted call flagged, if it ran the per-term queues (Sec. 4.3), by kind:
+ * set0 = soft counter-events (initial state) or sector-1 Borns (final state), set1 =
+ * collinear counter-events or sector-2 Borns.  (They are float64 at every point.)  Both 0
+ * after a call that ran the masked evaluation.  Synchronises the handle's stream. */
 int me_last_rescue_configs(me_handle* h, int64_t* set0, int64_t* set1);
 
 /* Monte-Carlo accumulators of all outputs since creation or the last set:

@@ -250,15 +250,16 @@ class Handle:
         return v.value
 
     def last_rescue_work(self) -> tuple[int, int, int]:
-        """(flagged points, real blocks, Born-value sets) re-evaluated in float64 by the
-        last subtracted-real call (item rescue)."""
+        """Float64 work of the last subtracted-real call (item rescue): flagged points, real
+        blocks re-evaluated, and counterterm Born sets of the flagged points (float64 at every
+        point)."""
         v = [ctypes.c_int64() for _ in range(3)]
         _check(self.lib.me_last_rescue_work(self.h, *(ctypes.byref(x) for x in v)))
         return tuple(x.value for x in v)
 
     def last_rescue_configs(self) -> tuple[int, int]:
-        """Float64 Born configurations of the last subtracted-real call that ran the
-        per-term queues: (soft or sector-1, collinear or sector-2)."""
+        """Active Born configurations of the flagged points, of the last subtracted-real call that
+        ran the per-term queues: (soft or sector-1, collinear or sector-2)."""
         v = [ctypes.c_int64() for _ in range(2)]
         _check(self.lib.me_last_rescue_configs(self.h, *(ctypes.byref(x) for x in v)))
         return tuple(x.value for x in v)
